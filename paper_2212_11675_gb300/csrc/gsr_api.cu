@@ -122,8 +122,9 @@ static void release(gsr_handle_t *h)
         cudaGraphExecDestroy(h->cg_exec);
     if (h->cg64_exec)
         cudaGraphExecDestroy(h->cg64_exec);
-    if (h->b_exec)
-        cudaGraphExecDestroy(h->b_exec);
+    for (cudaGraphExec_t g : h->b_exec)
+        if (g)
+            cudaGraphExecDestroy(g);
     if (h->h_bs)
         cudaFreeHost(h->h_bs);
     if (h->h_bargs)
@@ -147,7 +148,7 @@ static void release(gsr_handle_t *h)
                    h->d_xp64, h->d_q64, h->d_iseg, h->d_cseg, h->d_cseg32, h->d_irow, h->d_ival32, h->d_ival, h->d_ipart, h->d_gpart, h->d_a2ctr, h->d_bX32, h->d_bQ32,
                    h->d_bC, h->d_bS_, h->d_bD, h->d_bZ, h->d_bT, h->d_bS, h->d_bXcm,
                    h->d_bCcm, h->d_bB, h->d_bnorms, h->d_bpartial, h->d_bcounter, h->d_bs,
-                   h->d_bipart,
+                   h->d_bipart, h->d_bticket,
                    h->d_bargs};
     for (void *p : dev)
         if (p)
@@ -1056,6 +1057,15 @@ extern "C" int gsr_lsq_backward(void *hv, const double *b, const double *x, cons
     return GSR_OK;
 }
 
+static void drop_batched_graphs(gsr_handle_t *h)
+{
+    for (cudaGraphExec_t &g : h->b_exec)
+        if (g) {
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+}
+
 // buffers of the batched solve for k columns (leading dimension rounded up
 // to 8 so that the column-tile loads are aligned) and its inner graph
 static int ensure_batched(gsr_handle_t *h, int k)
@@ -1063,12 +1073,17 @@ static int ensure_batched(gsr_handle_t *h, int k)
     const SysView &A = h->sys;
     const int ldk = (k + 7) / 8 * 8;
     if (ldk > h->bk) {
-        void *old[] = {h->d_bX32, h->d_bQ32, h->d_bC, h->d_bS_, h->d_bD, h->d_bZ, h->d_bT};
-        for (void *p : old)
-            if (p)
-                cudaFree(p);
-        h->d_bX32 = nullptr; h->d_bQ32 = nullptr; h->d_bC = nullptr; h->d_bS_ = nullptr;
-        h->d_bD = nullptr; h->d_bZ = nullptr; h->d_bT = nullptr;
+        drop_batched_graphs(h);  // they hold the old buffers
+        void **old[] = {(void **)&h->d_bX32, (void **)&h->d_bQ32, (void **)&h->d_bC,
+                        (void **)&h->d_bS_, (void **)&h->d_bD, (void **)&h->d_bZ,
+                        (void **)&h->d_bT, (void **)&h->d_bS, (void **)&h->d_bipart,
+                        (void **)&h->d_bticket};
+        for (void **p : old) {
+            if (*p)
+                cudaFree(*p);
+            *p = nullptr;
+        }
+        h->bk = 0;
         TRY(dalloc(h, &h->d_bX32, A.n * ldk));
         TRY(dalloc(h, &h->d_bQ32, A.m * ldk));
         TRY(dalloc(h, &h->d_bC, A.n * ldk));
@@ -1076,28 +1091,33 @@ static int ensure_batched(gsr_handle_t *h, int k)
         TRY(dalloc(h, &h->d_bD, A.n * ldk));
         TRY(dalloc(h, &h->d_bZ, A.n * ldk));
         TRY(dalloc(h, &h->d_bT, A.n * ldk));
+        TRY(dalloc(h, &h->d_bS, A.nseg * kNAtt * batched_att_pieces(h) * ldk));
+        TRY(dalloc(h, &h->d_bipart, A.I * batched_instr_pieces(h) * ldk));
+        TRY(dalloc(h, &h->d_bticket, A.I * ldk));
+        // on the legacy stream, before the caller's: waited for below
+        CK(cudaMemset(h->d_bticket, 0, A.I * ldk * sizeof(unsigned)));
+        CK(cudaStreamSynchronize(cudaStreamLegacy));
         h->bk = ldk;
     }
-    if (!h->d_bS) {
-        TRY(dalloc(h, &h->d_bS, A.nseg * kNAtt * 8));
-        TRY(dalloc(h, &h->d_bipart, A.I * 4 * 8));
-        TRY(dalloc(h, &h->d_bpartial, (int64_t)8 * kMaxPartials));
-        TRY(dalloc(h, &h->d_bcounter, 1));
+    if (!h->d_bpartial) {
+        TRY(dalloc(h, &h->d_bcounter, kMaxBatch));
         TRY(dalloc(h, &h->d_bs, 1));
         TRY(dalloc(h, &h->d_bargs, 1));
         TRY(dalloc(h, &h->d_bnorms, 2 * kMaxBatch));
-        CK(cudaMemset(h->d_bcounter, 0, sizeof(unsigned)));
+        CK(cudaMemset(h->d_bcounter, 0, kMaxBatch * sizeof(unsigned)));
+        CK(cudaStreamSynchronize(cudaStreamLegacy));
         CK(cudaMallocHost((void **)&h->h_bs, sizeof(BatchState)));
         CK(cudaMallocHost((void **)&h->h_bargs, sizeof(BatchArgs)));
         CK(cudaMallocHost((void **)&h->h_bnorms, 2 * kMaxBatch * sizeof(double)));
-        h->grid_b1 = batched_grid_rows(h);
-        h->grid_b2 = batched_grid_stars(h);
-        if (h->grid_b1 <= 0 || h->grid_b2 <= 0)
-            return cuda_fail(cudaGetLastError(), "batched occupancy");
+        TRY(dalloc(h, &h->d_bpartial, (int64_t)kMaxBatch * kMaxPartials));
     }
-    if (!h->b_exec || h->b_graph_k != h->bk || h->b_graph_kt != h->b_kt ||
-        h->b_graph_lanes != h->b_lanes) {
-        cudaError_t e = build_batched_graph(h, h->bk);
+    if (h->b_graph_kt != h->b_kt || h->b_graph_lanes != h->b_lanes) {
+        drop_batched_graphs(h);
+        h->b_graph_kt = h->b_kt;
+        h->b_graph_lanes = h->b_lanes;
+    }
+    if (!h->b_exec[k]) {
+        cudaError_t e = build_batched_graph(h, k);
         if (e != cudaSuccess)
             return cuda_fail(e, "build_batched_graph");
     }
@@ -1257,7 +1277,7 @@ extern "C" int gsr_batched_products(void *hv, int k, const double *X, const doub
     }
     cudaError_t e = cudaMemsetAsync(h->d_bC, 0, A.n * h->bk * sizeof(double), st);
     if (e == cudaSuccess)
-        e = launch_b_products(h, h->bk, h->d_bX32, Q32, Y32, h->d_bC, st);
+        e = launch_b_products(h, k, h->d_bX32, Q32, Y32, h->d_bC, st);
     if (e == cudaSuccess)
         e = launch_b_layout(h, 0, (const double *)Q32, Q, 2, A.m, k, st);
     if (e == cudaSuccess)
@@ -1341,7 +1361,7 @@ extern "C" int gsr_batched_solve(void *hv, int k, const double *B, int max_outer
         // inner solve of all columns (converged ones have a tiny right-hand side)
         CK(cudaMemsetAsync(h->d_bC, 0, A.n * h->bk * sizeof(double), st));
         CK(launch_b_layout(h, 1, h->d_bCcm, h->d_bC, 0, A.n, k, st));
-        CK(run_batched_inner(h, h->bk, max_inner, st));
+        CK(run_batched_inner(h, k, max_inner, st));
         CK(launch_b_update_x(h, h->d_bXcm, k, st));
         CK(cudaMemcpyAsync(h->h_bs, h->d_bs, sizeof(BatchState), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));

@@ -31,7 +31,33 @@
 
 namespace gsr {
 
-constexpr int kInstrSplit = 4;  // warps per instrument in the batched instrumental pass
+// Streams and events that fork the passes of aprod 2 while the inner loop is
+// captured; they are released with the object, the graph keeps the branches.
+struct BatchSide {
+    cudaStream_t s[2] = {nullptr, nullptr};
+    cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+    cudaError_t make()
+    {
+        cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        for (int i = 0; i < 2 && e == cudaSuccess; i++) {
+            e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
+            if (e == cudaSuccess)
+                e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
+        }
+        return e;
+    }
+    ~BatchSide()
+    {
+        if (fork)
+            cudaEventDestroy(fork);
+        for (int i = 0; i < 2; i++) {
+            if (join[i])
+                cudaEventDestroy(join[i]);
+            if (s[i])
+                cudaStreamDestroy(s[i]);
+        }
+    }
+};
 
 constexpr int kPanel = 8;  // columns per panel of the dense blocks
 
@@ -41,100 +67,143 @@ __host__ __device__ __forceinline__ int64_t pidx(int64_t r, int64_t rows, int c)
     return ((int64_t)(c / kPanel) * rows + r) * kPanel + (c % kPanel);
 }
 
-__device__ __forceinline__ uint32_t instr_b(const uint4 &rc, int j)
-{
-    const uint32_t w = (j < 2) ? rc.y : ((j < 4) ? rc.z : rc.w);
-    return (j & 1) ? (w >> 16) : (w & 0xffffu);
-}
-
+// KT consecutive columns of one row as packed pairs (one scalar for KT = 1)
 template <int KT>
-__device__ __forceinline__ void load_cols(const float *__restrict__ p, float (&v)[KT])
+struct Cols {
+    typedef f32x2 V;
+    static constexpr int N = KT / 2;
+};
+template <>
+struct Cols<1> {
+    typedef float V;
+    static constexpr int N = 1;
+};
+
+__device__ __forceinline__ void v_bcast(float &d, float a) { d = a; }
+__device__ __forceinline__ void v_bcast(f32x2 &d, float a) { d = pack2(a, a); }
+
+// The KT = 8 row is one aligned 32-byte sector, fetched by one 256-bit load:
+// random rows arrive at 0.93 per clock and SM from L2 (1.6 from L1) against
+// 0.56 with two 128-bit loads.
+template <int KT>
+__device__ __forceinline__ void load_cols(const float *__restrict__ p,
+                                          typename Cols<KT>::V (&v)[Cols<KT>::N])
 {
     if constexpr (KT == 8) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+            : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
     } else if constexpr (KT == 4) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "l"(p));
     } else if constexpr (KT == 2) {
-        const float2 a = __ldg(reinterpret_cast<const float2 *>(p));
-        v[0] = a.x; v[1] = a.y;
+        asm("ld.global.nc.b64 %0, [%1];" : "=l"(v[0]) : "l"(p));
     } else {
         v[0] = __ldg(p);
     }
 }
 
-// grid reduction of KT per-column sums into bs->sums[c0 .. c0+KT)
 template <int KT>
-__device__ __forceinline__ bool grid_reduce_cols(double (&v)[KT], double *partial, unsigned *counter)
+__device__ __forceinline__ void store_cols(float *p, const typename Cols<KT>::V (&v)[Cols<KT>::N])
 {
-    return grid_reduce<KT>(v, partial, counter);
+    if constexpr (KT == 1) {
+        *p = v[0];
+    } else if constexpr (KT == 2) {
+        *reinterpret_cast<f32x2 *>(p) = v[0];
+    } else {
+        ulonglong2 *d = reinterpret_cast<ulonglong2 *>(p);
+#pragma unroll
+        for (int i = 0; i < Cols<KT>::N / 2; i++)
+            d[i] = make_ulonglong2(v[2 * i], v[2 * i + 1]);
+    }
 }
+
+// column c (compile time) of a packed row
+template <int KT>
+__device__ __forceinline__ float col_of(const typename Cols<KT>::V (&v)[Cols<KT>::N], int c)
+{
+    if constexpr (KT == 1) {
+        return v[0];
+    } else {
+        float a, b;
+        unpack2(v[c / 2], a, b);
+        return (c & 1) ? b : a;
+    }
+}
+
+// Tiles of KT columns: every kernel below takes the tiles of one launch from
+// blockIdx.y (tile y: columns c_first + y KT ...).  Tiles are independent, so
+// one launch covers all of them: on a system too small to fill the chip with
+// one tile they run side by side, on a large one the blocks of a tile are
+// dispatched before those of the next and keep its panel in L2.
 
 // ---------------------------------------------------------------------------
 // aprod 1 on KT columns: Q32[:, c0+c] = fl32(A32 X32[:, c0+c]), with
-// |Q[:, c]|^2 and alpha_c = gamma_c / |Q[:, c]|^2 (0 for a finished column)
+// |Q[:, c]|^2 and alpha_c = gamma_c / |Q[:, c]|^2 (0 for a finished column).
+// Bound by the FP32 pipe (8 lane operations per product: 0.27 ms at 7.0e6
+// rows and 8 columns) and the gathers of 24 rows of X per matrix row.
 // ---------------------------------------------------------------------------
-// three blocks per SM: at four the 8-column tile spills (measured 3% slower)
 template <int KT>
 __global__ void __launch_bounds__(kThreads, 3)
-k_b_aprod1(SysView A, const float *__restrict__ X, float *__restrict__ Q, int c0,
+k_b_aprod1(SysView A, const float *__restrict__ X, float *__restrict__ Q, int c_first,
            BatchState *bs, double *partial, unsigned *counter)
 {
+    typedef typename Cols<KT>::V V;
+    constexpr int N = Cols<KT>::N;
+    const int c0 = c_first + blockIdx.y * KT;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t ntiles = (A.m + 31) >> 5;
-    float nh[KT], nl[KT];  // |Q[:, c]|^2 of this thread (double-float)
+    const float *Xp = X + pidx(0, A.n, c0);  // row j of the panel at Xp + 8 j
+    V nh[N], nl[N];                          // |Q[:, c]|^2 of this thread (double-float)
 #pragma unroll
-    for (int c = 0; c < KT; c++)
-        nh[c] = nl[c] = 0.f;
+    for (int c = 0; c < N; c++)
+        nh[c] = nl[c] = V(0);
     for (int64_t t = warp; t < ntiles; t += nwarps) {
         const int64_t r = (t << 5) + lane;
         if (r >= A.m)
             continue;
         const uint32_t s = star_of_row(A, t, r);
         const uint4 rc = __ldcs(A.rec + r);
-        float h[KT], l[KT];
+        V h[N], l[N];
 #pragma unroll
-        for (int c = 0; c < KT; c++)
-            h[c] = l[c] = 0.f;
+        for (int c = 0; c < N; c++)
+            h[c] = l[c] = V(0);
         const float *v = A.val32 + tidx<kNPar>(0, r);  // plane k at v + 32 k
+        const float *xs = Xp + (int64_t)kPanel * kNAstro * s;
+        const float *xa = Xp + kPanel * (A.att0 + rc.x);
 #pragma unroll
         for (int k = 0; k < kNPar; k++) {
-            int64_t col;
+            const float *xr;
             if (k < kNAstro)
-                col = (int64_t)kNAstro * s + k;
+                xr = xs + kPanel * k;
             else if (k < kNAstro + kNAtt)
-                col = A.att0 + ((k - kNAstro) >> 2) * A.D + rc.x + ((k - kNAstro) & 3);
+                xr = xa + kPanel * (((k - kNAstro) >> 2) * A.D + ((k - kNAstro) & 3));
             else if (k < kNPar - 1)
-                col = A.ins0 + instr_b(rc, k - kNAstro - kNAtt);
+                xr = Xp + kPanel * (A.ins0 + instr_at32(rc, k - kNAstro - kNAtt));
             else
-                col = A.glb0;
-            const float a = __ldcs(v + 32 * k);
-            float xv[KT];
-            load_cols<KT>(X + pidx(col, A.n, c0), xv);
+                xr = Xp + kPanel * A.glb0;
+            V a, xv[N];
+            v_bcast(a, __ldcs(v + 32 * k));
+            load_cols<KT>(xr, xv);
 #pragma unroll
-            for (int c = 0; c < KT; c++)
-                df_acc(h[c], l[c], __fmul_rn(a, xv[c]));
+            for (int c = 0; c < N; c++)
+                df_acc_v(h[c], l[c], v_mul(a, xv[c]));
         }
-        float *q = Q + pidx(r, A.m, c0);
 #pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const float qv = __fadd_rn(h[c], l[c]);
-            q[c] = qv;
-            const float pq = __fmul_rn(qv, qv);  // q^2 = pq + fma(q, q, -pq) exactly
-            df_acc(nh[c], nl[c], pq);
-            nl[c] = __fadd_rn(nl[c], __fmaf_rn(qv, qv, -pq));
+        for (int c = 0; c < N; c++) {
+            h[c] = v_add(h[c], l[c]);  // the row's q
+            const V pq = v_mul(h[c], h[c]);  // q^2 = pq + fma(q, q, -pq) exactly
+            df_acc_v(nh[c], nl[c], pq);
+            nl[c] = v_add(nl[c], v_fma(h[c], h[c], v_neg(pq)));
         }
+        store_cols<KT>(Q + pidx(r, A.m, c0), h);
     }
     double nrm[KT];
 #pragma unroll
     for (int c = 0; c < KT; c++)
-        nrm[c] = df_to_d(nh[c], nl[c]);
-    if (grid_reduce_cols<KT>(nrm, partial, counter) && threadIdx.x == 0) {
+        nrm[c] = df_to_d(col_of<KT>(nh, c), col_of<KT>(nl, c));
+    if (grid_reduce<KT>(nrm, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
+        threadIdx.x == 0) {
 #pragma unroll
         for (int c = 0; c < KT; c++) {
             const int cc = c0 + c;
@@ -146,22 +215,26 @@ k_b_aprod1(SysView A, const float *__restrict__ X, float *__restrict__ Q, int c0
 
 // ---------------------------------------------------------------------------
 // aprod 2, astrometric and global nonzeros on KT columns (star-parallel):
-// T[astro rows] written, T[global] accumulated into zeroed memory
+// T[astro rows] and T[global] written (the global sums block by block in
+// block order: deterministic)
 // ---------------------------------------------------------------------------
 template <int KT, int G>
 __global__ void __launch_bounds__(kThreads)
-k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c0)
+k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_first,
+          double *partial, unsigned *counter)
 {
-    __shared__ double s_g[kThreads / 32][KT];
+    typedef typename Cols<KT>::V V;
+    constexpr int N = Cols<KT>::N;
     constexpr int GPW = 32 / G;
+    const int c0 = c_first + blockIdx.y * KT;
     const int lane = threadIdx.x & (G - 1);
     const int gw = (threadIdx.x & 31) / G;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    float gh[KT], gl[KT];
+    V gh[N], gl[N];
 #pragma unroll
-    for (int c = 0; c < KT; c++)
-        gh[c] = gl[c] = 0.f;
+    for (int c = 0; c < N; c++)
+        gh[c] = gl[c] = V(0);
     for (int64_t s0 = warp * GPW; s0 < A.S; s0 += nwarps * GPW) {
         const int64_t s = s0 + gw;
         uint32_t r0 = 0, r1 = 0;
@@ -169,83 +242,104 @@ k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c0
             r0 = A.star_ptr[s];
             r1 = A.star_ptr[s + 1];
         }
-        float ah[kNAstro][KT], al[kNAstro][KT];
+        V ah[kNAstro][N], al[kNAstro][N];
 #pragma unroll
         for (int k = 0; k < kNAstro; k++)
 #pragma unroll
-            for (int c = 0; c < KT; c++)
-                ah[k][c] = al[k][c] = 0.f;
+            for (int c = 0; c < N; c++)
+                ah[k][c] = al[k][c] = V(0);
         for (uint32_t r = r0 + lane; r < r1; r += G) {
             const float *v = A.val32 + tidx<kNPar>(0, r);
-            float yv[KT];
+            V yv[N];
             load_cols<KT>(Y + pidx(r, A.m, c0), yv);
 #pragma unroll
             for (int k = 0; k < kNAstro; k++) {
-                const float a = __ldcs(v + 32 * k);
+                V a;
+                v_bcast(a, __ldcs(v + 32 * k));
 #pragma unroll
-                for (int c = 0; c < KT; c++)
-                    df_acc(ah[k][c], al[k][c], __fmul_rn(a, yv[c]));
+                for (int c = 0; c < N; c++)
+                    df_acc_v(ah[k][c], al[k][c], v_mul(a, yv[c]));
             }
-            const float ag = __ldcs(v + 32 * 23);
+            V ag;
+            v_bcast(ag, __ldcs(v + 32 * 23));
 #pragma unroll
-            for (int c = 0; c < KT; c++)
-                df_acc(gh[c], gl[c], __fmul_rn(ag, yv[c]));
+            for (int c = 0; c < N; c++)
+                df_acc_v(gh[c], gl[c], v_mul(ag, yv[c]));
         }
         // the star's 5 KT sums over its G lanes: double-float reduce-scatter
-        // of the values padded to P (value v = k KT + c)
+        // of the values padded to P (value v = k KT + c), 32 at a time
         constexpr int NV = kNAstro * KT;
         constexpr int P = NV <= 8 ? 8 : (NV <= 16 ? 16 : 32);
-        float rh[P], rl[P];
 #pragma unroll
-        for (int v = 0; v < P; v++) {
-            rh[v] = v < NV ? ah[v / KT][v % KT] : 0.f;
-            rl[v] = v < NV ? al[v / KT][v % KT] : 0.f;
-        }
-        df_reduce_scatter<P, G>(rh, rl, lane);
-        constexpr int PER = P >= G ? P / G : 1;
+        for (int v0 = 0; v0 < NV; v0 += P) {
+            float rh[P], rl[P];
 #pragma unroll
-        for (int k = 0; k < PER; k++) {
-            const int v = P >= G ? lane * PER + k : lane / (G / P);
-            const bool owner = P >= G || (lane % (G / P)) == 0;
-            if (owner && v < NV && s < A.S)
-                T[pidx((int64_t)kNAstro * s + v / KT, A.n, c0) + v % KT] = df_to_d(rh[k], rl[k]);
+            for (int v = 0; v < P; v++) {
+                const int w = v0 + v;
+                rh[v] = w < NV ? col_of<KT>(ah[w < NV ? w / KT : 0], w % KT) : 0.f;
+                rl[v] = w < NV ? col_of<KT>(al[w < NV ? w / KT : 0], w % KT) : 0.f;
+            }
+            df_reduce_scatter<P, G>(rh, rl, lane);
+            constexpr int PER = P >= G ? P / G : 1;
+#pragma unroll
+            for (int k = 0; k < PER; k++) {
+                const int w = v0 + (P >= G ? lane * PER + k : lane / (G / P));
+                const bool owner = P >= G || (lane % (G / P)) == 0;
+                if (owner && w < NV && s < A.S)
+                    T[pidx((int64_t)kNAstro * s + w / KT, A.n, c0) + w % KT] =
+                        df_to_d(rh[k], rl[k]);
+            }
         }
     }
+    double g[KT];
 #pragma unroll
-    for (int c = 0; c < KT; c++) {
-        const double g = warp_sum(df_to_d(gh[c], gl[c]));
-        if ((threadIdx.x & 31) == 0)
-            s_g[threadIdx.x >> 5][c] = g;
-    }
-    __syncthreads();
-    if (threadIdx.x < KT) {
-        double t = 0.0;
-        for (int w = 0; w < kThreads / 32; w++)
-            t += s_g[w][threadIdx.x];
-        atomicAdd(T + pidx(A.glb0, A.n, c0) + threadIdx.x, t);
+    for (int c = 0; c < KT; c++)
+        g[c] = df_to_d(col_of<KT>(gh, c), col_of<KT>(gl, c));
+    if (grid_reduce<KT>(g, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
+        threadIdx.x == 0) {
+#pragma unroll
+        for (int c = 0; c < KT; c++)
+            T[pidx(A.glb0, A.n, c0) + c] = g[c];
     }
 }
 
 // ---------------------------------------------------------------------------
-// aprod 2, attitude nonzeros on KT columns: one warp per offset o and axis a
-// sums tap j of column c into S[((o * 3 + a) * 4 + j) * KT + c]
+// aprod 2, attitude nonzeros on KT columns: one warp per offset o, axis a and
+// piece q (np pieces of an offset's entries) sums tap j of column c into
+// S[((q nseg + o) 3 + a) 4 + j][c] of the tile's block
 // ---------------------------------------------------------------------------
 template <int KT>
 __global__ void __launch_bounds__(kThreads)
-k_b_att(SysView A, const float *__restrict__ Y, double *__restrict__ S, int c0)
+k_b_att(SysView A, const float *__restrict__ Y, double *__restrict__ Sall, int c_first, int np)
 {
+    typedef typename Cols<KT>::V V;
+    constexpr int N = Cols<KT>::N;
+    const int c0 = c_first + blockIdx.y * KT;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const float *Yp = Y + pidx(0, A.m, c0);
+    double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
     constexpr int NV = 4 * KT;  // sums per (offset, axis)
-    for (int64_t oa = warp; oa < A.nseg * 3; oa += nwarps) {
-        const int64_t o = oa / 3;
-        const int a = (int)(oa - o * 3);
-        const uint32_t e0 = A.seg[o], e1 = A.seg[o + 1];
-        float h[NV], l[NV];
+    const int64_t units = A.nseg * 3 * np;
+    for (int64_t w = warp; w < units; w += nwarps) {
+        // the axes of one (piece, offset) follow each other: their second and
+        // third readings of perm and of the rows of Y hit L2
+        const int64_t qo = w / 3;
+        const int a = (int)(w - qo * 3);
+        // pieces only where an offset has hundreds of entries: 32-bit counts
+        const uint32_t q = np == 1 ? 0u : (uint32_t)qo / (uint32_t)A.nseg;
+        const int64_t o = qo - q * A.nseg;
+        const uint32_t s0 = A.seg[o];
+        const uint64_t len = A.seg[o + 1] - s0;
+        const uint32_t e0 = s0 + (uint32_t)(len * q / np);
+        const uint32_t e1 = s0 + (uint32_t)(len * (q + 1) / np);
+        V h[4][N], l[4][N];
 #pragma unroll
-        for (int k = 0; k < NV; k++)
-            h[k] = l[k] = 0.f;
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int c = 0; c < N; c++)
+                h[j][c] = l[j][c] = V(0);
         // two entries per lane in flight (the row index, then the row of Y,
         // is a chain of two dependent loads); the sums take the entries in
         // the same order as one at a time
@@ -258,95 +352,126 @@ k_b_att(SysView A, const float *__restrict__ Y, double *__restrict__ S, int c0)
                 va[j] = __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e));
                 vb[j] = __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e + 32));
             }
-            float ya[KT], yb[KT];
-            load_cols<KT>(Y + pidx(ra, A.m, c0), ya);
-            load_cols<KT>(Y + pidx(rb, A.m, c0), yb);
-#pragma unroll
-            for (int j = 0; j < 4; j++)
-#pragma unroll
-                for (int c = 0; c < KT; c++)
-                    df_acc(h[j * KT + c], l[j * KT + c], __fmul_rn(va[j], ya[c]));
-#pragma unroll
-            for (int j = 0; j < 4; j++)
-#pragma unroll
-                for (int c = 0; c < KT; c++)
-                    df_acc(h[j * KT + c], l[j * KT + c], __fmul_rn(vb[j], yb[c]));
-        }
-        if (e < e1) {
-            float yv[KT];
-            load_cols<KT>(Y + pidx(__ldcs(A.perm + e), A.m, c0), yv);
+            V ya[N], yb[N];
+            load_cols<KT>(Yp + (int64_t)kPanel * ra, ya);
+            load_cols<KT>(Yp + (int64_t)kPanel * rb, yb);
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                const float v = __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e));
+                V av;
+                v_bcast(av, va[j]);
 #pragma unroll
-                for (int c = 0; c < KT; c++)
-                    df_acc(h[j * KT + c], l[j * KT + c], __fmul_rn(v, yv[c]));
+                for (int c = 0; c < N; c++)
+                    df_acc_v(h[j][c], l[j][c], v_mul(av, ya[c]));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                V av;
+                v_bcast(av, vb[j]);
+#pragma unroll
+                for (int c = 0; c < N; c++)
+                    df_acc_v(h[j][c], l[j][c], v_mul(av, yb[c]));
+            }
+        }
+        if (e < e1) {
+            V yv[N];
+            load_cols<KT>(Yp + (int64_t)kPanel * __ldcs(A.perm + e), yv);
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                V av;
+                v_bcast(av, __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e)));
+#pragma unroll
+                for (int c = 0; c < N; c++)
+                    df_acc_v(h[j][c], l[j][c], v_mul(av, yv[c]));
             }
         }
         // double-float reduce-scatter of the NV sums (a power of two <= 32)
         // over the warp: lane l ends with the total of index l / (32 / NV)
-        df_reduce_scatter<NV, 32>(h, l, lane);
+        float rh[NV], rl[NV];
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            rh[k] = col_of<KT>(h[k / KT], k % KT);
+            rl[k] = col_of<KT>(l[k / KT], k % KT);
+        }
+        df_reduce_scatter<NV, 32>(rh, rl, lane);
         constexpr int REST = 32 / NV;
         if ((lane % REST) == 0)
-            S[(o * 3 + a) * NV + lane / REST] = df_to_d(h[0], l[0]);
+            S[(qo * 3 + a) * NV + lane / REST] = df_to_d(rh[0], rl[0]);
     }
 }
 
-// attitude columns of T from S, column tile c0
+// attitude column colrow = a D + k of T, column c of the tile whose sums are S
 template <int KT>
-__global__ void k_b_att_combine(SysView A, const double *__restrict__ S, double *__restrict__ T,
-                                int c0)
+__device__ __forceinline__ double att_total(const SysView &A, const double *__restrict__ S,
+                                            int np, int64_t colrow, int c)
 {
+    const int64_t a = (colrow >= A.D) + (colrow >= 2 * A.D), k = colrow - a * A.D;
+    double t = 0.0;
+    for (int q = 0; q < np; q++) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int64_t o = k - j;
+            if (o >= 0 && o < A.nseg)
+                t += S[((((int64_t)q * A.nseg + o) * 3 + a) * 4 + j) * KT + c];
+        }
+    }
+    return t;
+}
+
+// attitude columns of T (products alone; the CG pass combines them itself)
+template <int KT>
+__global__ void k_b_att_combine(SysView A, const double *__restrict__ Sall, double *__restrict__ T,
+                                int c_first, int np)
+{
+    const int c0 = c_first + blockIdx.y * KT;
+    const double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
     const int64_t total = 3 * A.D * KT;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(i % KT);
         const int64_t colrow = i / KT;  // a * D + k
-        const int64_t a = colrow / A.D, k = colrow - a * A.D;
-        double t = 0.0;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int64_t o = k - j;
-            if (o >= 0 && o < A.nseg)
-                t += S[((o * 3 + a) * 4 + j) * KT + c];
-        }
-        T[pidx(A.att0 + colrow, A.n, c0) + c] = t;
+        T[pidx(A.att0 + colrow, A.n, c0) + c] = att_total<KT>(A, S, np, colrow, c);
     }
 }
 
 // ---------------------------------------------------------------------------
-// aprod 2, instrumental nonzeros on KT columns: one warp per instrument f
-// over its entries (row ibrow[e], value ibval32[e]) in the instrument-sorted
-// copy of the whole matrix
+// aprod 2, instrumental nonzeros on KT columns: one warp per piece q of
+// instrument f's entries (row irow[e], value ival[e]) in the
+// instrument-sorted copy of the whole matrix; the warp that finishes an
+// instrument's last piece (ticket) adds its np pieces in order into T
 // ---------------------------------------------------------------------------
 template <int KT>
 __global__ void __launch_bounds__(kThreads)
 k_b_instr(SysView A, const uint32_t *__restrict__ iseg, const uint32_t *__restrict__ irow,
-          const float *__restrict__ ival, const float *__restrict__ Y, double *__restrict__ part,
-          int c0)
+          const float *__restrict__ ival, const float *__restrict__ Y, double *__restrict__ part_all,
+          unsigned *__restrict__ ticket_all, double *__restrict__ T, int c_first, int np)
 {
-    // warp w takes chunk (w % kInstrSplit) of instrument w / kInstrSplit; two
-    // entries per lane are in flight to hide the dependent row -> Y gathers
+    typedef typename Cols<KT>::V V;
+    constexpr int N = Cols<KT>::N;
+    const int c0 = c_first + blockIdx.y * KT;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t wi = warp; wi < A.I * kInstrSplit; wi += nwarps) {
-        const int64_t f = wi / kInstrSplit;
-        const int q = (int)(wi - f * kInstrSplit);
-        const uint32_t s0 = iseg[f], s1 = iseg[f + 1];
-        const uint32_t len = s1 - s0;
-        const uint32_t e0 = s0 + (uint32_t)(((uint64_t)len * q) / kInstrSplit);
-        const uint32_t e1 = s0 + (uint32_t)(((uint64_t)len * (q + 1)) / kInstrSplit);
-        float h[KT], l[KT];
+    const float *Yp = Y + pidx(0, A.m, c0);
+    double *part = part_all + (int64_t)c0 * A.I * np;
+    unsigned *ticket = ticket_all + (int64_t)c0 * A.I;
+    for (uint32_t wi = (uint32_t)warp; wi < (uint32_t)A.I * np; wi += (uint32_t)nwarps) {
+        const uint32_t f = wi / np;
+        const uint32_t q = wi - f * np;
+        const uint32_t s0 = iseg[f];
+        const uint64_t len = iseg[f + 1] - s0;
+        const uint32_t e0 = s0 + (uint32_t)(len * q / np);
+        const uint32_t e1 = s0 + (uint32_t)(len * (q + 1) / np);
+        V h[N], l[N];
 #pragma unroll
-        for (int c = 0; c < KT; c++)
-            h[c] = l[c] = 0.f;
+        for (int c = 0; c < N; c++)
+            h[c] = l[c] = V(0);
         uint32_t e = e0 + lane;
-        // four entries per lane in flight, then pairs, then one (the sums
-        // take the entries in order either way)
+        // four entries per lane in flight (the gathers of Y depend on the row
+        // indices); the sums take the entries in order
         for (; e + 96 < e1; e += 128) {
             uint32_t r4[4];
-            float v4[4], y4[4][KT];
+            float v4[4];
+            V y4[4][N];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 r4[u] = __ldcs(irow + e + 32 * u);
@@ -354,143 +479,183 @@ k_b_instr(SysView A, const uint32_t *__restrict__ iseg, const uint32_t *__restri
             }
 #pragma unroll
             for (int u = 0; u < 4; u++)
-                load_cols<KT>(Y + pidx(r4[u], A.m, c0), y4[u]);
+                load_cols<KT>(Yp + (int64_t)kPanel * r4[u], y4[u]);
 #pragma unroll
-            for (int u = 0; u < 4; u++)
+            for (int u = 0; u < 4; u++) {
+                V a;
+                v_bcast(a, v4[u]);
 #pragma unroll
-                for (int c = 0; c < KT; c++)
-                    df_acc(h[c], l[c], __fmul_rn(v4[u], y4[u][c]));
-        }
-        for (; e + 32 < e1; e += 64) {
-            const uint32_t ra = __ldcs(irow + e), rb = __ldcs(irow + e + 32);
-            const float va = __ldcs(ival + e), vb = __ldcs(ival + e + 32);
-            float ya[KT], yb[KT];
-            load_cols<KT>(Y + pidx(ra, A.m, c0), ya);
-            load_cols<KT>(Y + pidx(rb, A.m, c0), yb);
-#pragma unroll
-            for (int c = 0; c < KT; c++) {
-                df_acc(h[c], l[c], __fmul_rn(va, ya[c]));
-                df_acc(h[c], l[c], __fmul_rn(vb, yb[c]));
+                for (int c = 0; c < N; c++)
+                    df_acc_v(h[c], l[c], v_mul(a, y4[u][c]));
             }
         }
-        if (e < e1) {
-            float yv[KT];
-            load_cols<KT>(Y + pidx(__ldcs(irow + e), A.m, c0), yv);
-            const float v = __ldcs(ival + e);
+        for (; e < e1; e += 32) {
+            V yv[N], a;
+            load_cols<KT>(Yp + (int64_t)kPanel * __ldcs(irow + e), yv);
+            v_bcast(a, __ldcs(ival + e));
 #pragma unroll
-            for (int c = 0; c < KT; c++)
-                df_acc(h[c], l[c], __fmul_rn(v, yv[c]));
+            for (int c = 0; c < N; c++)
+                df_acc_v(h[c], l[c], v_mul(a, yv[c]));
         }
+        float rh[KT], rl[KT];
 #pragma unroll
         for (int c = 0; c < KT; c++) {
-            df_warp_sum(h[c], l[c]);
-            if (lane == 0)
-                part[(f * kInstrSplit + q) * KT + c] = df_to_d(h[c], l[c]);
+            rh[c] = col_of<KT>(h, c);
+            rl[c] = col_of<KT>(l, c);
         }
+        // lane groups of 32 / KT lanes end with the total of one column
+        df_reduce_scatter<KT, 32>(rh, rl, lane);
+        constexpr int REST = 32 / KT;
+        const int c = lane / REST;
+        if ((lane % REST) == 0)
+            part[((int64_t)f * np + q) * KT + c] = df_to_d(rh[0], rl[0]);
+        __threadfence();
+        __syncwarp();
+        unsigned last = 0;
+        if (lane == 0)
+            last = atomicAdd(ticket + f, 1u) == (unsigned)np - 1;
+        if (!__shfl_sync(0xffffffffu, last, 0))
+            continue;
+        __threadfence();
+        // fixed order: lane (c, i) adds pieces i, i + REST, ..., then the lanes
+        double t = 0.0;
+        for (int k = lane % REST; k < np; k += REST)
+            t += __ldcg(part + ((int64_t)f * np + k) * KT + c);
+#pragma unroll
+        for (int off = REST / 2; off > 0; off >>= 1)
+            t += __shfl_xor_sync(0xffffffffu, t, off);
+        if ((lane % REST) == 0)
+            T[pidx(A.ins0 + f, A.n, c0) + c] = t;
+        if (lane == 0)
+            ticket[f] = 0u;
     }
 }
 
-// instrumental rows of T from the per-chunk partials (fixed order)
+// ---------------------------------------------------------------------------
+// batched CG vector kernels: n x k panelled FP64 blocks, per-column scalars.
+// Thread i takes entry (row i / KT, column i % KT) of its tile, so a warp
+// reads consecutive doubles and a thread keeps one column (one thread per row
+// and all its columns read 8-byte words 64 bytes apart and reduced 8 sums:
+// 88 against 58 us at n = 562,001 and 8 columns).
+// ---------------------------------------------------------------------------
+// sum over the grid of one value per thread, by column (thread t holds column
+// t % KT); true in the last block, whose threads 0 .. KT-1 hold the totals
 template <int KT>
-__global__ void k_b_instr_combine(SysView A, const double *__restrict__ part, double *__restrict__ T,
-                                  int c0)
+__device__ __forceinline__ bool grid_reduce_col(double &v, double *partial, unsigned *counter)
 {
-    const int64_t total = A.I * KT;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t f = i / KT;
-        const int c = (int)(i - f * KT);
+    constexpr int NW = kThreads / 32;
+    __shared__ double sh[NW][KT];
+    __shared__ bool am_last;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 16; off >= KT; off >>= 1)
+        v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane < KT)
+        sh[threadIdx.x >> 5][lane] = v;
+    __syncthreads();
+    if (threadIdx.x < KT) {
         double t = 0.0;
 #pragma unroll
-        for (int q = 0; q < kInstrSplit; q++)
-            t += part[(f * kInstrSplit + q) * KT + c];
-        T[pidx(A.ins0 + f, A.n, c0) + c] = t;
+        for (int w = 0; w < NW; w++)
+            t += sh[w][threadIdx.x];
+        partial[(int64_t)threadIdx.x * kMaxPartials + blockIdx.x] = t;
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        am_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!am_last)
+        return false;
+    __threadfence();
+    double t = 0.0;  // thread t: column t % KT, blocks t / KT, + kThreads / KT, ...
+    for (unsigned b = threadIdx.x / KT; b < gridDim.x; b += kThreads / KT)
+        t += __ldcg(partial + (int64_t)(threadIdx.x % KT) * kMaxPartials + b);
+#pragma unroll
+    for (int off = 16; off >= KT; off >>= 1)
+        t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (lane < KT)
+        sh[threadIdx.x >> 5][lane] = t;
+    __syncthreads();
+    if (threadIdx.x < KT) {
+        v = 0.0;
+#pragma unroll
+        for (int w = 0; w < NW; w++)
+            v += sh[w][threadIdx.x];
+    }
+    if (threadIdx.x == 0)
+        *counter = 0u;
+    return true;
 }
 
-// ---------------------------------------------------------------------------
-// batched CG vector kernels: n x k panelled FP64 blocks, per-column scalars
-// ---------------------------------------------------------------------------
-// S = p o C, Dd = S, Z = 0, X32 = fl32(p o Dd), gamma_c = |S_c|^2; zeroes the
-// global row of T.  One launch per column tile (c0, KT).
+// S = p o C, Dd = S, Z = 0, X32 = fl32(p o Dd), gamma_c = |S_c|^2
 template <int KT>
 __global__ void __launch_bounds__(kThreads)
 k_b_init(const double *__restrict__ p, const double *__restrict__ C, double *__restrict__ Sv,
-         double *__restrict__ Dd, double *__restrict__ Z, float *__restrict__ X32,
-         double *__restrict__ T, int64_t n, int64_t glb0, int c0, BatchState *bs,
-         const BatchArgs *args, double *partial, unsigned *counter)
+         double *__restrict__ Dd, double *__restrict__ Z, float *__restrict__ X32, int64_t n,
+         int c_first, BatchState *bs, const BatchArgs *args, double *partial, unsigned *counter)
 {
-    double acc[KT];
-#pragma unroll
-    for (int c = 0; c < KT; c++)
-        acc[c] = 0.0;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x) {
+    const int c0 = c_first + blockIdx.y * KT;
+    const int64_t base = pidx(0, n, c0);
+    double acc = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * KT;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = i / KT, e = base + j * kPanel + (i % KT);
         const double pj = p[j];
-#pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int64_t i = pidx(j, n, c0) + c;
-            const double sj = pj * C[i];
-            Sv[i] = sj;
-            Dd[i] = sj;
-            Z[i] = 0.0;
-            X32[i] = (float)(pj * sj);
-            acc[c] = fma(sj, sj, acc[c]);
-        }
+        const double sj = pj * C[e];
+        Sv[e] = sj;
+        Dd[e] = sj;
+        Z[e] = 0.0;
+        X32[e] = (float)(pj * sj);
+        acc = fma(sj, sj, acc);
     }
-    if (blockIdx.x == 0 && threadIdx.x < KT)
-        T[pidx(glb0, n, c0) + threadIdx.x] = 0.0;
-    if (grid_reduce<KT>(acc, partial, counter) && threadIdx.x == 0) {
-        if (c0 == 0) {
+    if (grid_reduce_col<KT>(acc, partial + (int64_t)c0 * kMaxPartials, counter + c0)) {
+        if (c0 == 0 && threadIdx.x == 0) {
             bs->nonfinite = 0;
             bs->all_done = 0;
         }
-#pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int cc = c0 + c;
-            bs->gamma[cc] = acc[c];
-            bs->gamma0[cc] = acc[c];
+        if (threadIdx.x < KT) {
+            const int cc = c0 + threadIdx.x;
+            bs->gamma[cc] = acc;
+            bs->gamma0[cc] = acc;
             bs->beta[cc] = 0.0;
-            bs->done[cc] = (acc[c] > 0.0) ? 0 : 1;
+            bs->done[cc] = (acc > 0.0) ? 0 : 1;
             bs->it[cc] = 0;
         }
     }
 }
 
-// S_c -= alpha_c p o T_c, Z_c += alpha_c Dd_c, gamma'_c = |S_c|^2
+// S_c -= alpha_c p o T_c, Z_c += alpha_c Dd_c, gamma'_c = |S_c|^2; the
+// attitude columns of T come from the segment sums Sall
 template <int KT>
 __global__ void __launch_bounds__(kThreads)
-k_b_vec1(const double *__restrict__ p, const double *__restrict__ T, double *__restrict__ Sv,
-         const double *__restrict__ Dd, double *__restrict__ Z, int64_t n, int c0,
-         BatchState *bs, const BatchArgs *args, double *partial, unsigned *counter)
+k_b_vec1(SysView A, const double *__restrict__ p, const double *__restrict__ T,
+         const double *__restrict__ Sall, int np, double *__restrict__ Sv,
+         const double *__restrict__ Dd, double *__restrict__ Z, int c_first, BatchState *bs,
+         const BatchArgs *args, double *partial, unsigned *counter)
 {
-    double al[KT], acc[KT];
-#pragma unroll
-    for (int c = 0; c < KT; c++) {
-        al[c] = bs->alpha[c0 + c];
-        acc[c] = 0.0;
+    const int c0 = c_first + blockIdx.y * KT;
+    const int c = threadIdx.x % KT;
+    const int64_t base = pidx(0, A.n, c0);
+    const double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
+    const double al = bs->alpha[c0 + c];
+    double acc = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n * KT;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = i / KT, e = base + j * kPanel + c;
+        const double tj = (j < A.att0 || j >= A.ins0) ? T[e] : att_total<KT>(A, S, np, j - A.att0, c);
+        const double sj = fma(-al, p[j] * tj, Sv[e]);
+        Sv[e] = sj;
+        Z[e] = fma(al, Dd[e], Z[e]);
+        acc = fma(sj, sj, acc);
     }
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const double pj = p[j];
-#pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int64_t i = pidx(j, n, c0) + c;
-            const double sj = fma(-al[c], pj * T[i], Sv[i]);
-            Sv[i] = sj;
-            Z[i] = fma(al[c], Dd[i], Z[i]);
-            acc[c] = fma(sj, sj, acc[c]);
-        }
-    }
-    if (grid_reduce<KT>(acc, partial, counter) && threadIdx.x == 0) {
-#pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int cc = c0 + c;
-            if (bs->done[cc]) {
-                bs->beta[cc] = 0.0;
-                continue;
-            }
-            const double gnew = acc[c];
+    if (grid_reduce_col<KT>(acc, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
+        threadIdx.x < KT) {
+        const int cc = c0 + threadIdx.x;
+        if (bs->done[cc]) {
+            bs->beta[cc] = 0.0;
+        } else {
+            const double gnew = acc;
             bs->beta[cc] = gnew / bs->gamma[cc];
             bs->gamma[cc] = gnew;
             bs->it[cc] += 1;
@@ -503,32 +668,37 @@ k_b_vec1(const double *__restrict__ p, const double *__restrict__ T, double *__r
     }
 }
 
-// Dd = S + beta_c Dd, X32 = fl32(p o Dd); zeroes the global row of T
+// Dd = S + beta_c Dd, X32 = fl32(p o Dd); with last set (every tile's vec1 of
+// the iteration has run) one thread clears the loop flag when every one of
+// the k columns is done
 template <int KT>
 __global__ void k_b_vec2(const double *__restrict__ p, const double *__restrict__ Sv,
-                         double *__restrict__ Dd, float *__restrict__ X32, double *__restrict__ T,
-                         int64_t n, int64_t glb0, int c0, const BatchState *bs)
+                         double *__restrict__ Dd, float *__restrict__ X32, int64_t n, int c_first,
+                         BatchState *bs, int k, cudaGraphConditionalHandle loop, int in_graph,
+                         int last)
 {
-    double be[KT];
-#pragma unroll
-    for (int c = 0; c < KT; c++)
-        be[c] = bs->beta[c0 + c];
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const double pj = p[j];
-#pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int64_t i = pidx(j, n, c0) + c;
-            const double dj = fma(be[c], Dd[i], Sv[i]);
-            Dd[i] = dj;
-            X32[i] = (float)(pj * dj);
-        }
+    const int c0 = c_first + blockIdx.y * KT;
+    const int c = threadIdx.x % KT;
+    const int64_t base = pidx(0, n, c0);
+    const double be = bs->beta[c0 + c];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * KT;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = i / KT, e = base + j * kPanel + c;
+        const double dj = fma(be, Dd[e], Sv[e]);
+        Dd[e] = dj;
+        X32[e] = (float)(p[j] * dj);
     }
-    if (blockIdx.x == 0 && threadIdx.x < KT)
-        T[pidx(glb0, n, c0) + threadIdx.x] = 0.0;
+    if (last && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        int all = 1;
+        for (int q = 0; q < k; q++)
+            all &= bs->done[q];
+        bs->all_done = all;
+        if (all && in_graph)
+            cudaGraphSetConditional(loop, 0u);
+    }
 }
 
-// loop flag: clear when every column is done
+// loop flag before the first iteration: clear when every column is done
 __global__ void k_b_flag(BatchState *bs, int k, cudaGraphConditionalHandle loop, int in_graph)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -603,88 +773,176 @@ __global__ void k_b_update_x(const double *__restrict__ p, const double *__restr
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-template <int KT>
-static cudaError_t b_aprod1(const gsr_handle_t *h, const float *X, float *Q, int c0,
-                            cudaStream_t st)
+// blocks for `warps` warps of work, at most the resident ones
+static int b_blocks(const gsr_handle_t *h, int occ, int64_t warps)
 {
-    k_b_aprod1<KT><<<h->grid_b1, kThreads, 0, st>>>(h->sys, X, Q, c0, h->d_bs,
-                                                    h->d_bpartial, h->d_bcounter);
-    return cudaGetLastError();
+    const int64_t need = (warps + kThreads / 32 - 1) / (kThreads / 32);
+    int64_t g = (int64_t)h->nsm * (occ < 1 ? 1 : occ);
+    if (g > need)
+        g = need;
+    if (g > kMaxPartials)
+        g = kMaxPartials;
+    return (int)(g < 1 ? 1 : g);
 }
 
-// all resident blocks of the star pass for this column tile and lane count
-template <int KS, int G>
-static int stars_grid(const gsr_handle_t *h)
+template <typename F>
+static int b_occ(F f)
 {
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_b_stars<KS, G>, kThreads, 0) !=
-            cudaSuccess ||
-        occ <= 0)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kThreads, 0) != cudaSuccess)
         occ = 1;
-    return h->nsm * occ;
+    return occ;
+}
+
+// pieces per attitude offset: one up to a mean of 512 entries (as many as one
+// warp takes in 8 steps), so that few long offsets still give every SM work
+int batched_att_pieces(const gsr_handle_t *h)
+{
+    const int64_t mean = h->sys.m / h->sys.nseg;
+    const int64_t np = (mean + 511) / 512;
+    return (int)(np < 1 ? 1 : (np > 64 ? 64 : np));
+}
+
+// pieces per instrument: about 2048 entries each
+int batched_instr_pieces(const gsr_handle_t *h)
+{
+    const int64_t mean = kNInstr * h->sys.m / h->sys.I;
+    const int64_t np = (mean + 2047) / 2048;
+    return (int)(np < 1 ? 1 : (np > 256 ? 256 : np));
 }
 
 template <int KT>
-static cudaError_t b_aprod2(const gsr_handle_t *h, const float *Y, double *T, int c0,
+static cudaError_t b_aprod1(const gsr_handle_t *h, const float *X, float *Q, int c0, int ny,
                             cudaStream_t st)
 {
-    // the star pass keeps at most 4 columns per lane (register pressure);
-    // wider tiles are split
-    constexpr int KS = (KT > 4) ? 4 : KT;
-    for (int cs = c0; cs < c0 + KT; cs += KS) {
-        switch (h->b_lanes) {
-        case 8: k_b_stars<KS, 8><<<stars_grid<KS, 8>(h), kThreads, 0, st>>>(h->sys, Y, T, cs); break;
-        case 32: k_b_stars<KS, 32><<<stars_grid<KS, 32>(h), kThreads, 0, st>>>(h->sys, Y, T, cs); break;
-        default: k_b_stars<KS, 16><<<stars_grid<KS, 16>(h), kThreads, 0, st>>>(h->sys, Y, T, cs); break;
-        }
+    const int occ = b_occ(k_b_aprod1<KT>);
+    k_b_aprod1<KT><<<dim3(b_blocks(h, occ, (h->sys.m + 31) / 32), ny), kThreads, 0, st>>>(
+        h->sys, X, Q, c0, h->d_bs, h->d_bpartial, h->d_bcounter);
+    return cudaGetLastError();
+}
+
+template <int KT, int G>
+static void b_stars(const gsr_handle_t *h, const float *Y, double *T, int c0, int ny,
+                    cudaStream_t st)
+{
+    const int occ = b_occ(k_b_stars<KT, G>);
+    const int gx = b_blocks(h, occ, (h->sys.S + 32 / G - 1) / (32 / G));
+    k_b_stars<KT, G><<<dim3(gx, ny), kThreads, 0, st>>>(h->sys, Y, T, c0, h->d_bpartial,
+                                                        h->d_bcounter);
+}
+
+// The three passes of aprod 2 write different sums and run side by side when
+// side streams are given (graph capture): one bound by its gathers shares the
+// SMs with one bound by the FP32 pipe.
+template <int KT>
+static cudaError_t b_aprod2(const gsr_handle_t *h, const float *Y, double *T, int c0, int ny,
+                            cudaStream_t st, const BatchSide *side)
+{
+    cudaStream_t sa = st, si = st;
+    cudaError_t e = cudaSuccess;
+    if (side) {
+        sa = side->s[0];
+        si = side->s[1];
+        e = cudaEventRecord(side->fork, st);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(sa, side->fork, 0);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(si, side->fork, 0);
+        if (e != cudaSuccess)
+            return e;
     }
-    // the attitude pass takes the whole tile at once: reading each entry's
-    // values and gathering its row of Y once for 8 columns (128 registers,
-    // 2 blocks per SM) beat two 4-column passes at 3 blocks per SM (batched
-    // solve at medium size, k = 8: 78.3 -> 68.5 ms; k = 32: 312.6 -> 272.8 ms)
-    k_b_att<KT><<<h->grid_att, kThreads, 0, st>>>(h->sys, Y, h->d_bS, c0);
-    k_b_att_combine<KT><<<h->nsm * 4, kThreads, 0, st>>>(h->sys, h->d_bS, T, c0);
-    k_b_instr<KT><<<h->nsm * 8, kThreads, 0, st>>>(h->sys, h->d_iseg, h->d_irow, h->d_ival32, Y,
-                                                  h->d_bipart, c0);
-    k_b_instr_combine<KT><<<h->nsm * 2, kThreads, 0, st>>>(h->sys, h->d_bipart, T, c0);
+    const int occ_a = b_occ(k_b_att<KT>), occ_i = b_occ(k_b_instr<KT>);
+    const int npa = batched_att_pieces(h), npi = batched_instr_pieces(h);
+    k_b_instr<KT><<<dim3(b_blocks(h, 2 * occ_i, h->sys.I * npi), ny), kThreads, 0, si>>>(
+        h->sys, h->d_iseg, h->d_irow, h->d_ival32, Y, h->d_bipart, h->d_bticket, T, c0, npi);
+    k_b_att<KT><<<dim3(b_blocks(h, 4 * occ_a, h->sys.nseg * 3 * npa), ny), kThreads, 0, sa>>>(
+        h->sys, Y, h->d_bS, c0, npa);
+    switch (h->b_lanes) {
+    case 8: b_stars<KT, 8>(h, Y, T, c0, ny, st); break;
+    case 32: b_stars<KT, 32>(h, Y, T, c0, ny, st); break;
+    default: b_stars<KT, 16>(h, Y, T, c0, ny, st); break;
+    }
+    if (side) {
+        for (int i = 0; i < 2 && e == cudaSuccess; i++) {
+            e = cudaEventRecord(side->join[i], side->s[i]);
+            if (e == cudaSuccess)
+                e = cudaStreamWaitEvent(st, side->join[i], 0);
+        }
+        if (e != cudaSuccess)
+            return e;
+    }
     return cudaGetLastError();
 }
 
 template <int KT>
-static cudaError_t b_prologue_tile(const gsr_handle_t *h, int c0, cudaStream_t s)
+static int vec_blocks(const gsr_handle_t *h)
 {
-    k_b_init<KT><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_bC, h->d_bS_, h->d_bD, h->d_bZ,
-                                                   h->d_bX32, h->d_bT, h->sys.n, h->sys.glb0,
-                                                   c0, h->d_bs, h->d_bargs, h->d_bpartial,
-                                                   h->d_bcounter);
+    const int64_t need = (h->sys.n * KT + kThreads - 1) / kThreads;
+    const int64_t g = (int64_t)h->nsm * 4;
+    return (int)(g < need ? g : need);
+}
+
+template <int KT>
+static cudaError_t b_prologue_tiles(const gsr_handle_t *h, int c0, int ny, cudaStream_t s)
+{
+    k_b_init<KT><<<dim3(vec_blocks<KT>(h), ny), kThreads, 0, s>>>(
+        h->d_p, h->d_bC, h->d_bS_, h->d_bD, h->d_bZ, h->d_bX32, h->sys.n, c0, h->d_bs, h->d_bargs,
+        h->d_bpartial, h->d_bcounter);
     return cudaGetLastError();
 }
 
 template <int KT>
-static cudaError_t b_iteration_tile_a(const gsr_handle_t *h, int c0, cudaStream_t s)
+static cudaError_t b_products_tiles(const gsr_handle_t *h, const float *X, float *Q, const float *Y,
+                                    double *T, int c0, int ny, cudaStream_t s)
 {
-    cudaError_t e = b_aprod1<KT>(h, h->d_bX32, h->d_bQ32, c0, s);
+    cudaError_t e = b_aprod1<KT>(h, X, Q, c0, ny, s);
     if (e == cudaSuccess)
-        e = b_aprod2<KT>(h, h->d_bQ32, h->d_bT, c0, s);
+        e = b_aprod2<KT>(h, Y, T, c0, ny, s, nullptr);
+    if (e == cudaSuccess) {
+        k_b_att_combine<KT><<<dim3(h->nsm, ny), kThreads, 0, s>>>(h->sys, h->d_bS, T, c0,
+                                                                  batched_att_pieces(h));
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+template <int KT>
+static cudaError_t b_iteration_tiles(const gsr_handle_t *h, int c0, int ny, cudaStream_t s, int k,
+                                     cudaGraphConditionalHandle loop, int in_graph, int last,
+                                     const BatchSide *side)
+{
+    cudaError_t e = b_aprod1<KT>(h, h->d_bX32, h->d_bQ32, c0, ny, s);
+    if (e == cudaSuccess)
+        e = b_aprod2<KT>(h, h->d_bQ32, h->d_bT, c0, ny, s, side);
     if (e != cudaSuccess)
         return e;
-    k_b_vec1<KT><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_bT, h->d_bS_, h->d_bD, h->d_bZ,
-                                                   h->sys.n, c0, h->d_bs, h->d_bargs,
-                                                   h->d_bpartial, h->d_bcounter);
-    k_b_vec2<KT><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_bS_, h->d_bD, h->d_bX32, h->d_bT,
-                                                   h->sys.n, h->sys.glb0, c0, h->d_bs);
+    const dim3 g(vec_blocks<KT>(h), ny);
+    k_b_vec1<KT><<<g, kThreads, 0, s>>>(h->sys, h->d_p, h->d_bT, h->d_bS, batched_att_pieces(h),
+                                        h->d_bS_, h->d_bD, h->d_bZ, c0, h->d_bs, h->d_bargs,
+                                        h->d_bpartial, h->d_bcounter);
+    k_b_vec2<KT><<<g, kThreads, 0, s>>>(h->d_p, h->d_bS_, h->d_bD, h->d_bX32, h->sys.n, c0, h->d_bs,
+                                        k, loop, in_graph, last);
     return cudaGetLastError();
 }
 
-static cudaError_t b_dispatch(const gsr_handle_t *h, int kt, int which, int c0,
-                              cudaStream_t s)
+// The k columns as runs of equal tiles: whole tiles of the chosen width, then
+// the rest in tiles of at most that width (11 columns at width 8: one tile of
+// 8, one of 2, one of 1), so no column of padding is computed.  f(kt, c0, ny)
+// per run; the last run is told.
+template <typename F>
+static cudaError_t for_runs(const gsr_handle_t *h, int k, F f)
 {
-    switch (kt) {
-    case 1: return which ? b_iteration_tile_a<1>(h, c0, s) : b_prologue_tile<1>(h, c0, s);
-    case 2: return which ? b_iteration_tile_a<2>(h, c0, s) : b_prologue_tile<2>(h, c0, s);
-    case 4: return which ? b_iteration_tile_a<4>(h, c0, s) : b_prologue_tile<4>(h, c0, s);
-    default: return which ? b_iteration_tile_a<8>(h, c0, s) : b_prologue_tile<8>(h, c0, s);
+    int c0 = 0;
+    for (int kt = h->b_kt; kt >= 1; kt >>= 1) {
+        const int ny = (k - c0) / kt;
+        if (ny > 0) {
+            cudaError_t e = f(kt, c0, ny, c0 + ny * kt == k);
+            if (e != cudaSuccess)
+                return e;
+            c0 += ny * kt;
+        }
     }
+    return cudaSuccess;
 }
 
 // the inner solve of the k columns: prologue, then iterations until every
@@ -692,25 +950,32 @@ static cudaError_t b_dispatch(const gsr_handle_t *h, int kt, int which, int c0,
 static cudaError_t b_prologue(const gsr_handle_t *h, int k, cudaStream_t s,
                               cudaGraphConditionalHandle loop, int in_graph)
 {
-    for (int c0 = 0; c0 < k; c0 += h->b_kt) {
-        cudaError_t e = b_dispatch(h, h->b_kt, 0, c0, s);
-        if (e != cudaSuccess)
-            return e;
-    }
+    cudaError_t e = for_runs(h, k, [&](int kt, int c0, int ny, bool) {
+        switch (kt) {
+        case 1: return b_prologue_tiles<1>(h, c0, ny, s);
+        case 2: return b_prologue_tiles<2>(h, c0, ny, s);
+        case 4: return b_prologue_tiles<4>(h, c0, ny, s);
+        default: return b_prologue_tiles<8>(h, c0, ny, s);
+        }
+    });
+    if (e != cudaSuccess)
+        return e;
     k_b_flag<<<1, 32, 0, s>>>(h->d_bs, k, loop, in_graph);
     return cudaGetLastError();
 }
 
 static cudaError_t b_iteration(const gsr_handle_t *h, int k, cudaStream_t s,
-                               cudaGraphConditionalHandle loop, int in_graph)
+                               cudaGraphConditionalHandle loop, int in_graph,
+                               const BatchSide *side)
 {
-    for (int c0 = 0; c0 < k; c0 += h->b_kt) {
-        cudaError_t e = b_dispatch(h, h->b_kt, 1, c0, s);
-        if (e != cudaSuccess)
-            return e;
-    }
-    k_b_flag<<<1, 32, 0, s>>>(h->d_bs, k, loop, in_graph);
-    return cudaGetLastError();
+    return for_runs(h, k, [&](int kt, int c0, int ny, bool last) {
+        switch (kt) {
+        case 1: return b_iteration_tiles<1>(h, c0, ny, s, k, loop, in_graph, last, side);
+        case 2: return b_iteration_tiles<2>(h, c0, ny, s, k, loop, in_graph, last, side);
+        case 4: return b_iteration_tiles<4>(h, c0, ny, s, k, loop, in_graph, last, side);
+        default: return b_iteration_tiles<8>(h, c0, ny, s, k, loop, in_graph, last, side);
+        }
+    });
 }
 
 #define B_TRY(x)                        \
@@ -733,14 +998,12 @@ cudaError_t build_batched_graph(gsr_handle_t *h, int k)
     cudaGraphNodeParams cp = {};
     cudaGraph_t body;
     cudaStream_t s = h->cap_stream;
-    if (h->b_exec) {
-        cudaGraphExecDestroy(h->b_exec);
-        h->b_exec = nullptr;
-    }
+    BatchSide side;
+    B_TRY(side.make());
     B_TRY(cudaGraphCreate(&g, 0));
     B_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
     B_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    b_prologue(h, k, s, loop, 1);
+    B_TRY(b_prologue(h, k, s, loop, 1));
     B_TRY(cudaStreamEndCapture(s, &g));
     B_TRY(find_graph_leaf(g, &pre_leaf));
     cp.type = cudaGraphNodeTypeConditional;
@@ -750,13 +1013,10 @@ cudaError_t build_batched_graph(gsr_handle_t *h, int k)
     B_TRY(cudaGraphAddNode(&wnode, g, &pre_leaf, nullptr, 1, &cp));
     body = cp.conditional.phGraph_out[0];
     B_TRY(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    b_iteration(h, k, s, loop, 1);
+    B_TRY(b_iteration(h, k, s, loop, 1, &side));
     B_TRY(cudaStreamEndCapture(s, &body));
-    B_TRY(cudaGraphInstantiate(&h->b_exec, g, 0));
+    B_TRY(cudaGraphInstantiate(&h->b_exec[k], g, 0));
     cudaGraphDestroy(g);
-    h->b_graph_k = k;
-    h->b_graph_kt = h->b_kt;
-    h->b_graph_lanes = h->b_lanes;
     return cudaSuccess;
 fail:
     {
@@ -777,7 +1037,7 @@ fail:
 cudaError_t run_batched_inner(gsr_handle_t *h, int k, int max_inner, cudaStream_t st)
 {
     if (!h->cfg.eager)
-        return cudaGraphLaunch(h->b_exec, st);
+        return cudaGraphLaunch(h->b_exec[k], st);
     cudaError_t e = b_prologue(h, k, st, 0, 0);
     for (int it = 0; e == cudaSuccess && it < max_inner + 1; it++) {
         e = cudaMemcpyAsync(h->h_bs, h->d_bs, sizeof(BatchState), cudaMemcpyDeviceToHost, st);
@@ -785,7 +1045,7 @@ cudaError_t run_batched_inner(gsr_handle_t *h, int k, int max_inner, cudaStream_
             e = cudaStreamSynchronize(st);
         if (e != cudaSuccess || h->h_bs->all_done)
             break;
-        e = b_iteration(h, k, st, 0, 0);
+        e = b_iteration(h, k, st, 0, 0, nullptr);
     }
     return e;
 }
@@ -801,33 +1061,14 @@ cudaError_t launch_b_update_x(const gsr_handle_t *h, double *X, int k, cudaStrea
 cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, const float *Y,
                               double *T, cudaStream_t st)
 {
-    for (int c0 = 0; c0 < k; c0 += h->b_kt) {
-        cudaError_t e;
-        switch (h->b_kt) {
-        case 1: e = b_aprod1<1>(h, X, Q, c0, st); if (e == cudaSuccess) e = b_aprod2<1>(h, Y, T, c0, st); break;
-        case 2: e = b_aprod1<2>(h, X, Q, c0, st); if (e == cudaSuccess) e = b_aprod2<2>(h, Y, T, c0, st); break;
-        case 4: e = b_aprod1<4>(h, X, Q, c0, st); if (e == cudaSuccess) e = b_aprod2<4>(h, Y, T, c0, st); break;
-        default: e = b_aprod1<8>(h, X, Q, c0, st); if (e == cudaSuccess) e = b_aprod2<8>(h, Y, T, c0, st); break;
+    return for_runs(h, k, [&](int kt, int c0, int ny, bool) {
+        switch (kt) {
+        case 1: return b_products_tiles<1>(h, X, Q, Y, T, c0, ny, st);
+        case 2: return b_products_tiles<2>(h, X, Q, Y, T, c0, ny, st);
+        case 4: return b_products_tiles<4>(h, X, Q, Y, T, c0, ny, st);
+        default: return b_products_tiles<8>(h, X, Q, Y, T, c0, ny, st);
         }
-        if (e != cudaSuccess)
-            return e;
-    }
-    return cudaSuccess;
-}
-
-int batched_grid_rows(const gsr_handle_t *h)
-{
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_b_aprod1<8>, kThreads, 0) != cudaSuccess ||
-        occ <= 0)
-        return -1;
-    int64_t g = (int64_t)h->nsm * occ;
-    return (int)(g > kMaxPartials ? kMaxPartials : g);
-}
-
-int batched_grid_stars(const gsr_handle_t *h)
-{
-    return stars_grid<4, 16>(h);
+    });
 }
 
 }  // namespace gsr

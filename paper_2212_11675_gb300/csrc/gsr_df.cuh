@@ -19,6 +19,71 @@ __device__ __forceinline__ void df_acc(float &hi, float &lo, float p)
     lo = __fadd_rn(lo, err);
 }
 
+// Two binary32 values in one 64-bit register pair, for the packed f32x2
+// instructions (each half rounds like the scalar instruction).  GB300 runs
+// them at the scalar lane rate (measured: 127 lane operations per clock and
+// SM packed, 122 scalar) from half the issue slots, which the double-float
+// accumulations on several columns need for their gathers.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+
+// add, subtract, multiply, a b + c with round to nearest, scalar or packed
+__device__ __forceinline__ float v_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float v_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float v_neg(float a) { return -a; }
+__device__ __forceinline__ f32x2 v_add(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 v_sub(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// two scalar multiplications: the compiler contracts a packed mul.rn with the
+// packed add that follows it into one FMA (its result is then not the sum of
+// the rounded product), and never a scalar mul.rn; measured at the same speed
+__device__ __forceinline__ f32x2 v_mul(f32x2 a, f32x2 b)
+{
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1);
+    unpack2(b, b0, b1);
+    return pack2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ f32x2 v_fma(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 v_neg(f32x2 a) { return a ^ 0x8000000080000000ull; }
+
+// df_acc on one value or on a packed pair of independent accumulators
+template <typename V>
+__device__ __forceinline__ void df_acc_v(V &hi, V &lo, V p)
+{
+    const V s = v_add(hi, p);
+    const V bp = v_sub(s, hi);
+    const V err = v_add(v_sub(hi, v_sub(s, bp)), v_sub(p, bp));
+    hi = s;
+    lo = v_add(lo, err);
+}
+
 // Sum of two double-float numbers (ah + al) + (bh + bl), Joldes, Muller &
 // Popescu, "Tight and rigorous error bounds for basic building blocks of
 // double-word arithmetic", ACM TOMS 44 (2017), Algorithm 6 ("AccurateDWPlusDW"):

@@ -239,17 +239,17 @@ struct gsr_handle_t {
     int bkB = 0;                                      // columns of the staged right-hand sides
     float *d_bX32 = nullptr, *d_bQ32 = nullptr;
     double *d_bC = nullptr, *d_bS_ = nullptr, *d_bD = nullptr, *d_bZ = nullptr, *d_bT = nullptr;
-    double *d_bS = nullptr;                           // attitude sums of one column tile
-    double *d_bipart = nullptr;                       // [I][4][8] instrumental partials
+    double *d_bS = nullptr;                           // attitude sums, [nseg][12] per piece, column
+    double *d_bipart = nullptr;                       // [I] partials per piece and column
     double *d_bXcm = nullptr, *d_bCcm = nullptr, *d_bB = nullptr;
     double *d_bnorms = nullptr, *h_bnorms = nullptr;
     double *d_bpartial = nullptr;
     unsigned *d_bcounter = nullptr;
     gsr::BatchState *d_bs = nullptr, *h_bs = nullptr;
     gsr::BatchArgs *d_bargs = nullptr, *h_bargs = nullptr;
-    cudaGraphExec_t b_exec = nullptr;
-    int b_kt = 8, b_lanes = 16, b_graph_k = 0, b_graph_kt = 0, b_graph_lanes = 0;
-    int grid_b1 = 0, grid_b2 = 0;
+    unsigned *d_bticket = nullptr;                    // [I] per column: finished pieces
+    cudaGraphExec_t b_exec[gsr::kMaxBatch + 1] = {};  // inner solve of k columns
+    int b_kt = 8, b_lanes = 16, b_graph_kt = 0, b_graph_lanes = 0;  // the graphs' tiling
     double *d_xp64 = nullptr, *d_q64 = nullptr;
     int grid_rows32 = 0, grid_rows2_32 = 0, grid_fused32 = 0;
     double n_nonempty = 0.0;
@@ -298,8 +298,8 @@ cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, floa
                               double *T, cudaStream_t st);
 cudaError_t launch_b_layout(const gsr_handle_t *h, int to_rm, const double *src, void *dst,
                             int dst_f32, int64_t rows, int k, cudaStream_t st);
-int batched_grid_rows(const gsr_handle_t *h);
-int batched_grid_stars(const gsr_handle_t *h);
+int batched_att_pieces(const gsr_handle_t *h);
+int batched_instr_pieces(const gsr_handle_t *h);
 cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out,
                           int mode, cudaStream_t st);
 cudaError_t launch_validate(const gsr_handle_t *h, cudaStream_t st);

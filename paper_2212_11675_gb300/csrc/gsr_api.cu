@@ -143,12 +143,15 @@ static void release(gsr_handle_t *h)
                    h->d_seg, h->d_attS, h->d_irep, h->d_p, h->d_u, h->d_v, h->d_w, h->d_z,
                    h->d_var, h->d_q, h->d_vp, h->d_vt, h->d_bstage, h->d_xstage, h->d_sestage,
                    h->d_ystage, h->d_state, h->d_args, h->d_partial, h->d_counter, h->d_err,
-                   h->d_val32, h->d_tval32, h->d_x32, h->d_xatt4, h->d_q32, h->d_c, h->d_s, h->d_d, h->d_t,
+                   h->d_atile, h->d_sv32, h->d_unit, h->d_useg, h->d_attS32,
+                   h->d_x32, h->d_x8, h->d_q32, h->d_c, h->d_s, h->d_d, h->d_t,
                    h->d_zc, h->d_xm, h->d_r, h->d_xneg, h->d_onorm, h->d_cg, h->d_cgargs,
                    h->d_xp64, h->d_q64, h->d_iseg, h->d_cseg, h->d_cseg32, h->d_irow, h->d_ival32, h->d_ival, h->d_ipart, h->d_gpart, h->d_a2ctr, h->d_bX32, h->d_bQ32,
                    h->d_bC, h->d_bS_, h->d_bD, h->d_bZ, h->d_bT, h->d_bS, h->d_bXcm,
                    h->d_bCcm, h->d_bB, h->d_bnorms, h->d_bpartial, h->d_bcounter, h->d_bs,
                    h->d_bipart, h->d_bticket,
+                   h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin,
+                   h->d_epos, h->d_eptr, h->d_epart,
                    h->d_bargs};
     for (void *p : dev)
         if (p)
@@ -161,6 +164,226 @@ static void release(gsr_handle_t *h)
     if (cur >= 0)
         cudaSetDevice(cur);
     delete h;
+}
+
+// Rows per window of the FP64 instrument units: R = 4096 I / 6 (about 4096
+// entries per instrument and window), at most 4 Mi rows (32 MB of FP64 y), at
+// least 64 Ki rows
+static int64_t instr_window(const gsr_handle_t *h)
+{
+    return std::max<int64_t>((int64_t)1 << 16,
+                             std::min<int64_t>(4096 * h->sys.I / kNInstr, (int64_t)1 << 22));
+}
+
+// the window bounds cseg of the instrument-sorted copy, its partial sums and
+// the grid of the separate instrument pass
+static int finish_instr(gsr_handle_t *h, const std::vector<uint32_t> &cseg, int64_t nq, int64_t nparts)
+{
+    const int64_t I = h->sys.I;
+    TRY(dalloc(h, &h->d_cseg, (nq + 1) * I));
+    CK(cudaMemcpy(h->d_cseg, cseg.data(), (nq + 1) * I * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    h->isplit = (int)nq;
+    TRY(dalloc(h, &h->d_ipart, nparts * I));
+    CK(cudaMemset(h->d_ipart, 0, (size_t)nparts * I * sizeof(double)));
+    const int64_t units_blocks = (I * nq + kThreads / 32 - 1) / (kThreads / 32);
+    const int64_t cap = (int64_t)h->nsm * 16;
+    h->grid_ins = (int)(units_blocks < cap ? units_blocks : cap);
+    return GSR_OK;
+}
+
+// Instrumental nonzeros of a mixed-precision handle in row windows (Ell): the
+// columns of every window and the place of every entry are worked out on the
+// host, window by window, the values gathered on the device; the
+// instrument-sorted copy (FP64 aprod 2, batched form) is written from them.
+static int build_ell(gsr_handle_t *h, cudaStream_t st)
+{
+    SysView &A = h->sys;
+    const int64_t m = A.m, I = A.I;
+    // one window per SM on a small system, a whole number of rounds of them
+    // on a large one, eight entries per instrument and window or more
+    int64_t W = (m + h->nsm - 1) / h->nsm;
+    const int64_t wmin = (8 * I + kNInstr - 1) / kNInstr;
+    if (W < wmin)
+        W = wmin;
+    if (W > kEllRowsMax) {
+        const int64_t rounds = (m + kEllRowsMax * h->nsm - 1) / (kEllRowsMax * h->nsm);
+        W = (m + rounds * h->nsm - 1) / (rounds * h->nsm);
+        if (W < wmin)
+            W = wmin;
+    }
+    W = (W + 31) / 32 * 32;
+    if (W > kEllRowsMax)
+        W = kEllRowsMax;
+    const int64_t nwin = (m + W - 1) / W;
+    const int64_t nblk = std::min<int64_t>(nwin, h->nsm);
+    // entries per column at most: about two slices for each of the 16 warps of
+    // a block where there are few instruments
+    const uint32_t L = (uint32_t)std::min<int64_t>(
+        kEllLen, std::max<int64_t>(kEllStep, kNInstr * W / 1024 / kEllStep * kEllStep));
+    std::vector<uint4> rec((size_t)m);
+    CK(cudaMemcpy(rec.data(), h->d_rec, m * sizeof(uint4), cudaMemcpyDeviceToHost));
+    std::vector<uint32_t> code, win((size_t)nwin + 1), vf, vloc, vrank;
+    std::vector<uint2> slice;
+    code.reserve((size_t)(kNInstr * m + kNInstr * m / 8 + 4096));
+    // columns of instrument f in a window of block b: at most nchunk[b I + f],
+    // each with a partial of its own
+    std::vector<uint32_t> cnt((size_t)I), rank((size_t)I, 0), nchunk((size_t)(nblk * I), 0);
+    std::vector<uint32_t> cur((size_t)I), idx((size_t)I), first((size_t)I), order, len;
+    std::vector<uint64_t> base;
+    uint64_t groups = 0;  // 32-entry groups so far
+    // the FP64 units' windows: whole ones of these
+    const int64_t per = std::max<int64_t>(1, (instr_window(h) + W / 2) / W);
+    std::vector<uint32_t> cseg;
+    for (int64_t w = 0; w < nwin; w++) {
+        if (w % per == 0)
+            cseg.insert(cseg.end(), rank.begin(), rank.end());
+        const int64_t r0 = w * W, r1 = std::min(m, r0 + W);
+        std::fill(cnt.begin(), cnt.end(), 0u);
+        for (int64_t i = r0; i < r1; i++)
+            for (int j = 0; j < kNInstr; j++)
+                cnt[instr_of(rec[i], j)]++;
+        // columns in (instrument, piece) order, then by decreasing length
+        len.clear();
+        std::vector<uint32_t> cf;
+        for (int64_t f = 0; f < I; f++) {
+            first[f] = (uint32_t)len.size();
+            for (uint32_t c = cnt[f]; c > 0;) {
+                const uint32_t l = std::min<uint32_t>(c, L);
+                len.push_back(l);
+                cf.push_back((uint32_t)f);
+                c -= l;
+            }
+        }
+        uint32_t start[kEllLen + 2] = {0};
+        for (uint32_t l : len)
+            start[kEllLen - l + 1]++;
+        for (int l = 0; l <= kEllLen; l++)
+            start[l + 1] += start[l];
+        order.resize(len.size());
+        for (size_t v = 0; v < len.size(); v++)
+            order[start[kEllLen - len[v]]++] = (uint32_t)v;
+        win[w] = (uint32_t)slice.size();
+        const size_t lane0 = vf.size();
+        const size_t nsl = (len.size() + 31) / 32;
+        vf.resize(lane0 + 32 * nsl, kEllNone);
+        vloc.resize(lane0 + 32 * nsl, 0);
+        vrank.resize(lane0 + 32 * nsl, 0);
+        base.resize(len.size());
+        for (size_t q = 0; q < nsl; q++) {
+            const uint32_t l = (len[order[32 * q]] + kEllStep - 1) / kEllStep * kEllStep;
+            slice.push_back(make_uint2((uint32_t)groups, l));
+            for (size_t t = 0; t < 32 && 32 * q + t < len.size(); t++)
+                base[order[32 * q + t]] = groups * 32 + t;
+            for (size_t t = 0; t < 32 && 32 * q + t < len.size(); t++)
+                vf[lane0 + 32 * q + t] = order[32 * q + t];  // column for now
+            groups += l;
+        }
+        // piece number (with kEllFirst where its partial is new) and first
+        // entry of every column, in column order
+        uint32_t *nc = nchunk.data() + (w % nblk) * I;
+        std::vector<uint32_t> cloc(len.size()), crank(len.size());
+        for (size_t v = 0; v < len.size(); v++) {
+            const uint32_t f = cf[v], c = (uint32_t)v - first[f];
+            cloc[v] = c;
+            if (c >= nc[f]) {
+                nc[f] = c + 1;
+                cloc[v] |= kEllFirst;
+            }
+            crank[v] = rank[f];
+            rank[f] += len[v];
+        }
+        for (size_t t = lane0; t < vf.size(); t++)
+            if (vf[t] != kEllNone) {
+                const uint32_t v = vf[t];
+                vloc[t] = cloc[v];
+                vrank[t] = crank[v];
+                vf[t] = cf[v];
+            }
+        code.resize(groups * 32, kEllNone);
+        for (int64_t f = 0; f < I; f++) {
+            cur[f] = first[f];
+            idx[f] = 0;
+        }
+        for (int64_t i = r0; i < r1; i++)
+            for (int j = 0; j < kNInstr; j++) {
+                const uint32_t f = instr_of(rec[i], j);
+                code[base[cur[f]] + 32ull * idx[f]] = (uint32_t)(kNInstr * i + j);
+                if (++idx[f] == L) {
+                    idx[f] = 0;
+                    cur[f]++;
+                }
+            }
+    }
+    win[nwin] = (uint32_t)slice.size();
+    std::vector<uint4>().swap(rec);
+    // partials of instrument f: block after block, those of f - 1 before them
+    std::vector<uint32_t> ptr((size_t)I + 1), seg((size_t)I + 1);
+    ptr[0] = seg[0] = 0;
+    for (int64_t f = 0; f < I; f++) {
+        uint32_t t = ptr[f];
+        for (int64_t b = 0; b < nblk; b++) {
+            const uint32_t c = nchunk[b * I + f];
+            nchunk[b * I + f] = t;
+            t += c;
+        }
+        ptr[f + 1] = t;
+        seg[f + 1] = seg[f] + rank[f];
+    }
+    cseg.insert(cseg.end(), rank.begin(), rank.end());
+    const int64_t nq = (nwin + per - 1) / per;
+    for (int64_t q = 0; q <= nq; q++)
+        for (int64_t f = 0; f < I; f++)
+            cseg[q * I + f] += seg[f];
+    const int64_t npart = ptr[I], nslots = (int64_t)vf.size();
+    std::vector<uint32_t> pos((size_t)nslots, kEllNone), sorted((size_t)nslots, kEllNone);
+    for (int64_t w = 0; w < nwin; w++)
+        for (int64_t t = 32 * (int64_t)win[w]; t < 32 * (int64_t)win[w + 1]; t++)
+            if (vf[t] != kEllNone) {
+                pos[t] = (nchunk[(w % nblk) * I + vf[t]] + (vloc[t] & ~kEllFirst)) |
+                         (vloc[t] & kEllFirst);
+                sorted[t] = seg[vf[t]] + vrank[t];
+            }
+    const int64_t total = (int64_t)code.size();
+    TRY(dalloc(h, &h->d_eidx, total));
+    TRY(dalloc(h, &h->d_eval32, total));
+    TRY(dalloc(h, &h->d_eslice, (int64_t)slice.size()));
+    TRY(dalloc(h, &h->d_ewin, nwin + 1));
+    TRY(dalloc(h, &h->d_epos, nslots));
+    TRY(dalloc(h, &h->d_eptr, I + 1));
+    TRY(dalloc(h, &h->d_epart, npart));
+    TRY(dalloc(h, &h->d_iseg, I + 1));
+    TRY(dalloc(h, &h->d_irow, kNInstr * m));
+    TRY(dalloc(h, &h->d_ival, kNInstr * m));
+    TRY(dalloc(h, &h->d_ival32, kNInstr * m));
+    CK(cudaMemcpy(h->d_eslice, slice.data(), slice.size() * sizeof(uint2), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_ewin, win.data(), (nwin + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_epos, pos.data(), nslots * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_eptr, ptr.data(), (I + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_iseg, seg.data(), (I + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    h->ell = Ell{h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin, h->d_epos, h->d_eptr, h->d_epart,
+                 nwin, W, nblk};
+    uint32_t *d_tmp = nullptr;
+    const size_t bytes = (size_t)std::max(total, nslots) * sizeof(uint32_t);
+    if (cudaMalloc(&d_tmp, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return GSR_ERR_OOM;
+    }
+    cudaError_t e = cudaMemcpy(d_tmp, code.data(), total * sizeof(uint32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = launch_ell_fill(h, d_tmp, total, st);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(d_tmp, sorted.data(), nslots * sizeof(uint32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = launch_ell_sorted(h, d_tmp, st);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(st);
+    cudaFree(d_tmp);
+    if (e != cudaSuccess)
+        return cuda_fail(e, "instrument windows");
+    h->ell_on = true;
+    return finish_instr(h, cseg, nq, nq);
 }
 
 // Instrument-sorted copy of the instrumental nonzeros: a stable counting
@@ -210,14 +433,7 @@ static int build_instr_sorted(gsr_handle_t *h, cudaStream_t st)
     cudaFree(d_code);
     if (e != cudaSuccess)
         return cuda_fail(e, "instrument-sorted layout");
-    // row windows: R = 4096 I / 6 rows (about 4096 entries per instrument and
-    // window), at most 4 Mi rows (32 MB of FP64 y), at least 64 Ki rows
-    int64_t R = 4096 * I / kNInstr;
-    if (R > ((int64_t)1 << 22))
-        R = (int64_t)1 << 22;
-    if (R < ((int64_t)1 << 16))
-        R = (int64_t)1 << 16;
-    const int64_t nq = (m + R - 1) / R;
+    const int64_t R = instr_window(h), nq = (m + R - 1) / R;
     std::vector<uint32_t> cseg((size_t)((nq + 1) * I));
     for (int64_t f = 0; f < I; f++) {
         uint32_t e = seg[f];
@@ -229,9 +445,6 @@ static int build_instr_sorted(gsr_handle_t *h, cudaStream_t st)
         }
         cseg[nq * I + f] = seg[f + 1];
     }
-    TRY(dalloc(h, &h->d_cseg, (nq + 1) * I));
-    CK(cudaMemcpy(h->d_cseg, cseg.data(), (nq + 1) * I * sizeof(uint32_t), cudaMemcpyHostToDevice));
-    h->isplit = (int)nq;
     int64_t nparts = nq;
     if (h->cfg.precision == GSR_PREC_MIXED) {
         // binary32 units: windows of 32 MB of binary32 y (8 Mi rows), each
@@ -258,32 +471,70 @@ static int build_instr_sorted(gsr_handle_t *h, cudaStream_t st)
         if (nq32 * ks32 > nparts)
             nparts = nq32 * ks32;
     }
-    TRY(dalloc(h, &h->d_ipart, nparts * I));
-    CK(cudaMemset(h->d_ipart, 0, (size_t)nparts * I * sizeof(double)));
-    const int64_t units_blocks = (I * h->isplit + kThreads / 32 - 1) / (kThreads / 32);
-    const int64_t cap = (int64_t)h->nsm * 16;
-    h->grid_ins = (int)(units_blocks < cap ? units_blocks : cap);
+    return finish_instr(h, cseg, nq, nparts);
+}
+
+// the units of the offset-ordered binary32 layout (Att32)
+static int build_units(gsr_handle_t *h)
+{
+    const SysView &A = h->sys;
+    std::vector<uint32_t> seg((size_t)A.nseg + 1), useg((size_t)A.nseg + 1);
+    CK(cudaMemcpy(seg.data(), h->d_seg, (A.nseg + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    // tiles per unit: about four units for each of the 16 warps of every SM,
+    // at most kUnitTiles (the unit's reduction is then a small share)
+    const uint64_t want = (uint64_t)((A.m / 32) / ((int64_t)h->nsm * 64));
+    const uint64_t ut = want < 1 ? 1 : (want > kUnitTiles ? kUnitTiles : want);
+    std::vector<uint4> unit;
+    unit.reserve((size_t)(A.nseg + A.m / 32 / ut + 1));
+    for (int64_t o = 0; o < A.nseg; o++) {
+        useg[o] = (uint32_t)unit.size();
+        const uint64_t e0 = seg[o], e1 = seg[o + 1];
+        if (e0 == e1)
+            continue;
+        // tiles t0 .. t1-1 in np runs of like length
+        const uint64_t t0 = e0 >> 5, t1 = ((e1 - 1) >> 5) + 1, nt = t1 - t0;
+        const uint64_t np = (nt + ut - 1) / ut;
+        for (uint64_t q = 0; q < np; q++) {
+            const uint64_t a = (t0 + nt * q / np) << 5, b = (t0 + nt * (q + 1) / np) << 5;
+            unit.push_back(make_uint4((uint32_t)o, (uint32_t)std::max(a, e0),
+                                      (uint32_t)std::min(b, e1), 0u));
+        }
+    }
+    useg[A.nseg] = (uint32_t)unit.size();
+    const int64_t nu = (int64_t)unit.size();
+    TRY(dalloc(h, &h->d_unit, nu));
+    TRY(dalloc(h, &h->d_useg, A.nseg + 1));
+    TRY(dalloc(h, &h->d_attS32, nu * kNAtt));
+    CK(cudaMemcpy(h->d_unit, unit.data(), nu * sizeof(uint4), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_useg, useg.data(), (A.nseg + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    h->att32.unit = h->d_unit;
+    h->att32.useg = h->d_useg;
+    h->att32.nunits = nu;
     return GSR_OK;
 }
 
-// binary32 copies of the value planes and of the offset-sorted attitude
-// values, the mixed-precision workspace and the inner CG graph
+// the binary32 copies of the values, the mixed-precision workspace and the
+// inner CG graph
 static int create_mixed(gsr_handle_t *h, cudaStream_t st)
 {
     SysView &A = h->sys;
     const int64_t m = A.m, n = A.n, mp = A.mp;
-    TRY(dalloc(h, &h->d_val32, kNPar * mp));
-    TRY(dalloc(h, &h->d_tval32, (int64_t)kNAtt * mp));
-    TRY(dalloc(h, &h->d_ival32, kNInstr * m));
+    TRY(dalloc(h, &h->d_atile, mp / 32 * kAttTileBytes));
+    TRY(dalloc(h, &h->d_sv32, kNAstro * mp));
     TRY(dalloc(h, &h->d_x32, n));
-    TRY(dalloc(h, &h->d_xatt4, 3 * A.D * 4));
-    CK(cudaMemset(h->d_xatt4, 0, 3 * A.D * 4 * sizeof(float)));
+    TRY(dalloc(h, &h->d_x8, 8 * A.S));
     TRY(dalloc(h, &h->d_q32, m));
-    CK(launch_to_f32(h, h->d_val, h->d_val32, kNPar * mp, st));
-    CK(launch_to_f32(h, h->d_tval, h->d_tval32, kNAtt * mp, st));
-    A.val32 = h->d_val32;
-    A.tval32 = h->d_tval32;
-    CK(launch_to_f32(h, h->d_ival, h->d_ival32, kNInstr * m, st));
+    CK(cudaMemsetAsync(h->d_x8, 0, 8 * A.S * sizeof(float), st));
+    // whole tiles are copied: the entries beyond m are zero
+    CK(cudaMemsetAsync(h->d_atile, 0, mp / 32 * kAttTileBytes, st));
+    TRY(build_units(h));
+    h->att32.tile = h->d_atile;
+    h->att32.sv = h->d_sv32;
+    CK(build_att32(h, st));
+    if (!h->ell_on) {
+        TRY(dalloc(h, &h->d_ival32, kNInstr * m));
+        CK(launch_to_f32(h, h->d_ival, h->d_ival32, kNInstr * m, st));
+    }
     // ||A diag(p)||_F^2 = number of nonempty columns (column sums of squares > 0)
     CK(cudaMemsetAsync(h->d_s, 0, n * sizeof(double), st));
     CK(launch_aprod2(h, nullptr, h->d_s, kA2Squares, st));
@@ -291,10 +542,9 @@ static int create_mixed(gsr_handle_t *h, cudaStream_t st)
     CK(cudaMemcpyAsync(h->h_onorm, h->d_onorm, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     h->n_nonempty = h->h_onorm[0];
-    h->grid_rows32 = aprod1_f32_grid(h);
-    h->grid_rows2_32 = aprod2_f32_grid(h);
-    h->grid_fused32 = aprod2_f32_fused_grid(h);
-    if (h->grid_rows32 <= 0 || h->grid_rows2_32 <= 0 || h->grid_fused32 <= 0)
+    h->grid_main32 = f32_main_grid(h);
+    h->grid_rest32 = f32_rest_grid(h);
+    if (h->grid_main32 <= 0 || h->grid_rest32 <= 0)
         return cuda_fail(cudaGetLastError(), "mixed occupancy");
     cudaError_t e = build_cg_graph(h);
     if (e != cudaSuccess)
@@ -475,7 +725,8 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
     // instrumental part of aprod 2 and its layout
     h->ipath = instr_path(h->cfg, I);
     if (h->ipath == kIpSorted || h->cfg.precision == GSR_PREC_MIXED)
-        TRY(build_instr_sorted(h, st));
+        TRY(h->cfg.precision == GSR_PREC_MIXED && I <= kEllInstrMax ? build_ell(h, st)
+                                                                    : build_instr_sorted(h, st));
 
     // launch geometry
     // measured at the medium size: 8 lanes per star with shared-memory
@@ -498,7 +749,7 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
     h->grid_lsqr_vec = lsqr_vec_grid(h);
     if (h->grid_lsqr_vec <= 0)
         return cuda_fail(cudaGetLastError(), "vector pass occupancy");
-    if (h->ipath == kIpReplicas || (h->cfg.precision == GSR_PREC_MIXED && !instr_in_smem(h))) {
+    if (h->ipath == kIpReplicas) {
         h->nrep = h->nsm;
         TRY(dalloc(h, &h->d_irep, (int64_t)h->nrep * I));
         CK(cudaMemset(h->d_irep, 0, (size_t)h->nrep * I * sizeof(double)));
@@ -511,19 +762,17 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
         h->grid_fused = aprod2_fused_grid(h);
         if (h->grid_fused <= 0)
             return cuda_fail(cudaGetLastError(), "fused aprod2 occupancy");
-        // star units of the FP64 and of the binary32 (4 stars each) launches
-        int64_t nsu = (h->sys.S + 32 / h->lanes - 1) / (32 / h->lanes);
-        const int64_t nsu32 = (h->sys.S + 3) / 4;
-        if (nsu32 > nsu)
-            nsu = nsu32;
+        const int64_t nsu = (h->sys.S + 32 / h->lanes - 1) / (32 / h->lanes);
         if (nsu > ((int64_t)1 << 30) || a2_queue(h, h->lanes).total >= ((int64_t)1 << 32))
             h->a2_fused = 0;  // bounded partials buffer; 32-bit unit indices
         else if (nsu > ngp)
             ngp = (int)nsu;
-        TRY(dalloc(h, &h->d_a2ctr, 1));
-        CK(cudaMemset(h->d_a2ctr, 0, sizeof(unsigned long long)));
     } else {
         h->a2_fused = 0;
+    }
+    if (h->ipath == kIpSorted || h->cfg.precision == GSR_PREC_MIXED) {
+        TRY(dalloc(h, &h->d_a2ctr, 1));
+        CK(cudaMemset(h->d_a2ctr, 0, sizeof(unsigned long long)));
     }
     TRY(dalloc(h, &h->d_gpart, ngp));
 
@@ -966,6 +1215,8 @@ extern "C" int gsr_set_values(void *hv, int k, const double *values, void *strea
     double *dv;
     TRY(stage(h, &h->d_ystage, h->sys.m, values, &dv, true, st));
     CK(launch_set_plane(h, k, dv, st));
+    if (h->ell_on && k >= kNAstro + kNAtt && k < kNAstro + kNAtt + kNInstr)
+        CK(launch_ell_plane(h, k - kNAstro - kNAtt, st));
     if (h->cfg.precision == GSR_PREC_MIXED)
         CK(launch_f32_plane(h, k, st));
     if (dv != values)
@@ -1091,7 +1342,7 @@ static int ensure_batched(gsr_handle_t *h, int k)
         TRY(dalloc(h, &h->d_bD, A.n * ldk));
         TRY(dalloc(h, &h->d_bZ, A.n * ldk));
         TRY(dalloc(h, &h->d_bT, A.n * ldk));
-        TRY(dalloc(h, &h->d_bS, A.nseg * kNAtt * batched_att_pieces(h) * ldk));
+        TRY(dalloc(h, &h->d_bS, h->att32.nunits * kNAtt * ldk));
         TRY(dalloc(h, &h->d_bipart, A.I * batched_instr_pieces(h) * ldk));
         TRY(dalloc(h, &h->d_bticket, A.I * ldk));
         // on the legacy stream, before the caller's: waited for below
@@ -1100,16 +1351,16 @@ static int ensure_batched(gsr_handle_t *h, int k)
         h->bk = ldk;
     }
     if (!h->d_bpartial) {
-        TRY(dalloc(h, &h->d_bcounter, kMaxBatch));
+        TRY(dalloc(h, &h->d_bcounter, 2 * kMaxBatch));
         TRY(dalloc(h, &h->d_bs, 1));
         TRY(dalloc(h, &h->d_bargs, 1));
         TRY(dalloc(h, &h->d_bnorms, 2 * kMaxBatch));
-        CK(cudaMemset(h->d_bcounter, 0, kMaxBatch * sizeof(unsigned)));
+        CK(cudaMemset(h->d_bcounter, 0, 2 * kMaxBatch * sizeof(unsigned)));
         CK(cudaStreamSynchronize(cudaStreamLegacy));
         CK(cudaMallocHost((void **)&h->h_bs, sizeof(BatchState)));
         CK(cudaMallocHost((void **)&h->h_bargs, sizeof(BatchArgs)));
         CK(cudaMallocHost((void **)&h->h_bnorms, 2 * kMaxBatch * sizeof(double)));
-        TRY(dalloc(h, &h->d_bpartial, (int64_t)kMaxBatch * kMaxPartials));
+        TRY(dalloc(h, &h->d_bpartial, (int64_t)2 * kMaxBatch * kMaxPartials));
     }
     if (h->b_graph_kt != h->b_kt || h->b_graph_lanes != h->b_lanes) {
         drop_batched_graphs(h);

@@ -13,49 +13,46 @@
 // columns spread a tile's sectors over four times the address range and its
 // products ran 1.7x slower than at 8 columns).
 //
-// Column sections:
-//   aprod 1: row-parallel, one row per lane (as the single form)
-//   aprod 2: astrometric + global: star-parallel, G lanes per star;
-//            attitude: offset-sorted copy, one warp per offset, one axis at a
-//            time (4 taps x KT columns of double-float sums per lane);
-//            instrumental: instrument-sorted copy of the whole matrix, one
-//            warp per instrument.  No atomics except the global column.
+// Column sections (Att32 layout, gsr_internal.cuh):
+//   A X with the attitude and global part of A^T Q: one pass over the
+//            offset-ordered values (k_b_main);
+//   astrometric: star-parallel, G lanes per star, in row order;
+//   instrumental: instrument-sorted copy, pieces of one instrument per warp.
+// Every sum has a fixed order: no atomics on values.
 // CG: k independent Hestenes-Stiefel recurrences with per-column scalars.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
+#include "gsr_att32.cuh"
 #include "gsr_df.cuh"
 #include "gsr_internal.cuh"
 #include "gsr_reduce.cuh"
 
 namespace gsr {
 
-// Streams and events that fork the passes of aprod 2 while the inner loop is
+// The stream and events that fork a pass of aprod 2 while the inner loop is
 // captured; they are released with the object, the graph keeps the branches.
 struct BatchSide {
-    cudaStream_t s[2] = {nullptr, nullptr};
-    cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+    cudaStream_t s = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     cudaError_t make()
     {
         cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-        for (int i = 0; i < 2 && e == cudaSuccess; i++) {
-            e = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking);
-            if (e == cudaSuccess)
-                e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
-        }
+        if (e == cudaSuccess)
+            e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+        if (e == cudaSuccess)
+            e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
         return e;
     }
     ~BatchSide()
     {
         if (fork)
             cudaEventDestroy(fork);
-        for (int i = 0; i < 2; i++) {
-            if (join[i])
-                cudaEventDestroy(join[i]);
-            if (s[i])
-                cudaStreamDestroy(s[i]);
-        }
+        if (join)
+            cudaEventDestroy(join);
+        if (s)
+            cudaStreamDestroy(s);
     }
 };
 
@@ -135,93 +132,240 @@ __device__ __forceinline__ float col_of(const typename Cols<KT>::V (&v)[Cols<KT>
 // one tile they run side by side, on a large one the blocks of a tile are
 // dispatched before those of the next and keep its panel in L2.
 
+// the products of one launch of the main kernel
+constexpr int kBA1 = 1;  // Q = A32 X
+constexpr int kBA2 = 2;  // attitude and global part of A32^T Q
+
 // ---------------------------------------------------------------------------
-// aprod 1 on KT columns: Q32[:, c0+c] = fl32(A32 X32[:, c0+c]), with
-// |Q[:, c]|^2 and alpha_c = gamma_c / |Q[:, c]|^2 (0 for a finished column).
-// Bound by the FP32 pipe (8 lane operations per product: 0.27 ms at 7.0e6
-// rows and 8 columns) and the gathers of 24 rows of X per matrix row.
+// Main pass over the offset-ordered values on KT columns, units as in
+// k_f32_main.  A1: Q32[row, c0+c] = fl32(A32 X32[:, c0+c]) with |Q[:, c]|^2
+// and alpha_c = gamma_c / |Q[:, c]|^2 (0 for a finished column); A2: the
+// attitude sums of A32^T Q into S[unit][4a + j][c] of the tile's block and
+// T[global], on the Q just formed (or on Q itself without A1).
+// The row sums take one row per lane.  The attitude sums take one output per
+// lane (tap 4a + j, column c), 12 KT of them in NI rounds: their accumulators
+// are a few registers instead of 24 KT, and a unit needs no reduction over
+// the warp.  They read the values from the tile's stage and the rows of Q
+// through shared memory, two rows per packed operation (even and odd rows are
+// two chains); the lanes of different taps start 8 rows apart, so that they
+// read different banks.
+// Bound by the FP32 pipe: 8 lane operations per product, 37 products a row
+// and column (0.47 ms at 7.0e6 rows and 8 columns with all lanes busy).
 // ---------------------------------------------------------------------------
+constexpr int kBWarps = 16;  // one block per SM
+constexpr int kBThreads = 32 * kBWarps;
+constexpr int kBStages = 2;
+constexpr int kBRow = 34;  // row stride of Q in shared memory: distinct banks, 8-byte aligned pairs
+
+// one warp's shared memory
 template <int KT>
-__global__ void __launch_bounds__(kThreads, 3)
-k_b_aprod1(SysView A, const float *__restrict__ X, float *__restrict__ Q, int c_first,
-           BatchState *bs, double *partial, unsigned *counter)
+struct alignas(128) BWarp {
+    unsigned char stage[kBStages * kAttTileBytes];
+    float x[kNAtt][KT];  // attitude rows of X of the unit
+    float q[KT][kBRow];  // Q of the tile's rows
+    uint64_t bar[kBStages];
+};
+
+// this lane's attitude sums over the rows of a tile; rows outside lo .. hi-1
+// (a tile shared with another offset) are skipped
+template <int KT, int NI, bool FULL>
+__device__ __forceinline__ void b_att_tile(const float *__restrict__ val, const BWarp<KT> &W,
+                                           int lane, int lo, int hi, f32x2 (&sh)[NI], f32x2 (&sl)[NI])
+{
+    const int g = lane / KT;
+#pragma unroll 4
+    for (int i2 = 0; i2 < 32; i2 += 2) {
+        const int rr = (i2 + 8 * g) & 31;
+        f32x2 qv = *reinterpret_cast<const f32x2 *>(&W.q[lane % KT][rr]);
+#pragma unroll
+        for (int i = 0; i < NI; i++) {
+            const int k = g + i * (32 / KT);
+            f32x2 av = *reinterpret_cast<const f32x2 *>(val + 32 * (kNAstro + (k < kNAtt ? k : 0)) + rr);
+            if (!FULL) {
+                float a0, a1;
+                unpack2(av, a0, a1);
+                av = pack2(rr >= lo && rr < hi ? a0 : 0.f, rr + 1 >= lo && rr + 1 < hi ? a1 : 0.f);
+            }
+            df_acc_v(sh[i], sl[i], v_mul(av, qv));
+        }
+    }
+}
+
+template <int KT, int MODE>
+__global__ void __launch_bounds__(kBThreads, 1)
+k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
+         double *__restrict__ Sall, double *__restrict__ T, int c_first, BatchState *bs,
+         double *partial, unsigned *counter, int *kerr)
 {
     typedef typename Cols<KT>::V V;
     constexpr int N = Cols<KT>::N;
+    constexpr bool A1 = (MODE & kBA1) != 0, A2 = (MODE & kBA2) != 0;
+    constexpr int NOUT = kNAtt * KT, NI = (NOUT + 31) / 32;
+    extern __shared__ __align__(128) unsigned char smem[];
     const int c0 = c_first + blockIdx.y * KT;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t ntiles = (A.m + 31) >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    BWarp<KT> &W = reinterpret_cast<BWarp<KT> *>(smem)[wib];
     const float *Xp = X + pidx(0, A.n, c0);  // row j of the panel at Xp + 8 j
-    V nh[N], nl[N];                          // |Q[:, c]|^2 of this thread (double-float)
+    float *Qp = Q + pidx(0, A.m, c0);
+    double *S = Sall + (int64_t)c0 * U.nunits * kNAtt;
+    const int64_t stride = (int64_t)gridDim.x * kBWarps;
+    int64_t u = blockIdx.x + (int64_t)gridDim.x * wib;
+    AttWalk<kBStages> walk(U, W.stage, W.bar, u, stride);
+    V nh[N], nl[N], gh[N], gl[N];  // |Q[:, c]|^2 and the global sums of this thread
 #pragma unroll
     for (int c = 0; c < N; c++)
-        nh[c] = nl[c] = V(0);
-    for (int64_t t = warp; t < ntiles; t += nwarps) {
-        const int64_t r = (t << 5) + lane;
-        if (r >= A.m)
-            continue;
-        const uint32_t s = star_of_row(A, t, r);
-        const uint4 rc = __ldcs(A.rec + r);
+        nh[c] = nl[c] = gh[c] = gl[c] = V(0);
+    f32x2 sh[NI], sl[NI];  // this lane's attitude sums, even and odd rows
+    bool ok = walk.d[0].ok && walk.arrived(0, kerr);
+    while (ok) {
+        const Visit v = walk.d[0];
+        if (v.first()) {
+            if (A1) {
+                for (int i = lane; i < NOUT; i += 32) {
+                    const int k = i / KT, c = i % KT;
+                    W.x[k][c] =
+                        __ldg(Xp + kPanel * (A.att0 + (k >> 2) * A.D + v.un.x + (k & 3)) + c);
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (int i = 0; i < NI; i++)
+                sh[i] = sl[i] = 0ull;
+        }
+        const uint32_t e = (v.t << 5) + lane;
+        const float *val = walk.val();  // plane k of the tile at val + 32 k
         V h[N], l[N];
 #pragma unroll
         for (int c = 0; c < N; c++)
             h[c] = l[c] = V(0);
-        const float *v = A.val32 + tidx<kNPar>(0, r);  // plane k at v + 32 k
-        const float *xs = Xp + (int64_t)kPanel * kNAstro * s;
-        const float *xa = Xp + kPanel * (A.att0 + rc.x);
+        if (e >= v.un.y && e < v.un.z) {
+            const float *vk = val + lane;
+            const uint32_t r = walk.row();
+            V ag;
+            v_bcast(ag, vk[32 * (kNPar - 1)]);
+            if constexpr (A1) {
+                // the rows of X of the star are on their way while the
+                // attitude products are formed, those of the instruments
+                // while the astrometric ones are
+                const uint4 rc = walk.rec(0);
+                const float *xs = Xp + (int64_t)kPanel * kNAstro * rc.x;
+                V xv[kNAstro][N], xi[kNInstr][N], xg[N];
 #pragma unroll
-        for (int k = 0; k < kNPar; k++) {
-            const float *xr;
-            if (k < kNAstro)
-                xr = xs + kPanel * k;
-            else if (k < kNAstro + kNAtt)
-                xr = xa + kPanel * (((k - kNAstro) >> 2) * A.D + ((k - kNAstro) & 3));
-            else if (k < kNPar - 1)
-                xr = Xp + kPanel * (A.ins0 + instr_at32(rc, k - kNAstro - kNAtt));
+                for (int k = 0; k < kNAstro; k++)
+                    load_cols<KT>(xs + kPanel * k, xv[k]);
+#pragma unroll
+                for (int k = 0; k < kNAtt; k++) {
+                    V a;
+                    v_bcast(a, vk[32 * (kNAstro + k)]);
+#pragma unroll
+                    for (int c = 0; c < N; c++)
+                        df_acc_v(h[c], l[c], v_mul(a, reinterpret_cast<const V *>(W.x[k])[c]));
+                }
+#pragma unroll
+                for (int j = 0; j < kNInstr; j++)
+                    load_cols<KT>(Xp + kPanel * (A.ins0 + instr_at32(rc, j)), xi[j]);
+#pragma unroll
+                for (int k = 0; k < kNAstro; k++) {
+                    V a;
+                    v_bcast(a, vk[32 * k]);
+#pragma unroll
+                    for (int c = 0; c < N; c++)
+                        df_acc_v(h[c], l[c], v_mul(a, xv[k][c]));
+                }
+                load_cols<KT>(Xp + kPanel * A.glb0, xg);
+#pragma unroll
+                for (int j = 0; j < kNInstr; j++) {
+                    V a;
+                    v_bcast(a, vk[32 * (17 + j)]);
+#pragma unroll
+                    for (int c = 0; c < N; c++)
+                        df_acc_v(h[c], l[c], v_mul(a, xi[j][c]));
+                }
+#pragma unroll
+                for (int c = 0; c < N; c++)
+                    df_acc_v(h[c], l[c], v_mul(ag, xg[c]));
+#pragma unroll
+                for (int c = 0; c < N; c++) {
+                    h[c] = v_add(h[c], l[c]);        // the row's q
+                    const V pq = v_mul(h[c], h[c]);  // q^2 = pq + fma(q, q, -pq) exactly
+                    df_acc_v(nh[c], nl[c], pq);
+                    nl[c] = v_add(nl[c], v_fma(h[c], h[c], v_neg(pq)));
+                }
+                store_cols<KT>(Qp + (int64_t)kPanel * r, h);
+            } else {
+                load_cols<KT>(Qp + (int64_t)kPanel * r, h);
+            }
+            if constexpr (A2) {
+#pragma unroll
+                for (int c = 0; c < N; c++)
+                    df_acc_v(gh[c], gl[c], v_mul(ag, h[c]));
+            }
+        }
+        if constexpr (A2) {
+#pragma unroll
+            for (int c = 0; c < KT; c++)
+                W.q[c][lane] = col_of<KT>(h, c);
+            __syncwarp();
+            const uint32_t b = v.t << 5;
+            if (v.un.y <= b && v.un.z >= b + 32)
+                b_att_tile<KT, NI, true>(val, W, lane, 0, 32, sh, sl);
             else
-                xr = Xp + kPanel * A.glb0;
-            V a, xv[N];
-            v_bcast(a, __ldcs(v + 32 * k));
-            load_cols<KT>(xr, xv);
+                b_att_tile<KT, NI, false>(val, W, lane, (int)(max(v.un.y, b) - b),
+                                          (int)(min(v.un.z, b + 32) - b), sh, sl);
+            if (v.last()) {
 #pragma unroll
-            for (int c = 0; c < N; c++)
-                df_acc_v(h[c], l[c], v_mul(a, xv[c]));
+                for (int i = 0; i < NI; i++) {
+                    float h0, h1, l0, l1;
+                    unpack2(sh[i], h0, h1);
+                    unpack2(sl[i], l0, l1);
+                    df_add(h0, l0, h1, l1);
+                    if (lane + 32 * i < NOUT)
+                        S[u * NOUT + lane + 32 * i] = df_to_d(h0, l0);
+                }
+            }
         }
-#pragma unroll
-        for (int c = 0; c < N; c++) {
-            h[c] = v_add(h[c], l[c]);  // the row's q
-            const V pq = v_mul(h[c], h[c]);  // q^2 = pq + fma(q, q, -pq) exactly
-            df_acc_v(nh[c], nl[c], pq);
-            nl[c] = v_add(nl[c], v_fma(h[c], h[c], v_neg(pq)));
-        }
-        store_cols<KT>(Q + pidx(r, A.m, c0), h);
+        if (v.last())
+            u += stride;
+        if (!walk.d[1].ok)
+            break;
+        walk.advance();
+        ok = walk.arrived(0, kerr);
     }
-    double nrm[KT];
+    double v[KT];
+    if constexpr (A1) {
 #pragma unroll
-    for (int c = 0; c < KT; c++)
-        nrm[c] = df_to_d(col_of<KT>(nh, c), col_of<KT>(nl, c));
-    if (grid_reduce<KT>(nrm, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
-        threadIdx.x == 0) {
+        for (int c = 0; c < KT; c++)
+            v[c] = df_to_d(col_of<KT>(nh, c), col_of<KT>(nl, c));
+        if (grid_reduce<KT, kBThreads>(v, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
+            threadIdx.x == 0) {
 #pragma unroll
-        for (int c = 0; c < KT; c++) {
-            const int cc = c0 + c;
-            bs->xi[cc] = nrm[c];
-            bs->alpha[cc] = (!bs->done[cc] && nrm[c] > 0.0) ? bs->gamma[cc] / nrm[c] : 0.0;
+            for (int c = 0; c < KT; c++) {
+                const int cc = c0 + c;
+                bs->xi[cc] = v[c];
+                bs->alpha[cc] = (!bs->done[cc] && v[c] > 0.0) ? bs->gamma[cc] / v[c] : 0.0;
+            }
+        }
+    }
+    if constexpr (A2) {
+#pragma unroll
+        for (int c = 0; c < KT; c++)
+            v[c] = df_to_d(col_of<KT>(gh, c), col_of<KT>(gl, c));
+        if (grid_reduce<KT, kBThreads>(v, partial + (int64_t)(kMaxBatch + c0) * kMaxPartials,
+                                       counter + kMaxBatch + c0) && threadIdx.x == 0) {
+#pragma unroll
+            for (int c = 0; c < KT; c++)
+                T[pidx(A.glb0, A.n, c0) + c] = v[c];
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// aprod 2, astrometric and global nonzeros on KT columns (star-parallel):
-// T[astro rows] and T[global] written (the global sums block by block in
-// block order: deterministic)
+// aprod 2, astrometric nonzeros on KT columns (star-parallel): T[astro rows]
 // ---------------------------------------------------------------------------
 template <int KT, int G>
 __global__ void __launch_bounds__(kThreads)
-k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_first,
-          double *partial, unsigned *counter)
+k_b_stars(SysView A, const float *__restrict__ sv, const float *__restrict__ Y,
+          double *__restrict__ T, int c_first)
 {
     typedef typename Cols<KT>::V V;
     constexpr int N = Cols<KT>::N;
@@ -231,10 +375,6 @@ k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_
     const int gw = (threadIdx.x & 31) / G;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    V gh[N], gl[N];
-#pragma unroll
-    for (int c = 0; c < N; c++)
-        gh[c] = gl[c] = V(0);
     for (int64_t s0 = warp * GPW; s0 < A.S; s0 += nwarps * GPW) {
         const int64_t s = s0 + gw;
         uint32_t r0 = 0, r1 = 0;
@@ -249,7 +389,7 @@ k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_
             for (int c = 0; c < N; c++)
                 ah[k][c] = al[k][c] = V(0);
         for (uint32_t r = r0 + lane; r < r1; r += G) {
-            const float *v = A.val32 + tidx<kNPar>(0, r);
+            const float *v = sv + tidx<kNAstro>(0, r);
             V yv[N];
             load_cols<KT>(Y + pidx(r, A.m, c0), yv);
 #pragma unroll
@@ -260,11 +400,6 @@ k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_
                 for (int c = 0; c < N; c++)
                     df_acc_v(ah[k][c], al[k][c], v_mul(a, yv[c]));
             }
-            V ag;
-            v_bcast(ag, __ldcs(v + 32 * 23));
-#pragma unroll
-            for (int c = 0; c < N; c++)
-                df_acc_v(gh[c], gl[c], v_mul(ag, yv[c]));
         }
         // the star's 5 KT sums over its G lanes: double-float reduce-scatter
         // of the values padded to P (value v = k KT + c), 32 at a time
@@ -291,127 +426,23 @@ k_b_stars(SysView A, const float *__restrict__ Y, double *__restrict__ T, int c_
             }
         }
     }
-    double g[KT];
-#pragma unroll
-    for (int c = 0; c < KT; c++)
-        g[c] = df_to_d(col_of<KT>(gh, c), col_of<KT>(gl, c));
-    if (grid_reduce<KT>(g, partial + (int64_t)c0 * kMaxPartials, counter + c0) &&
-        threadIdx.x == 0) {
-#pragma unroll
-        for (int c = 0; c < KT; c++)
-            T[pidx(A.glb0, A.n, c0) + c] = g[c];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// aprod 2, attitude nonzeros on KT columns: one warp per offset o, axis a and
-// piece q (np pieces of an offset's entries) sums tap j of column c into
-// S[((q nseg + o) 3 + a) 4 + j][c] of the tile's block
-// ---------------------------------------------------------------------------
-template <int KT>
-__global__ void __launch_bounds__(kThreads)
-k_b_att(SysView A, const float *__restrict__ Y, double *__restrict__ Sall, int c_first, int np)
-{
-    typedef typename Cols<KT>::V V;
-    constexpr int N = Cols<KT>::N;
-    const int c0 = c_first + blockIdx.y * KT;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const float *Yp = Y + pidx(0, A.m, c0);
-    double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
-    constexpr int NV = 4 * KT;  // sums per (offset, axis)
-    const int64_t units = A.nseg * 3 * np;
-    for (int64_t w = warp; w < units; w += nwarps) {
-        // the axes of one (piece, offset) follow each other: their second and
-        // third readings of perm and of the rows of Y hit L2
-        const int64_t qo = w / 3;
-        const int a = (int)(w - qo * 3);
-        // pieces only where an offset has hundreds of entries: 32-bit counts
-        const uint32_t q = np == 1 ? 0u : (uint32_t)qo / (uint32_t)A.nseg;
-        const int64_t o = qo - q * A.nseg;
-        const uint32_t s0 = A.seg[o];
-        const uint64_t len = A.seg[o + 1] - s0;
-        const uint32_t e0 = s0 + (uint32_t)(len * q / np);
-        const uint32_t e1 = s0 + (uint32_t)(len * (q + 1) / np);
-        V h[4][N], l[4][N];
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int c = 0; c < N; c++)
-                h[j][c] = l[j][c] = V(0);
-        // two entries per lane in flight (the row index, then the row of Y,
-        // is a chain of two dependent loads); the sums take the entries in
-        // the same order as one at a time
-        uint32_t e = e0 + lane;
-        for (; e + 32 < e1; e += 64) {
-            const uint32_t ra = __ldcs(A.perm + e), rb = __ldcs(A.perm + e + 32);
-            float va[4], vb[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                va[j] = __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e));
-                vb[j] = __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e + 32));
-            }
-            V ya[N], yb[N];
-            load_cols<KT>(Yp + (int64_t)kPanel * ra, ya);
-            load_cols<KT>(Yp + (int64_t)kPanel * rb, yb);
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                V av;
-                v_bcast(av, va[j]);
-#pragma unroll
-                for (int c = 0; c < N; c++)
-                    df_acc_v(h[j][c], l[j][c], v_mul(av, ya[c]));
-            }
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                V av;
-                v_bcast(av, vb[j]);
-#pragma unroll
-                for (int c = 0; c < N; c++)
-                    df_acc_v(h[j][c], l[j][c], v_mul(av, yb[c]));
-            }
-        }
-        if (e < e1) {
-            V yv[N];
-            load_cols<KT>(Yp + (int64_t)kPanel * __ldcs(A.perm + e), yv);
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                V av;
-                v_bcast(av, __ldcs(A.tval32 + tidx<kNAtt>(4 * a + j, e)));
-#pragma unroll
-                for (int c = 0; c < N; c++)
-                    df_acc_v(h[j][c], l[j][c], v_mul(av, yv[c]));
-            }
-        }
-        // double-float reduce-scatter of the NV sums (a power of two <= 32)
-        // over the warp: lane l ends with the total of index l / (32 / NV)
-        float rh[NV], rl[NV];
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            rh[k] = col_of<KT>(h[k / KT], k % KT);
-            rl[k] = col_of<KT>(l[k / KT], k % KT);
-        }
-        df_reduce_scatter<NV, 32>(rh, rl, lane);
-        constexpr int REST = 32 / NV;
-        if ((lane % REST) == 0)
-            S[(qo * 3 + a) * NV + lane / REST] = df_to_d(rh[0], rl[0]);
-    }
 }
 
 // attitude column colrow = a D + k of T, column c of the tile whose sums are S
 template <int KT>
-__device__ __forceinline__ double att_total(const SysView &A, const double *__restrict__ S,
-                                            int np, int64_t colrow, int c)
+__device__ __forceinline__ double att_total(const SysView &A, const uint32_t *__restrict__ useg,
+                                            const double *__restrict__ S, int64_t colrow, int c)
 {
     const int64_t a = (colrow >= A.D) + (colrow >= 2 * A.D), k = colrow - a * A.D;
     double t = 0.0;
-    for (int q = 0; q < np; q++) {
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int64_t o = k - j;
-            if (o >= 0 && o < A.nseg)
-                t += S[((((int64_t)q * A.nseg + o) * 3 + a) * 4 + j) * KT + c];
+    for (int j = 0; j < 4; j++) {
+        const int64_t o = k - j;
+        if (o >= 0 && o < A.nseg) {
+            const uint32_t u0 = __ldg(useg + o), u1 = __ldg(useg + o + 1);
+#pragma unroll 4
+            for (uint32_t u = u0; u < u1; u++)
+                t += S[((int64_t)u * kNAtt + 4 * a + j) * KT + c];
         }
     }
     return t;
@@ -419,17 +450,17 @@ __device__ __forceinline__ double att_total(const SysView &A, const double *__re
 
 // attitude columns of T (products alone; the CG pass combines them itself)
 template <int KT>
-__global__ void k_b_att_combine(SysView A, const double *__restrict__ Sall, double *__restrict__ T,
-                                int c_first, int np)
+__global__ void k_b_att_combine(SysView A, Att32 U, const double *__restrict__ Sall,
+                                double *__restrict__ T, int c_first)
 {
     const int c0 = c_first + blockIdx.y * KT;
-    const double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
+    const double *S = Sall + (int64_t)c0 * U.nunits * kNAtt;
     const int64_t total = 3 * A.D * KT;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(i % KT);
         const int64_t colrow = i / KT;  // a * D + k
-        T[pidx(A.att0 + colrow, A.n, c0) + c] = att_total<KT>(A, S, np, colrow, c);
+        T[pidx(A.att0 + colrow, A.n, c0) + c] = att_total<KT>(A, U.useg, S, colrow, c);
     }
 }
 
@@ -455,8 +486,11 @@ k_b_instr(SysView A, const uint32_t *__restrict__ iseg, const uint32_t *__restri
     double *part = part_all + (int64_t)c0 * A.I * np;
     unsigned *ticket = ticket_all + (int64_t)c0 * A.I;
     for (uint32_t wi = (uint32_t)warp; wi < (uint32_t)A.I * np; wi += (uint32_t)nwarps) {
-        const uint32_t f = wi / np;
-        const uint32_t q = wi - f * np;
+        // piece-major: at any time the warps take one quantile of every
+        // instrument's rows, so their gathers stay within about 1/np of Y
+        // (which need not fit in L2: 224 MB at 7.0e6 rows and 8 columns)
+        const uint32_t q = wi / (uint32_t)A.I;
+        const uint32_t f = wi - q * (uint32_t)A.I;
         const uint32_t s0 = iseg[f];
         const uint64_t len = iseg[f + 1] - s0;
         const uint32_t e0 = s0 + (uint32_t)(len * q / np);
@@ -629,21 +663,21 @@ k_b_init(const double *__restrict__ p, const double *__restrict__ C, double *__r
 // attitude columns of T come from the segment sums Sall
 template <int KT>
 __global__ void __launch_bounds__(kThreads)
-k_b_vec1(SysView A, const double *__restrict__ p, const double *__restrict__ T,
-         const double *__restrict__ Sall, int np, double *__restrict__ Sv,
+k_b_vec1(SysView A, Att32 U, const double *__restrict__ p, const double *__restrict__ T,
+         const double *__restrict__ Sall, double *__restrict__ Sv,
          const double *__restrict__ Dd, double *__restrict__ Z, int c_first, BatchState *bs,
          const BatchArgs *args, double *partial, unsigned *counter)
 {
     const int c0 = c_first + blockIdx.y * KT;
     const int c = threadIdx.x % KT;
     const int64_t base = pidx(0, A.n, c0);
-    const double *S = Sall + (int64_t)c0 * A.nseg * kNAtt * np;
+    const double *S = Sall + (int64_t)c0 * U.nunits * kNAtt;
     const double al = bs->alpha[c0 + c];
     double acc = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n * KT;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = i / KT, e = base + j * kPanel + c;
-        const double tj = (j < A.att0 || j >= A.ins0) ? T[e] : att_total<KT>(A, S, np, j - A.att0, c);
+        const double tj = (j < A.att0 || j >= A.ins0) ? T[e] : att_total<KT>(A, U.useg, S, j - A.att0, c);
         const double sj = fma(-al, p[j] * tj, Sv[e]);
         Sv[e] = sj;
         Z[e] = fma(al, Dd[e], Z[e]);
@@ -794,15 +828,6 @@ static int b_occ(F f)
     return occ;
 }
 
-// pieces per attitude offset: one up to a mean of 512 entries (as many as one
-// warp takes in 8 steps), so that few long offsets still give every SM work
-int batched_att_pieces(const gsr_handle_t *h)
-{
-    const int64_t mean = h->sys.m / h->sys.nseg;
-    const int64_t np = (mean + 511) / 512;
-    return (int)(np < 1 ? 1 : (np > 64 ? 64 : np));
-}
-
 // pieces per instrument: about 2048 entries each
 int batched_instr_pieces(const gsr_handle_t *h)
 {
@@ -811,13 +836,19 @@ int batched_instr_pieces(const gsr_handle_t *h)
     return (int)(np < 1 ? 1 : (np > 256 ? 256 : np));
 }
 
-template <int KT>
-static cudaError_t b_aprod1(const gsr_handle_t *h, const float *X, float *Q, int c0, int ny,
-                            cudaStream_t st)
+template <int KT, int MODE>
+static cudaError_t b_main(const gsr_handle_t *h, const float *X, float *Q, double *T, int c0, int ny,
+                          cudaStream_t st)
 {
-    const int occ = b_occ(k_b_aprod1<KT>);
-    k_b_aprod1<KT><<<dim3(b_blocks(h, occ, (h->sys.m + 31) / 32), ny), kThreads, 0, st>>>(
-        h->sys, X, Q, c0, h->d_bs, h->d_bpartial, h->d_bcounter);
+    constexpr size_t smem = kBWarps * sizeof(BWarp<KT>);
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_b_main<KT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    const int gx = (int)(h->att32.nunits < h->nsm ? h->att32.nunits : h->nsm);
+    k_b_main<KT, MODE><<<dim3(gx, ny), kBThreads, smem, st>>>(h->sys, h->att32, X, Q, h->d_bS, T, c0,
+                                                              h->d_bs, h->d_bpartial,
+                                                              h->d_bcounter, h->d_kerr);
     return cudaGetLastError();
 }
 
@@ -827,51 +858,42 @@ static void b_stars(const gsr_handle_t *h, const float *Y, double *T, int c0, in
 {
     const int occ = b_occ(k_b_stars<KT, G>);
     const int gx = b_blocks(h, occ, (h->sys.S + 32 / G - 1) / (32 / G));
-    k_b_stars<KT, G><<<dim3(gx, ny), kThreads, 0, st>>>(h->sys, Y, T, c0, h->d_bpartial,
-                                                        h->d_bcounter);
+    k_b_stars<KT, G><<<dim3(gx, ny), kThreads, 0, st>>>(h->sys, h->att32.sv, Y, T, c0);
 }
 
-// The three passes of aprod 2 write different sums and run side by side when
-// side streams are given (graph capture): one bound by its gathers shares the
-// SMs with one bound by the FP32 pipe.
+// The star and instrument passes write different sums and run side by side
+// when a side stream is given (graph capture): one bound by its gathers
+// shares the SMs with one bound by the FP32 pipe.
 template <int KT>
-static cudaError_t b_aprod2(const gsr_handle_t *h, const float *Y, double *T, int c0, int ny,
-                            cudaStream_t st, const BatchSide *side)
+static cudaError_t b_rest(const gsr_handle_t *h, const float *Y, double *T, int c0, int ny,
+                          cudaStream_t st, const BatchSide *side)
 {
-    cudaStream_t sa = st, si = st;
+    cudaStream_t si = st;
     cudaError_t e = cudaSuccess;
     if (side) {
-        sa = side->s[0];
-        si = side->s[1];
+        si = side->s;
         e = cudaEventRecord(side->fork, st);
-        if (e == cudaSuccess)
-            e = cudaStreamWaitEvent(sa, side->fork, 0);
         if (e == cudaSuccess)
             e = cudaStreamWaitEvent(si, side->fork, 0);
         if (e != cudaSuccess)
             return e;
     }
-    const int occ_a = b_occ(k_b_att<KT>), occ_i = b_occ(k_b_instr<KT>);
-    const int npa = batched_att_pieces(h), npi = batched_instr_pieces(h);
+    const int occ_i = b_occ(k_b_instr<KT>);
+    const int npi = batched_instr_pieces(h);
     k_b_instr<KT><<<dim3(b_blocks(h, 2 * occ_i, h->sys.I * npi), ny), kThreads, 0, si>>>(
         h->sys, h->d_iseg, h->d_irow, h->d_ival32, Y, h->d_bipart, h->d_bticket, T, c0, npi);
-    k_b_att<KT><<<dim3(b_blocks(h, 4 * occ_a, h->sys.nseg * 3 * npa), ny), kThreads, 0, sa>>>(
-        h->sys, Y, h->d_bS, c0, npa);
     switch (h->b_lanes) {
     case 8: b_stars<KT, 8>(h, Y, T, c0, ny, st); break;
     case 32: b_stars<KT, 32>(h, Y, T, c0, ny, st); break;
     default: b_stars<KT, 16>(h, Y, T, c0, ny, st); break;
     }
-    if (side) {
-        for (int i = 0; i < 2 && e == cudaSuccess; i++) {
-            e = cudaEventRecord(side->join[i], side->s[i]);
-            if (e == cudaSuccess)
-                e = cudaStreamWaitEvent(st, side->join[i], 0);
-        }
-        if (e != cudaSuccess)
-            return e;
+    e = cudaGetLastError();
+    if (side && e == cudaSuccess) {
+        e = cudaEventRecord(side->join, si);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(st, side->join, 0);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 template <int KT>
@@ -892,15 +914,16 @@ static cudaError_t b_prologue_tiles(const gsr_handle_t *h, int c0, int ny, cudaS
 }
 
 template <int KT>
-static cudaError_t b_products_tiles(const gsr_handle_t *h, const float *X, float *Q, const float *Y,
+static cudaError_t b_products_tiles(const gsr_handle_t *h, const float *X, float *Q, float *Y,
                                     double *T, int c0, int ny, cudaStream_t s)
 {
-    cudaError_t e = b_aprod1<KT>(h, X, Q, c0, ny, s);
+    cudaError_t e = b_main<KT, kBA1>(h, X, Q, T, c0, ny, s);
     if (e == cudaSuccess)
-        e = b_aprod2<KT>(h, Y, T, c0, ny, s, nullptr);
+        e = b_main<KT, kBA2>(h, nullptr, Y, T, c0, ny, s);
+    if (e == cudaSuccess)
+        e = b_rest<KT>(h, Y, T, c0, ny, s, nullptr);
     if (e == cudaSuccess) {
-        k_b_att_combine<KT><<<dim3(h->nsm, ny), kThreads, 0, s>>>(h->sys, h->d_bS, T, c0,
-                                                                  batched_att_pieces(h));
+        k_b_att_combine<KT><<<dim3(h->nsm, ny), kThreads, 0, s>>>(h->sys, h->att32, h->d_bS, T, c0);
         e = cudaGetLastError();
     }
     return e;
@@ -911,38 +934,40 @@ static cudaError_t b_iteration_tiles(const gsr_handle_t *h, int c0, int ny, cuda
                                      cudaGraphConditionalHandle loop, int in_graph, int last,
                                      const BatchSide *side)
 {
-    cudaError_t e = b_aprod1<KT>(h, h->d_bX32, h->d_bQ32, c0, ny, s);
+    cudaError_t e = b_main<KT, kBA1 | kBA2>(h, h->d_bX32, h->d_bQ32, h->d_bT, c0, ny, s);
     if (e == cudaSuccess)
-        e = b_aprod2<KT>(h, h->d_bQ32, h->d_bT, c0, ny, s, side);
+        e = b_rest<KT>(h, h->d_bQ32, h->d_bT, c0, ny, s, side);
     if (e != cudaSuccess)
         return e;
     const dim3 g(vec_blocks<KT>(h), ny);
-    k_b_vec1<KT><<<g, kThreads, 0, s>>>(h->sys, h->d_p, h->d_bT, h->d_bS, batched_att_pieces(h),
-                                        h->d_bS_, h->d_bD, h->d_bZ, c0, h->d_bs, h->d_bargs,
-                                        h->d_bpartial, h->d_bcounter);
+    k_b_vec1<KT><<<g, kThreads, 0, s>>>(h->sys, h->att32, h->d_p, h->d_bT, h->d_bS, h->d_bS_,
+                                        h->d_bD, h->d_bZ, c0, h->d_bs, h->d_bargs, h->d_bpartial,
+                                        h->d_bcounter);
     k_b_vec2<KT><<<g, kThreads, 0, s>>>(h->d_p, h->d_bS_, h->d_bD, h->d_bX32, h->sys.n, c0, h->d_bs,
                                         k, loop, in_graph, last);
     return cudaGetLastError();
 }
 
 // The k columns as runs of equal tiles: whole tiles of the chosen width, then
-// the rest in tiles of at most that width (11 columns at width 8: one tile of
-// 8, one of 2, one of 1), so no column of padding is computed.  f(kt, c0, ny)
-// per run; the last run is told.
+// the rest in one tile of the least width that holds it (its further columns
+// are zero: 19 columns at width 8 are two tiles of 8 and one of 4).
+// f(kt, c0, ny) per run; the last run is told.
 template <typename F>
 static cudaError_t for_runs(const gsr_handle_t *h, int k, F f)
 {
-    int c0 = 0;
-    for (int kt = h->b_kt; kt >= 1; kt >>= 1) {
-        const int ny = (k - c0) / kt;
-        if (ny > 0) {
-            cudaError_t e = f(kt, c0, ny, c0 + ny * kt == k);
-            if (e != cudaSuccess)
-                return e;
-            c0 += ny * kt;
-        }
+    const int whole = k / h->b_kt;
+    if (whole > 0) {
+        const cudaError_t e = f(h->b_kt, 0, whole, whole * h->b_kt == k);
+        if (e != cudaSuccess)
+            return e;
     }
-    return cudaSuccess;
+    const int rest = k - whole * h->b_kt;
+    if (rest == 0)
+        return cudaSuccess;
+    int kt = 1;
+    while (kt < rest)
+        kt *= 2;
+    return f(kt, whole * h->b_kt, 1, true);
 }
 
 // the inner solve of the k columns: prologue, then iterations until every
@@ -1058,7 +1083,7 @@ cudaError_t launch_b_update_x(const gsr_handle_t *h, double *X, int k, cudaStrea
 
 // single products on the binary32 copy for k columns (panelled blocks),
 // for the parity tests and the tuner: Q = A32 X and T = A32^T Y
-cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, const float *Y,
+cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, float *Y,
                               double *T, cudaStream_t st)
 {
     return for_runs(h, k, [&](int kt, int c0, int ny, bool) {

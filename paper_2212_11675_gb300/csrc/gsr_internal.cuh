@@ -23,8 +23,6 @@ struct SysView {
     const uint32_t *star_ptr;  // [S+1]
     const uint4 *rec;          // [m]
     const double *val;         // 24 value planes, tiled (tidx<24>; plane k = nonzero k)
-    const float *val32;        // binary32 copy (mixed precision), same tiling, or null
-    const float *tval32;       // binary32 offset-sorted attitude copy (tidx<12>), or null
     const uint32_t *tile_star; // [ceil(m/32)] star of the first row of each 32-row tile
     const uint16_t *sdelta;    // [m] star of row r minus tile_star[r/32]; 0xffff: walk on
     const uint32_t *sorder;    // [S] stars by decreasing row count (star groups of aprod 2)
@@ -38,6 +36,29 @@ struct SysView {
     int64_t att0, ins0, glb0;  // first column of each section
     int64_t nseg;              // D-3 attitude offsets
 };
+
+// Binary32 layout of the mixed and batched forms.  All 24 values of a row sit
+// in the order of the attitude copy (entry e is row perm[e]), so the rows that
+// a warp takes share their attitude offset: the 12 attitude unknowns of x are
+// the same for the whole warp and its attitude sums of A^T q stay in
+// registers, which lets one pass over the values serve A x and the attitude
+// part of A^T (A x).  A unit is a run of a few 32-entry tiles of one offset
+// (its first and last tile may be shared with the neighbouring offset), so
+// the units are of like size whatever the offsets hold.
+struct Att32 {
+    // per 32 entries one block of kAttTileBytes: the 24 value planes (32
+    // floats each), the records (star, then the instrument words of
+    // SysView::rec) and the rows, so that one bulk copy stages a tile
+    const unsigned char *tile;
+    const uint4 *unit;     // [nunits] offset, first entry, last entry + 1, 0
+    const uint32_t *useg;  // [nseg+1] units of offset o: useg[o] .. useg[o+1]-1
+    const float *sv;       // the 5 astrometric planes in row order (tidx<5>)
+    int64_t nunits;
+};
+constexpr uint32_t kAttRecAt = 32 * kNPar * sizeof(float);               // 3072
+constexpr uint32_t kAttRowAt = kAttRecAt + 32 * sizeof(uint4);           // 3584
+constexpr uint32_t kAttTileBytes = kAttRowAt + 32 * sizeof(uint32_t);    // 3712
+constexpr int kUnitTiles = 8;  // at most; fewer where that leaves warps without a unit
 
 // The value planes are stored in tiles of 32 rows (or sorted entries): tile
 // t holds the K planes of its rows contiguously, plane k of the tile being
@@ -66,16 +87,41 @@ __device__ __forceinline__ uint32_t star_of_row(const SysView &A, int64_t t, int
     return s;
 }
 
+// Instrumental nonzeros in row windows (gsr_ell.cu): slices of 32 columns, the
+// entries of slice s at (slice[s].x + i) * 32 + lane for i < slice[s].y
+// (a multiple of kEllStep).
+constexpr uint32_t kEllRowBits = 13;
+constexpr uint32_t kEllRowMask = (1u << kEllRowBits) - 1;
+constexpr uint32_t kEllPad = kEllRowMask;     // window row of a padding entry (y = 0)
+constexpr uint32_t kEllNone = 0xffffffffu;    // no column in this lane
+constexpr uint32_t kEllFirst = 0x80000000u;   // flag of a partial: the block's first column of it
+constexpr int kEllLen = 64;                   // entries per column at most
+constexpr int kEllStep = 8;                   // entries loaded at a time
+constexpr int64_t kEllRowsMax = 8160;         // rows per window at most
+constexpr int64_t kEllInstrMax = 6144;
+struct Ell {
+    const uint16_t *idx;  // row of the window | slot << kEllRowBits
+    const float *val32;
+    const uint2 *slice;
+    const uint32_t *win;  // [nwin+1] slices of each window
+    const uint32_t *pos;  // [32 slices] partial of each column, with kEllFirst
+    const uint32_t *ptr;  // [I+1] partials of instrument f: ptr[f] .. ptr[f+1]-1
+    double *part;
+    int64_t nwin, W;      // windows, rows per window
+    int64_t nblk;         // block b takes windows b, b + nblk, ...
+};
+
 // Partial sums of the single-launch aprod 2 that a following vector pass
 // combines itself (no combine launch): attitude segment sums S, instrument window
 // totals, per-star-unit global partials, and the work counter to reset.
 struct A2Parts {
     const double *S;
     const double *ipart;
-    int isplit;
+    int isplit;  // 0: the instrumental sums are in the row windows' partials
     const double *gpart;
     int ngpart;
     unsigned long long *ctr;
+    Ell ell;
 };
 
 // q_j of the non-astrometric columns from the partial sums: column a D + k of
@@ -218,14 +264,27 @@ struct gsr_handle_t {
     // into ks32 pieces; partial sums at d_ipart[(q ks32 + k) I + f]
     uint32_t *d_cseg32 = nullptr;       // [nq32+1][I] window bounds as d_cseg
     int nq32 = 1, ks32 = 1;
+    // row windows of the binary32 form where I <= kEllInstrMax
+    gsr::Ell ell = {};
+    bool ell_on = false;
+    uint16_t *d_eidx = nullptr;
+    double *d_epart = nullptr;
+    float *d_eval32 = nullptr;
+    uint2 *d_eslice = nullptr;
+    uint32_t *d_ewin = nullptr, *d_epos = nullptr, *d_eptr = nullptr;
     double *d_gpart = nullptr;          // per-block partials of the global column (star pass)
     int a2_fused = 1;                   // aprod 2 in one launch (sorted path), else separate passes
     unsigned long long *d_a2ctr = nullptr;  // work counter of the single-launch aprod 2
     int grid_fused = 0;
     // mixed precision
-    float *d_val32 = nullptr, *d_tval32 = nullptr;
+    gsr::Att32 att32 = {};
+    unsigned char *d_atile = nullptr;
+    float *d_sv32 = nullptr;
+    uint4 *d_unit = nullptr;
+    uint32_t *d_useg = nullptr;
+    double *d_attS32 = nullptr;         // [nunits][12] attitude sums of the units
     float *d_x32 = nullptr, *d_q32 = nullptr;
-    float *d_xatt4 = nullptr;           // [3D][4] attitude part of x32 as one float4 per offset
+    float *d_x8 = nullptr;              // [S][8] astrometric part of x32, one sector per star
     double *d_c = nullptr, *d_s = nullptr, *d_d = nullptr, *d_t = nullptr, *d_zc = nullptr;
     double *d_xm = nullptr, *d_r = nullptr, *d_xneg = nullptr, *d_onorm = nullptr;
     gsr::CgState *d_cg = nullptr, *h_cg = nullptr;
@@ -251,7 +310,7 @@ struct gsr_handle_t {
     cudaGraphExec_t b_exec[gsr::kMaxBatch + 1] = {};  // inner solve of k columns
     int b_kt = 8, b_lanes = 16, b_graph_kt = 0, b_graph_lanes = 0;  // the graphs' tiling
     double *d_xp64 = nullptr, *d_q64 = nullptr;
-    int grid_rows32 = 0, grid_rows2_32 = 0, grid_fused32 = 0;
+    int grid_main32 = 0, grid_rest32 = 0;
     double n_nonempty = 0.0;
     double *d_p = nullptr;              // preconditioner
     double *d_u = nullptr;              // m
@@ -294,11 +353,10 @@ cudaError_t launch_f32_plane(const gsr_handle_t *h, int k, cudaStream_t st);
 cudaError_t build_batched_graph(gsr_handle_t *h, int k);
 cudaError_t run_batched_inner(gsr_handle_t *h, int k, int max_inner, cudaStream_t st);
 cudaError_t launch_b_update_x(const gsr_handle_t *h, double *X, int k, cudaStream_t st);
-cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, const float *Y,
+cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, float *Y,
                               double *T, cudaStream_t st);
 cudaError_t launch_b_layout(const gsr_handle_t *h, int to_rm, const double *src, void *dst,
                             int dst_f32, int64_t rows, int k, cudaStream_t st);
-int batched_att_pieces(const gsr_handle_t *h);
 int batched_instr_pieces(const gsr_handle_t *h);
 cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out,
                           int mode, cudaStream_t st);
@@ -318,17 +376,21 @@ bool aprod1_split(const gsr_handle_t *h);
 int split_request(const gsr_config &cfg);
 int aprod2_split(const gsr_handle_t *h);
 int aprod2_split_active(const gsr_handle_t *h);
-bool instr_in_smem(const gsr_handle_t *h);
 cudaError_t launch_att_combine(const gsr_handle_t *h, double *out, int nb_att, int nb_ins,
                                double *rep, int nrep, const double *gpart, int ngpart,
                                bool accumulate, cudaStream_t st, unsigned long long *ctr = nullptr);
 int instr_path(const gsr_config &cfg, int64_t I);
-A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units = -1);
+A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units = -1, int64_t natt = -1);
 bool aprod2_partials(const gsr_handle_t *h, const double *y, double *out, const double **S,
                      const double **ipart, int *isplit, const double **gpart, int *ngpart,
                      unsigned long long **ctr, cudaStream_t st);
 cudaError_t launch_gather_instr64(const gsr_handle_t *h, const uint32_t *code, double *out,
                                   cudaStream_t st);
+// instrument pass over row windows (gsr_ell.cu)
+cudaError_t launch_ell_fill(const gsr_handle_t *h, const uint32_t *code, int64_t total,
+                            cudaStream_t st);
+cudaError_t launch_ell_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
+cudaError_t launch_ell_sorted(const gsr_handle_t *h, const uint32_t *start, cudaStream_t st);
 // mixed precision (gsr_mixed.cu)
 cudaError_t launch_aprod1_f32_api(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
 cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double *x, cudaStream_t st);
@@ -341,9 +403,9 @@ cudaError_t launch_norms2(const gsr_handle_t *h, const double *c, const double *
 cudaError_t launch_neg(const gsr_handle_t *h, const double *a, double *b, int64_t n, cudaStream_t st);
 cudaError_t launch_count_pos(const gsr_handle_t *h, const double *a, double *out, cudaStream_t st);
 cudaError_t launch_to_f32(const gsr_handle_t *h, const double *a, float *b, int64_t n, cudaStream_t st);
-int aprod1_f32_grid(const gsr_handle_t *h);
-int aprod2_f32_grid(const gsr_handle_t *h);
-int aprod2_f32_fused_grid(const gsr_handle_t *h);
+cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st);
+int f32_main_grid(const gsr_handle_t *h);
+int f32_rest_grid(const gsr_handle_t *h);
 cudaError_t enqueue_precondition(const gsr_handle_t *h, double *p, cudaStream_t st);
 // LSQR pieces (gsr_lsqr.cu)
 cudaError_t build_solve_graph(gsr_handle_t *h);

@@ -34,6 +34,7 @@
 #include "gsr_internal.cuh"
 #include "gsr_reduce.cuh"
 #include "gsr_split.cuh"
+#include "gsr_tma.cuh"
 
 namespace gsr {
 
@@ -357,7 +358,6 @@ constexpr uint32_t kTileDeltaBytes = 32 * sizeof(uint16_t);         // 64
 constexpr uint32_t kTileBytes = kTileValBytes + kTileRecBytes + kTileDeltaBytes;
 constexpr uint32_t kTileYBytes = 32 * sizeof(double);               // 256
 constexpr uint32_t kStageBytes = (kTileBytes + kTileYBytes + 127) / 128 * 128;  // 7040
-constexpr uint64_t kWaitNs = 1000000000ull;                         // 1 s
 
 // block shape of the staged form, measured on the medium workload (in-solve
 // aprod 1, ms): 18 warps with one stage each and y staged 0.305; 20 warps
@@ -377,38 +377,6 @@ constexpr size_t tma_smem_bytes(int64_t I)
            (size_t)kTmaWarps * kTmaStages * (kStageBytes + sizeof(uint64_t));
 }
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t global_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// true when the mbarrier at bar completed the phase with this parity within
-// kWaitNs
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t done = 0;
-    uint64_t t0 = 0;
-    for (int it = 0; !done; it++) {
-        asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; "
-                     "selp.u32 %0, 1, 0, p; }"
-                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done)
-            break;
-        if (it == 0)
-            t0 = global_ns();
-        else if (global_ns() - t0 > kWaitNs)
-            return false;
-    }
-    return true;
-}
-
 // lane 0 of the warp: stage tile t (values, records, star deltas) into the
 // stage at sbase, completing on the mbarrier bar.  drop: a test hook, the
 // tile whose copies are announced to the barrier but never issued (its wait
@@ -416,22 +384,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ void tma_stage_tile(const SysView &A, int64_t t, uint32_t sbase,
                                                uint32_t bar, int64_t drop, const double *ys)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                 "r"(kTileBytes + (ys ? kTileYBytes : 0u)) : "memory");
+    mbar_expect(bar, kTileBytes + (ys ? kTileYBytes : 0u));
     if (t == drop)
         return;
     if (ys)
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(sbase + kTileBytes), "l"(ys + t * 32), "r"(kTileYBytes), "r"(bar)
-                     : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(sbase), "l"(A.val + t * 32 * kNPar), "r"(kTileValBytes), "r"(bar) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(sbase + kTileValBytes), "l"(A.rec + t * 32), "r"(kTileRecBytes), "r"(bar)
-                 : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(sbase + kTileValBytes + kTileRecBytes), "l"(A.sdelta + t * 32),
-                 "r"(kTileDeltaBytes), "r"(bar) : "memory");
+        bulk_copy(sbase + kTileBytes, ys + t * 32, kTileYBytes, bar);
+    bulk_copy(sbase, A.val + t * 32 * kNPar, kTileValBytes, bar);
+    bulk_copy(sbase + kTileValBytes, A.rec + t * 32, kTileRecBytes, bar);
+    bulk_copy(sbase + kTileValBytes + kTileRecBytes, A.sdelta + t * 32, kTileDeltaBytes, bar);
 }
 
 template <int MODE, bool ASTRO>
@@ -467,7 +427,7 @@ k_aprod1_tma(SysView A, const double *__restrict__ x, double *__restrict__ y, So
     const uint32_t sb0 = smem_addr(my);
     if (lane == 0) {
         for (int j = 0; j < NS; j++)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * j) : "memory");
+            mbar_init(bar0 + 8 * j);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();  // x pieces and barriers ready
@@ -1480,14 +1440,6 @@ cudaError_t launch_aprod1_with_slots(const gsr_handle_t *h, const double *x, dou
     return a1_launch<1>(h, x, y, st_slot, partial, counter, st);
 }
 
-// shared-memory instrument sums of the binary32 star pass
-bool instr_in_smem(const gsr_handle_t *h)
-{
-    if (h->cfg.instr_mode == GSR_INSTR_REPLICAS)
-        return false;
-    return h->sys.I <= kSmemInstrMax;
-}
-
 int instr_path(const gsr_config &cfg, int64_t I)
 {
     switch (cfg.instr_mode) {
@@ -1568,7 +1520,8 @@ static cudaError_t launch_aprod2_split(const gsr_handle_t *h, const double *y, d
 // attitude segment at the medium size)
 constexpr int kStarGroupsPerUnit = 4;
 
-A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units)
+// (natt: the attitude units, nseg by default)
+A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units, int64_t natt)
 {
     A2Queue q;
     q.ctr = h->d_a2ctr;
@@ -1576,7 +1529,7 @@ A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units)
     q.nstar_groups = (h->sys.S + 32 / G - 1) / (32 / G);
     q.nstar_units = (q.nstar_groups + q.star_k - 1) / q.star_k;
     q.ninstr_units = ninstr_units >= 0 ? ninstr_units : h->sys.I * h->isplit;
-    const int64_t n[3] = {q.nstar_units, h->sys.nseg, q.ninstr_units};
+    const int64_t n[3] = {q.nstar_units, natt >= 0 ? natt : h->sys.nseg, q.ninstr_units};
     const int64_t tot = n[0] + n[1] + n[2];
     int sl[3];
     for (int t = 0; t < 3; t++) {

@@ -28,295 +28,265 @@
 #include "gsr_internal.cuh"
 #include "gsr_reduce.cuh"
 #include "gsr_df.cuh"
+#include "gsr_att32.cuh"
+#include "gsr_ell.cuh"
 
 namespace gsr {
 
 constexpr int64_t kSmemInstrMax32 = 12288;  // binary32 instrument entries in shared memory
 
+__device__ __forceinline__ int64_t gtid32() { return blockIdx.x * (int64_t)blockDim.x + threadIdx.x; }
+__device__ __forceinline__ int64_t gstride32() { return (int64_t)gridDim.x * blockDim.x; }
+
+// the passes of the main kernel
+constexpr int kF32A1 = 1;  // q = A32 x
+constexpr int kF32A2 = 2;  // attitude and global part of A32^T q
+
 // ---------------------------------------------------------------------------
-// inner aprod 1: row-parallel, binary32 products, double-float sums.
-// MODE 0: y (FP64) += A32 x32.  MODE 1 (CG): q32 = fl32(A32 x32), |q|^2
-// reduced and alpha = gamma / |q|^2 stored by the last block.
+// Main pass of the inner operator over the offset-ordered values, one row per
+// lane (binary32 products, double-float sums).
+// A1 and A2 (CG): q32[row] = fl32(A32 x32) with |q|^2 (alpha = gamma / |q|^2
+// by the last block), the attitude sums of A32^T q into S[unit][4a + j] and
+// its global column into *glb.  A1 alone: y[row] += A32 x32 in FP64.  A2
+// alone: q is read from q32, *glb += its global column.
+// One reading of the values (96 B a row) serves both products, the row's q is
+// scattered to row order (28 MB at 7.0e6 rows: it stays in L2); the
+// astrometric x of a random star is one 32-byte sector of x8.  Bound by HBM:
+// 120 B a row.
 // ---------------------------------------------------------------------------
-template <int MODE, bool SMEMX, int U>
-__global__ void __launch_bounds__(kThreads, U == 1 ? 4 : 2)
-k_aprod1_f32(SysView A, const float *__restrict__ x32, const float4 *__restrict__ xatt4,
-             double *__restrict__ y, float *__restrict__ q32, CgState *cg, double *partial,
-             unsigned *counter)
+constexpr int kMainWarps = 16;  // one block per SM: 16 warps of three stages
+constexpr int kMainThreads = 32 * kMainWarps;
+constexpr int kMainStages = 3;
+
+// [stages][x of the attitude taps: 16 floats a warp][barriers][instrument x]
+constexpr size_t kMainSmem =
+    kMainWarps * (kMainStages * (kAttTileBytes + sizeof(uint64_t)) + 16 * sizeof(float));
+
+template <int MODE, bool SMEMX>
+__global__ void __launch_bounds__(kMainThreads, 1)
+k_f32_main(SysView A, Att32 U, const float *__restrict__ x32, const float *__restrict__ x8,
+           float *__restrict__ q32, double *__restrict__ y, double *__restrict__ S,
+           double *__restrict__ glb, CgState *cg, double *partial, unsigned *counter, int *kerr)
 {
-    extern __shared__ float s_x32[];
-    if (SMEMX) {
+    constexpr bool A1 = (MODE & kF32A1) != 0, A2 = (MODE & kF32A2) != 0;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    unsigned char *stages = smem + wib * kMainStages * kAttTileBytes;
+    float *s_xa = reinterpret_cast<float *>(smem + kMainWarps * kMainStages * kAttTileBytes) + 16 * wib;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kMainWarps * (kMainStages * kAttTileBytes +
+                                                                       16 * sizeof(float))) +
+                     kMainStages * wib;
+    float *s_x32 = reinterpret_cast<float *>(smem + kMainSmem);
+    // units are dealt to the warps of all blocks round-robin, blocks first, so
+    // that a small system spreads over the SMs
+    AttWalk<kMainStages> walk(U, stages, bars, blockIdx.x + (int64_t)gridDim.x * wib,
+                 (int64_t)gridDim.x * kMainWarps);
+    if (A1 && SMEMX) {
         for (int64_t f = threadIdx.x; f < A.I; f += blockDim.x)
             s_x32[f] = x32[A.ins0 + f];
         __syncthreads();
     }
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t ntiles = (A.m + 31) >> 5;
-    const int64_t mp = A.mp;
-    const float xg = __ldg(x32 + A.glb0);
-    float nh = 0.f, nl = 0.f;  // ||q||^2 of this thread (double-float)
-    // U tiles per step: all loads of the U rows are issued before the sums
-    for (int64_t t0 = warp; t0 < ntiles; t0 += U * nwarps) {
-        float vk[U][kNPar];
-        uint4 rc[U];
-        uint32_t st[U];
-        bool ok[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int64_t t = t0 + u * nwarps;
-            const int64_t r = (t << 5) + lane;
-            ok[u] = (t < ntiles) && (r < A.m);
-            st[u] = 0;
-            if (ok[u]) {
-                st[u] = star_of_row(A, t, r);
-                rc[u] = __ldcs(A.rec + r);
-                const float *v = A.val32 + tidx<kNPar>(0, r);  // plane k at v + 32 k
-#pragma unroll
-                for (int k = 0; k < kNPar; k++)
-                    vk[u][k] = __ldcs(v + 32 * k);
-            }
+    const float xg = A1 ? __ldg(x32 + A.glb0) : 0.f;
+    const float *xk = x32 + A.att0 + (lane >> 2) * A.D + (lane & 3);  // lane k < 12: tap k
+    float nh = 0.f, nl = 0.f;  // |q|^2 of this thread (double-float)
+    float gh = 0.f, gl = 0.f;  // its global sum
+    f32x2 sh[kNAtt / 2], sl[kNAtt / 2];  // attitude sums, taps k and k + 1 packed
+    int64_t u = blockIdx.x + (int64_t)gridDim.x * wib;
+    // astrometric x of the row (one sector), or its q, one visit ahead
+    f32x2 s01 = 0ull, s23 = 0ull;
+    float s4 = 0.f, xt = 0.f;
+    auto prefetch = [&](int j, f32x2 &a, f32x2 &b, float &c, float &x) {
+        if (A1) {
+            asm("{ .reg .b32 a, b, c, d, f, g, h, i;\n"
+                "ld.global.nc.v8.b32 {a, b, c, d, f, g, h, i}, [%3];\n"
+                "mov.b64 %0, {a, b}; mov.b64 %1, {c, d}; mov.b32 %2, f; }"
+                : "=l"(a), "=l"(b), "=f"(c) : "l"(x8 + 8 * (int64_t)walk.rec(j).x));
+            x = (lane < kNAtt && walk.d[j].first()) ? __ldg(xk + walk.d[j].un.x) : 0.f;
+        } else {
+            c = __ldg(q32 + walk.row(j));
         }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (!ok[u])
-                continue;
-            const int64_t r = ((t0 + u * nwarps) << 5) + lane;
-            float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;  // two independent pairs
-            const float *xs = x32 + (int64_t)kNAstro * st[u];
-#pragma unroll
-            for (int k = 0; k < kNAstro; k++)
-                df_acc(h0, l0, __fmul_rn(vk[u][k], __ldg(xs + k)));
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                const float4 xa = __ldg(xatt4 + a * A.D + rc[u].x);
-                df_acc(h1, l1, __fmul_rn(vk[u][5 + 4 * a + 0], xa.x));
-                df_acc(h1, l1, __fmul_rn(vk[u][5 + 4 * a + 1], xa.y));
-                df_acc(h1, l1, __fmul_rn(vk[u][5 + 4 * a + 2], xa.z));
-                df_acc(h1, l1, __fmul_rn(vk[u][5 + 4 * a + 3], xa.w));
+    };
+    bool ok = walk.d[0].ok && walk.arrived(0, kerr);
+    if (ok)
+        prefetch(0, s01, s23, s4, xt);
+    while (ok) {
+        f32x2 n01 = 0ull, n23 = 0ull;
+        float n4 = 0.f, nt = 0.f;
+        const bool more = walk.d[1].ok;
+        if (more) {
+            ok = walk.arrived(1, kerr);
+            if (ok)
+                prefetch(1, n01, n23, n4, nt);
+        }
+        const Visit v = walk.d[0];
+        if (v.first()) {
+            if (A1) {
+                if (lane < kNAtt)
+                    s_xa[lane] = xt;
+                __syncwarp();
             }
 #pragma unroll
-            for (int j = 0; j < kNInstr; j++) {
-                const uint32_t f = instr_at32(rc[u], j);
-                df_acc(h0, l0,
-                       __fmul_rn(vk[u][17 + j], SMEMX ? s_x32[f] : __ldg(x32 + A.ins0 + f)));
-            }
-            df_acc(h1, l1, __fmul_rn(vk[u][23], xg));
-            df_acc(h0, l0, h1);
-            l0 = __fadd_rn(l0, l1);
-            if (MODE == 0) {
-                y[r] += df_to_d(h0, l0);
+            for (int k = 0; k < kNAtt / 2; k++)
+                sh[k] = sl[k] = 0ull;
+        }
+        const uint32_t e = (v.t << 5) + lane;
+        if (e >= v.un.y && e < v.un.z) {
+            const float *vk = walk.val() + lane;  // plane k at vk[32 k]
+            const uint32_t r = walk.row();
+            float q;
+            if constexpr (A1) {
+                const uint4 rc = walk.rec(0);
+                float xi[kNInstr];
+#pragma unroll
+                for (int j = 0; j < kNInstr; j++) {
+                    const uint32_t f = instr_at32(rc, j);
+                    xi[j] = SMEMX ? s_x32[f] : __ldg(x32 + A.ins0 + f);
+                }
+                // the 24 products as 12 pairs: two chains of sums, packed
+                f32x2 h = 0ull, l = 0ull;
+#pragma unroll
+                for (int k = 0; k < kNAtt; k += 2)
+                    df_acc_v(h, l, v_mul(pack2(vk[32 * (5 + k)], vk[32 * (6 + k)]),
+                                         *reinterpret_cast<const f32x2 *>(s_xa + k)));
+                df_acc_v(h, l, v_mul(pack2(vk[0], vk[32]), s01));
+                df_acc_v(h, l, v_mul(pack2(vk[64], vk[96]), s23));
+                df_acc_v(h, l, v_mul(pack2(vk[128], vk[32 * 23]), pack2(s4, xg)));
+#pragma unroll
+                for (int j = 0; j < kNInstr; j += 2)
+                    df_acc_v(h, l, v_mul(pack2(vk[32 * (17 + j)], vk[32 * (18 + j)]),
+                                         pack2(xi[j], xi[j + 1])));
+                float h0, h1, l0, l1;
+                unpack2(h, h0, h1);
+                unpack2(l, l0, l1);
+                df_acc(h0, l0, h1);
+                l0 = __fadd_rn(l0, l1);
+                if constexpr (A2) {
+                    q = __fadd_rn(h0, l0);
+                    q32[r] = q;
+                    // q^2 = pq + eq exactly (product error by FMA), accumulated
+                    // in double-float on the FP32 pipe
+                    const float pq = __fmul_rn(q, q);
+                    df_acc(nh, nl, pq);
+                    nl = __fadd_rn(nl, __fmaf_rn(q, q, -pq));
+                } else {
+                    q = 0.f;
+                    y[r] += df_to_d(h0, l0);
+                }
             } else {
-                const float qv = __fadd_rn(h0, l0);
-                q32[r] = qv;
-                // q^2 = pq + eq exactly (product error by FMA), accumulated
-                // in double-float on the FP32 pipe
-                const float pq = __fmul_rn(qv, qv);
-                df_acc(nh, nl, pq);
-                nl = __fadd_rn(nl, __fmaf_rn(qv, qv, -pq));
+                q = s4;
+            }
+            if constexpr (A2) {
+                const f32x2 qq = pack2(q, q);
+#pragma unroll
+                for (int k = 0; k < kNAtt; k += 2)
+                    df_acc_v(sh[k / 2], sl[k / 2],
+                             v_mul(pack2(vk[32 * (5 + k)], vk[32 * (6 + k)]), qq));
+                df_acc(gh, gl, __fmul_rn(vk[32 * 23], q));
             }
         }
+        if (v.last()) {
+            if constexpr (A2) {
+                // reduce-scatter over the warp in double-float (FP32 pipe):
+                // after the butterfly, lane pair (2k, 2k+1) holds sum k
+                __syncwarp();
+                float rh[16], rl[16];
+#pragma unroll
+                for (int k = 0; k < 16; k += 2) {
+                    rh[k] = rh[k + 1] = rl[k] = rl[k + 1] = 0.f;
+                    if (k < kNAtt) {
+                        unpack2(sh[k / 2], rh[k], rh[k + 1]);
+                        unpack2(sl[k / 2], rl[k], rl[k + 1]);
+                    }
+                }
+                df_reduce_scatter<16, 32>(rh, rl, lane);
+                const int kk = lane >> 1;
+                if ((lane & 1) == 0 && kk < kNAtt)
+                    S[u * kNAtt + kk] = df_to_d(rh[0], rl[0]);
+            }
+            u += (int64_t)gridDim.x * kMainWarps;
+        }
+        if (!more || !ok)
+            break;
+        walk.advance();
+        s01 = n01;
+        s23 = n23;
+        s4 = n4;
+        xt = nt;
     }
-    if (MODE == 1) {
-        double v1[1] = {df_to_d(nh, nl)};
-        if (grid_reduce<1>(v1, partial, counter) && threadIdx.x == 0) {
-            const double xi = v1[0];
-            cg->xi = xi;
-            cg->alpha = (xi > 0.0) ? cg->gamma / xi : 0.0;
+    if constexpr (A2) {
+        double v2[2] = {df_to_d(nh, nl), df_to_d(gh, gl)};
+        if (grid_reduce<2, kMainThreads>(v2, partial, counter) && threadIdx.x == 0) {
+            if (A1) {
+                cg->xi = v2[0];
+                cg->alpha = (v2[0] > 0.0) ? cg->gamma / v2[0] : 0.0;
+                *glb = v2[1];
+            } else {
+                *glb += v2[1];
+            }
         }
     }
 }
 
 // ---------------------------------------------------------------------------
-// inner aprod 2, star-parallel over astrometric, instrumental and global
-// nonzeros.  MODE kA2Accumulate: out += A32^T y32.  kA2Overwrite: astro
-// part written, instrumental/global accumulated into zeroed memory.
-// Instrumental products go to per-SM replicas (FP64 reductions in L2).
+// Astrometric part of the inner aprod 2, one star group of the rest kernel:
+// G lanes per star over the row-ordered q.  MODE kA2Accumulate: out += ,
+// kA2Overwrite: written.
 // ---------------------------------------------------------------------------
-// Star-group part of warp `warp` of `nwarps` (binary32 products, double-float
-// sums): astrometric sums, instrumental products unless the sorted path
-// takes them, and this thread's share of the global column (returned).
-template <int G, int MODE, int IP>
-__device__ __forceinline__ double stars_body_f32(const SysView &A, const float *__restrict__ y32,
-                                                 double *__restrict__ out, double *myrep,
-                                                 double *s_ins, int64_t warp, int64_t nwarps)
+template <int G, int MODE>
+__device__ __forceinline__ void stars_body_f32(const SysView &A, const float *__restrict__ sv,
+                                               const float *__restrict__ y32,
+                                               double *__restrict__ out, int64_t grp)
 {
     static_assert(G >= kNAstro, "a star group needs a lane per astrometric sum");
     constexpr int GPW = 32 / G;
-    constexpr bool INS = IP != kIpSorted;
     const int lane = threadIdx.x & (G - 1);
     const int gw = (threadIdx.x & 31) / G;
-    const int64_t mp = A.mp;
-    float gh = 0.f, gl = 0.f;
-    for (int64_t s0 = warp * GPW; s0 < A.S; s0 += nwarps * GPW) {
-        // the GPW stars of a warp have similar row counts (stars taken in
-        // decreasing row count), so its lane groups finish together
-        const int64_t s = (s0 + gw < A.S) ? (int64_t)A.sorder[s0 + gw] : A.S;
-        uint32_t r0 = 0, r1 = 0;
-        if (s < A.S) {
-            r0 = A.star_ptr[s];
-            r1 = A.star_ptr[s + 1];
-        }
-        float ah[kNAstro], al[kNAstro];
+    const int64_t s0 = grp * GPW;
+    // the GPW stars of a warp have similar row counts (stars taken in
+    // decreasing row count), so its lane groups finish together
+    const int64_t s = (s0 + gw < A.S) ? (int64_t)A.sorder[s0 + gw] : A.S;
+    uint32_t r0 = 0, r1 = 0;
+    if (s < A.S) {
+        r0 = A.star_ptr[s];
+        r1 = A.star_ptr[s + 1];
+    }
+    float ah[kNAstro], al[kNAstro];
+#pragma unroll
+    for (int k = 0; k < kNAstro; k++)
+        ah[k] = al[k] = 0.f;
+#pragma unroll 2
+    for (uint32_t r = r0 + lane; r < r1; r += G) {
+        const float *v = sv + tidx<kNAstro>(0, r);
+        const float yi = __ldg(y32 + r);
 #pragma unroll
         for (int k = 0; k < kNAstro; k++)
-            ah[k] = al[k] = 0.f;
-        for (uint32_t r = r0 + lane; r < r1; r += G) {
-            const float *v = A.val32 + tidx<kNPar>(0, r);
-            const float yi = __ldcs(y32 + r);
+            df_acc(ah[k], al[k], __fmul_rn(__ldcs(v + 32 * k), yi));
+    }
+    // the star's five sums over its G lanes, in double-float
 #pragma unroll
-            for (int k = 0; k < kNAstro; k++)
-                df_acc(ah[k], al[k], __fmul_rn(__ldcs(v + 32 * k), yi));
-            if (INS) {
-                const uint4 rc = __ldcs(A.rec + r);
+    for (int off = G / 2; off > 0; off >>= 1) {
 #pragma unroll
-                for (int j = 0; j < kNInstr; j++) {
-                    const float pr = __fmul_rn(__ldcs(v + 32 * (17 + j)), yi);
-                    if (IP == kIpSmem)
-                        atomicAdd(&s_ins[instr_at32(rc, j)], f2d(pr));
-                    else
-                        atomicAdd(myrep + instr_at32(rc, j), f2d(pr));
-                }
-            }
-            df_acc(gh, gl, __fmul_rn(__ldcs(v + 32 * 23), yi));
-        }
-        // the star's five sums over its G lanes, in double-float
-#pragma unroll
-        for (int off = G / 2; off > 0; off >>= 1) {
-#pragma unroll
-            for (int k = 0; k < kNAstro; k++) {
-                const float oh = __shfl_xor_sync(0xffffffffu, ah[k], off);
-                const float ol = __shfl_xor_sync(0xffffffffu, al[k], off);
-                df_add(ah[k], al[k], oh, ol);
-            }
-        }
-        if (lane < kNAstro && s < A.S) {
-            // lane k writes sum k (all lanes of the group hold all five)
-            float kh = ah[0], kl = al[0];
-#pragma unroll
-            for (int k = 1; k < kNAstro; k++)
-                if (lane == k) {
-                    kh = ah[k];
-                    kl = al[k];
-                }
-            double *xs = out + kNAstro * s + lane;
-            if (MODE == kA2Accumulate)
-                *xs += df_to_d(kh, kl);
-            else
-                *xs = df_to_d(kh, kl);
+        for (int k = 0; k < kNAstro; k++) {
+            const float oh = __shfl_xor_sync(0xffffffffu, ah[k], off);
+            const float ol = __shfl_xor_sync(0xffffffffu, al[k], off);
+            df_add(ah[k], al[k], oh, ol);
         }
     }
-    return df_to_d(gh, gl);
-}
-
-template <int G, int MODE, bool SMEM_INSTR>
-__global__ void __launch_bounds__(kThreads)
-k_aprod2_f32_stars(SysView A, const float *__restrict__ y32, double *__restrict__ out,
-                   double *__restrict__ rep, int nrep)
-{
-    extern __shared__ double s_ins[];
-    __shared__ double s_red[kThreads / 32];
-    if (SMEM_INSTR) {
-        for (int64_t f = threadIdx.x; f < A.I; f += blockDim.x)
-            s_ins[f] = 0.0;
-        __syncthreads();
-    }
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    double *myrep = rep + (int64_t)(blockIdx.x % nrep) * A.I;
-    const double gpart = stars_body_f32<G, MODE, SMEM_INSTR ? kIpSmem : kIpReplicas>(
-        A, y32, out, myrep, s_ins, warp, nwarps);
-    double g = warp_sum(gpart);
-    if ((threadIdx.x & 31) == 0)
-        s_red[threadIdx.x >> 5] = g;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kThreads / 32; w++)
-            t += s_red[w];
-        atomicAdd(out + A.glb0, t);
-    }
-    if (SMEM_INSTR) {
-        for (int64_t f = threadIdx.x; f < A.I; f += blockDim.x) {
-            const double t = s_ins[f];
-            if (t != 0.0)
-                atomicAdd(out + A.ins0 + f, t);
-        }
-    }
-}
-
-// inner aprod 2, attitude part over the offset-sorted binary32 copy
-__device__ __forceinline__ void att_body_f32(const SysView &A, const float *__restrict__ y32,
-                                             double *__restrict__ S, int64_t warp, int64_t nwarps)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t mp = A.mp;
-    for (int64_t o = warp; o < A.nseg; o += nwarps) {
-        const uint32_t e0 = A.seg[o], e1 = A.seg[o + 1];
-        float h[kNAtt], l[kNAtt];
+    if (lane < kNAstro && s < A.S) {
+        // lane k writes sum k (all lanes of the group hold all five)
+        float kh = ah[0], kl = al[0];
 #pragma unroll
-        for (int k = 0; k < kNAtt; k++)
-            h[k] = l[k] = 0.f;
-        uint32_t e = e0 + lane;
-        for (; e + 32 < e1; e += 64) {  // two entries per lane in flight
-            const uint32_t ra = __ldcs(A.perm + e), rb = __ldcs(A.perm + e + 32);
-            float va[kNAtt], vb[kNAtt];
-#pragma unroll
-            for (int k = 0; k < kNAtt; k++) {
-                va[k] = __ldcs(A.tval32 + tidx<kNAtt>(k, e));
-                vb[k] = __ldcs(A.tval32 + tidx<kNAtt>(k, e + 32));
+        for (int k = 1; k < kNAstro; k++)
+            if (lane == k) {
+                kh = ah[k];
+                kl = al[k];
             }
-            const float ya = __ldg(y32 + ra), yb = __ldg(y32 + rb);
-#pragma unroll
-            for (int k = 0; k < kNAtt; k++) {
-                df_acc(h[k], l[k], __fmul_rn(va[k], ya));
-                df_acc(h[k], l[k], __fmul_rn(vb[k], yb));
-            }
-        }
-        if (e < e1) {
-            const float yi = __ldg(y32 + __ldcs(A.perm + e));
-#pragma unroll
-            for (int k = 0; k < kNAtt; k++)
-                df_acc(h[k], l[k], __fmul_rn(__ldcs(A.tval32 + tidx<kNAtt>(k, e)), yi));
-        }
-        // reduce-scatter over the warp in double-float (FP32 pipe): after
-        // the butterfly, lane pair (2k, 2k+1) holds sum k
-        float rh[16], rl[16];
-#pragma unroll
-        for (int k = 0; k < 16; k++) {
-            rh[k] = k < kNAtt ? h[k] : 0.f;
-            rl[k] = k < kNAtt ? l[k] : 0.f;
-        }
-#pragma unroll
-        for (int half = 8; half >= 1; half >>= 1) {
-            const bool upper = (lane & (2 * half)) != 0;
-#pragma unroll
-            for (int k = 0; k < half; k++) {
-                const float sh = upper ? rh[k] : rh[k + half];
-                const float sl = upper ? rl[k] : rl[k + half];
-                float kh = upper ? rh[k + half] : rh[k];
-                float kl = upper ? rl[k + half] : rl[k];
-                df_add(kh, kl, __shfl_xor_sync(0xffffffffu, sh, 2 * half),
-                       __shfl_xor_sync(0xffffffffu, sl, 2 * half));
-                rh[k] = kh;
-                rl[k] = kl;
-            }
-        }
-        float th = rh[0], tl = rl[0];
-        df_add(th, tl, __shfl_xor_sync(0xffffffffu, rh[0], 1), __shfl_xor_sync(0xffffffffu, rl[0], 1));
-        const int kk = lane >> 1;
-        if ((lane & 1) == 0 && kk < kNAtt)
-            S[o * kNAtt + kk] = df_to_d(th, tl);
+        double *xs = out + kNAstro * s + lane;
+        if (MODE == kA2Accumulate)
+            *xs += df_to_d(kh, kl);
+        else
+            *xs = df_to_d(kh, kl);
     }
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_att_segments_f32(SysView A, const float *__restrict__ y32, double *__restrict__ S)
-{
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    att_body_f32(A, y32, S, warp, nwarps);
 }
 
 // inner aprod 2, instrumental part over the instrument-sorted binary32 copy,
@@ -415,18 +385,16 @@ __device__ __forceinline__ void instr_body_f32_win(const SysView &A, const uint3
     }
 }
 
-// inner aprod 2 in one launch (sorted instrumental path), the binary32 form
-// of k_aprod2_fused: units of the three kinds from one work queue, one
-// global-column partial per star unit
+// Rest of the inner aprod 2 in one launch: star units and instrument units
+// from one work queue (as k_aprod2_fused, without attitude units)
 template <int G, int MODE, bool WIN>
 __global__ void __launch_bounds__(kThreads)
-k_aprod2_f32_fused(SysView A, const float *__restrict__ y32, double *__restrict__ out,
-                   double *__restrict__ S, const uint32_t *__restrict__ cseg,
-                   const uint32_t *__restrict__ irow, const float *__restrict__ ival32,
-                   double *__restrict__ part, int nwin, int ks, double *__restrict__ gpart, A2Queue q)
+k_f32_rest(SysView A, Att32 U, const float *__restrict__ y32, double *__restrict__ out,
+           const uint32_t *__restrict__ cseg, const uint32_t *__restrict__ irow,
+           const float *__restrict__ ival32, double *__restrict__ part, int nwin, int ks, A2Queue q)
 {
     const int lane = threadIdx.x & 31;
-    const int L = q.ns + q.na + q.ni;
+    const int L = q.ns + q.ni;
     for (;;) {
         unsigned long long u = 0;
         if (lane == 0)
@@ -448,23 +416,14 @@ k_aprod2_f32_fused(SysView A, const float *__restrict__ y32, double *__restrict_
         if (slot < q.ns) {
             const int64_t i = c * q.ns + slot;
             if (i < q.nstar_units) {
-                double g = 0.0;
                 for (int k = 0; k < q.star_k; k++) {
                     const int64_t grp = i * q.star_k + k;
                     if (grp < q.nstar_groups)
-                        g += stars_body_f32<G, MODE, kIpSorted>(A, y32, out, nullptr, nullptr, grp,
-                                                                q.nstar_groups);
+                        stars_body_f32<G, MODE>(A, U.sv, y32, out, grp);
                 }
-                g = warp_sum(g);
-                if (lane == 0)
-                    gpart[i] = g;
             }
-        } else if (slot < q.ns + q.na) {
-            const int64_t i = c * q.na + (slot - q.ns);
-            if (i < A.nseg)
-                att_body_f32(A, y32, S, i, A.nseg);
         } else {
-            const int64_t i = c * q.ni + (slot - q.ns - q.na);
+            const int64_t i = c * q.ni + (slot - q.ns);
             if (i < q.ninstr_units)
                 if (WIN)
                     instr_body_f32_win(A, cseg, irow, ival32, y32, part, nwin, ks, i,
@@ -475,11 +434,93 @@ k_aprod2_f32_fused(SysView A, const float *__restrict__ y32, double *__restrict_
     }
 }
 
+// The rest of the inner aprod 2 with the instruments in row windows: 16 warps
+// of a block sum its windows, the others take star units, and the first 16
+// join them (as k_aprod2_win)
+constexpr int kRestThreads = 1024;
+
+template <int G, int MODE>
+__global__ void __launch_bounds__(kRestThreads, 1)
+k_f32_rest_win(SysView A, Att32 U, Ell E, const float *__restrict__ y32, double *__restrict__ out,
+               A2Queue q, int *kerr)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ EllShared sh;
+    const uint32_t nfix = gridDim.x * (kRestThreads / 32 - kEllWarps);
+    uint32_t u = 0xffffffffu;
+    if (threadIdx.x < kEllThreads)
+        ell32_part(E, y32, A.m, smem, &sh, kerr);
+    else
+        u = blockIdx.x + gridDim.x * ((threadIdx.x - kEllThreads) >> 5);
+    for (;;) {
+        if (u != 0xffffffffu && (int64_t)u < q.nstar_units)
+            for (int k = 0; k < q.star_k; k++) {
+                const int64_t grp = (int64_t)u * q.star_k + k;
+                if (grp < q.nstar_groups)
+                    stars_body_f32<G, MODE>(A, U.sv, y32, out, grp);
+            }
+        if ((int64_t)nfix >= q.nstar_units)
+            break;
+        if ((threadIdx.x & 31) == 0)
+            u = nfix + (uint32_t)atomicAdd(q.ctr, 1ull);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if ((int64_t)u >= q.nstar_units)
+            break;
+    }
+}
+
+// attitude or instrument column j of A32^T q from the units' sums and the
+// instrument totals (fixed order)
+__device__ __forceinline__ double q_from_units(const SysView &A, const uint32_t *__restrict__ useg,
+                                               const double *__restrict__ S,
+                                               const double *__restrict__ ipart, int npart,
+                                               int64_t j)
+{
+    double t = 0.0;
+    if (j < A.ins0) {
+        const int64_t c = j - A.att0;
+        const int64_t a = (c >= A.D) + (c >= 2 * A.D), k = c - a * A.D;
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) {
+            const int64_t o = k - jj;
+            if (o >= 0 && o < A.nseg) {
+                const uint32_t u0 = __ldg(useg + o), u1 = __ldg(useg + o + 1);
+#pragma unroll 4
+                for (uint32_t u = u0; u < u1; u++)
+                    t += S[(int64_t)u * kNAtt + 4 * a + jj];
+            }
+        }
+    } else {
+        const int64_t f = j - A.ins0;
+        for (int q = 0; q < npart; q++)
+            t += ipart[(int64_t)q * A.I + f];
+    }
+    return t;
+}
+
+// out += the attitude and instrument columns of A32^T q; resets the counter
+__global__ void __launch_bounds__(kThreads)
+k_f32_combine(SysView A, const uint32_t *__restrict__ useg, const double *__restrict__ S,
+              const double *__restrict__ ipart, int npart, double *__restrict__ out,
+              unsigned long long *ctr, Ell E)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *ctr = 0ull;
+    if (npart == 0)  // the instruments' partials of the row windows
+        for (int64_t f = gtid32() >> 5; f < A.I; f += gstride32() >> 5) {
+            const double t = ell_total(E, f);
+            if ((threadIdx.x & 31) == 0)
+                out[A.ins0 + f] += t;
+        }
+    const int64_t end = npart ? A.glb0 : A.ins0;
+    for (int64_t j = A.att0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < end;
+         j += (int64_t)gridDim.x * blockDim.x)
+        out[j] += q_from_units(A, useg, S, ipart, npart, j);
+}
+
 // ---------------------------------------------------------------------------
 // vector kernels (FP64)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int64_t gtid32() { return blockIdx.x * (int64_t)blockDim.x + threadIdx.x; }
-__device__ __forceinline__ int64_t gstride32() { return (int64_t)gridDim.x * blockDim.x; }
 
 __global__ void k_to_f32(const double *__restrict__ a, float *__restrict__ b, int64_t n)
 {
@@ -487,32 +528,30 @@ __global__ void k_to_f32(const double *__restrict__ a, float *__restrict__ b, in
         b[j] = __double2float_rn(a[j]);
 }
 
-// Attitude part of a binary32 x, also stored as one float4 per (axis a,
-// offset o) holding x[a D + o .. a D + o + 3], so that a row reads its 12
-// attitude entries with 3 aligned vector loads.  Entry j of x (attitude
-// column a D + o) is component jj of the float4 of offset o - jj.
-__device__ __forceinline__ void att4_scatter(float *__restrict__ xatt4, int64_t j, float v,
-                                             int64_t att0, int64_t D)
+// Entry j of a binary32 x: the astrometric part as 8 floats (one sector) per
+// star, the rest in place
+__device__ __forceinline__ void store_x32(float *__restrict__ x32, float *__restrict__ x8,
+                                          int64_t att0, int64_t j, float v)
 {
-    const int64_t c = j - att0;
-    if (c < 0 || c >= 3 * D)
-        return;
-    const int64_t a = c / D, o = c - a * D;
-#pragma unroll
-    for (int jj = 0; jj < 4; jj++)
-        if (o - jj >= 0)
-            xatt4[((a * D + o - jj) << 2) + jj] = v;
+    if (j < att0) {
+        const int64_t s = j / kNAstro;
+        x8[8 * s + (j - kNAstro * s)] = v;
+    } else {
+        x32[j] = v;
+    }
+}
+__device__ __forceinline__ void store_x32(double *__restrict__ xp, float *, int64_t, int64_t j,
+                                          double v)
+{
+    xp[j] = v;
 }
 
-// API form: x32 = fl32(x) and its attitude float4 copy
+// API form: x32 = fl32(x)
 __global__ void k_x_to_f32(const double *__restrict__ x, float *__restrict__ x32,
-                           float *__restrict__ xatt4, int64_t n, int64_t att0, int64_t D)
+                           float *__restrict__ x8, int64_t n, int64_t att0)
 {
-    for (int64_t j = gtid32(); j < n; j += gstride32()) {
-        const float v = __double2float_rn(x[j]);
-        x32[j] = v;
-        att4_scatter(xatt4, j, v, att0, D);
-    }
+    for (int64_t j = gtid32(); j < n; j += gstride32())
+        store_x32(x32, x8, att0, j, __double2float_rn(x[j]));
 }
 
 // s = p o c, d = s, z = 0, xp32 = fl32(p o d), gamma = |s|^2; clears the
@@ -523,7 +562,7 @@ k_cg_init(const double *__restrict__ p, const double *__restrict__ c, double *__
           double *__restrict__ d, double *__restrict__ z, XT *__restrict__ xp32,
           double *__restrict__ t, int64_t n, int64_t ins0, CgState *cg, const CgArgs *args,
           double *partial, unsigned *counter, cudaGraphConditionalHandle loop, int in_graph,
-          float *__restrict__ xatt4, int64_t att0, int64_t D)
+          float *__restrict__ x8, int64_t att0)
 {
     double acc[1] = {0.0};
     for (int64_t j = gtid32(); j < n; j += gstride32()) {
@@ -531,10 +570,7 @@ k_cg_init(const double *__restrict__ p, const double *__restrict__ c, double *__
         s[j] = sj;
         d[j] = sj;
         z[j] = 0.0;
-        const XT xv = (XT)(p[j] * sj);
-        xp32[j] = xv;
-        if (xatt4)
-            att4_scatter(xatt4, j, (float)xv, att0, D);
+        store_x32(xp32, x8, att0, j, (XT)(p[j] * sj));
         if (j >= ins0)
             t[j] = 0.0;
         acc[0] = fma(sj, sj, acc[0]);
@@ -554,45 +590,48 @@ k_cg_init(const double *__restrict__ p, const double *__restrict__ c, double *__
 }
 
 // s -= alpha p o t, z += alpha d, gamma' = |s|^2; the last block forms beta
-// and applies the inner stopping rule.  INL: t holds only the astrometric
-// part of A^T q (single-launch aprod 2); the other columns come from its
-// partial sums, the global column from one fixed slice of the per-unit
-// partials per block, updated by the last block (which also resets the
-// aprod 2 work counter).
+// and applies the inner stopping rule.  INL: t holds the astrometric part and
+// the global column of A32^T q; the other columns come from the sums of the
+// units and instruments (the last block resets the work counter).
 template <bool INL>
 __global__ void __launch_bounds__(kThreads)
 k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restrict__ t,
           double *__restrict__ s, const double *__restrict__ d, double *__restrict__ z, CgState *cg,
           const CgArgs *args, double *partial, unsigned *counter,
-          cudaGraphConditionalHandle loop, int in_graph, A2Parts P)
+          cudaGraphConditionalHandle loop, int in_graph, const uint32_t *__restrict__ useg, A2Parts P)
 {
-    const int64_t n = A.n, glb0 = A.glb0;
+    const int64_t n = A.n;
     const double alpha = cg->alpha;
-    double acc[2] = {0.0, 0.0};
-    for (int64_t j = gtid32(); j < n; j += gstride32()) {
-        z[j] = fma(alpha, d[j], z[j]);
-        if (INL && j == glb0)
-            continue;  // the global column: the last block
-        const double tj = (!INL || j < A.att0) ? t[j] : q_from_parts(A, P, j);
-        const double sj = fma(-alpha, p[j] * tj, s[j]);
+    double acc[1] = {0.0};
+    // column j with t_j = tf(): the loads of the vectors come first
+    auto update = [&](int64_t j, auto tf) {
+        const double dj = d[j], zo = z[j], pj = p[j], so = s[j];
+        const double sj = fma(-alpha, pj * tf(), so);
+        z[j] = fma(alpha, dj, zo);
         s[j] = sj;
         acc[0] = fma(sj, sj, acc[0]);
-    }
-    if (INL) {
-        const int64_t per = (P.ngpart + gridDim.x - 1) / gridDim.x;
-        const int64_t b0 = blockIdx.x * per, b1 = min((int64_t)P.ngpart, b0 + per);
-        for (int64_t b = b0 + threadIdx.x; b < b1; b += blockDim.x)
-            acc[1] += P.gpart[b];
-    }
-    if (grid_reduce<2>(acc, partial, counter) && threadIdx.x == 0) {
-        CgState g = *cg;
-        double gnew = acc[0];
-        if (INL) {
-            const double sj = fma(-alpha, p[glb0] * acc[1], s[glb0]);
-            s[glb0] = sj;
-            gnew = fma(sj, sj, gnew);
-            *P.ctr = 0ull;
+    };
+    const bool win = INL && P.isplit == 0;  // instruments in row windows
+    if (win) {
+        for (int64_t f = gtid32() >> 5; f < A.I; f += gstride32() >> 5) {
+            const double t = ell_total(P.ell, f);
+            if ((threadIdx.x & 31) == 0)
+                update(A.ins0 + f, [&] { return t; });
         }
+    }
+    for (int64_t j = gtid32(); j < n; j += gstride32()) {
+        if (win && j >= A.ins0 && j < A.glb0)
+            continue;
+        update(j, [&] {
+            return (!INL || j < A.att0 || j >= A.glb0)
+                       ? t[j] : q_from_units(A, useg, P.S, P.ipart, P.isplit, j);
+        });
+    }
+    if (grid_reduce<1>(acc, partial, counter) && threadIdx.x == 0) {
+        CgState g = *cg;
+        const double gnew = acc[0];
+        if (INL)
+            *P.ctr = 0ull;
         g.beta = gnew / g.gamma;
         g.gamma = gnew;
         g.it += 1;
@@ -608,22 +647,19 @@ k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restric
     }
 }
 
-// d = s + beta d, xp32 = fl32(p o d) (and its attitude float4 copy when
-// xatt4 is set); clears the instrumental/global part of t
+// d = s + beta d, xp32 = fl32(p o d); clears the instrumental/global part of t
+// (the FP64 form: the binary32 products write theirs)
 template <typename XT>
 __global__ void k_cg_vec2(const double *__restrict__ p, const double *__restrict__ s,
                           double *__restrict__ d, XT *__restrict__ xp32, double *__restrict__ t,
-                          int64_t n, int64_t ins0, const CgState *cg, float *__restrict__ xatt4,
-                          int64_t att0, int64_t D)
+                          int64_t n, int64_t ins0, const CgState *cg, float *__restrict__ x8,
+                          int64_t att0)
 {
     const double beta = cg->beta;
     for (int64_t j = gtid32(); j < n; j += gstride32()) {
         const double dj = fma(beta, d[j], s[j]);
         d[j] = dj;
-        const XT xv = (XT)(p[j] * dj);
-        xp32[j] = xv;
-        if (xatt4)
-            att4_scatter(xatt4, j, (float)xv, att0, D);
+        store_x32(xp32, x8, att0, j, (XT)(p[j] * dj));
         if (j >= ins0)
             t[j] = 0.0;
     }
@@ -677,82 +713,90 @@ __global__ void k_count_pos(const double *__restrict__ a, int64_t n, double *par
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-bool x32_in_smem(const gsr_handle_t *h) { return h->sys.I <= kSmemInstrMax32; }
+static bool x32_in_smem(const gsr_handle_t *h) { return h->sys.I <= kSmemInstrMax32; }
+static size_t main_smem(const gsr_handle_t *h)
+{
+    return kMainSmem + (x32_in_smem(h) ? (size_t)h->sys.I * sizeof(float) : 0);
+}
 
-// rows in flight per lane of the binary32 aprod 1: one row at 4 blocks per
-// SM (64 registers) measured 5% faster than two rows at 2 blocks per SM on
-// the 100,000-star system
-constexpr int kA1f32Tiles = 1;
+static A2Queue rest_queue(const gsr_handle_t *h)
+{
+    return a2_queue(h, 8, (int64_t)h->sys.I * h->nq32 * h->ks32, 0);
+}
 
 template <int MODE>
-static cudaError_t a1f_launch(const gsr_handle_t *h, const float *x32, double *y, float *q32,
-                              cudaStream_t st)
+static cudaError_t f32_main(const gsr_handle_t *h, double *y, double *glb, cudaStream_t st)
 {
     double *part = h->d_partial + kRedU * kPartialsPerKind;
     unsigned *cnt = h->d_counter + kRedU;
-    constexpr int U = kA1f32Tiles;
     if (x32_in_smem(h))
-        k_aprod1_f32<MODE, true, U><<<h->grid_rows32, kThreads, (size_t)h->sys.I * sizeof(float),
-                                      st>>>(h->sys, x32, (const float4 *)h->d_xatt4, y, q32,
-                                            h->d_cg, part, cnt);
+        k_f32_main<MODE, true><<<h->grid_main32, kMainThreads, main_smem(h), st>>>(
+            h->sys, h->att32, h->d_x32, h->d_x8, h->d_q32, y, h->d_attS32, glb, h->d_cg, part, cnt,
+            h->d_kerr);
     else
-        k_aprod1_f32<MODE, false, U><<<h->grid_rows32, kThreads, 0, st>>>(
-            h->sys, x32, (const float4 *)h->d_xatt4, y, q32, h->d_cg, part, cnt);
+        k_f32_main<MODE, false><<<h->grid_main32, kMainThreads, main_smem(h), st>>>(
+            h->sys, h->att32, h->d_x32, h->d_x8, h->d_q32, y, h->d_attS32, glb, h->d_cg, part, cnt,
+            h->d_kerr);
+    return cudaGetLastError();
+}
+
+// the rest of aprod 2 over the row-ordered q32: stars and instruments; *P:
+// where the attitude and instrument sums are (isplit 0: in the row windows'
+// partials)
+template <int MODE, int G>
+static cudaError_t rest_win(const gsr_handle_t *h, double *out, cudaStream_t st)
+{
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_f32_rest_win<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEllSmem32);
+    if (e != cudaSuccess)
+        return e;
+    k_f32_rest_win<G, MODE><<<h->nsm, kRestThreads, kEllSmem32, st>>>(
+        h->sys, h->att32, h->ell, h->d_q32, out, a2_queue(h, G, 0, 0), h->d_kerr);
     return cudaGetLastError();
 }
 
 template <int MODE>
-static cudaError_t a2f_launch(const gsr_handle_t *h, const float *y32, double *out, cudaStream_t st)
+static cudaError_t f32_rest(const gsr_handle_t *h, double *out, A2Parts *P, cudaStream_t st)
 {
-    const int G = 8;
-    if (h->ipath == kIpSorted && h->a2_fused) {
-        const A2Queue q = a2_queue(h, G, (int64_t)h->sys.I * h->nq32 * h->ks32);
-        if (h->nq32 > 1)
-            k_aprod2_f32_fused<G, MODE, true><<<h->grid_fused32, kThreads, 0, st>>>(
-                h->sys, y32, out, h->d_attS, h->d_cseg32, h->d_irow, h->d_ival32, h->d_ipart,
-                h->nq32, h->ks32, h->d_gpart, q);
-        else
-            k_aprod2_f32_fused<G, MODE, false><<<h->grid_fused32, kThreads, 0, st>>>(
-                h->sys, y32, out, h->d_attS, h->d_iseg, h->d_irow, h->d_ival32, h->d_ipart, 1,
-                h->ks32, h->d_gpart, q);
-        const int nb_att = (int)((3 * h->sys.D + kThreads - 1) / kThreads < 4 * h->nsm
-                                     ? (3 * h->sys.D + kThreads - 1) / kThreads
-                                     : 4 * h->nsm);
-        const int nb_ins = (int)((h->sys.I + kThreads / 32 - 1) / (kThreads / 32));
-        launch_att_combine(h, out, nb_att, nb_ins, h->d_ipart, h->nq32 * h->ks32, h->d_gpart,
-                           (int)q.nstar_units, MODE == kA2Accumulate, st, h->d_a2ctr);
-        return cudaGetLastError();
+    *P = {h->d_attS32, h->d_ipart, h->ell_on ? 0 : h->nq32 * h->ks32, nullptr, 0, h->d_a2ctr, h->ell};
+    if (h->ell_on) {
+        // a lane takes about as many rows of long stars with more lanes
+        const int64_t mean = h->sys.m / h->sys.S;
+        return mean >= 256 ? rest_win<MODE, 32>(h, out, st)
+                           : (mean >= 128 ? rest_win<MODE, 16>(h, out, st)
+                                          : rest_win<MODE, 8>(h, out, st));
     }
-    const bool smem = instr_in_smem(h);
-    if (smem)
-        k_aprod2_f32_stars<G, MODE, true><<<h->grid_rows2_32, kThreads,
-                                             (size_t)h->sys.I * sizeof(double), st>>>(
-            h->sys, y32, out, h->d_irep, h->nrep);
+    const A2Queue q = rest_queue(h);
+    if (h->nq32 > 1)
+        k_f32_rest<8, MODE, true><<<h->grid_rest32, kThreads, 0, st>>>(
+            h->sys, h->att32, h->d_q32, out, h->d_cseg32, h->d_irow, h->d_ival32, h->d_ipart,
+            h->nq32, h->ks32, q);
     else
-        k_aprod2_f32_stars<G, MODE, false><<<h->grid_rows2_32, kThreads, 0, st>>>(
-            h->sys, y32, out, h->d_irep, h->nrep);
-    k_att_segments_f32<<<h->grid_att, kThreads, 0, st>>>(h->sys, y32, h->d_attS);
-    const int nb_att = (int)((3 * h->sys.D + kThreads - 1) / kThreads < 4 * h->nsm
-                                 ? (3 * h->sys.D + kThreads - 1) / kThreads
-                                 : 4 * h->nsm);
-    const int nb_ins = smem ? 0 : (int)((h->sys.I + kThreads / 32 - 1) / (kThreads / 32));
-    launch_att_combine(h, out, nb_att, nb_ins, h->d_irep, h->nrep, nullptr, 0, MODE == kA2Accumulate,
-                       st);
+        k_f32_rest<8, MODE, false><<<h->grid_rest32, kThreads, 0, st>>>(
+            h->sys, h->att32, h->d_q32, out, h->d_iseg, h->d_irow, h->d_ival32, h->d_ipart, 1,
+            h->ks32, q);
     return cudaGetLastError();
 }
 
 // API forms (FP64 vectors in and out)
 cudaError_t launch_aprod1_f32_api(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st)
 {
-    k_x_to_f32<<<h->grid_vec, kThreads, 0, st>>>(x, h->d_x32, h->d_xatt4, h->sys.n, h->sys.att0,
-                                                  h->sys.D);
-    return a1f_launch<0>(h, h->d_x32, y, nullptr, st);
+    k_x_to_f32<<<h->grid_vec, kThreads, 0, st>>>(x, h->d_x32, h->d_x8, h->sys.n, h->sys.att0);
+    return f32_main<kF32A1>(h, y, nullptr, st);
 }
 
 cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double *x, cudaStream_t st)
 {
     k_to_f32<<<h->grid_vec, kThreads, 0, st>>>(y, h->d_q32, h->sys.m);
-    return a2f_launch<kA2Accumulate>(h, h->d_q32, x, st);
+    cudaError_t e = f32_main<kF32A2>(h, nullptr, x + h->sys.glb0, st);
+    A2Parts P;
+    if (e == cudaSuccess)
+        e = f32_rest<kA2Accumulate>(h, x, &P, st);
+    if (e != cudaSuccess)
+        return e;
+    k_f32_combine<<<h->nsm * 2, kThreads, 0, st>>>(h->sys, h->d_useg, P.S, P.ipart, P.isplit, x,
+                                                   P.ctr, P.ell);
+    return cudaGetLastError();
 }
 
 static cudaError_t cg_prologue(const gsr_handle_t *h, cudaStream_t s, cudaGraphConditionalHandle loop,
@@ -763,7 +807,7 @@ static cudaError_t cg_prologue(const gsr_handle_t *h, cudaStream_t s, cudaGraphC
                                                 h->d_t, A.n, A.ins0, h->d_cg, h->d_cgargs,
                                                 h->d_partial + kRedBnorm * kPartialsPerKind,
                                                 h->d_counter + kRedBnorm, loop, in_graph,
-                                                h->d_xatt4, A.att0, A.D);
+                                                h->d_x8, A.att0);
     return cudaGetLastError();
 }
 
@@ -771,37 +815,19 @@ static cudaError_t cg_iteration(const gsr_handle_t *h, cudaStream_t s, cudaGraph
                                 int in_graph)
 {
     const SysView &A = h->sys;
-    cudaError_t e = a1f_launch<1>(h, h->d_x32, nullptr, h->d_q32, s);
+    A2Parts P;
+    cudaError_t e = f32_main<kF32A1 | kF32A2>(h, nullptr, h->d_t + A.glb0, s);
+    if (e == cudaSuccess)
+        e = f32_rest<kA2Overwrite>(h, h->d_t, &P, s);
     if (e != cudaSuccess)
         return e;
-    A2Parts P = {};
-    double *part = h->d_partial + kRedV * kPartialsPerKind;
-    unsigned *cnt = h->d_counter + kRedV;
-    if (h->ipath == kIpSorted && h->a2_fused) {
-        // single-launch aprod 2 without the combine; the CG pass combines
-        const A2Queue q = a2_queue(h, 8, (int64_t)A.I * h->nq32 * h->ks32);
-        if (h->nq32 > 1)
-            k_aprod2_f32_fused<8, kA2Overwrite, true><<<h->grid_fused32, kThreads, 0, s>>>(
-                h->sys, h->d_q32, h->d_t, h->d_attS, h->d_cseg32, h->d_irow, h->d_ival32,
-                h->d_ipart, h->nq32, h->ks32, h->d_gpart, q);
-        else
-            k_aprod2_f32_fused<8, kA2Overwrite, false><<<h->grid_fused32, kThreads, 0, s>>>(
-                h->sys, h->d_q32, h->d_t, h->d_attS, h->d_iseg, h->d_irow, h->d_ival32, h->d_ipart,
-                1, h->ks32, h->d_gpart, q);
-        P = {h->d_attS, h->d_ipart, h->nq32 * h->ks32, h->d_gpart, (int)q.nstar_units, h->d_a2ctr};
-        k_cg_vec1<true><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d, h->d_zc,
-                                                         h->d_cg, h->d_cgargs, part, cnt, loop,
-                                                         in_graph, P);
-    } else {
-        e = a2f_launch<kA2Overwrite>(h, h->d_q32, h->d_t, s);
-        if (e != cudaSuccess)
-            return e;
-        k_cg_vec1<false><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
-                                                          h->d_zc, h->d_cg, h->d_cgargs, part, cnt,
-                                                          loop, in_graph, P);
-    }
-    k_cg_vec2<float><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_x32, h->d_t, A.n, A.ins0,
-                                                h->d_cg, h->d_xatt4, A.att0, A.D);
+    k_cg_vec1<true><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d, h->d_zc, h->d_cg,
+                                                     h->d_cgargs,
+                                                     h->d_partial + kRedV * kPartialsPerKind,
+                                                     h->d_counter + kRedV, loop, in_graph,
+                                                     h->d_useg, P);
+    k_cg_vec2<float><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_x32, h->d_t, A.n, A.n,
+                                                h->d_cg, h->d_x8, A.att0);
     return cudaGetLastError();
 }
 
@@ -920,44 +946,75 @@ cudaError_t launch_to_f32(const gsr_handle_t *h, const double *a, float *b, int6
     return cudaGetLastError();
 }
 
-int aprod1_f32_grid(const gsr_handle_t *h)
+// one block per SM, no more than the units need
+int f32_main_grid(const gsr_handle_t *h)
 {
-    int occ = 0;
-    cudaError_t e = x32_in_smem(h)
-                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &occ, k_aprod1_f32<1, true, kA1f32Tiles>, kThreads,
-                              (size_t)h->sys.I * sizeof(float))
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &occ, k_aprod1_f32<1, false, kA1f32Tiles>, kThreads, 0);
-    if (e != cudaSuccess || occ <= 0)
-        return -1;
-    int64_t g = (int64_t)h->nsm * occ;
-    return (int)(g > kMaxPartials ? kMaxPartials : g);
+    const void *fns[6] = {(const void *)k_f32_main<1, true>, (const void *)k_f32_main<1, false>,
+                          (const void *)k_f32_main<2, true>, (const void *)k_f32_main<2, false>,
+                          (const void *)k_f32_main<3, true>, (const void *)k_f32_main<3, false>};
+    for (const void *f : fns) {
+        // the most that any handle of this process asks for: the attribute is
+        // shared by all of them
+        const size_t most = kMainSmem + kSmemInstrMax32 * sizeof(float);
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
+            cudaSuccess)
+            return -1;
+    }
+    const int64_t nu = h->att32.nunits;
+    return (int)(nu < h->nsm ? nu : h->nsm);
 }
 
-int aprod2_f32_fused_grid(const gsr_handle_t *h)
+int f32_rest_grid(const gsr_handle_t *h)
 {
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &occ, k_aprod2_f32_fused<8, kA2Overwrite, true>, kThreads, 0);
+        &occ, k_f32_rest<8, kA2Overwrite, true>, kThreads, 0);
     if (e != cudaSuccess || occ <= 0)
         return -1;
-    return h->nsm * occ;
+    const A2Queue q = rest_queue(h);
+    const int64_t need = (q.total + kThreads / 32 - 1) / (kThreads / 32);
+    const int64_t g = (int64_t)h->nsm * occ;
+    return (int)(g < need ? g : need);
 }
 
-int aprod2_f32_grid(const gsr_handle_t *h)
+// the binary32 copies from the FP64 values: the offset-ordered tiles, the
+// astrometric planes in row order; one plane when k1 >= 0
+__global__ void k_atile(SysView A, unsigned char *__restrict__ tile, int k1)
 {
-    int occ = 0;
-    cudaError_t e = instr_in_smem(h)
-                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &occ, k_aprod2_f32_stars<8, kA2Overwrite, true>, kThreads,
-                              (size_t)h->sys.I * sizeof(double))
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                              &occ, k_aprod2_f32_stars<8, kA2Overwrite, false>, kThreads, 0);
-    if (e != cudaSuccess || occ <= 0)
-        return -1;
-    int64_t g = (int64_t)h->nsm * occ;
-    return (int)(g > kMaxPartials ? kMaxPartials : g);
+    for (int64_t e = gtid32(); e < A.m; e += gstride32()) {
+        const int64_t r = A.perm[e];
+        const int l = (int)(e & 31);
+        unsigned char *tp = tile + (e >> 5) * kAttTileBytes;
+        float *v = reinterpret_cast<float *>(tp) + l;
+        if (k1 >= 0) {
+            v[32 * k1] = (float)A.val[tidx<kNPar>(k1, r)];
+            continue;
+        }
+#pragma unroll
+        for (int k = 0; k < kNPar; k++)
+            v[32 * k] = (float)A.val[tidx<kNPar>(k, r)];
+        uint4 rc = A.rec[r];
+        rc.x = star_of_row(A, r >> 5, r);
+        reinterpret_cast<uint4 *>(tp + kAttRecAt)[l] = rc;
+        reinterpret_cast<uint32_t *>(tp + kAttRowAt)[l] = (uint32_t)r;
+    }
+}
+
+__global__ void k_sv32(SysView A, float *__restrict__ sv, int k1)
+{
+    for (int64_t r = gtid32(); r < A.m; r += gstride32()) {
+#pragma unroll
+        for (int k = 0; k < kNAstro; k++)
+            if (k1 < 0 || k == k1)
+                sv[tidx<kNAstro>(k, r)] = (float)A.val[tidx<kNPar>(k, r)];
+    }
+}
+
+cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st)
+{
+    k_atile<<<h->nsm * 8, kThreads, 0, st>>>(h->sys, h->d_atile, -1);
+    k_sv32<<<h->nsm * 8, kThreads, 0, st>>>(h->sys, h->d_sv32, -1);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -975,7 +1032,7 @@ static cudaError_t cg64_prologue(const gsr_handle_t *h, cudaStream_t s,
                                                         h->d_cgargs,
                                                         h->d_partial + kRedBnorm * kPartialsPerKind,
                                                         h->d_counter + kRedBnorm, loop, in_graph,
-                                                        nullptr, 0, 0);
+                                                        nullptr, 0);
     return cudaGetLastError();
 }
 
@@ -992,9 +1049,9 @@ static cudaError_t cg64_iteration(const gsr_handle_t *h, cudaStream_t s,
                                                       h->d_cg, h->d_cgargs,
                                                       h->d_partial + kRedV * kPartialsPerKind,
                                                       h->d_counter + kRedV, loop, in_graph,
-                                                      A2Parts{});
+                                                      nullptr, A2Parts{});
     k_cg_vec2<double><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_xp64, h->d_t,
-                                                        A.n, A.ins0, h->d_cg, nullptr, 0, 0);
+                                                        A.n, A.ins0, h->d_cg, nullptr, 0);
     return cudaGetLastError();
 }
 
@@ -1064,24 +1121,12 @@ cudaError_t run_cg64(gsr_handle_t *h, cudaStream_t st, int max_iter)
     return e;
 }
 
-// binary32 copy of plane k of K tiled planes (k_to_f32 over one plane)
-template <int K>
-__global__ void k_plane_to_f32(const double *__restrict__ a, float *__restrict__ b, int k, int64_t m)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = tidx<K>(k, i);
-        b[j] = (float)a[j];
-    }
-}
-
 // binary32 copies of plane k after it changed
 cudaError_t launch_f32_plane(const gsr_handle_t *h, int k, cudaStream_t st)
 {
-    k_plane_to_f32<kNPar><<<h->nsm * 8, kThreads, 0, st>>>(h->d_val, h->d_val32, k, h->sys.m);
-    if (k >= kNAstro && k < kNAstro + kNAtt)
-        k_plane_to_f32<kNAtt><<<h->nsm * 8, kThreads, 0, st>>>(h->d_tval, h->d_tval32, k - kNAstro,
-                                                              h->sys.m);
+    k_atile<<<h->nsm * 8, kThreads, 0, st>>>(h->sys, h->d_atile, k);
+    if (k < kNAstro)
+        k_sv32<<<h->nsm * 8, kThreads, 0, st>>>(h->sys, h->d_sv32, k);
     return cudaGetLastError();
 }
 

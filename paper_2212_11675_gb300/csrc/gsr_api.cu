@@ -166,13 +166,17 @@ static void release(gsr_handle_t *h)
     delete h;
 }
 
-// Rows per window of the FP64 instrument units: R = 4096 I / 6 (about 4096
-// entries per instrument and window), at most 4 Mi rows (32 MB of FP64 y), at
-// least 64 Ki rows
+// Rows per window of the FP64 instrument units (a unit is one instrument in
+// one window): 4096 entries a unit on a large system (units of about 1,024 or
+// 2,048 entries were slower at m = 7.0e6), fewer, down to 256, where that
+// would leave the resident warps (32 per SM) without a unit; at most
+// 4 Mi rows, so that L2 holds the 32 MB of y that a window's units gather.
 static int64_t instr_window(const gsr_handle_t *h)
 {
-    return std::max<int64_t>((int64_t)1 << 16,
-                             std::min<int64_t>(4096 * h->sys.I / kNInstr, (int64_t)1 << 22));
+    const int64_t m = h->sys.m, I = h->sys.I;
+    int64_t e = kNInstr * m / ((int64_t)h->nsm * 32);
+    e = std::max<int64_t>(256, std::min<int64_t>(4096, e));
+    return std::max<int64_t>(32, std::min<int64_t>(e * I / kNInstr, (int64_t)1 << 22));
 }
 
 // the window bounds cseg of the instrument-sorted copy, its partial sums and
@@ -569,6 +573,11 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
     A.ins0 = A.att0 + 3 * D;
     A.glb0 = A.ins0 + I;
     A.nseg = D - 3;
+    // pieces of an offset's rows, one warp each: of 512 rows or fewer on
+    // average, so that a few long offsets still give every SM work
+    A.attp = (m / A.nseg + 511) / 512;
+    if (A.attp < 1)
+        A.attp = 1;
     const int64_t ntiles = (m + 31) / 32;
 
     TRY(dalloc(h, &h->d_star_ptr, S + 1));
@@ -582,7 +591,7 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
     TRY(dalloc(h, &h->d_tval, (int64_t)kNAtt * mp));
     TRY(dalloc(h, &h->d_perm, m));
     TRY(dalloc(h, &h->d_seg, A.nseg + 1));
-    TRY(dalloc(h, &h->d_attS, A.nseg * kNAtt));
+    TRY(dalloc(h, &h->d_attS, A.nseg * A.attp * kNAtt));
     TRY(dalloc(h, &h->d_p, n));
     TRY(dalloc(h, &h->d_u, m));
     TRY(dalloc(h, &h->d_v, n));
@@ -729,9 +738,12 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
                                                                     : build_instr_sorted(h, st));
 
     // launch geometry
-    // measured at the medium size: 8 lanes per star with shared-memory
-    // instrument sums or the sorted pass, 32 with replicas
-    h->lanes = h->cfg.lanes_per_star ? h->cfg.lanes_per_star : (h->ipath == kIpReplicas ? 32 : 8);
+    // measured at the medium size (70 rows a star): 8 lanes per star with
+    // shared-memory instrument sums or the sorted pass, 32 with replicas;
+    // a lane takes about as many rows of longer stars with more lanes
+    const int64_t mean = m / S;
+    h->lanes = h->cfg.lanes_per_star ? h->cfg.lanes_per_star
+               : (h->ipath == kIpReplicas || mean >= 256) ? 32 : (mean >= 128 ? 16 : 8);
     // aprod 1 staged by the bulk-copy engine wherever it applies (measured
     // faster in the solve on the medium workload: 0.305 against 0.328 ms)
     CK(aprod1_tma_prepare(h));

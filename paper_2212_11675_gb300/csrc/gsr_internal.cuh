@@ -35,6 +35,7 @@ struct SysView {
     int64_t S, D, I, m, n;
     int64_t att0, ins0, glb0;  // first column of each section
     int64_t nseg;              // D-3 attitude offsets
+    int64_t attp;              // pieces per offset of the FP64 attitude sums
 };
 
 // Binary32 layout of the mixed and batched forms.  All 24 values of a row sit
@@ -124,28 +125,51 @@ struct A2Parts {
     Ell ell;
 };
 
-// q_j of the non-astrometric columns from the partial sums: column a D + k of
-// the attitude block is sum_{jj<4} S[k-jj][4a+jj]; instrument f the sum of its
-// window totals (both in the combine kernel's order)
-__device__ __forceinline__ double q_from_parts(const SysView &A, const A2Parts &P, int64_t j)
+// Attitude column a D + k from the segment sums: sum_{jj<4} S[k-jj][4a+jj],
+// the pieces of an offset in order
+__device__ __forceinline__ double att_column(const SysView &A, const double *__restrict__ S, int64_t a,
+                                             int64_t k)
 {
     double t = 0.0;
-    if (j < A.ins0) {
-        // axis a and knot k of attitude column c by two comparisons (a 64-bit
-        // division is a long instruction sequence on the GPU)
-        const int64_t c = j - A.att0;
-        const int64_t a = (c >= A.D) + (c >= 2 * A.D), k = c - a * A.D;
+    if (A.attp == 1) {  // without the loops: four loads in flight
 #pragma unroll
         for (int jj = 0; jj < 4; jj++) {
             const int64_t o = k - jj;
             if (o >= 0 && o < A.nseg)
-                t += P.S[o * kNAtt + 4 * a + jj];
+                t += S[o * kNAtt + 4 * a + jj];
         }
     } else {
-        const int64_t f = j - A.ins0;
-        for (int qq = 0; qq < P.isplit; qq++)
-            t += P.ipart[(int64_t)qq * A.I + f];
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) {
+            const int64_t o = k - jj;
+            if (o >= 0 && o < A.nseg) {
+                const double *s = S + o * A.attp * kNAtt + 4 * a + jj;
+#pragma unroll 4
+                for (int q = 0; q < (int)A.attp; q++)
+                    t += s[q * kNAtt];
+            }
+        }
     }
+    return t;
+}
+
+// q_j of the non-astrometric columns from the partial sums: an attitude column
+// as above; instrument f the sum of its window totals (both in the combine
+// kernel's order)
+__device__ __forceinline__ double q_from_parts(const SysView &A, const A2Parts &P, int64_t j)
+{
+    if (j < A.ins0) {
+        // axis a and knot k of attitude column c by two comparisons (a 64-bit
+        // division is a long instruction sequence on the GPU)
+        const int64_t c = j - A.att0;
+        const int64_t a = (c >= A.D) + (c >= 2 * A.D);
+        return att_column(A, P.S, a, c - a * A.D);
+    }
+    const int64_t f = j - A.ins0;
+    double t = 0.0;
+#pragma unroll 4
+    for (int qq = 0; qq < P.isplit; qq++)
+        t += P.ipart[(int64_t)qq * A.I + f];
     return t;
 }
 

@@ -985,26 +985,53 @@ cudaError_t launch_gather_instr64(const gsr_handle_t *h, const uint32_t *code, d
 // products of the rows with that offset into S[o][4a + j].  SQ: squares of
 // the values (preconditioner) instead of products with y.
 // ---------------------------------------------------------------------------
+// Entries of attitude unit u: piece u % attp of offset u / attp, sums at S[u]
+__device__ __forceinline__ void att_range(const SysView &A, int64_t u, uint32_t &e0, uint32_t &e1)
+{
+    if (A.attp == 1) {
+        e0 = A.seg[u];
+        e1 = A.seg[u + 1];
+        return;
+    }
+    // only where offsets have hundreds of rows: fewer than 2^32 units
+    const uint32_t np = (uint32_t)A.attp, o = (uint32_t)u / np, q = (uint32_t)u - o * np;
+    const uint32_t s0 = A.seg[o];
+    const uint64_t len = A.seg[o + 1] - s0;
+    e0 = s0 + (uint32_t)(len * q / np);
+    e1 = s0 + (uint32_t)(len * (q + 1) / np);
+}
+
 template <bool SQ>
 __device__ __forceinline__ void att_body(const SysView &A, const double *__restrict__ y,
                                          double *__restrict__ S, int64_t warp, int64_t nwarps)
 {
     const int lane = threadIdx.x & 31;
-    for (int64_t o = warp; o < A.nseg; o += nwarps) {
-        const uint32_t e0 = A.seg[o], e1 = A.seg[o + 1];
+    for (int64_t o = warp; o < A.nseg * A.attp; o += nwarps) {
+        uint32_t e0, e1;
+        att_range(A, o, e0, e1);
         double acc[kNAtt];
 #pragma unroll
         for (int k = 0; k < kNAtt; k++)
             acc[k] = 0.0;
-        for (uint32_t e = e0 + lane; e < e1; e += 32) {
-            const double yi = SQ ? 1.0 : __ldg(y + __ldcs(A.perm + e));
+        // the y of the next entry (row number, then the gather: two dependent
+        // loads) is on its way while the current one is summed
+        uint32_t e = e0 + lane;
+        double yn = (SQ || e >= e1) ? 1.0 : __ldg(y + __ldcs(A.perm + e));
+        uint32_t rn = (SQ || e + 32 >= e1) ? 0u : __ldcs(A.perm + e + 32);
+        for (; e < e1; e += 32) {
+            const double yi = yn;
+            double v[kNAtt];
 #pragma unroll
-            for (int k = 0; k < kNAtt; k++) {
-                double v = __ldcs(A.tval + tidx<kNAtt>(k, e));
-                if (SQ)
-                    v *= v;
-                acc[k] = fma(v, yi, acc[k]);
+            for (int k = 0; k < kNAtt; k++)
+                v[k] = __ldcs(A.tval + tidx<kNAtt>(k, e));
+            if (!SQ && e + 32 < e1) {
+                yn = __ldg(y + rn);
+                if (e + 64 < e1)
+                    rn = __ldcs(A.perm + e + 64);
             }
+#pragma unroll
+            for (int k = 0; k < kNAtt; k++)
+                acc[k] = fma(SQ ? v[k] * v[k] : v[k], yi, acc[k]);
         }
         // reduce-scatter over the warp: after the butterfly, lane pair
         // (2k, 2k+1) holds the total of sum k (16 adds per lane, not 60).
@@ -1096,7 +1123,8 @@ __device__ __forceinline__ bool att_unit_split(const SysView &A, const double *_
     constexpr int NN = kNAtt - NAS;
     static_assert(NAS > 0 && NAS <= 8, "the split taps pair with native ones at xor 16");
     const int lane = threadIdx.x & 31;
-    const uint32_t e0 = A.seg[o], e1 = A.seg[o + 1];
+    uint32_t e0, e1;
+    att_range(A, o, e0, e1);
     double acc[NN];
     Acc3 c[NAS];
 #pragma unroll
@@ -1205,13 +1233,11 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
     constexpr bool SQ = MODE == kA2Squares;
     const int lane = threadIdx.x & 31;
     const uint32_t L = (uint32_t)(q.ns + q.na + q.ni);
-    for (;;) {
-        unsigned long long u = 0;
-        if (lane == 0)
-            u = atomicAdd(q.ctr, 1ull);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if ((int64_t)u >= q.total)
-            break;
+    // every warp's first unit is fixed (a small system needs no counter: the
+    // numbers of 4,864 warps from one address took about 8 us), the others
+    // come from the counter
+    const unsigned nfix = gridDim.x * (kThreads / 32);
+    for (unsigned long long u = blockIdx.x + gridDim.x * (threadIdx.x >> 5); (int64_t)u < q.total;) {
         // q.total < 2^32 (checked at creation): 32-bit unit decode
         const int64_t c = (uint32_t)u / L;
         const int slot = (int)((uint32_t)u - (uint32_t)c * L);
@@ -1239,14 +1265,14 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
             }
         } else if (slot < q.ns + q.na) {
             const int64_t i = c * q.na + (slot - q.ns);
-            if (i < A.nseg) {
+            if (i < A.nseg * A.attp) {
                 bool done = false;
                 if constexpr ((SPL & kSplitAtt2) != 0)
                     done = att_unit_split<8>(A, y, S, i);
                 else if constexpr ((SPL & kSplitAtt) != 0)
                     done = att_unit_split<4>(A, y, S, i);
                 if (!done)  // native FP64 products (an operand outside the split range)
-                    att_body<SQ>(A, y, S, i, A.nseg);
+                    att_body<SQ>(A, y, S, i, A.nseg * A.attp);
             }
         } else {
             const int64_t i = c * q.ni + (slot - q.ns - q.na);
@@ -1262,6 +1288,12 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
                     instr_body<SQ>(A, cseg, irow, ival, y, part, nwin, i, q.ninstr_units);
             }
         }
+        if ((int64_t)nfix >= q.total)
+            break;
+        unsigned long long t = 0;
+        if (lane == 0)
+            t = atomicAdd(q.ctr, 1ull);
+        u = nfix + __shfl_sync(0xffffffffu, t, 0);
     }
 }
 
@@ -1304,14 +1336,8 @@ k_att_combine(SysView A, const double *__restrict__ S, double *__restrict__ out,
         const int64_t total = 3 * A.D;
         for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < total;
              c += (int64_t)nb_att * blockDim.x) {
-            const int64_t a = c / A.D, k = c - a * A.D;
-            double t = 0.0;
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int64_t o = k - j;
-                if (o >= 0 && o < A.nseg)
-                    t += S[o * kNAtt + 4 * a + j];
-            }
+            const int64_t a = (c >= A.D) + (c >= 2 * A.D);
+            const double t = att_column(A, S, a, c - a * A.D);
             double *dst = out + A.att0 + c;
             if (ACC)
                 *dst += t;
@@ -1520,16 +1546,22 @@ static cudaError_t launch_aprod2_split(const gsr_handle_t *h, const double *y, d
 // attitude segment at the medium size)
 constexpr int kStarGroupsPerUnit = 4;
 
-// (natt: the attitude units, nseg by default)
+// (natt: the attitude units, all pieces by default)
 A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units, int64_t natt)
 {
     A2Queue q;
     q.ctr = h->d_a2ctr;
-    q.star_k = kStarGroupsPerUnit;
     q.nstar_groups = (h->sys.S + 32 / G - 1) / (32 / G);
+    // fewer where that leaves the resident warps (32 per SM) without a unit
+    q.star_k = (int)(q.nstar_groups / ((int64_t)h->nsm * 32));
+    if (q.star_k < 1)
+        q.star_k = 1;
+    if (q.star_k > kStarGroupsPerUnit)
+        q.star_k = kStarGroupsPerUnit;
     q.nstar_units = (q.nstar_groups + q.star_k - 1) / q.star_k;
     q.ninstr_units = ninstr_units >= 0 ? ninstr_units : h->sys.I * h->isplit;
-    const int64_t n[3] = {q.nstar_units, natt >= 0 ? natt : h->sys.nseg, q.ninstr_units};
+    const int64_t n[3] = {q.nstar_units, natt >= 0 ? natt : h->sys.nseg * h->sys.attp,
+                          q.ninstr_units};
     const int64_t tot = n[0] + n[1] + n[2];
     int sl[3];
     for (int t = 0; t < 3; t++) {
@@ -1923,7 +1955,7 @@ static int a2_occupancy(const gsr_handle_t *h)
     return e == cudaSuccess ? occ : -1;
 }
 
-// blocks of the fused aprod 2: all resident blocks, a multiple of 8
+// blocks of the fused aprod 2: the resident blocks
 template <int G>
 static cudaError_t fused_occupancy(const gsr_handle_t *h, int *occ)
 {
@@ -1965,9 +1997,13 @@ int aprod2_fused_grid(const gsr_handle_t *h)
     if (e != cudaSuccess || occ <= 0)
         return -1;
     int64_t g = (int64_t)h->nsm * occ / 8 * 8;
+    // no more warps than units
+    const int64_t need = (a2_queue(h, h->lanes).total + kThreads / 32 - 1) / (kThreads / 32);
+    if (g > need)
+        g = need;
     if (g > kMaxPartials)
         g = kMaxPartials;
-    return (int)(g < 8 ? 8 : g);
+    return (int)(g < 1 ? 1 : g);
 }
 
 int aprod2_grid(const gsr_handle_t *h)

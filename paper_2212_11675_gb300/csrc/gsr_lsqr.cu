@@ -41,6 +41,7 @@
 namespace gsr {
 
 constexpr int kIstopNonfinite = 8;
+constexpr int kThreadParts = 8;  // window totals of an instrument that one thread adds
 
 __device__ __forceinline__ int64_t gtid() { return blockIdx.x * (int64_t)blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
@@ -114,14 +115,18 @@ __device__ void init_scalars(SolveState *st, const SolveArgs *args, double vnorm
 }
 
 // Scalar recurrences of one LSQR iteration, run by the whole last block of
-// the vector pass.  The four independent square roots go to four different warps;
-// everything else is one thread, with products by reciprocals already
-// known (1/rho from the aprod 1 pass) instead of divisions, because FP64
-// divisions and square roots are long instruction sequences on this part.
+// the vector pass.  The independent square roots and the reciprocal of the new
+// alpha go to different warps; everything else is one thread, with products by
+// reciprocals already known (1/rho from the aprod 1 pass) instead of
+// divisions, because FP64 divisions and square roots take a third of a
+// microsecond each on this part and every dependent operation 65 clocks.  The
+// tests of the machine-precision rules are multiplied out:
+// 1 + a / b <= 1 exactly when a <= 2^-53 b (up to the rounding of a / b).
 __device__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm2,
                              double dd, double zz, cudaGraphConditionalHandle loop, int in_graph)
 {
-    __shared__ double sq[4];
+    __shared__ double sq[6];
+    constexpr double kHalfEps = 1.0 / 9007199254740992.0;  // 2^-53
     const double beta = st->bnext;
     const bool upd = beta > 0.0;
     const double anorm2 = upd ? st->anorm2 + st->alpha * st->alpha + beta * beta : st->anorm2;
@@ -134,13 +139,19 @@ __device__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm
         sq[2] = sqrt(anorm2);
     if (threadIdx.x == 96)
         sq[3] = sqrt(ddnorm);
+    if (threadIdx.x == 128) {
+        const double a = upd ? sqrt(vnorm2) : st->alpha;
+        sq[4] = (a > 0.0) ? 1.0 / a : 1.0;
+    }
+    if (threadIdx.x == 160)
+        sq[5] = sqrt(st->rhobar * st->rhobar + beta * beta);
     __syncthreads();
     if (threadIdx.x != 0)
         return;
     SolveState s = *st;
     const double alpha = sq[0];
     const double irho = s.irho;
-    const double rho = sqrt(s.rhobar * s.rhobar + beta * beta);
+    const double rho = sq[5];
     const double c = s.rhobar * irho;
     const double sn = beta * irho;
     const double phi = c * s.phibar;
@@ -160,7 +171,7 @@ __device__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm
     s.xnorm = sq[1];
     s.anorm = sq[2];
     s.acond = s.anorm * sq[3];
-    s.ia = (alpha > 0.0) ? 1.0 / alpha : 1.0;
+    s.ia = sq[4];
     s.rnorm = s.phibar;
     s.arnorm = alpha * fabs(tau);
     s.itn += 1;
@@ -172,9 +183,9 @@ __device__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm
     const double anr = s.anorm * s.rnorm;
     int istop = 0;
     if (s.itn >= args->itmax) istop = 7;
-    if (1.0 + 1.0 / s.acond <= 1.0) istop = 6;
-    if (anr != 0.0 && 1.0 + s.arnorm / anr <= 1.0) istop = 5;
-    if (1.0 + s.rnorm / (s.bnorm + anx) <= 1.0) istop = 4;
+    if (s.acond * kHalfEps >= 1.0) istop = 6;
+    if (anr != 0.0 && s.arnorm <= kHalfEps * anr) istop = 5;
+    if (s.bnorm + anx > 0.0 && s.rnorm <= kHalfEps * (s.bnorm + anx)) istop = 4;
     if (args->ctol * s.acond >= 1.0 && args->ctol > 0.0) istop = 3;
     if (anr != 0.0 && s.arnorm <= args->atol * anr) istop = 2;
     if (s.rnorm <= rtol_b) istop = 1;
@@ -231,23 +242,23 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
     Acc3 c[3] = {Acc3{0.f, 0.f, 0.f}, Acc3{0.f, 0.f, 0.f}, Acc3{0.f, 0.f, 0.f}};
     double fb[3] = {0.0, 0.0, 0.0};
     double gacc = 0.0;
-#pragma unroll 2
-    for (int64_t j = gtid(); j < n; j += gstride()) {
+    // column j with q_j = qf(): the loads of the vectors come first, so that
+    // they are in flight together with those of the partial sums
+    auto update = [&](int64_t j, auto qf) {
         const double pj = p[j];
-        double qj;
-        if (INL) {
-            qj = (j < att0) ? q[j] : (j < glb0 ? q_from_parts(A, P, j) : 0.0);
-        } else {
-            qj = q[j];
-            if (j >= att0)
-                q[j] = 0.0;
+        double vo = 0.0, wo = 0.0, zo = 0.0, ro = 0.0;
+        if (!first) {
+            vo = v[j];
+            wo = w[j];
+            zo = z[j];
+            ro = var[j];
         }
-        const double vo = first ? 0.0 : v[j];
+        const double qj = qf();
         double wj = 0.0, zj = 0.0, vr = 0.0;
         if (!first) {
-            wj = fma(c2, w[j], vo * c1);
-            vr = fma(wj, wj, var[j]);
-            zj = fma(phi, wj, z[j]);
+            wj = fma(c2, wo, vo * c1);
+            vr = fma(wj, wj, ro);
+            zj = fma(phi, wj, zo);
             acc3_sqr_or(c[1], fb[1], wj);
             acc3_sqr_or(c[2], fb[2], zj);
         }
@@ -255,11 +266,39 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
         z[j] = zj;
         var[j] = vr;
         if (INL && j == glb0)
-            continue;  // V at the global column: the last block
+            return;  // V at the global column: the last block
         const double vn = upd ? fma(pj * qj, k1, k2 * vo) : vo;
         v[j] = vn;
         vp[j] = pj * vn;
         acc3_sqr_or(c[0], fb[0], vn);
+    };
+    // an instrument with many window totals is summed by a warp, which then
+    // updates its column
+    const bool warp_instr = INL && P.isplit > kThreadParts;
+    if (warp_instr) {
+        for (int64_t f = gtid() >> 5; f < A.I; f += gstride() >> 5) {
+            double t = 0.0;
+            for (int qq = threadIdx.x & 31; qq < P.isplit; qq += 32)
+                t += P.ipart[(int64_t)qq * A.I + f];
+            t = warp_sum(t);
+            if ((threadIdx.x & 31) == 0)
+                update(A.ins0 + f, [&] { return t; });
+        }
+    }
+#pragma unroll 2
+    for (int64_t j = gtid(); j < n; j += gstride()) {
+        if (INL) {
+            if (warp_instr && j >= A.ins0 && j < glb0)
+                continue;
+            update(j, [&] { return (j < att0) ? q[j] : (j < glb0 ? q_from_parts(A, P, j) : 0.0); });
+        } else {
+            update(j, [&] {
+                const double qj = q[j];
+                if (j >= att0)
+                    q[j] = 0.0;
+                return qj;
+            });
+        }
     }
     if (INL) {  // this block's fixed slice of the global-column partials
         const uint32_t per = ((uint32_t)P.ngpart + gridDim.x - 1) / gridDim.x;

@@ -1385,16 +1385,18 @@ int split_request(const gsr_config &cfg)
     return GSR_SPLIT_APROD1;
 }
 
+// the staged form (one block per SM) holds the pieces of more instruments than
+// the register form: whatever its stages leave, I <= 6,598
 bool aprod1_split(const gsr_handle_t *h)
 {
-    return (split_request(h->cfg) & GSR_SPLIT_APROD1) && h->sys.I <= kSplitInstrMax;
+    return (split_request(h->cfg) & GSR_SPLIT_APROD1) && (h->sys.I <= kSplitInstrMax || h->a1_tma);
 }
 
-// the staged form of aprod 1: its shared memory, 0 when the split products
-// do not apply
+// the staged form of aprod 1: its shared memory, 0 when split products are
+// not asked for
 size_t aprod1_tma_smem(const gsr_handle_t *h)
 {
-    return aprod1_split(h) ? tma_smem_bytes(h->sys.I) : 0;
+    return (split_request(h->cfg) & GSR_SPLIT_APROD1) ? tma_smem_bytes(h->sys.I) : 0;
 }
 
 // the staged form needs the split products and its stages in the opt-in
@@ -1411,8 +1413,18 @@ cudaError_t aprod1_tma_prepare(gsr_handle_t *h)
     const void *fns[6] = {(const void *)k_aprod1_tma<0, false>, (const void *)k_aprod1_tma<1, false>,
                           (const void *)k_aprod1_tma<2, false>, (const void *)k_aprod1_tma<0, true>,
                           (const void *)k_aprod1_tma<1, true>, (const void *)k_aprod1_tma<2, true>};
-    for (int i = 0; i < 6 && e == cudaSuccess; i++)
-        e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    for (int i = 0; i < 6 && e == cudaSuccess; i++) {
+        // all that a block may have, for every handle: the attribute belongs
+        // to the kernel, and handles ask for different sizes
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, fns[i]);
+        if (e != cudaSuccess)
+            return e;
+        const size_t most = (size_t)optin - fa.sharedSizeBytes;
+        if (need > most)
+            return cudaSuccess;
+        e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    }
     if (e == cudaSuccess)
         h->a1_tma_avail = 1;
     return e;

@@ -149,7 +149,7 @@ static void release(gsr_handle_t *h)
                    h->d_xp64, h->d_q64, h->d_iseg, h->d_cseg, h->d_cseg32, h->d_irow, h->d_ival32, h->d_ival, h->d_ipart, h->d_gpart, h->d_a2ctr, h->d_bX32, h->d_bQ32,
                    h->d_bC, h->d_bS_, h->d_bD, h->d_bZ, h->d_bT, h->d_bS, h->d_bXcm,
                    h->d_bCcm, h->d_bB, h->d_bnorms, h->d_bpartial, h->d_bcounter, h->d_bs,
-                   h->d_bipart, h->d_bticket,
+                   h->d_bipart, h->d_bticket, h->d_bar,
                    h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin,
                    h->d_epos, h->d_eptr, h->d_epart,
                    h->d_bargs};
@@ -606,6 +606,7 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
     TRY(dalloc(h, &h->d_counter, kRedCount));
     TRY(dalloc(h, &h->d_err, 1));
     TRY(dalloc(h, &h->d_kerr, 1));
+    TRY(dalloc(h, &h->d_bar, 1));
     CK(cudaMemset(h->d_counter, 0, kRedCount * sizeof(unsigned)));
     CK(cudaMemset(h->d_err, 0, sizeof(int)));
     CK(cudaMemset(h->d_kerr, 0, sizeof(int)));

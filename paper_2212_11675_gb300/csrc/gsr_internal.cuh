@@ -125,8 +125,21 @@ struct A2Parts {
     Ell ell;
 };
 
+// A load of data that other blocks of the same launch write (CG: from L2,
+// after a barrier of the grid) or that no block does
+template <bool CG>
+__device__ __forceinline__ double ld_shared(const double *p)
+{
+    if (!CG)
+        return __ldg(p);
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+
 // Attitude column a D + k from the segment sums: sum_{jj<4} S[k-jj][4a+jj],
 // the pieces of an offset in order
+template <bool CG = false>
 __device__ __forceinline__ double att_column(const SysView &A, const double *__restrict__ S, int64_t a,
                                              int64_t k)
 {
@@ -136,7 +149,7 @@ __device__ __forceinline__ double att_column(const SysView &A, const double *__r
         for (int jj = 0; jj < 4; jj++) {
             const int64_t o = k - jj;
             if (o >= 0 && o < A.nseg)
-                t += S[o * kNAtt + 4 * a + jj];
+                t += ld_shared<CG>(S + o * kNAtt + 4 * a + jj);
         }
     } else {
 #pragma unroll
@@ -146,7 +159,7 @@ __device__ __forceinline__ double att_column(const SysView &A, const double *__r
                 const double *s = S + o * A.attp * kNAtt + 4 * a + jj;
 #pragma unroll 4
                 for (int q = 0; q < (int)A.attp; q++)
-                    t += s[q * kNAtt];
+                    t += ld_shared<CG>(s + q * kNAtt);
             }
         }
     }
@@ -156,6 +169,7 @@ __device__ __forceinline__ double att_column(const SysView &A, const double *__r
 // q_j of the non-astrometric columns from the partial sums: an attitude column
 // as above; instrument f the sum of its window totals (both in the combine
 // kernel's order)
+template <bool CG = false>
 __device__ __forceinline__ double q_from_parts(const SysView &A, const A2Parts &P, int64_t j)
 {
     if (j < A.ins0) {
@@ -163,13 +177,13 @@ __device__ __forceinline__ double q_from_parts(const SysView &A, const A2Parts &
         // division is a long instruction sequence on the GPU)
         const int64_t c = j - A.att0;
         const int64_t a = (c >= A.D) + (c >= 2 * A.D);
-        return att_column(A, P.S, a, c - a * A.D);
+        return att_column<CG>(A, P.S, a, c - a * A.D);
     }
     const int64_t f = j - A.ins0;
     double t = 0.0;
 #pragma unroll 4
     for (int qq = 0; qq < P.isplit; qq++)
-        t += P.ipart[(int64_t)qq * A.I + f];
+        t += ld_shared<CG>(P.ipart + (int64_t)qq * A.I + f);
     return t;
 }
 
@@ -357,6 +371,7 @@ struct gsr_handle_t {
     // aprod 1 with its tiles staged by the bulk-copy engine (k_aprod1_tma)
     int a1_tma = 0;                     // 1: the staged form runs
     int a1_tma_avail = 0;               // 1: the staged form applies on this device
+    unsigned *d_bar = nullptr;          // barrier count of k_lsqr_loop
     int *d_kerr = nullptr;              // set by a kernel whose bounded wait expired
     int64_t drop_tile = -1;             // test hook: the tile whose bulk copy is not issued
 };
@@ -431,6 +446,9 @@ cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st);
 int f32_main_grid(const gsr_handle_t *h);
 int f32_rest_grid(const gsr_handle_t *h);
 cudaError_t enqueue_precondition(const gsr_handle_t *h, double *p, cudaStream_t st);
+// all LSQR iterations of a small system in one launch (gsr_kernels.cu)
+bool lsqr_loop_fits(const gsr_handle_t *h);
+cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st);
 // LSQR pieces (gsr_lsqr.cu)
 cudaError_t build_solve_graph(gsr_handle_t *h);
 cudaError_t enqueue_prologue(const gsr_handle_t *h, cudaStream_t s,

@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "gsr_internal.cuh"
+#include "gsr_lsqr.cuh"
 #include "gsr_reduce.cuh"
 #include "gsr_split.cuh"
 #include "gsr_tma.cuh"
@@ -120,7 +121,7 @@ __device__ __forceinline__ uint32_t instr_at(const uint4 &rc, int j)
 // binary32 pipes (x pieces s_x4 in shared memory, global pieces g1..g3).
 // ASTRO (with SPLIT): the five astrometric products too, with the star's x
 // split per row.
-template <bool SMEMX, bool SPLIT, bool ASTRO = false>
+template <bool SMEMX, bool SPLIT, bool ASTRO = false, bool CG = false>
 __device__ __forceinline__ double row_sum(const SysView &A, const double *__restrict__ x,
                                           const double (&vk)[kNPar], const uint4 &rc, uint32_t s,
                                           const float4 *s_x4, const double *s_xi, bool split_x,
@@ -158,7 +159,7 @@ __device__ __forceinline__ double row_sum(const SysView &A, const double *__rest
                 for (int k = 0; k < kNAstro; k++) {
                     float a1, a2, a3, x1, x2, x3;
                     rng = max(rng, split3z(vk[k], a1, a2, a3));
-                    rng = max(rng, split3z(__ldg(xs + k), x1, x2, x3));
+                    rng = max(rng, split3z(ld_shared<CG>(xs + k), x1, x2, x3));
                     acc3_fma(c, a1, a2, a3, x1, x2, x3);
                 }
             }
@@ -171,47 +172,47 @@ __device__ __forceinline__ double row_sum(const SysView &A, const double *__rest
             s0 = vk[23] * xg;
 #pragma unroll
             for (int j = 0; j < kNInstr; j++)
-                s0 = fma(vk[17 + j], __ldg(x + A.ins0 + instr_at(rc, j)), s0);
+                s0 = fma(vk[17 + j], ld_shared<CG>(x + A.ins0 + instr_at(rc, j)), s0);
             s1 = 0.0;
             if constexpr (ASTRO) {
 #pragma unroll
                 for (int k = 0; k < kNAstro; k++)
-                    s0 = fma(vk[k], __ldg(xs + k), s0);
+                    s0 = fma(vk[k], ld_shared<CG>(xs + k), s0);
             }
         }
         if constexpr (!ASTRO) {
 #pragma unroll
             for (int k = 0; k < kNAstro; k++)
-                s0 = fma(vk[k], __ldg(xs + k), s0);
+                s0 = fma(vk[k], ld_shared<CG>(xs + k), s0);
         }
         const double *xa = x + A.att0 + rc.x;
 #pragma unroll
         for (int a = 0; a < 3; a++)
 #pragma unroll
             for (int j = 0; j < 4; j++)
-                s1 = fma(vk[5 + 4 * a + j], __ldg(xa + a * A.D + j), s1);
+                s1 = fma(vk[5 + 4 * a + j], ld_shared<CG>(xa + a * A.D + j), s1);
     } else {
         const double *xs = x + (int64_t)kNAstro * s;
-        s0 = vk[0] * __ldg(xs);
+        s0 = vk[0] * ld_shared<CG>(xs);
 #pragma unroll
         for (int k = 1; k < kNAstro; k++)
-            s0 = fma(vk[k], __ldg(xs + k), s0);
+            s0 = fma(vk[k], ld_shared<CG>(xs + k), s0);
         const double *xa = x + A.att0 + rc.x;
-        s1 = vk[5] * __ldg(xa);
+        s1 = vk[5] * ld_shared<CG>(xa);
 #pragma unroll
         for (int j = 1; j < 4; j++)
-            s1 = fma(vk[5 + j], __ldg(xa + j), s1);
+            s1 = fma(vk[5 + j], ld_shared<CG>(xa + j), s1);
 #pragma unroll
         for (int j = 0; j < 4; j++)
-            s1 = fma(vk[9 + j], __ldg(xa + A.D + j), s1);
+            s1 = fma(vk[9 + j], ld_shared<CG>(xa + A.D + j), s1);
         s0 = fma(vk[23], xg, s0);
 #pragma unroll
         for (int j = 0; j < 4; j++)
-            s1 = fma(vk[13 + j], __ldg(xa + 2 * A.D + j), s1);
+            s1 = fma(vk[13 + j], ld_shared<CG>(xa + 2 * A.D + j), s1);
 #pragma unroll
         for (int j = 0; j < kNInstr; j++) {
             const uint32_t f = instr_at(rc, j);
-            s0 = fma(vk[17 + j], SMEMX ? s_xi[f] : __ldg(x + A.ins0 + f), s0);
+            s0 = fma(vk[17 + j], SMEMX ? s_xi[f] : ld_shared<CG>(x + A.ins0 + f), s0);
         }
     }
     return s0 + s1;
@@ -241,6 +242,26 @@ __device__ __forceinline__ void lsqr_beta_rotation(SolveState *st, double unorm2
     __syncthreads();
     if (threadIdx.x == 0)
         st->t1 = rhobar * sq[1] * st->phibar;  // phi = c phibar, c = rhobar / rho
+}
+
+// the same by one warp, in two lanes
+__device__ __forceinline__ void lsqr_beta_rotation_warp(SolveState *st, double unorm2)
+{
+    const int lane = threadIdx.x & 31;
+    const double rhobar = st->rhobar, ia = st->ia, phibar = st->phibar;
+    const double r = sqrt(lane == 0 ? unorm2 : rhobar * rhobar + unorm2 * ia * ia);
+    const double d = lane == 0 ? r * ia : r;  // beta, rho
+    const double inv = 1.0 / d;
+    const double irho = __shfl_sync(0xffffffffu, inv, 1);
+    __syncwarp();
+    if (lane == 0) {
+        st->beta_new = r;
+        st->bnext = d;
+        st->ib = (d > 0.0) ? inv : 0.0;
+        st->irho = irho;
+        st->t1 = rhobar * irho * phibar;  // phi = c phibar, c = rhobar / rho
+    }
+    __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
@@ -530,7 +551,7 @@ k_aprod1_tma(SysView A, const double *__restrict__ x, double *__restrict__ y, So
 // per star (rows are star-grouped), the instrumental products unless the
 // sorted path (IP == kIpSorted) takes them, and this thread's share of the
 // global column, which is returned.
-template <int G, int MODE, int IP>
+template <int G, int MODE, int IP, bool CG = false>
 __device__ __forceinline__ double stars_body(const SysView &A, const double *__restrict__ y,
                                              double *__restrict__ out, double *__restrict__ rep,
                                              int nrep, double *s_ins, int64_t warp, int64_t nwarps)
@@ -573,7 +594,7 @@ __device__ __forceinline__ double stars_body(const SysView &A, const double *__r
                     vi[j] *= vi[j];
                 vg *= vg;
             } else {
-                yi = __ldcs(y + r);
+                yi = CG ? ld_shared<true>(y + r) : __ldcs(y + r);
             }
             a0 = fma(va[0], yi, a0);
             a1 = fma(va[1], yi, a1);
@@ -899,7 +920,7 @@ k_aprod2_stars(SysView A, const double *__restrict__ y, double *__restrict__ out
 // adds the nwin window totals of each instrument in a fixed order: no
 // atomics, deterministic.  SQ: squares of the values.
 // ---------------------------------------------------------------------------
-template <bool SQ>
+template <bool SQ, bool CG = false>
 __device__ __forceinline__ void instr_body(const SysView &A, const uint32_t *__restrict__ cseg,
                                            const uint32_t *__restrict__ irow,
                                            const double *__restrict__ ival,
@@ -933,7 +954,7 @@ __device__ __forceinline__ void instr_body(const SysView &A, const uint32_t *__r
                     r[u] = __ldcs(irow + e + 32 * u);
 #pragma unroll
                 for (int u = 0; u < 4; u++)
-                    yv[u] = __ldg(y + r[u]);
+                    yv[u] = ld_shared<CG>(y + r[u]);
             }
 #pragma unroll
             for (int u = 0; u < 4; u++)
@@ -941,7 +962,7 @@ __device__ __forceinline__ void instr_body(const SysView &A, const uint32_t *__r
         }
         for (int u = 0; e < e1; e += 32, u++) {
             const double v = __ldcs(ival + e);
-            acc[u & 3] = fma(v, SQ ? v : __ldg(y + __ldcs(irow + e)), acc[u & 3]);
+            acc[u & 3] = fma(v, SQ ? v : ld_shared<CG>(y + __ldcs(irow + e)), acc[u & 3]);
         }
         const double t = warp_sum_split<4>(acc);
         if (lane == 0)
@@ -1001,7 +1022,7 @@ __device__ __forceinline__ void att_range(const SysView &A, int64_t u, uint32_t 
     e1 = s0 + (uint32_t)(len * (q + 1) / np);
 }
 
-template <bool SQ>
+template <bool SQ, bool CG = false>
 __device__ __forceinline__ void att_body(const SysView &A, const double *__restrict__ y,
                                          double *__restrict__ S, int64_t warp, int64_t nwarps)
 {
@@ -1016,7 +1037,7 @@ __device__ __forceinline__ void att_body(const SysView &A, const double *__restr
         // the y of the next entry (row number, then the gather: two dependent
         // loads) is on its way while the current one is summed
         uint32_t e = e0 + lane;
-        double yn = (SQ || e >= e1) ? 1.0 : __ldg(y + __ldcs(A.perm + e));
+        double yn = (SQ || e >= e1) ? 1.0 : ld_shared<CG>(y + __ldcs(A.perm + e));
         uint32_t rn = (SQ || e + 32 >= e1) ? 0u : __ldcs(A.perm + e + 32);
         for (; e < e1; e += 32) {
             const double yi = yn;
@@ -1025,7 +1046,7 @@ __device__ __forceinline__ void att_body(const SysView &A, const double *__restr
             for (int k = 0; k < kNAtt; k++)
                 v[k] = __ldcs(A.tval + tidx<kNAtt>(k, e));
             if (!SQ && e + 32 < e1) {
-                yn = __ldg(y + rn);
+                yn = ld_shared<CG>(y + rn);
                 if (e + 64 < e1)
                     rn = __ldcs(A.perm + e + 64);
             }
@@ -1295,6 +1316,252 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
             t = atomicAdd(q.ctr, 1ull);
         u = nfix + __shfl_sync(0xffffffffu, t, 0);
     }
+}
+
+// ---------------------------------------------------------------------------
+// All LSQR iterations of a small system in one launch (cooperative: every
+// block is resident).  An iteration as three launches costs about 35 us on
+// the 1,000-star system however little work it has: three launch ramps, three
+// grid reductions whose last block works alone.  Here its three parts are
+// separated by barriers of the grid, and every block works out the sums of
+// the blocks' partials and the scalar recurrences for itself, in the same
+// order, so no block waits for another's result (20,000 rows: 36.6 -> 27 us an
+// iteration; 280,000: 80.7 -> 74; from 500,000 rows on the launches win).
+//   1. U = A vp + cy U, ||U||^2 (rows as in k_aprod1's split form)
+//   2. star, attitude and instrument units of A^T U, one after the other
+//   3. the columns; block 0 adds the global column
+// One warp of each block works out the scalars beside the others' work: the
+// rotation during part 2, the recurrences and stopping rules during part 1 of
+// the next iteration (which changes only U, so it may be one too many).
+// Data that other blocks write is read from L2 (ld_shared).  Each wait of the
+// barrier is bounded: when it runs out the block sets *kerr and ends.
+// Taken up to kLoopRows rows: beyond, the staged aprod 1 and the dynamic unit
+// queue of the separate launches win.
+// ---------------------------------------------------------------------------
+constexpr int kLoopThreads = 512;
+constexpr int64_t kLoopRows = 400000;
+
+struct LoopArgs {
+    double *u, *q, *S, *ipart, *gpart;
+    VecPass X;
+    const uint32_t *cseg, *irow;
+    const double *ival;
+    int isplit;
+    int64_t ngroups, ninstr;  // star groups (units), instrument units
+    SolveState *st;
+    const SolveArgs *args;
+    double *partial;          // [4][kMaxPartials]
+    unsigned *bar;            // zero on entry
+    int *kerr;
+};
+
+// Barrier of the grid: false when the others did not arrive in time
+__device__ __forceinline__ bool loop_sync(unsigned *bar, unsigned &target, int *kerr)
+{
+    __shared__ int s_ok;
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        bool ok = true;
+        uint64_t t0 = 0;
+        for (int it = 0;; it++) {
+            unsigned c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(bar) : "memory");
+            if ((int)(c - target) >= 0)
+                break;
+            if (it == 0)
+                t0 = global_ns();
+            else if ((it & 63) == 0 && global_ns() - t0 > kWaitNs) {
+                atomicExch(kerr, 1);
+                ok = false;
+                break;
+            }
+        }
+        __threadfence();
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// Sums over the grid of K values per thread, without a last block: block sums
+// into partial (loop_part), a barrier of the grid, then every block adds the
+// blocks' partials for itself, sum k by warp k (loop_total).  The FP64 pipe
+// takes 16 clocks for a warp's addition, so only warps that have something to
+// add do so (busy: the same for a whole warp): 16 warps reducing three zeros
+// each cost 2 us, and every warp adding the partials for itself 5 us.
+template <int K>
+__device__ __forceinline__ void loop_part(double (&v)[K], bool busy, double *partial)
+{
+    constexpr int NW = kLoopThreads / 32;
+    __shared__ double sh[K][NW];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        const double t = busy ? warp_sum(v[k]) : 0.0;
+        if (lane == 0)
+            sh[k][wib] = t;
+    }
+    __syncthreads();
+    if (wib < K) {
+        double t = lane < NW ? sh[wib][lane] : 0.0;
+#pragma unroll
+        for (int off = NW / 2; off > 0; off >>= 1)
+            t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (lane == 0)
+            partial[wib * kMaxPartials + blockIdx.x] = t;
+    }
+}
+
+template <int K>
+__device__ __forceinline__ void loop_total(double (&v)[K], const double *partial)
+{
+    __shared__ double sh[K];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    if (wib < K) {
+        double t = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32)
+            t += ld_shared<true>(partial + wib * kMaxPartials + b);
+        t = warp_sum(t);
+        if (lane == 0)
+            sh[wib] = t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; k++)
+        v[k] = sh[k];
+}
+
+template <int G>
+__global__ void __launch_bounds__(kLoopThreads, 1)
+k_lsqr_loop(SysView A, LoopArgs L)
+{
+    constexpr int NW = kLoopThreads / 32;
+    extern __shared__ float4 s_x4[];
+    __shared__ SolveState s;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // warps (and threads) numbered blocks first, so that few units spread
+    // over the SMs
+    const int64_t gw = blockIdx.x + (int64_t)gridDim.x * wib, nw = (int64_t)gridDim.x * NW;
+    const int64_t ntiles = (A.m + 31) >> 5;
+    unsigned target = 0;
+    if (threadIdx.x == 0)
+        s = *L.st;
+    __syncthreads();
+    double cy = s.cy;
+    if (s.done)
+        return;
+    for (;;) {
+        // 1. rows
+        const double *x = L.X.vp;
+        const double xg = ld_shared<true>(x + A.glb0);
+        float g1, g2, g3;
+        const bool split_x = split3z(xg, g1, g2, g3) < kSplitRangeSpan;
+        for (int64_t f = threadIdx.x; f < A.I; f += kLoopThreads) {
+            float p1, p2, p3;
+            const bool ok = split3z(ld_shared<true>(x + A.ins0 + f), p1, p2, p3) < kSplitRangeSpan;
+            s_x4[f] = make_float4(p1, p2, p3, ok ? 0.f : 1.f);
+        }
+        __syncthreads();
+        double nrm[1] = {0.0};
+        for (int64_t t = gw; t < ntiles; t += nw) {
+            const int64_t r = (t << 5) + lane;
+            if (r < A.m) {
+                const uint32_t star = star_of_row(A, t, r);
+                const uint4 rc = __ldg(A.rec + r);
+                const double *v = A.val + tidx<kNPar>(0, r);
+                double vk[kNPar];
+#pragma unroll
+                for (int k = 0; k < kNPar; k++)
+                    vk[k] = __ldg(v + 32 * k);
+                const double sum = row_sum<true, true, false, true>(A, x, vk, rc, star, s_x4, nullptr,
+                                                                    split_x, xg, g1, g2, g3);
+                const double yn = fma(cy, L.u[r], sum);
+                nrm[0] = fma(yn, yn, nrm[0]);
+                L.u[r] = yn;
+            }
+        }
+        loop_part<1>(nrm, gw < ntiles, L.partial);
+        if (!loop_sync(L.bar, target, L.kerr))
+            return;
+        if (s.done)  // by the recurrences of the iteration before
+            break;
+        if (wib == NW - 1) {
+            double t = 0.0;
+            for (unsigned b = lane; b < gridDim.x; b += 32)
+                t += ld_shared<true>(L.partial + b);
+            lsqr_beta_rotation_warp(&s, warp_sum(t));
+        }
+        // 2. units
+        const int64_t natt = A.nseg * A.attp;
+        for (int64_t i = gw; i < natt + L.ninstr + L.ngroups; i += nw) {
+            if (i < natt) {
+                att_body<false, true>(A, L.u, L.S, i, natt);
+            } else if (i < natt + L.ninstr) {
+                instr_body<false, true>(A, L.cseg, L.irow, L.ival, L.u, L.ipart, L.isplit, i - natt,
+                                        L.ninstr);
+            } else {
+                const int64_t grp = i - natt - L.ninstr;
+                const double g[1] = {stars_body<G, kA2Overwrite, kIpSorted, true>(
+                    A, L.u, L.q, nullptr, 1, nullptr, grp, L.ngroups)};
+                const double t = warp_sum_split<1>(g);
+                if (lane == 0)
+                    L.gpart[grp] = t;
+            }
+        }
+        if (!loop_sync(L.bar, target, L.kerr))
+            return;
+        // 3. columns
+        const VecCoef k = vec_coef(&s, 0);
+        const A2Parts P = {L.S, L.ipart, L.isplit, nullptr, 0, nullptr, Ell{}};
+        VecSums S;
+        const bool warp_instr = L.isplit > kThreadParts;
+        if (warp_instr) {
+            for (int64_t f = gw; f < A.I; f += nw) {
+                double t = 0.0;
+                for (int qq = lane; qq < L.isplit; qq += 32)
+                    t += ld_shared<true>(L.ipart + (int64_t)qq * A.I + f);
+                t = warp_sum(t);
+                if (lane == 0)
+                    vec_column(L.X, k, S, A.ins0 + f, false, [&] { return t; });
+            }
+        }
+        const int64_t end = warp_instr ? A.ins0 : A.glb0;
+        for (int64_t j = gw * 32 + lane; j < end; j += nw * 32)
+            vec_column(L.X, k, S, j, false, [&] {
+                return j < A.att0 ? ld_shared<true>(L.q + j) : q_from_parts<true>(A, P, j);
+            });
+        if (blockIdx.x == 0 && wib == NW - 1) {  // the global column
+            double t = 0.0;
+#pragma unroll 4
+            for (int64_t b = lane; b < L.ngroups; b += 32)
+                t += ld_shared<true>(L.gpart + b);
+            t = warp_sum(t);
+            if (lane == 0)
+                vec_column(L.X, k, S, A.glb0, false, [&] { return t; });
+        }
+        const bool busy = gw * 32 < end || (warp_instr && gw < A.I) ||
+                          (blockIdx.x == 0 && wib == NW - 1);
+        double acc[3] = {0.0, 0.0, 0.0};
+        if (busy) {
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                acc[i] = S.total(i);
+        }
+        loop_part<3>(acc, busy, L.partial + kMaxPartials);
+        const double ia = s.ia, ib = s.ib, alpha = s.alpha, bn = s.bnext;
+        if (!loop_sync(L.bar, target, L.kerr))
+            return;
+        loop_total<3>(acc, L.partial + kMaxPartials);
+        // -alpha_{i+1}^2 / (alpha_i beta_{i+1})
+        cy = -(bn > 0.0 ? acc[0] : alpha * alpha) * ia * ib;
+        if (wib == NW - 1)
+            lsqr_scalars_warp(&s, L.args, acc[0], acc[1], acc[2]);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *L.st = s;
 }
 
 // Pass 2, fused with the instrumental replicas.  Blocks [0, nb_att) combine
@@ -1667,6 +1934,40 @@ cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out, i
                                   mode == kA2Accumulate, st, h->d_a2ctr);
     }
     return launch_aprod2_split(h, y, out, mode, st);
+}
+
+bool lsqr_loop_fits(const gsr_handle_t *h)
+{
+    return h->sys.m <= kLoopRows && h->sys.I <= kSplitInstrMax && h->ipath == kIpSorted &&
+           h->a2_fused && h->cfg.products == GSR_PRODUCTS_AUTO && h->drop_tile < 0 &&
+           h->nsm <= kMaxPartials;
+}
+
+template <int G>
+static cudaError_t loop_launch(const gsr_handle_t *h, cudaStream_t st)
+{
+    LoopArgs L = {h->d_u, h->d_q, h->d_attS, h->d_ipart, h->d_gpart,
+                  VecPass{h->d_p, h->d_v, h->d_vp, h->d_w, h->d_z, h->d_var},
+                  h->d_cseg, h->d_irow, h->d_ival, h->isplit,
+                  (h->sys.S + 32 / G - 1) / (32 / G), h->sys.I * h->isplit,
+                  h->d_state, h->d_args, h->d_partial, h->d_bar, h->d_kerr};
+    SysView A = h->sys;
+    void *args[] = {&A, &L};
+    cudaError_t e = cudaMemsetAsync(h->d_bar, 0, sizeof(unsigned), st);
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel(k_lsqr_loop<G>, dim3(h->nsm), dim3(kLoopThreads), args,
+                                        (size_t)A.I * sizeof(float4), st);
+    return e;
+}
+
+cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st)
+{
+    switch (h->lanes) {
+    case 4: return loop_launch<4>(h, st);
+    case 8: return loop_launch<8>(h, st);
+    case 32: return loop_launch<32>(h, st);
+    default: return loop_launch<16>(h, st);
+    }
 }
 
 // With the single-launch aprod 2: launch it without the combine, writing the

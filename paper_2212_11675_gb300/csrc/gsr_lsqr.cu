@@ -35,13 +35,12 @@
 #include <math.h>
 
 #include "gsr_internal.cuh"
+#include "gsr_lsqr.cuh"
 #include "gsr_reduce.cuh"
 #include "gsr_split.cuh"
 
 namespace gsr {
 
-constexpr int kIstopNonfinite = 8;
-constexpr int kThreadParts = 8;  // window totals of an instrument that one thread adds
 
 __device__ __forceinline__ int64_t gtid() { return blockIdx.x * (int64_t)blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
@@ -114,98 +113,6 @@ __device__ void init_scalars(SolveState *st, const SolveArgs *args, double vnorm
         cudaGraphSetConditional(loop, 0u);
 }
 
-// Scalar recurrences of one LSQR iteration, run by the whole last block of
-// the vector pass.  The independent square roots and the reciprocal of the new
-// alpha go to different warps; everything else is one thread, with products by
-// reciprocals already known (1/rho from the aprod 1 pass) instead of
-// divisions, because FP64 divisions and square roots take a third of a
-// microsecond each on this part and every dependent operation 65 clocks.  The
-// tests of the machine-precision rules are multiplied out:
-// 1 + a / b <= 1 exactly when a <= 2^-53 b (up to the rounding of a / b).
-__device__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm2,
-                             double dd, double zz, cudaGraphConditionalHandle loop, int in_graph)
-{
-    __shared__ double sq[6];
-    constexpr double kHalfEps = 1.0 / 9007199254740992.0;  // 2^-53
-    const double beta = st->bnext;
-    const bool upd = beta > 0.0;
-    const double anorm2 = upd ? st->anorm2 + st->alpha * st->alpha + beta * beta : st->anorm2;
-    const double ddnorm = st->ddnorm + dd;
-    if (threadIdx.x == 0)
-        sq[0] = upd ? sqrt(vnorm2) : st->alpha;
-    if (threadIdx.x == 32)
-        sq[1] = sqrt(zz);
-    if (threadIdx.x == 64)
-        sq[2] = sqrt(anorm2);
-    if (threadIdx.x == 96)
-        sq[3] = sqrt(ddnorm);
-    if (threadIdx.x == 128) {
-        const double a = upd ? sqrt(vnorm2) : st->alpha;
-        sq[4] = (a > 0.0) ? 1.0 / a : 1.0;
-    }
-    if (threadIdx.x == 160)
-        sq[5] = sqrt(st->rhobar * st->rhobar + beta * beta);
-    __syncthreads();
-    if (threadIdx.x != 0)
-        return;
-    SolveState s = *st;
-    const double alpha = sq[0];
-    const double irho = s.irho;
-    const double rho = sq[5];
-    const double c = s.rhobar * irho;
-    const double sn = beta * irho;
-    const double phi = c * s.phibar;
-    s.anorm2 = anorm2;
-    s.theta = sn * alpha;
-    s.rhobar = -c * alpha;
-    s.phibar = sn * s.phibar;
-    const double tau = sn * phi;
-    s.rho = rho;
-    s.cs = c;
-    s.sn = sn;
-    s.phi = phi;
-    s.alpha = alpha;
-    s.beta = beta;
-    s.cy = -alpha * alpha * s.ia * s.ib;  // -alpha_{i+1}^2 / (alpha_i beta_{i+1})
-    s.ddnorm = ddnorm;
-    s.xnorm = sq[1];
-    s.anorm = sq[2];
-    s.acond = s.anorm * sq[3];
-    s.ia = sq[4];
-    s.rnorm = s.phibar;
-    s.arnorm = alpha * fabs(tau);
-    s.itn += 1;
-    s.t = s.rnorm * args->isdof;
-
-    // stopping rules (P&S 1982 §6) in multiplied form; a later rule wins
-    const double anx = s.anorm * s.xnorm;
-    const double rtol_b = args->btol * s.bnorm + args->atol * anx;  // rtol * bnorm
-    const double anr = s.anorm * s.rnorm;
-    int istop = 0;
-    if (s.itn >= args->itmax) istop = 7;
-    if (s.acond * kHalfEps >= 1.0) istop = 6;
-    if (anr != 0.0 && s.arnorm <= kHalfEps * anr) istop = 5;
-    if (s.bnorm + anx > 0.0 && s.rnorm <= kHalfEps * (s.bnorm + anx)) istop = 4;
-    if (args->ctol * s.acond >= 1.0 && args->ctol > 0.0) istop = 3;
-    if (anr != 0.0 && s.arnorm <= args->atol * anr) istop = 2;
-    if (s.rnorm <= rtol_b) istop = 1;
-    const bool bad = !isfinite(rho) || !isfinite(alpha) || !isfinite(s.phibar) ||
-                     !isfinite(s.xnorm) || !isfinite(s.ddnorm) || rho == 0.0;
-    if (bad) {
-        s.nonfinite = 1;
-        istop = kIstopNonfinite;
-    }
-    if (args->force_itmax && !bad && s.itn < args->itmax)
-        istop = 0;
-    s.istop = istop;
-    if (istop != 0) {
-        s.done = 1;
-        if (in_graph)
-            cudaGraphSetConditional(loop, 0u);
-    }
-    *st = s;
-}
-
 // The vector pass of iteration i (first: the start, V_1 = p o A^T b / beta_1
 // with w, z, var cleared).  The stored w is W_i = w_i / rho_i of the paper's
 // recurrence, which takes the division by rho out of three updates:
@@ -230,48 +137,10 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
       unsigned *counter, cudaGraphConditionalHandle loop, int in_graph, int first, A2Parts P)
 {
     const int64_t n = A.n, att0 = A.att0, glb0 = A.glb0;
-    const double ia = st->ia;           // 1/alpha_i
-    const double ib = st->ib;           // 1/beta_{i+1}
-    const double bn = st->bnext;        // beta_{i+1}
-    const double irho = first ? 0.0 : st->irho;  // 1/rho_i
-    const double c1 = ia * irho;                 // 1/(alpha_i rho_i)
-    const double c2 = first ? 0.0 : -st->theta * irho;
-    const double phi = first ? 0.0 : st->t1;     // phi_i
-    const bool upd = bn > 0.0;
-    const double k1 = ia * ib, k2 = -bn * ia;
-    Acc3 c[3] = {Acc3{0.f, 0.f, 0.f}, Acc3{0.f, 0.f, 0.f}, Acc3{0.f, 0.f, 0.f}};
-    double fb[3] = {0.0, 0.0, 0.0};
+    const VecCoef k = vec_coef(st, first);
+    const VecPass X = {p, v, vp, w, z, var};
+    VecSums S;
     double gacc = 0.0;
-    // column j with q_j = qf(): the loads of the vectors come first, so that
-    // they are in flight together with those of the partial sums
-    auto update = [&](int64_t j, auto qf) {
-        const double pj = p[j];
-        double vo = 0.0, wo = 0.0, zo = 0.0, ro = 0.0;
-        if (!first) {
-            vo = v[j];
-            wo = w[j];
-            zo = z[j];
-            ro = var[j];
-        }
-        const double qj = qf();
-        double wj = 0.0, zj = 0.0, vr = 0.0;
-        if (!first) {
-            wj = fma(c2, wo, vo * c1);
-            vr = fma(wj, wj, ro);
-            zj = fma(phi, wj, zo);
-            acc3_sqr_or(c[1], fb[1], wj);
-            acc3_sqr_or(c[2], fb[2], zj);
-        }
-        w[j] = wj;
-        z[j] = zj;
-        var[j] = vr;
-        if (INL && j == glb0)
-            return;  // V at the global column: the last block
-        const double vn = upd ? fma(pj * qj, k1, k2 * vo) : vo;
-        v[j] = vn;
-        vp[j] = pj * vn;
-        acc3_sqr_or(c[0], fb[0], vn);
-    };
     // an instrument with many window totals is summed by a warp, which then
     // updates its column
     const bool warp_instr = INL && P.isplit > kThreadParts;
@@ -282,7 +151,7 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
                 t += P.ipart[(int64_t)qq * A.I + f];
             t = warp_sum(t);
             if ((threadIdx.x & 31) == 0)
-                update(A.ins0 + f, [&] { return t; });
+                vec_column(X, k, S, A.ins0 + f, false, [&] { return t; });
         }
     }
 #pragma unroll 2
@@ -290,9 +159,11 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
         if (INL) {
             if (warp_instr && j >= A.ins0 && j < glb0)
                 continue;
-            update(j, [&] { return (j < att0) ? q[j] : (j < glb0 ? q_from_parts(A, P, j) : 0.0); });
+            vec_column(X, k, S, j, j == glb0, [&] {
+                return (j < att0) ? q[j] : (j < glb0 ? q_from_parts(A, P, j) : 0.0);
+            });
         } else {
-            update(j, [&] {
+            vec_column(X, k, S, j, false, [&] {
                 const double qj = q[j];
                 if (j >= att0)
                     q[j] = 0.0;
@@ -309,8 +180,8 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
     }
     double acc[4];
 #pragma unroll
-    for (int k = 0; k < 3; k++)
-        acc[k] = acc3_to_double(c[k]) + fb[k];
+    for (int i = 0; i < 3; i++)
+        acc[i] = S.total(i);
     acc[3] = gacc;
     if (grid_reduce<4>(acc, partial, counter)) {
         __shared__ double vn2;
@@ -319,7 +190,7 @@ k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, dou
             if (INL) {
                 const double vo = first ? 0.0 : v[glb0];
                 const double pj = p[glb0];
-                const double vn = upd ? fma(pj * acc[3], k1, k2 * vo) : vo;
+                const double vn = k.upd ? fma(pj * acc[3], k.k1, k.k2 * vo) : vo;
                 v[glb0] = vn;
                 vp[glb0] = pj * vn;
                 vn2 = fma(vn, vn, vn2);
@@ -508,6 +379,8 @@ cudaError_t enqueue_epilogue(const gsr_handle_t *h, cudaStream_t s)
 // Build and instantiate the graph of one whole solve:
 //   [precondition, U_1 = b, q = A^T U_1, V_1]  ->  WHILE(flag) { iteration }
 //   ->  [x = p o z, se]
+// or, for a small system, with one launch for all iterations in place of the
+// loop (k_lsqr_loop).
 cudaError_t build_solve_graph(gsr_handle_t *h)
 {
     cudaError_t err = cudaSuccess;
@@ -519,6 +392,18 @@ cudaError_t build_solve_graph(gsr_handle_t *h)
     cudaStream_t s = h->cap_stream;
 
     GSR_TRY(cudaGraphCreate(&g, 0));
+    if (lsqr_loop_fits(h)) {
+        // a small system: all iterations in one launch
+        GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0,
+                                              cudaStreamCaptureModeThreadLocal));
+        GSR_TRY(enqueue_prologue(h, s, 0, 0));
+        GSR_TRY(launch_lsqr_loop(h, s));
+        GSR_TRY(enqueue_epilogue(h, s));
+        GSR_TRY(cudaStreamEndCapture(s, &g));
+        GSR_TRY(cudaGraphInstantiate(&h->solve_exec, g, 0));
+        cudaGraphDestroy(g);
+        return cudaSuccess;
+    }
     GSR_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
 
     GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));

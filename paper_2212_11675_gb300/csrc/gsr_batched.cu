@@ -360,21 +360,29 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
 }
 
 // ---------------------------------------------------------------------------
-// aprod 2, astrometric nonzeros on KT columns (star-parallel): T[astro rows]
+// aprod 2, astrometric nonzeros on KT columns (star-parallel): T[astro rows].
+// G lanes own a star: KT / 2 lanes take a pair of columns each of one row, G
+// over that many rows at a time.  A lane holds five packed sums, so that
+// enough warps and rows are in flight (with a whole row of 8 columns per lane:
+// 144 registers, 8 warps per SM, 276 us at 7.0e6 rows).
 // ---------------------------------------------------------------------------
 template <int KT, int G>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_b_stars(SysView A, const float *__restrict__ sv, const float *__restrict__ Y,
           double *__restrict__ T, int c_first)
 {
-    typedef typename Cols<KT>::V V;
-    constexpr int N = Cols<KT>::N;
+    constexpr int KP = KT > 1 ? 2 : 1;  // columns per lane
+    typedef typename Cols<KP>::V V;
+    constexpr int CL = KT / KP;  // lanes per row
+    constexpr int RS = G / CL;   // rows at a time
     constexpr int GPW = 32 / G;
     const int c0 = c_first + blockIdx.y * KT;
     const int lane = threadIdx.x & (G - 1);
     const int gw = (threadIdx.x & 31) / G;
+    const int cl = lane % CL, slot = lane / CL;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const float *Yp = Y + pidx(0, A.m, c0) + KP * cl;
     for (int64_t s0 = warp * GPW; s0 < A.S; s0 += nwarps * GPW) {
         const int64_t s = s0 + gw;
         uint32_t r0 = 0, r1 = 0;
@@ -382,48 +390,47 @@ k_b_stars(SysView A, const float *__restrict__ sv, const float *__restrict__ Y,
             r0 = A.star_ptr[s];
             r1 = A.star_ptr[s + 1];
         }
-        V ah[kNAstro][N], al[kNAstro][N];
+        V h[kNAstro], l[kNAstro];
 #pragma unroll
         for (int k = 0; k < kNAstro; k++)
-#pragma unroll
-            for (int c = 0; c < N; c++)
-                ah[k][c] = al[k][c] = V(0);
-        for (uint32_t r = r0 + lane; r < r1; r += G) {
+            h[k] = l[k] = V(0);
+#pragma unroll 2
+        for (uint32_t r = r0 + slot; r < r1; r += RS) {
             const float *v = sv + tidx<kNAstro>(0, r);
-            V yv[N];
-            load_cols<KT>(Y + pidx(r, A.m, c0), yv);
+            V yv[Cols<KP>::N];
+            load_cols<KP>(Yp + (int64_t)kPanel * r, yv);
 #pragma unroll
             for (int k = 0; k < kNAstro; k++) {
                 V a;
                 v_bcast(a, __ldcs(v + 32 * k));
-#pragma unroll
-                for (int c = 0; c < N; c++)
-                    df_acc_v(ah[k][c], al[k][c], v_mul(a, yv[c]));
+                df_acc_v(h[k], l[k], v_mul(a, yv[0]));
             }
         }
-        // the star's 5 KT sums over its G lanes: double-float reduce-scatter
-        // of the values padded to P (value v = k KT + c), 32 at a time
-        constexpr int NV = kNAstro * KT;
-        constexpr int P = NV <= 8 ? 8 : (NV <= 16 ? 16 : 32);
+        // over the RS rows in double-float; slot q writes sums q, q + RS, ...
+        float rh[kNAstro][KP], rl[kNAstro][KP];
 #pragma unroll
-        for (int v0 = 0; v0 < NV; v0 += P) {
-            float rh[P], rl[P];
+        for (int k = 0; k < kNAstro; k++)
 #pragma unroll
-            for (int v = 0; v < P; v++) {
-                const int w = v0 + v;
-                rh[v] = w < NV ? col_of<KT>(ah[w < NV ? w / KT : 0], w % KT) : 0.f;
-                rl[v] = w < NV ? col_of<KT>(al[w < NV ? w / KT : 0], w % KT) : 0.f;
+            for (int c = 0; c < KP; c++) {
+                const V hv[1] = {h[k]}, lv[1] = {l[k]};
+                rh[k][c] = col_of<KP>(hv, c);
+                rl[k][c] = col_of<KP>(lv, c);
+#pragma unroll
+                for (int off = CL; off < G; off <<= 1) {
+                    const float oh = __shfl_xor_sync(0xffffffffu, rh[k][c], off);
+                    const float ol = __shfl_xor_sync(0xffffffffu, rl[k][c], off);
+                    df_add(rh[k][c], rl[k][c], oh, ol);
+                }
             }
-            df_reduce_scatter<P, G>(rh, rl, lane);
-            constexpr int PER = P >= G ? P / G : 1;
+        if (s < A.S) {
 #pragma unroll
-            for (int k = 0; k < PER; k++) {
-                const int w = v0 + (P >= G ? lane * PER + k : lane / (G / P));
-                const bool owner = P >= G || (lane % (G / P)) == 0;
-                if (owner && w < NV && s < A.S)
-                    T[pidx((int64_t)kNAstro * s + w / KT, A.n, c0) + w % KT] =
-                        df_to_d(rh[k], rl[k]);
-            }
+            for (int k = 0; k < kNAstro; k++)
+                if (k % RS == slot) {
+                    double *t = T + pidx((int64_t)kNAstro * s + k, A.n, c0) + KP * cl;
+#pragma unroll
+                    for (int c = 0; c < KP; c++)
+                        t[c] = df_to_d(rh[k][c], rl[k][c]);
+                }
         }
     }
 }

@@ -151,7 +151,7 @@ static void release(gsr_handle_t *h)
                    h->d_bCcm, h->d_bB, h->d_bnorms, h->d_bpartial, h->d_bcounter, h->d_bs,
                    h->d_bipart, h->d_bticket, h->d_bar,
                    h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin,
-                   h->d_epos, h->d_eptr, h->d_epart,
+                   h->d_epos, h->d_estart, h->d_epart,
                    h->d_bargs};
     for (void *p : dev)
         if (p)
@@ -230,7 +230,7 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     std::vector<uint2> slice;
     code.reserve((size_t)(kNInstr * m + kNInstr * m / 8 + 4096));
     // columns of instrument f in a window of block b: at most nchunk[b I + f],
-    // each with a partial of its own
+    // each with a sum of its own
     std::vector<uint32_t> cnt((size_t)I), rank((size_t)I, 0), nchunk((size_t)(nblk * I), 0);
     std::vector<uint32_t> cur((size_t)I), idx((size_t)I), first((size_t)I), order, len;
     std::vector<uint64_t> base;
@@ -277,22 +277,19 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
             const uint32_t l = (len[order[32 * q]] + kEllStep - 1) / kEllStep * kEllStep;
             slice.push_back(make_uint2((uint32_t)groups, l));
             for (size_t t = 0; t < 32 && 32 * q + t < len.size(); t++)
-                base[order[32 * q + t]] = groups * 32 + t;
+                base[order[32 * q + t]] = groups * 32 + 2 * t;
             for (size_t t = 0; t < 32 && 32 * q + t < len.size(); t++)
                 vf[lane0 + 32 * q + t] = order[32 * q + t];  // column for now
             groups += l;
         }
-        // piece number (with kEllFirst where its partial is new) and first
-        // entry of every column, in column order
+        // piece number and first entry of every column, in column order
         uint32_t *nc = nchunk.data() + (w % nblk) * I;
         std::vector<uint32_t> cloc(len.size()), crank(len.size());
         for (size_t v = 0; v < len.size(); v++) {
             const uint32_t f = cf[v], c = (uint32_t)v - first[f];
             cloc[v] = c;
-            if (c >= nc[f]) {
+            if (c >= nc[f])
                 nc[f] = c + 1;
-                cloc[v] |= kEllFirst;
-            }
             crank[v] = rank[f];
             rank[f] += len[v];
         }
@@ -311,7 +308,8 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
         for (int64_t i = r0; i < r1; i++)
             for (int j = 0; j < kNInstr; j++) {
                 const uint32_t f = instr_of(rec[i], j);
-                code[base[cur[f]] + 32ull * idx[f]] = (uint32_t)(kNInstr * i + j);
+                code[base[cur[f]] + 64ull * (idx[f] >> 1) + (idx[f] & 1u)] =
+                    (uint32_t)(kNInstr * i + j);
                 if (++idx[f] == L) {
                     idx[f] = 0;
                     cur[f]++;
@@ -320,31 +318,30 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     }
     win[nwin] = (uint32_t)slice.size();
     std::vector<uint4>().swap(rec);
-    // partials of instrument f: block after block, those of f - 1 before them
-    std::vector<uint32_t> ptr((size_t)I + 1), seg((size_t)I + 1);
-    ptr[0] = seg[0] = 0;
-    for (int64_t f = 0; f < I; f++) {
-        uint32_t t = ptr[f];
-        for (int64_t b = 0; b < nblk; b++) {
-            const uint32_t c = nchunk[b * I + f];
-            nchunk[b * I + f] = t;
-            t += c;
-        }
-        ptr[f + 1] = t;
-        seg[f + 1] = seg[f] + rank[f];
+    // sums of a block: instrument after instrument
+    std::vector<uint32_t> start((size_t)(nblk * (I + 1))), seg((size_t)I + 1);
+    int64_t nacc = 0;
+    for (int64_t b = 0; b < nblk; b++) {
+        uint32_t *s0 = start.data() + b * (I + 1);
+        s0[0] = 0;
+        for (int64_t f = 0; f < I; f++)
+            s0[f + 1] = s0[f] + nchunk[b * I + f];
+        nacc = std::max<int64_t>(nacc, s0[I]);
     }
+    seg[0] = 0;
+    for (int64_t f = 0; f < I; f++)
+        seg[f + 1] = seg[f] + rank[f];
     cseg.insert(cseg.end(), rank.begin(), rank.end());
     const int64_t nq = (nwin + per - 1) / per;
     for (int64_t q = 0; q <= nq; q++)
         for (int64_t f = 0; f < I; f++)
             cseg[q * I + f] += seg[f];
-    const int64_t npart = ptr[I], nslots = (int64_t)vf.size();
+    const int64_t nslots = (int64_t)vf.size();
     std::vector<uint32_t> pos((size_t)nslots, kEllNone), sorted((size_t)nslots, kEllNone);
     for (int64_t w = 0; w < nwin; w++)
         for (int64_t t = 32 * (int64_t)win[w]; t < 32 * (int64_t)win[w + 1]; t++)
             if (vf[t] != kEllNone) {
-                pos[t] = (nchunk[(w % nblk) * I + vf[t]] + (vloc[t] & ~kEllFirst)) |
-                         (vloc[t] & kEllFirst);
+                pos[t] = start[(w % nblk) * (I + 1) + vf[t]] + vloc[t];
                 sorted[t] = seg[vf[t]] + vrank[t];
             }
     const int64_t total = (int64_t)code.size();
@@ -353,8 +350,8 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     TRY(dalloc(h, &h->d_eslice, (int64_t)slice.size()));
     TRY(dalloc(h, &h->d_ewin, nwin + 1));
     TRY(dalloc(h, &h->d_epos, nslots));
-    TRY(dalloc(h, &h->d_eptr, I + 1));
-    TRY(dalloc(h, &h->d_epart, npart));
+    TRY(dalloc(h, &h->d_estart, nblk * (I + 1)));
+    TRY(dalloc(h, &h->d_epart, nblk * I));
     TRY(dalloc(h, &h->d_iseg, I + 1));
     TRY(dalloc(h, &h->d_irow, kNInstr * m));
     TRY(dalloc(h, &h->d_ival, kNInstr * m));
@@ -362,10 +359,10 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     CK(cudaMemcpy(h->d_eslice, slice.data(), slice.size() * sizeof(uint2), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_ewin, win.data(), (nwin + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_epos, pos.data(), nslots * sizeof(uint32_t), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h->d_eptr, ptr.data(), (I + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h->d_estart, start.data(), start.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(h->d_iseg, seg.data(), (I + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
-    h->ell = Ell{h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin, h->d_epos, h->d_eptr, h->d_epart,
-                 nwin, W, nblk};
+    h->ell = Ell{h->d_eidx, h->d_eval32, h->d_eslice, h->d_ewin, h->d_epos, h->d_estart, h->d_epart,
+                 (int)nacc, nwin, W, nblk};
     uint32_t *d_tmp = nullptr;
     const size_t bytes = (size_t)std::max(total, nslots) * sizeof(uint32_t);
     if (cudaMalloc(&d_tmp, bytes) != cudaSuccess) {
@@ -386,8 +383,12 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     cudaFree(d_tmp);
     if (e != cudaSuccess)
         return cuda_fail(e, "instrument windows");
-    h->ell_on = true;
-    return finish_instr(h, cseg, nq, nq);
+    // (nacc is at most I + 6 W / L, below kEllAccMax, unless the instruments are
+    // used very unevenly: the sorted copy's units serve then)
+    h->ell_on = nacc <= kEllAccMax;
+    if (!h->ell_on)
+        h->ks32 = (int)((kNInstr * m / I + 4095) / 4096);
+    return finish_instr(h, cseg, nq, std::max<int64_t>(nq, h->ks32));
 }
 
 // Instrument-sorted copy of the instrumental nonzeros: a stable counting
@@ -484,9 +485,11 @@ static int build_units(gsr_handle_t *h)
     const SysView &A = h->sys;
     std::vector<uint32_t> seg((size_t)A.nseg + 1), useg((size_t)A.nseg + 1);
     CK(cudaMemcpy(seg.data(), h->d_seg, (A.nseg + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost));
-    // tiles per unit: about four units for each of the 16 warps of every SM,
+    // tiles per unit: about two units for each of the 16 warps of every SM (one
+    // warp with one unit of 8 tiles took 35 us at 700,000 rows, two with 4 took
+    // 32; smaller ones only add partial sums),
     // at most kUnitTiles (the unit's reduction is then a small share)
-    const uint64_t want = (uint64_t)((A.m / 32) / ((int64_t)h->nsm * 64));
+    const uint64_t want = (uint64_t)((A.m / 32) / ((int64_t)h->nsm * 32));
     const uint64_t ut = want < 1 ? 1 : (want > kUnitTiles ? kUnitTiles : want);
     std::vector<uint4> unit;
     unit.reserve((size_t)(A.nseg + A.m / 32 / ut + 1));
@@ -535,7 +538,7 @@ static int create_mixed(gsr_handle_t *h, cudaStream_t st)
     h->att32.tile = h->d_atile;
     h->att32.sv = h->d_sv32;
     CK(build_att32(h, st));
-    if (!h->ell_on) {
+    if (!h->d_ival32) {
         TRY(dalloc(h, &h->d_ival32, kNInstr * m));
         CK(launch_to_f32(h, h->d_ival, h->d_ival32, kNInstr * m, st));
     }

@@ -55,7 +55,7 @@ __global__ void k_ell_sorted(SysView A, Ell E, const uint32_t *__restrict__ star
             if (d == kEllNone)
                 continue;
             for (uint32_t i = 0; i < s.y; i++, d++) {
-                const int64_t p = ((int64_t)s.x + i) * 32 + lane;
+                const int64_t p = (int64_t)s.x * 32 + (i >> 1) * 64 + 2 * lane + (i & 1);
                 const uint32_t c = E.idx[p], r = c & kEllRowMask;
                 if (r == kEllPad)
                     break;

@@ -5,11 +5,12 @@
 // The rows are cut into windows of W <= 8160 rows.  Inside a window the
 // nonzeros of one instrument, in row order, form one or more columns of at
 // most kEllLen entries, one lane each; 32 columns of like length are one slice
-// (sliced ELL: entry i of the 32 lanes is contiguous), so a warp reads values
+// (sliced ELL: entries 2 i and 2 i + 1 of the 32 lanes are contiguous), so a warp reads values
 // and row numbers in whole segments and needs no reduction across lanes.  A
-// block stages the window of y in shared memory and gathers it from there;
-// every column keeps one partial sum per block, so an instrument has about as
-// many partials as there are SMs.  Every sum has a fixed order.
+// block stages the window of y in shared memory and gathers it from there; the
+// columns' sums of all its windows are added in shared memory too (added in
+// global memory they cost 50 of 128 us) and leave it as one partial per
+// instrument and block.  Every sum has a fixed order.
 //
 // Why: gathered from L2 (one instrument's rows spread over all of y) the 6 m
 // gathers alone take 0.145 ms at m = 7.0e6 (random 32-byte sectors arrive at
@@ -23,9 +24,10 @@
 //
 // kEllWarps warps of a block run the pass (the others, and these once they
 // have finished, take the star units).  The next window of y is copied by the
-// bulk-copy engine while the current one is summed, and every warp loads its
-// next eight entries (of this slice or the next) before it sums the current
-// eight.
+// bulk-copy engine while the current one is summed, and every warp has its next
+// sixteen entries (of this slice or the next) on their way while it sums
+// eight: with eight on their way the pass took 128 us of HBM latency for its
+// 300 MB.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -49,71 +51,66 @@ __device__ __forceinline__ void ell_sync()
     asm volatile("bar.sync 1, %0;" ::"n"(kEllThreads) : "memory");
 }
 
-// kEllStep entries of a column: values, window rows
-template <typename T>
+// kEllStep entries of each lane's column, and with the last ones of a slice
+// where their sum goes (pos; kEllMore: the column goes on)
 struct EllRun {
-    T v[kEllStep];
-    uint32_t r[kEllStep];
+    float2 v[kEllStep / 2];
+    uint32_t r[kEllStep / 2];  // two window rows
+    uint32_t pos;
 };
+constexpr uint32_t kEllMore = 0xfffffffeu;
 
-template <typename T>
-__device__ __forceinline__ void ell_load(EllRun<T> &a, const T *__restrict__ val,
-                                         const uint16_t *__restrict__ idx, int64_t p)
-{
-#pragma unroll
-    for (int k = 0; k < kEllStep; k++) {
-        a.v[k] = __ldcs(val + p + 32 * k);
-        a.r[k] = (uint32_t)__ldcs(idx + p + 32 * k) & kEllRowMask;
+// The slices sl, sl + kEllWarps, ... of one window as a sequence of runs, their
+// descriptions one slice ahead
+struct EllCursor {
+    const Ell &E;
+    uint32_t sl, sl1, i = 0;
+    uint2 s, sn;
+    uint32_t pos, pn;
+    int lane;
+
+    __device__ __forceinline__ EllCursor(const Ell &E_, uint32_t sl_, uint32_t sl1_)
+        : E(E_), sl(sl_), sl1(sl1_), lane(threadIdx.x & 31)
+    {
+        if (sl < sl1) {
+            s = __ldg(E.slice + sl);
+            pos = __ldcs(E.pos + (int64_t)sl * 32 + lane);
+            describe();
+        }
     }
-}
-
-// The slices of one window, dealt to the kEllWarps warps; body(a) sums
-// kEllStep entries, done() ends a column and returns its sum, which is added to
-// the column's partial (stored where the block has not written it yet).  A
-// slice's description and partials are loaded a slice ahead.
-template <typename T, typename Body, typename Done>
-__device__ __forceinline__ void ell_slices(const Ell &E, const T *__restrict__ val, uint32_t sl,
-                                           uint32_t sl1, Body body, Done done)
-{
-    const int lane = threadIdx.x & 31;
-    sl += threadIdx.x >> 5;
-    if (sl >= sl1)
-        return;
-    uint2 s = __ldg(E.slice + sl);
-    uint32_t pos = __ldcs(E.pos + (int64_t)sl * 32 + lane);
-    EllRun<T> a;
-    ell_load(a, val, E.idx, (int64_t)s.x * 32 + lane);
-    for (;;) {
-        const bool more = sl + kEllWarps < sl1;
-        uint2 sn = s;
-        uint32_t pn = kEllNone;
-        if (more) {
+    __device__ __forceinline__ void describe()
+    {
+        sn = s;
+        pn = pos;
+        if (sl + kEllWarps < sl1) {
             sn = __ldg(E.slice + sl + kEllWarps);
             pn = __ldcs(E.pos + (int64_t)(sl + kEllWarps) * 32 + lane);
         }
-        double *part = E.part + (pos & ~kEllFirst);
-        const double old = (pos & kEllFirst) ? 0.0 : *part;  // none: flagged too
-        const int64_t p0 = (int64_t)s.x * 32 + lane;
-        for (uint32_t i = kEllStep; i < s.y; i += kEllStep) {
-            EllRun<T> b;
-            ell_load(b, val, E.idx, p0 + 32 * (int64_t)i);
-            body(a);
-            a = b;
-        }
-        EllRun<T> b;
-        ell_load(b, val, E.idx, (int64_t)sn.x * 32 + lane);
-        body(a);
-        const double t = done();
-        if (pos != kEllNone)
-            *part = (pos & kEllFirst) ? t : old + t;
-        if (!more)
-            return;
-        a = b;
-        s = sn;
-        pos = pn;
-        sl += kEllWarps;
     }
-}
+    __device__ __forceinline__ bool fetch(EllRun &a)
+    {
+        if (sl >= sl1)
+            return false;
+        // the lane's first pair; its pairs are 32 pairs apart
+        const int64_t p = ((int64_t)s.x + i) * 32 + 2 * lane;
+#pragma unroll
+        for (int k = 0; k < kEllStep / 2; k++) {
+            a.v[k] = __ldcs(reinterpret_cast<const float2 *>(E.val32 + p + 64 * k));
+            a.r[k] = __ldcs(reinterpret_cast<const uint32_t *>(E.idx + p + 64 * k));
+        }
+        i += kEllStep;
+        a.pos = kEllMore;
+        if (i >= s.y) {
+            a.pos = pos;
+            sl += kEllWarps;
+            s = sn;
+            pos = pn;
+            i = 0;
+            describe();
+        }
+        return true;
+    }
+};
 
 struct EllShared {
     uint64_t bar[2];
@@ -197,8 +194,6 @@ __device__ __forceinline__ void ell_windows(const Ell &E, const T *y, int64_t m,
 {
     EllWindows<T> win;
     int64_t w = blockIdx.x;
-    if (w >= E.nblk)
-        return;
     win.init(buf, sh, y, m, E.W);
     int b = 0;
     win.fetch(w, 0);
@@ -221,41 +216,64 @@ __device__ __forceinline__ void ell_windows(const Ell &E, const T *y, int64_t m,
 // binary32 values and y: binary32 products, double-float sums (two entries per
 // packed operation), FP64 partials
 __device__ __forceinline__ void ell32_part(const Ell &E, const float *y, int64_t m,
-                                           unsigned char *smem, EllShared *sh, int *kerr)
+                                           unsigned char *smem, EllShared *sh, int *kerr, int64_t I)
 {
+    double *acc = reinterpret_cast<double *>(smem + kEllSmem32);  // [nacc]
+    if (blockIdx.x >= E.nblk)
+        return;
+    for (int i = threadIdx.x; i < E.nacc; i += kEllThreads)
+        acc[i] = 0.0;
     ell_windows<float>(E, y, m, reinterpret_cast<float *>(smem), sh, kerr,
                        [&](int64_t w, const float *yw) {
+        EllCursor cur(E, __ldg(E.win + w) + (threadIdx.x >> 5), __ldg(E.win + w + 1));
         f32x2 h[2] = {0ull, 0ull}, l[2] = {0ull, 0ull};
-        ell_slices<float>(E, E.val32, __ldg(E.win + w), __ldg(E.win + w + 1),
-                          [&](const EllRun<float> &a) {
+        EllRun a, b, c;
+        bool ok = cur.fetch(a), okb = cur.fetch(b);
+        while (ok) {
+            const bool okc = cur.fetch(c);
 #pragma unroll
-            for (int k = 0; k < kEllStep; k += 2)
-                df_acc_v(h[(k / 2) & 1], l[(k / 2) & 1],
-                         v_mul(pack2(a.v[k], a.v[k + 1]), pack2(yw[a.r[k]], yw[a.r[k + 1]])));
-        }, [&] {
-            float th[4], tl[4];
+            for (int k = 0; k < kEllStep / 2; k++)
+                df_acc_v(h[k & 1], l[k & 1],
+                         v_mul(pack2(a.v[k].x, a.v[k].y),
+                               pack2(yw[a.r[k] & kEllRowMask], yw[(a.r[k] >> 16) & kEllRowMask])));
+            if (a.pos != kEllMore) {
+                float th[4], tl[4];
 #pragma unroll
-            for (int k = 0; k < 2; k++) {
-                unpack2(h[k], th[2 * k], th[2 * k + 1]);
-                unpack2(l[k], tl[2 * k], tl[2 * k + 1]);
-                h[k] = l[k] = 0ull;
+                for (int k = 0; k < 2; k++) {
+                    unpack2(h[k], th[2 * k], th[2 * k + 1]);
+                    unpack2(l[k], tl[2 * k], tl[2 * k + 1]);
+                    h[k] = l[k] = 0ull;
+                }
+                df_add(th[0], tl[0], th[1], tl[1]);
+                df_add(th[2], tl[2], th[3], tl[3]);
+                df_add(th[0], tl[0], th[2], tl[2]);
+                const double t = df_to_d(th[0], tl[0]);
+                if (a.pos != kEllNone)  // one column of the window has this sum
+                    acc[a.pos] += t;
             }
-            df_add(th[0], tl[0], th[1], tl[1]);
-            df_add(th[2], tl[2], th[3], tl[3]);
-            df_add(th[0], tl[0], th[2], tl[2]);
-            return df_to_d(th[0], tl[0]);
-        });
+            a = b;
+            b = c;
+            ok = okb;
+            okb = okc;
+        }
     });
+    // the pieces of an instrument in order
+    const uint32_t *start = E.start + (int64_t)blockIdx.x * (I + 1);
+    for (int64_t f = threadIdx.x; f < I; f += kEllThreads) {
+        double t = 0.0;
+        for (uint32_t i = __ldg(start + f); i < __ldg(start + f + 1); i++)
+            t += acc[i];
+        E.part[(int64_t)blockIdx.x * I + f] = t;
+    }
 }
 
 // total of instrument f, by one warp (every lane has it), in a fixed order
-__device__ __forceinline__ double ell_total(const Ell &E, int64_t f)
+__device__ __forceinline__ double ell_total(const Ell &E, int64_t f, int64_t I)
 {
-    const uint32_t a = __ldg(E.ptr + f), b = __ldg(E.ptr + f + 1);
     double t = 0.0;
-#pragma unroll 4
-    for (uint32_t p = a + (threadIdx.x & 31); p < b; p += 32)
-        t += __ldcg(E.part + p);
+#pragma unroll 5
+    for (int64_t b = threadIdx.x & 31; b < E.nblk; b += 32)
+        t += __ldcg(E.part + b * I + f);
     __syncwarp();
     return warp_sum(t);
 }

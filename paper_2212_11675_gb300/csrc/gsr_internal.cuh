@@ -89,25 +89,27 @@ __device__ __forceinline__ uint32_t star_of_row(const SysView &A, int64_t t, int
 }
 
 // Instrumental nonzeros in row windows (gsr_ell.cu): slices of 32 columns, the
-// entries of slice s at (slice[s].x + i) * 32 + lane for i < slice[s].y
+// entry i < slice[s].y of its lane at slice[s].x * 32 + (i / 2) * 64 + 2 lane
+// + i % 2
 // (a multiple of kEllStep).
 constexpr uint32_t kEllRowBits = 13;
 constexpr uint32_t kEllRowMask = (1u << kEllRowBits) - 1;
 constexpr uint32_t kEllPad = kEllRowMask;     // window row of a padding entry (y = 0)
 constexpr uint32_t kEllNone = 0xffffffffu;    // no column in this lane
-constexpr uint32_t kEllFirst = 0x80000000u;   // flag of a partial: the block's first column of it
 constexpr int kEllLen = 64;                   // entries per column at most
 constexpr int kEllStep = 8;                   // entries loaded at a time
 constexpr int64_t kEllRowsMax = 8160;         // rows per window at most
 constexpr int64_t kEllInstrMax = 6144;
+constexpr int kEllAccMax = 16384;              // sums of a block in shared memory (128 KB)
 struct Ell {
     const uint16_t *idx;  // row of the window | slot << kEllRowBits
     const float *val32;
     const uint2 *slice;
     const uint32_t *win;  // [nwin+1] slices of each window
-    const uint32_t *pos;  // [32 slices] partial of each column, with kEllFirst
-    const uint32_t *ptr;  // [I+1] partials of instrument f: ptr[f] .. ptr[f+1]-1
-    double *part;
+    const uint32_t *pos;  // [32 slices] sum of the block that each column adds to
+    const uint32_t *start;  // [nblk][I+1] sums of instrument f: start[f] .. start[f+1]-1
+    double *part;         // [nblk][I]
+    int nacc;             // sums of a block at most
     int64_t nwin, W;      // windows, rows per window
     int64_t nblk;         // block b takes windows b, b + nblk, ...
 };
@@ -309,7 +311,7 @@ struct gsr_handle_t {
     double *d_epart = nullptr;
     float *d_eval32 = nullptr;
     uint2 *d_eslice = nullptr;
-    uint32_t *d_ewin = nullptr, *d_epos = nullptr, *d_eptr = nullptr;
+    uint32_t *d_ewin = nullptr, *d_epos = nullptr, *d_estart = nullptr;
     double *d_gpart = nullptr;          // per-block partials of the global column (star pass)
     int a2_fused = 1;                   // aprod 2 in one launch (sorted path), else separate passes
     unsigned long long *d_a2ctr = nullptr;  // work counter of the single-launch aprod 2

@@ -436,8 +436,8 @@ k_f32_rest(SysView A, Att32 U, const float *__restrict__ y32, double *__restrict
 
 // The rest of the inner aprod 2 with the instruments in row windows: 16 warps
 // of a block sum its windows, the others take star units, and the first 16
-// join them (as k_aprod2_win)
-constexpr int kRestThreads = 1024;
+// join them
+constexpr int kRestThreads = 768;
 
 template <int G, int MODE>
 __global__ void __launch_bounds__(kRestThreads, 1)
@@ -449,7 +449,7 @@ k_f32_rest_win(SysView A, Att32 U, Ell E, const float *__restrict__ y32, double 
     const uint32_t nfix = gridDim.x * (kRestThreads / 32 - kEllWarps);
     uint32_t u = 0xffffffffu;
     if (threadIdx.x < kEllThreads)
-        ell32_part(E, y32, A.m, smem, &sh, kerr);
+        ell32_part(E, y32, A.m, smem, &sh, kerr, A.I);
     else
         u = blockIdx.x + gridDim.x * ((threadIdx.x - kEllThreads) >> 5);
     for (;;) {
@@ -508,7 +508,7 @@ k_f32_combine(SysView A, const uint32_t *__restrict__ useg, const double *__rest
         *ctr = 0ull;
     if (npart == 0)  // the instruments' partials of the row windows
         for (int64_t f = gtid32() >> 5; f < A.I; f += gstride32() >> 5) {
-            const double t = ell_total(E, f);
+            const double t = ell_total(E, f, A.I);
             if ((threadIdx.x & 31) == 0)
                 out[A.ins0 + f] += t;
         }
@@ -614,7 +614,7 @@ k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restric
     const bool win = INL && P.isplit == 0;  // instruments in row windows
     if (win) {
         for (int64_t f = gtid32() >> 5; f < A.I; f += gstride32() >> 5) {
-            const double t = ell_total(P.ell, f);
+            const double t = ell_total(P.ell, f, A.I);
             if ((threadIdx.x & 31) == 0)
                 update(A.ins0 + f, [&] { return t; });
         }
@@ -746,12 +746,21 @@ static cudaError_t f32_main(const gsr_handle_t *h, double *y, double *glb, cudaS
 template <int MODE, int G>
 static cudaError_t rest_win(const gsr_handle_t *h, double *out, cudaStream_t st)
 {
+    // the most that any handle of the process may ask for
     const cudaError_t e = cudaFuncSetAttribute(
-        k_f32_rest_win<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEllSmem32);
+        k_f32_rest_win<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)(kEllSmem32 + kEllAccMax * sizeof(double)));
     if (e != cudaSuccess)
         return e;
-    k_f32_rest_win<G, MODE><<<h->nsm, kRestThreads, kEllSmem32, st>>>(
-        h->sys, h->att32, h->ell, h->d_q32, out, a2_queue(h, G, 0, 0), h->d_kerr);
+    // at most two star groups a unit: the 8 warps that start with stars end
+    // nearer to the 16 of the windows (113 -> 106 us at m = 7.0e6)
+    A2Queue q = a2_queue(h, G, 0, 0);
+    if (q.star_k > 2) {
+        q.star_k = 2;
+        q.nstar_units = (q.nstar_groups + 1) / 2;
+    }
+    k_f32_rest_win<G, MODE><<<h->nsm, kRestThreads, kEllSmem32 + h->ell.nacc * sizeof(double), st>>>(
+        h->sys, h->att32, h->ell, h->d_q32, out, q, h->d_kerr);
     return cudaGetLastError();
 }
 

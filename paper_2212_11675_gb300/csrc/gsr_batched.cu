@@ -31,28 +31,49 @@
 
 namespace gsr {
 
-// The stream and events that fork a pass of aprod 2 while the inner loop is
-// captured; they are released with the object, the graph keeps the branches.
-struct BatchSide {
+// A stream and the events that fork it from another one and join it again
+// while the inner loop is captured; released with the object, the graph keeps
+// the branch.
+struct Branch {
     cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
     cudaError_t make()
     {
-        cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-        if (e == cudaSuccess)
-            e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
-        if (e == cudaSuccess)
-            e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        for (int i = 0; i < 2 && e == cudaSuccess; i++)
+            e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
         return e;
     }
-    ~BatchSide()
+    cudaError_t fork(cudaStream_t from)
     {
-        if (fork)
-            cudaEventDestroy(fork);
-        if (join)
-            cudaEventDestroy(join);
+        const cudaError_t e = cudaEventRecord(ev[0], from);
+        return e == cudaSuccess ? cudaStreamWaitEvent(s, ev[0], 0) : e;
+    }
+    cudaError_t join(cudaStream_t to)
+    {
+        const cudaError_t e = cudaEventRecord(ev[1], s);
+        return e == cudaSuccess ? cudaStreamWaitEvent(to, ev[1], 0) : e;
+    }
+    ~Branch()
+    {
+        for (cudaEvent_t e : ev)
+            if (e)
+                cudaEventDestroy(e);
         if (s)
             cudaStreamDestroy(s);
+    }
+};
+
+// The branches of an iteration: the second run of tiles beside the first, in
+// each run the instrument pass beside the star pass
+struct BatchSide {
+    Branch run, instr[2];
+    cudaError_t make()
+    {
+        cudaError_t e = run.make();
+        for (int i = 0; i < 2 && e == cudaSuccess; i++)
+            e = instr[i].make();
+        return e;
     }
 };
 
@@ -869,22 +890,16 @@ static void b_stars(const gsr_handle_t *h, const float *Y, double *T, int c0, in
 }
 
 // The star and instrument passes write different sums and run side by side
-// when a side stream is given (graph capture): one bound by its gathers
-// shares the SMs with one bound by the FP32 pipe.
+// when a branch is given (graph capture): one bound by its gathers shares the
+// SMs with one bound by the FP32 pipe.
 template <int KT>
 static cudaError_t b_rest(const gsr_handle_t *h, const float *Y, double *T, int c0, int ny,
-                          cudaStream_t st, const BatchSide *side)
+                          cudaStream_t st, Branch *br)
 {
-    cudaStream_t si = st;
-    cudaError_t e = cudaSuccess;
-    if (side) {
-        si = side->s;
-        e = cudaEventRecord(side->fork, st);
-        if (e == cudaSuccess)
-            e = cudaStreamWaitEvent(si, side->fork, 0);
-        if (e != cudaSuccess)
-            return e;
-    }
+    cudaError_t e = br ? br->fork(st) : cudaSuccess;
+    if (e != cudaSuccess)
+        return e;
+    const cudaStream_t si = br ? br->s : st;
     const int occ_i = b_occ(k_b_instr<KT>);
     const int npi = batched_instr_pieces(h);
     k_b_instr<KT><<<dim3(b_blocks(h, 2 * occ_i, h->sys.I * npi), ny), kThreads, 0, si>>>(
@@ -895,12 +910,7 @@ static cudaError_t b_rest(const gsr_handle_t *h, const float *Y, double *T, int 
     default: b_stars<KT, 16>(h, Y, T, c0, ny, st); break;
     }
     e = cudaGetLastError();
-    if (side && e == cudaSuccess) {
-        e = cudaEventRecord(side->join, si);
-        if (e == cudaSuccess)
-            e = cudaStreamWaitEvent(st, side->join, 0);
-    }
-    return e;
+    return br && e == cudaSuccess ? br->join(st) : e;
 }
 
 template <int KT>
@@ -939,11 +949,11 @@ static cudaError_t b_products_tiles(const gsr_handle_t *h, const float *X, float
 template <int KT>
 static cudaError_t b_iteration_tiles(const gsr_handle_t *h, int c0, int ny, cudaStream_t s, int k,
                                      cudaGraphConditionalHandle loop, int in_graph, int last,
-                                     const BatchSide *side)
+                                     Branch *br)
 {
     cudaError_t e = b_main<KT, kBA1 | kBA2>(h, h->d_bX32, h->d_bQ32, h->d_bT, c0, ny, s);
     if (e == cudaSuccess)
-        e = b_rest<KT>(h, h->d_bQ32, h->d_bT, c0, ny, s, side);
+        e = b_rest<KT>(h, h->d_bQ32, h->d_bT, c0, ny, s, br);
     if (e != cudaSuccess)
         return e;
     const dim3 g(vec_blocks<KT>(h), ny);
@@ -996,18 +1006,34 @@ static cudaError_t b_prologue(const gsr_handle_t *h, int k, cudaStream_t s,
     return cudaGetLastError();
 }
 
+// With branches the runs are independent chains and the loop flag follows
+// their join; otherwise the last run's vector pass sets it.
 static cudaError_t b_iteration(const gsr_handle_t *h, int k, cudaStream_t s,
-                               cudaGraphConditionalHandle loop, int in_graph,
-                               const BatchSide *side)
+                               cudaGraphConditionalHandle loop, int in_graph, BatchSide *side)
 {
-    return for_runs(h, k, [&](int kt, int c0, int ny, bool last) {
+    const bool two = side && k > h->b_kt && k % h->b_kt != 0;
+    cudaError_t e = two ? side->run.fork(s) : cudaSuccess;
+    if (e != cudaSuccess)
+        return e;
+    e = for_runs(h, k, [&](int kt, int c0, int ny, bool last) {
+        const int i = c0 > 0;
+        const cudaStream_t st = two && i ? side->run.s : s;
+        Branch *br = side ? &side->instr[i] : nullptr;
+        const int flag = last && !two;
         switch (kt) {
-        case 1: return b_iteration_tiles<1>(h, c0, ny, s, k, loop, in_graph, last, side);
-        case 2: return b_iteration_tiles<2>(h, c0, ny, s, k, loop, in_graph, last, side);
-        case 4: return b_iteration_tiles<4>(h, c0, ny, s, k, loop, in_graph, last, side);
-        default: return b_iteration_tiles<8>(h, c0, ny, s, k, loop, in_graph, last, side);
+        case 1: return b_iteration_tiles<1>(h, c0, ny, st, k, loop, in_graph, flag, br);
+        case 2: return b_iteration_tiles<2>(h, c0, ny, st, k, loop, in_graph, flag, br);
+        case 4: return b_iteration_tiles<4>(h, c0, ny, st, k, loop, in_graph, flag, br);
+        default: return b_iteration_tiles<8>(h, c0, ny, st, k, loop, in_graph, flag, br);
         }
     });
+    if (e != cudaSuccess || !two)
+        return e;
+    e = side->run.join(s);
+    if (e != cudaSuccess)
+        return e;
+    k_b_flag<<<1, 32, 0, s>>>(h->d_bs, k, loop, in_graph);
+    return cudaGetLastError();
 }
 
 #define B_TRY(x)                        \

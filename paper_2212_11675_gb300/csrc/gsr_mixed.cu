@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include "gsr_internal.cuh"
+#include "gsr_lsqr.cuh"
 #include "gsr_reduce.cuh"
 #include "gsr_df.cuh"
 #include "gsr_att32.cuh"
@@ -589,11 +590,20 @@ k_cg_init(const double *__restrict__ p, const double *__restrict__ c, double *__
     }
 }
 
+// Where the column sums of aprod 2 are when k_cg_vec1 reads them
+enum CgSums {
+    kSumsDone = 0,   // all in t
+    kSumsUnits = 1,  // binary32 form: units of Att32 and the instruments' partials
+    kSumsParts = 2   // FP64 single-launch aprod 2: its partial sums
+};
+
 // s -= alpha p o t, z += alpha d, gamma' = |s|^2; the last block forms beta
-// and applies the inner stopping rule.  INL: t holds the astrometric part and
-// the global column of A32^T q; the other columns come from the sums of the
-// units and instruments (the last block resets the work counter).
-template <bool INL>
+// and applies the inner stopping rule.  SUMS: t holds the astrometric part
+// (and the global column but for kSumsParts), the other columns are added up
+// here (no combine launch); with kSumsParts the global column comes from one
+// fixed slice of the star units' partials per block, added by the last block.
+// The last block resets the work counter.
+template <int SUMS>
 __global__ void __launch_bounds__(kThreads)
 k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restrict__ t,
           double *__restrict__ s, const double *__restrict__ d, double *__restrict__ z, CgState *cg,
@@ -602,7 +612,7 @@ k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restric
 {
     const int64_t n = A.n;
     const double alpha = cg->alpha;
-    double acc[1] = {0.0};
+    double acc[SUMS == kSumsParts ? 2 : 1] = {};
     // column j with t_j = tf(): the loads of the vectors come first
     auto update = [&](int64_t j, auto tf) {
         const double dj = d[j], zo = z[j], pj = p[j], so = s[j];
@@ -611,26 +621,52 @@ k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restric
         s[j] = sj;
         acc[0] = fma(sj, sj, acc[0]);
     };
-    const bool win = INL && P.isplit == 0;  // instruments in row windows
-    if (win) {
+    // instruments in row windows, or with many window totals: a warp each
+    const bool win = SUMS == kSumsUnits && P.isplit == 0;
+    const bool warp_instr = win || (SUMS == kSumsParts && P.isplit > kThreadParts);
+    if (warp_instr) {
         for (int64_t f = gtid32() >> 5; f < A.I; f += gstride32() >> 5) {
-            const double t = ell_total(P.ell, f, A.I);
+            double v = 0.0;
+            if (win) {
+                v = ell_total(P.ell, f, A.I);
+            } else {
+                for (int qq = threadIdx.x & 31; qq < P.isplit; qq += 32)
+                    v += P.ipart[(int64_t)qq * A.I + f];
+                v = warp_sum(v);
+            }
             if ((threadIdx.x & 31) == 0)
-                update(A.ins0 + f, [&] { return t; });
+                update(A.ins0 + f, [&] { return v; });
         }
     }
     for (int64_t j = gtid32(); j < n; j += gstride32()) {
-        if (win && j >= A.ins0 && j < A.glb0)
+        if (warp_instr && j >= A.ins0 && j < A.glb0)
             continue;
+        if (SUMS == kSumsParts && j == A.glb0)
+            continue;  // the last block
         update(j, [&] {
-            return (!INL || j < A.att0 || j >= A.glb0)
-                       ? t[j] : q_from_units(A, useg, P.S, P.ipart, P.isplit, j);
+            if (SUMS == kSumsDone || j < A.att0 || j >= A.glb0)
+                return t[j];
+            return SUMS == kSumsUnits ? q_from_units(A, useg, P.S, P.ipart, P.isplit, j)
+                                      : q_from_parts(A, P, j);
         });
     }
-    if (grid_reduce<1>(acc, partial, counter) && threadIdx.x == 0) {
+    if constexpr (SUMS == kSumsParts) {
+        const uint32_t per = ((uint32_t)P.ngpart + gridDim.x - 1) / gridDim.x;
+        const uint32_t b0 = blockIdx.x * per, b1 = min((uint32_t)P.ngpart, b0 + per);
+        for (uint32_t b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+            acc[1] += P.gpart[b];
+    }
+    if (grid_reduce(acc, partial, counter) && threadIdx.x == 0) {
         CgState g = *cg;
-        const double gnew = acc[0];
-        if (INL)
+        double gnew = acc[0];
+        if constexpr (SUMS == kSumsParts) {
+            const int64_t j = A.glb0;
+            const double sj = fma(-alpha, p[j] * acc[1], s[j]);
+            z[j] = fma(alpha, d[j], z[j]);
+            s[j] = sj;
+            gnew = fma(sj, sj, gnew);
+        }
+        if (SUMS != kSumsDone)
             *P.ctr = 0ull;
         g.beta = gnew / g.gamma;
         g.gamma = gnew;
@@ -830,11 +866,11 @@ static cudaError_t cg_iteration(const gsr_handle_t *h, cudaStream_t s, cudaGraph
         e = f32_rest<kA2Overwrite>(h, h->d_t, &P, s);
     if (e != cudaSuccess)
         return e;
-    k_cg_vec1<true><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d, h->d_zc, h->d_cg,
-                                                     h->d_cgargs,
-                                                     h->d_partial + kRedV * kPartialsPerKind,
-                                                     h->d_counter + kRedV, loop, in_graph,
-                                                     h->d_useg, P);
+    k_cg_vec1<kSumsUnits><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
+                                                           h->d_zc, h->d_cg, h->d_cgargs,
+                                                           h->d_partial + kRedV * kPartialsPerKind,
+                                                           h->d_counter + kRedV, loop, in_graph,
+                                                           h->d_useg, P);
     k_cg_vec2<float><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_x32, h->d_t, A.n, A.n,
                                                 h->d_cg, h->d_x8, A.att0);
     return cudaGetLastError();
@@ -1050,15 +1086,24 @@ static cudaError_t cg64_iteration(const gsr_handle_t *h, cudaStream_t s,
 {
     const SysView &A = h->sys;
     cudaError_t e = launch_aprod1_cg(h, h->d_xp64, h->d_q64, s);
-    if (e == cudaSuccess)
-        e = launch_aprod2(h, h->d_q64, h->d_t, kA2Overwrite, s);
     if (e != cudaSuccess)
         return e;
-    k_cg_vec1<false><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d, h->d_zc,
-                                                      h->d_cg, h->d_cgargs,
-                                                      h->d_partial + kRedV * kPartialsPerKind,
-                                                      h->d_counter + kRedV, loop, in_graph,
-                                                      nullptr, A2Parts{});
+    double *part = h->d_partial + kRedV * kPartialsPerKind;
+    unsigned *cnt = h->d_counter + kRedV;
+    A2Parts P = {};
+    if (aprod2_partials(h, h->d_q64, h->d_t, &P.S, &P.ipart, &P.isplit, &P.gpart, &P.ngpart, &P.ctr,
+                        s)) {
+        k_cg_vec1<kSumsParts><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
+                                                               h->d_zc, h->d_cg, h->d_cgargs, part,
+                                                               cnt, loop, in_graph, nullptr, P);
+    } else {
+        e = launch_aprod2(h, h->d_q64, h->d_t, kA2Overwrite, s);
+        if (e != cudaSuccess)
+            return e;
+        k_cg_vec1<kSumsDone><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
+                                                              h->d_zc, h->d_cg, h->d_cgargs, part,
+                                                              cnt, loop, in_graph, nullptr, P);
+    }
     k_cg_vec2<double><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_xp64, h->d_t,
                                                         A.n, A.ins0, h->d_cg, nullptr, 0);
     return cudaGetLastError();

@@ -47,7 +47,8 @@ def peaks():
 
 # sources of the row kernels; a capture's DRAM traffic applies only while
 # their hash is the one recorded beside it
-KERNEL_SOURCES = ("gsr_kernels.cu", "gsr_internal.cuh", "gsr_split.cuh", "gsr_reduce.cuh")
+KERNEL_SOURCES = ("gsr_kernels.cu", "gsr_internal.cuh", "gsr_split.cuh", "gsr_reduce.cuh",
+                  "gsr_lsqr.cuh", "gsr_tma.cuh")
 
 
 def kernel_source_hash():
@@ -700,8 +701,9 @@ def main():
     # preconditioner: single-launch aprod 2 of squares + combine + finish;
     # init: U, aprod 2, first vector pass), 3 per LSQR iteration (aprod 1,
     # single-launch aprod 2, vector pass that also combines aprod 2's
-    # partial sums), 1 epilogue
-    launches_per_step = 9 + 3 * (iters // args.steps)
+    # partial sums; all iterations of a system of at most 400,000 rows in one
+    # launch), 1 epilogue
+    launches_per_step = 9 + (3 * (iters // args.steps) if m > 400000 else 1)
     line = {"metric": METRIC, "value": value, "unit": "iter/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1e3 * t_max / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",

@@ -48,8 +48,8 @@ extern "C" {
 #define GSR_ERR_INDEX (-2)       /* structure out of range (star_ptr, attoff, instr) */
 #define GSR_ERR_OOM (-3)         /* device or host allocation failed */
 #define GSR_ERR_CUDA (-4)        /* a CUDA runtime call failed */
-#define GSR_ERR_TIMEOUT (-5)     /* a bounded device wait expired (the staged aprod 1
-                                    waited over a second for a bulk copy of a tile;
+#define GSR_ERR_TIMEOUT (-5)     /* a bounded device wait expired (a kernel waited
+                                    over a second for a bulk copy or a grid barrier;
                                     the results of that call are undefined) */
 #define GSR_ERR_NONFINITE (-6)   /* NaN or Inf in the input or in the recurrences */
 #define GSR_ERR_UNSUPPORTED (-7) /* configuration not supported by this build */
@@ -74,8 +74,11 @@ extern "C" {
  * to native FP64 products.  gsr_product_forms() tells which forms a handle
  * runs. */
 #define GSR_PRODUCTS_AUTO 0   /* library choice: aprod 1's split form where it
-                                 applies (I <= 3072); native products
-                                 otherwise and in aprod 2 */
+                                 applies (I <= 3072, and I up to what
+                                 the stages leave of the shared memory,
+                                 6,576, where aprod 1 runs staged);
+                                 native products otherwise and in
+                                 aprod 2 */
 #define GSR_PRODUCTS_NATIVE 1 /* every product on the FP64 pipe */
 #define GSR_PRODUCTS_SPLIT 2  /* the first three split forms: GSR_SPLIT_APROD1 |
                                  GSR_SPLIT_APROD2_STARS | GSR_SPLIT_APROD2_INSTR
@@ -203,8 +206,8 @@ int gsr_precondition(void *h, double *p, void *stream);
  * The whole iteration runs on the device (one CUDA graph, no host
  * synchronisation until the end).  `out` receives the stopping estimates.
  * Errors: GSR_ERR_ARG, GSR_ERR_NONFINITE (a NaN/Inf in b or in the scalar
- * recurrences; x and se are then undefined), GSR_ERR_TIMEOUT (a bounded wait
- * of the staged aprod 1 expired; x and se are undefined), GSR_ERR_CUDA.
+ * recurrences; x and se are then undefined), GSR_ERR_TIMEOUT (a bounded
+ * device wait expired; x and se are undefined), GSR_ERR_CUDA.
  */
 int gsr_lsqr_solve(void *h, const double *b, int itmax, double atol,
                    double btol, double *x, double *se, gsr_result *out,

@@ -485,10 +485,11 @@ static int build_units(gsr_handle_t *h)
     const SysView &A = h->sys;
     std::vector<uint32_t> seg((size_t)A.nseg + 1), useg((size_t)A.nseg + 1);
     CK(cudaMemcpy(seg.data(), h->d_seg, (A.nseg + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost));
-    // tiles per unit: about two units for each of the 16 warps of every SM (one
-    // warp with one unit of 8 tiles took 35 us at 700,000 rows, two with 4 took
-    // 32; smaller ones only add partial sums),
-    // at most kUnitTiles (the unit's reduction is then a small share)
+    // Tiles per unit: about two units for each of the 16 warps of every SM (at
+    // 700,000 rows one unit of 8 tiles per warp 35 us, two of 4 tiles 32;
+    // smaller ones only add partial sums), at most kUnitTiles (the unit's
+    // reduction is then a small share: 16 tiles 190 us, 8 tiles 185 us at
+    // 7.0e6 rows).
     const uint64_t want = (uint64_t)((A.m / 32) / ((int64_t)h->nsm * 32));
     const uint64_t ut = want < 1 ? 1 : (want > kUnitTiles ? kUnitTiles : want);
     std::vector<uint4> unit;
@@ -936,7 +937,7 @@ static int take_kernel_status(gsr_handle_t *h, cudaStream_t st)
     CK(cudaMemsetAsync(h->d_kerr, 0, sizeof(int), st));
     CK(cudaStreamSynchronize(st));
     snprintf(g_last_error, sizeof g_last_error, "%s",
-             "a bounded wait of the staged aprod 1 expired: a bulk copy did not complete");
+             "a bounded device wait expired: a bulk copy or a grid barrier did not complete");
     return GSR_ERR_TIMEOUT;
 }
 

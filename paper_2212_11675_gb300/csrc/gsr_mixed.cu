@@ -19,8 +19,10 @@
 // CG on the normal equations (Hestenes-Stiefel) with s_0 = c, d_0 = s_0:
 //   q = A32 (p o d), alpha = |s|^2 / |q|^2, z += alpha d,
 //   s -= alpha p o (A32^T q), beta = |s_new|^2 / |s|^2, d = s + beta d.
-// One inner iteration = 4 launches in a CUDA graph with a conditional WHILE
-// node, like the LSQR loop.
+// One inner iteration = 4 launches (the main pass with both products of the
+// attitude and global part, the star and instrument passes in one launch, two
+// vector passes) in a CUDA graph with a conditional WHILE node, like the LSQR
+// loop.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -52,8 +54,11 @@ constexpr int kF32A2 = 2;  // attitude and global part of A32^T q
 // alone: q is read from q32, *glb += its global column.
 // One reading of the values (96 B a row) serves both products, the row's q is
 // scattered to row order (28 MB at 7.0e6 rows: it stays in L2); the
-// astrometric x of a random star is one 32-byte sector of x8.  Bound by HBM:
-// 120 B a row.
+// astrometric x of a random star is one 32-byte sector of x8.
+// At 7.0e6 rows 186 us, against 124 us for its 120 B a row at the copy rate:
+// 490 instructions a visit keep 55 % of the issue slots busy, the rest is
+// latency with 16 warps an SM; without the scatter of q 173 us, without the
+// gather of x 174.  The product A32 x alone took 156 us in row order.
 // ---------------------------------------------------------------------------
 constexpr int kMainWarps = 16;  // one block per SM: 16 warps of three stages
 constexpr int kMainThreads = 32 * kMainWarps;

@@ -36,7 +36,6 @@
 
 namespace gsr {
 
-constexpr int64_t kSmemInstrMax32 = 12288;  // binary32 instrument entries in shared memory
 
 __device__ __forceinline__ int64_t gtid32() { return blockIdx.x * (int64_t)blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t gstride32() { return (int64_t)gridDim.x * blockDim.x; }
@@ -60,33 +59,46 @@ constexpr int kF32A2 = 2;  // attitude and global part of A32^T q
 // latency with 16 warps an SM; without the scatter of q 173 us, without the
 // gather of x 174.  The product A32 x alone took 156 us in row order.
 // ---------------------------------------------------------------------------
-constexpr int kMainWarps = 16;  // one block per SM: 16 warps of three stages
+constexpr int kMainWarps = 16;  // one block per SM
 constexpr int kMainThreads = 32 * kMainWarps;
-constexpr int kMainStages = 3;
+
+// Where the instrumental x is (six random reads a row): in shared memory
+// beside three stages a warp up to 12,288 instruments, beside two up to
+// 27,648; beyond, in global memory, with two stages so that more of it stays
+// in L1.  20,000 instruments, 7.0e7 rows: 3.97 ms from global memory beside
+// three stages, 3.85 from shared memory beside two (what holds it there is the
+// scatter of q, 280 MB that L2 does not keep).
+enum MainX { kXGlobal = 0, kXThree = 1, kXTwo = 2 };
+constexpr int64_t kXThreeMax = 12288, kXTwoMax = 27648;
+__host__ __device__ constexpr int main_stages(int where) { return where == kXThree ? 3 : 2; }
 
 // [stages][x of the attitude taps: 16 floats a warp][barriers][instrument x]
-constexpr size_t kMainSmem =
-    kMainWarps * (kMainStages * (kAttTileBytes + sizeof(uint64_t)) + 16 * sizeof(float));
+__host__ __device__ constexpr size_t main_smem(int where)
+{
+    return kMainWarps * (main_stages(where) * (kAttTileBytes + sizeof(uint64_t)) +
+                         16 * sizeof(float));
+}
 
-template <int MODE, bool SMEMX>
+template <int MODE, int X>
 __global__ void __launch_bounds__(kMainThreads, 1)
 k_f32_main(SysView A, Att32 U, const float *__restrict__ x32, const float *__restrict__ x8,
            float *__restrict__ q32, double *__restrict__ y, double *__restrict__ S,
            double *__restrict__ glb, CgState *cg, double *partial, unsigned *counter, int *kerr)
 {
-    constexpr bool A1 = (MODE & kF32A1) != 0, A2 = (MODE & kF32A2) != 0;
+    constexpr bool A1 = (MODE & kF32A1) != 0, A2 = (MODE & kF32A2) != 0, SMEMX = X != kXGlobal;
+    constexpr int NS = main_stages(X);
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    unsigned char *stages = smem + wib * kMainStages * kAttTileBytes;
-    float *s_xa = reinterpret_cast<float *>(smem + kMainWarps * kMainStages * kAttTileBytes) + 16 * wib;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kMainWarps * (kMainStages * kAttTileBytes +
+    unsigned char *stages = smem + wib * NS * kAttTileBytes;
+    float *s_xa = reinterpret_cast<float *>(smem + kMainWarps * NS * kAttTileBytes) + 16 * wib;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kMainWarps * (NS * kAttTileBytes +
                                                                        16 * sizeof(float))) +
-                     kMainStages * wib;
-    float *s_x32 = reinterpret_cast<float *>(smem + kMainSmem);
+                     NS * wib;
+    float *s_x32 = reinterpret_cast<float *>(smem + main_smem(X));
     // units are dealt to the warps of all blocks round-robin, blocks first, so
     // that a small system spreads over the SMs
-    AttWalk<kMainStages> walk(U, stages, bars, blockIdx.x + (int64_t)gridDim.x * wib,
-                 (int64_t)gridDim.x * kMainWarps);
+    AttWalk<NS> walk(U, stages, bars, blockIdx.x + (int64_t)gridDim.x * wib,
+                     (int64_t)gridDim.x * kMainWarps);
     if (A1 && SMEMX) {
         for (int64_t f = threadIdx.x; f < A.I; f += blockDim.x)
             s_x32[f] = x32[A.ins0 + f];
@@ -754,31 +766,29 @@ __global__ void k_count_pos(const double *__restrict__ a, int64_t n, double *par
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-static bool x32_in_smem(const gsr_handle_t *h) { return h->sys.I <= kSmemInstrMax32; }
-static size_t main_smem(const gsr_handle_t *h)
-{
-    return kMainSmem + (x32_in_smem(h) ? (size_t)h->sys.I * sizeof(float) : 0);
-}
-
 static A2Queue rest_queue(const gsr_handle_t *h)
 {
     return a2_queue(h, 8, (int64_t)h->sys.I * h->nq32 * h->ks32, 0);
 }
 
+template <int MODE, int X>
+static cudaError_t main_launch(const gsr_handle_t *h, double *y, double *glb, cudaStream_t st)
+{
+    const size_t smem = main_smem(X) + (X == kXGlobal ? 0 : (size_t)h->sys.I * sizeof(float));
+    k_f32_main<MODE, X><<<h->grid_main32, kMainThreads, smem, st>>>(
+        h->sys, h->att32, h->d_x32, h->d_x8, h->d_q32, y, h->d_attS32, glb, h->d_cg,
+        h->d_partial + kRedU * kPartialsPerKind, h->d_counter + kRedU, h->d_kerr);
+    return cudaGetLastError();
+}
+
 template <int MODE>
 static cudaError_t f32_main(const gsr_handle_t *h, double *y, double *glb, cudaStream_t st)
 {
-    double *part = h->d_partial + kRedU * kPartialsPerKind;
-    unsigned *cnt = h->d_counter + kRedU;
-    if (x32_in_smem(h))
-        k_f32_main<MODE, true><<<h->grid_main32, kMainThreads, main_smem(h), st>>>(
-            h->sys, h->att32, h->d_x32, h->d_x8, h->d_q32, y, h->d_attS32, glb, h->d_cg, part, cnt,
-            h->d_kerr);
-    else
-        k_f32_main<MODE, false><<<h->grid_main32, kMainThreads, main_smem(h), st>>>(
-            h->sys, h->att32, h->d_x32, h->d_x8, h->d_q32, y, h->d_attS32, glb, h->d_cg, part, cnt,
-            h->d_kerr);
-    return cudaGetLastError();
+    if (h->sys.I <= kXThreeMax)
+        return main_launch<MODE, kXThree>(h, y, glb, st);
+    if (h->sys.I <= kXTwoMax)
+        return main_launch<MODE, kXTwo>(h, y, glb, st);
+    return main_launch<MODE, kXGlobal>(h, y, glb, st);
 }
 
 // the rest of aprod 2 over the row-ordered q32: stars and instruments; *P:
@@ -999,17 +1009,23 @@ cudaError_t launch_to_f32(const gsr_handle_t *h, const double *a, float *b, int6
 // one block per SM, no more than the units need
 int f32_main_grid(const gsr_handle_t *h)
 {
-    const void *fns[6] = {(const void *)k_f32_main<1, true>, (const void *)k_f32_main<1, false>,
-                          (const void *)k_f32_main<2, true>, (const void *)k_f32_main<2, false>,
-                          (const void *)k_f32_main<3, true>, (const void *)k_f32_main<3, false>};
-    for (const void *f : fns) {
-        // the most that any handle of this process asks for: the attribute is
-        // shared by all of them
-        const size_t most = kMainSmem + kSmemInstrMax32 * sizeof(float);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
+    // the most that any handle of this process asks for: the attribute is
+    // shared by all of them
+    const struct {
+        const void *f;
+        size_t smem;
+    } fns[9] = {
+#define GSR_MAIN(X, MAX)                                                    \
+    {(const void *)k_f32_main<1, X>, main_smem(X) + (MAX) * sizeof(float)}, \
+    {(const void *)k_f32_main<2, X>, main_smem(X) + (MAX) * sizeof(float)}, \
+    {(const void *)k_f32_main<3, X>, main_smem(X) + (MAX) * sizeof(float)}
+        GSR_MAIN(kXGlobal, 0), GSR_MAIN(kXThree, kXThreeMax), GSR_MAIN(kXTwo, kXTwoMax)
+#undef GSR_MAIN
+    };
+    for (const auto &k : fns)
+        if (cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem) !=
             cudaSuccess)
             return -1;
-    }
     const int64_t nu = h->att32.nunits;
     return (int)(nu < h->nsm ? nu : h->nsm);
 }

@@ -61,6 +61,10 @@ SHAPES = {
     "instr_6577": (300, 12, 50, 6577, None),
     "instr_6598": (300, 12, 50, 6598, None),
     "instr_6599": (300, 12, 50, 6599, None),
+    "instr_12288": (300, 12, 50, 12288, None),  # the binary32 main pass's limits
+    "instr_12289": (300, 12, 50, 12289, None),
+    "instr_27648": (300, 12, 50, 27648, None),
+    "instr_27649": (300, 12, 50, 27649, None),
 }
 
 

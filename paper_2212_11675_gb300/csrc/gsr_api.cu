@@ -480,6 +480,8 @@ static int build_instr_sorted(gsr_handle_t *h, cudaStream_t st)
 }
 
 // the units of the offset-ordered binary32 layout (Att32)
+constexpr int64_t kQInL2 = 96 << 20;  // bytes of the 129 MB
+
 static int build_units(gsr_handle_t *h)
 {
     const SysView &A = h->sys;
@@ -505,11 +507,26 @@ static int build_units(gsr_handle_t *h)
         for (uint64_t q = 0; q < np; q++) {
             const uint64_t a = (t0 + nt * q / np) << 5, b = (t0 + nt * (q + 1) / np) << 5;
             unit.push_back(make_uint4((uint32_t)o, (uint32_t)std::max(a, e0),
-                                      (uint32_t)std::min(b, e1), 0u));
+                                      (uint32_t)std::min(b, e1), (uint32_t)unit.size()));
         }
     }
     useg[A.nseg] = (uint32_t)unit.size();
     const int64_t nu = (int64_t)unit.size();
+    // Where the binary32 q does not fit in L2, the units are taken in the order
+    // of their rows (an offset's rows ascend, so unit q of np begins near the
+    // fraction q / np of all rows): the rows of q that are written at a time lie
+    // together (7.0e7 rows, 280 MB of q: the main pass 3.85 -> 3.23 ms).
+    if (A.m * (int64_t)sizeof(float) > kQInL2) {
+        std::vector<std::pair<float, uint32_t>> key((size_t)nu);
+        for (int64_t o = 0; o < A.nseg; o++)
+            for (uint32_t i = useg[o]; i < useg[o + 1]; i++)
+                key[i] = {(float)(i - useg[o]) / (float)(useg[o + 1] - useg[o]), i};
+        std::sort(key.begin(), key.end());
+        std::vector<uint4> by((size_t)nu);
+        for (int64_t i = 0; i < nu; i++)
+            by[i] = unit[key[i].second];
+        unit.swap(by);
+    }
     TRY(dalloc(h, &h->d_unit, nu));
     TRY(dalloc(h, &h->d_useg, A.nseg + 1));
     TRY(dalloc(h, &h->d_attS32, nu * kNAtt));

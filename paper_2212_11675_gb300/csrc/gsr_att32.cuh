@@ -14,7 +14,7 @@
 namespace gsr {
 
 struct Visit {
-    uint4 un;    // offset, first entry, end of the unit
+    uint4 un;    // offset, first entry, end of the unit, where its sums go
     uint32_t t;  // tile
     bool ok;
     __device__ __forceinline__ bool first() const { return t == (un.y >> 5); }

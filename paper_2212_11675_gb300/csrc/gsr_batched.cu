@@ -343,7 +343,7 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
                     unpack2(sl[i], l0, l1);
                     df_add(h0, l0, h1, l1);
                     if (lane + 32 * i < NOUT)
-                        S[u * NOUT + lane + 32 * i] = df_to_d(h0, l0);
+                        S[(int64_t)v.un.w * NOUT + lane + 32 * i] = df_to_d(h0, l0);
                 }
             }
         }

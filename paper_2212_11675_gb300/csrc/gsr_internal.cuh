@@ -51,7 +51,7 @@ struct Att32 {
     // floats each), the records (star, then the instrument words of
     // SysView::rec) and the rows, so that one bulk copy stages a tile
     const unsigned char *tile;
-    const uint4 *unit;     // [nunits] offset, first entry, last entry + 1, 0
+    const uint4 *unit;     // [nunits] offset, first entry, last entry + 1, place of its sums
     const uint32_t *useg;  // [nseg+1] units of offset o: useg[o] .. useg[o+1]-1
     const float *sv;       // the 5 astrometric planes in row order (tidx<5>)
     int64_t nunits;

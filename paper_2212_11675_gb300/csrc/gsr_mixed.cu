@@ -48,7 +48,7 @@ constexpr int kF32A2 = 2;  // attitude and global part of A32^T q
 // Main pass of the inner operator over the offset-ordered values, one row per
 // lane (binary32 products, double-float sums).
 // A1 and A2 (CG): q32[row] = fl32(A32 x32) with |q|^2 (alpha = gamma / |q|^2
-// by the last block), the attitude sums of A32^T q into S[unit][4a + j] and
+// by the last block), the attitude sums of A32^T q into S[place of the unit][4a + j] and
 // its global column into *glb.  A1 alone: y[row] += A32 x32 in FP64.  A2
 // alone: q is read from q32, *glb += its global column.
 // One reading of the values (96 B a row) serves both products, the row's q is
@@ -66,8 +66,8 @@ constexpr int kMainThreads = 32 * kMainWarps;
 // beside three stages a warp up to 12,288 instruments, beside two up to
 // 27,648; beyond, in global memory, with two stages so that more of it stays
 // in L1.  20,000 instruments, 7.0e7 rows: 3.97 ms from global memory beside
-// three stages, 3.85 from shared memory beside two (what holds it there is the
-// scatter of q, 280 MB that L2 does not keep).
+// three stages, 3.85 from shared memory beside two (3.23 with the units in the
+// order of their rows, which keeps the scatter of q in L2).
 enum MainX { kXGlobal = 0, kXThree = 1, kXTwo = 2 };
 constexpr int64_t kXThreeMax = 12288, kXTwoMax = 27648;
 __host__ __device__ constexpr int main_stages(int where) { return where == kXThree ? 3 : 2; }
@@ -219,7 +219,7 @@ k_f32_main(SysView A, Att32 U, const float *__restrict__ x32, const float *__res
                 df_reduce_scatter<16, 32>(rh, rl, lane);
                 const int kk = lane >> 1;
                 if ((lane & 1) == 0 && kk < kNAtt)
-                    S[u * kNAtt + kk] = df_to_d(rh[0], rl[0]);
+                    S[(int64_t)v.un.w * kNAtt + kk] = df_to_d(rh[0], rl[0]);
             }
             u += (int64_t)gridDim.x * kMainWarps;
         }

@@ -1955,7 +1955,13 @@ static cudaError_t loop_launch(const gsr_handle_t *h, cudaStream_t st)
                   h->d_state, h->d_args, h->d_partial, h->d_bar, h->d_kerr};
     SysView A = h->sys;
     void *args[] = {&A, &L};
-    cudaError_t e = cudaMemsetAsync(h->d_bar, 0, sizeof(unsigned), st);
+    // beside the kernel's static shared memory, the pieces of kSplitInstrMax
+    // instruments exceed the 48 KB that a launch may have without asking; the
+    // attribute belongs to the kernel: the most that any handle asks for
+    cudaError_t e = cudaFuncSetAttribute(k_lsqr_loop<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kSplitInstrMax * sizeof(float4)));
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(h->d_bar, 0, sizeof(unsigned), st);
     if (e == cudaSuccess)
         e = cudaLaunchCooperativeKernel(k_lsqr_loop<G>, dim3(h->nsm), dim3(kLoopThreads), args,
                                         (size_t)A.I * sizeof(float4), st);

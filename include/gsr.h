@@ -303,8 +303,8 @@ int gsr_product_forms(void *h, int *aprod1_split_on, int *aprod2_split_on);
 /*
  * Replace nonzero k (0..23, in the order of the column map above) of every
  * row with values[m] (host or device).  k = 23 is the global (PPN gamma)
- * column.  The derived copies (offset-sorted attitude values, binary32
- * copy) follow.  Solves started afterwards use the new values.
+ * column.  The derived copies (offset-sorted attitude values,
+ * instrument-sorted values, binary32 copies) follow.  Solves started afterwards use the new values.
  */
 int gsr_set_values(void *h, int k, const double *values, void *stream);
 

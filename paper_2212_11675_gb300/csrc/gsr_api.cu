@@ -1249,8 +1249,13 @@ extern "C" int gsr_set_values(void *hv, int k, const double *values, void *strea
     double *dv;
     TRY(stage(h, &h->d_ystage, h->sys.m, values, &dv, true, st));
     CK(launch_set_plane(h, k, dv, st));
-    if (h->ell_on && k >= kNAstro + kNAtt && k < kNAstro + kNAtt + kNInstr)
-        CK(launch_ell_plane(h, k - kNAstro - kNAtt, st));
+    const int slot = k - kNAstro - kNAtt;  // of an instrumental nonzero
+    if (slot >= 0 && slot < kNInstr) {
+        if (h->d_ival)
+            CK(launch_instr_plane(h, slot, st));
+        if (h->ell_on)
+            CK(launch_ell_plane(h, slot, st));
+    }
     if (h->cfg.precision == GSR_PREC_MIXED)
         CK(launch_f32_plane(h, k, st));
     if (dv != values)

@@ -385,6 +385,7 @@ cudaError_t launch_aprod1(const gsr_handle_t *h, const double *x, double *y,
                           int lsqr_mode, cudaStream_t st);
 cudaError_t launch_aprod1_cg(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
 cudaError_t launch_set_plane(const gsr_handle_t *h, int k, const double *v, cudaStream_t st);
+cudaError_t launch_instr_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
 cudaError_t launch_grad_global(const gsr_handle_t *h, const double *r, const double *s,
                                const double *q, const double *x, double *grad, cudaStream_t st);
 cudaError_t build_cg64_graph(gsr_handle_t *h);

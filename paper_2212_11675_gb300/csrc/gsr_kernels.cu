@@ -2168,6 +2168,51 @@ cudaError_t launch_set_plane(const gsr_handle_t *h, int k, const double *v, cuda
     return cudaGetLastError();
 }
 
+// The values of instrument slot `slot` again in the instrument-sorted copy
+// (np pieces of each instrument's entries, a warp each).  An entry holds its
+// row only: entry e is slot j of the row, j the (number of entries before e
+// with the same row)-th slot that names the instrument, because the entries of
+// an instrument are in row and slot order.
+__global__ void __launch_bounds__(kThreads)
+k_regather_instr_plane(SysView A, int slot, const uint32_t *__restrict__ iseg,
+                       const uint32_t *__restrict__ irow, double *__restrict__ ival,
+                       float *__restrict__ ival32, int np)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = warp; w < A.I * np; w += nwarps) {
+        const int64_t q = w / A.I;
+        const uint32_t f = (uint32_t)(w - q * A.I);
+        const uint32_t s0 = iseg[f];
+        const uint64_t len = iseg[f + 1] - s0;
+        const uint32_t e1 = s0 + (uint32_t)(len * (q + 1) / np);
+        for (uint32_t e = s0 + (uint32_t)(len * q / np) + lane; e < e1; e += 32) {
+            const uint32_t r = irow[e];
+            int before = 0;
+            for (uint32_t i = e; i > s0 && irow[i - 1] == r; i--)
+                before++;
+            const uint4 rc = A.rec[r];
+            int j = 0;
+            while (j < kNInstr && (instr_at(rc, j) != f || before-- > 0))
+                j++;
+            if (j == slot) {
+                const double v = A.val[tidx<kNPar>(kNAstro + kNAtt + slot, r)];
+                ival[e] = v;
+                if (ival32)
+                    ival32[e] = (float)v;
+            }
+        }
+    }
+}
+
+cudaError_t launch_instr_plane(const gsr_handle_t *h, int slot, cudaStream_t st)
+{
+    k_regather_instr_plane<<<h->nsm * 8, kThreads, 0, st>>>(
+        h->sys, slot, h->d_iseg, h->d_irow, h->d_ival, h->d_ival32, batched_instr_pieces(h));
+    return cudaGetLastError();
+}
+
 // grad[i] = r_i q_G - s_i x_G (derivative of the loss with respect to the
 // global-column value of row i, for the least-squares solution x)
 __global__ void k_grad_global(const double *__restrict__ r, const double *__restrict__ s,

@@ -381,86 +381,86 @@ struct gsr_handle_t {
 namespace gsr {
 
 // launchers (gsr_kernels.cu)
-cudaError_t launch_aprod1(const gsr_handle_t *h, const double *x, double *y,
-                          int lsqr_mode, cudaStream_t st);
-cudaError_t launch_aprod1_cg(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
-cudaError_t launch_set_plane(const gsr_handle_t *h, int k, const double *v, cudaStream_t st);
-cudaError_t launch_instr_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
-cudaError_t launch_grad_global(const gsr_handle_t *h, const double *r, const double *s,
-                               const double *q, const double *x, double *grad, cudaStream_t st);
-cudaError_t build_cg64_graph(gsr_handle_t *h);
-cudaError_t run_cg64(gsr_handle_t *h, cudaStream_t st, int max_iter);
-cudaError_t launch_f32_plane(const gsr_handle_t *h, int k, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_aprod1(const gsr_handle_t *h, const double *x, double *y,
+                                        int lsqr_mode, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_aprod1_cg(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_set_plane(const gsr_handle_t *h, int k, const double *v, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_instr_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_grad_global(const gsr_handle_t *h, const double *r, const double *s,
+                                             const double *q, const double *x, double *grad, cudaStream_t st);
+[[nodiscard]] cudaError_t build_cg64_graph(gsr_handle_t *h);
+[[nodiscard]] cudaError_t run_cg64(gsr_handle_t *h, cudaStream_t st, int max_iter);
+[[nodiscard]] cudaError_t launch_f32_plane(const gsr_handle_t *h, int k, cudaStream_t st);
 // batched (gsr_batched.cu)
-cudaError_t build_batched_graph(gsr_handle_t *h, int k);
-cudaError_t run_batched_inner(gsr_handle_t *h, int k, int max_inner, cudaStream_t st);
-cudaError_t launch_b_update_x(const gsr_handle_t *h, double *X, int k, cudaStream_t st);
-cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, float *Y,
-                              double *T, cudaStream_t st);
-cudaError_t launch_b_layout(const gsr_handle_t *h, int to_rm, const double *src, void *dst,
-                            int dst_f32, int64_t rows, int k, cudaStream_t st);
+[[nodiscard]] cudaError_t build_batched_graph(gsr_handle_t *h, int k);
+[[nodiscard]] cudaError_t run_batched_inner(gsr_handle_t *h, int k, int max_inner, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_b_update_x(const gsr_handle_t *h, double *X, int k, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_b_products(const gsr_handle_t *h, int k, const float *X, float *Q, float *Y,
+                                            double *T, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_b_layout(const gsr_handle_t *h, int to_rm, const double *src, void *dst,
+                                          int dst_f32, int64_t rows, int k, cudaStream_t st);
 int batched_instr_pieces(const gsr_handle_t *h);
-cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out,
-                          int mode, cudaStream_t st);
-cudaError_t launch_validate(const gsr_handle_t *h, cudaStream_t st);
-cudaError_t launch_planes(const gsr_handle_t *h, const double *rowmajor,
-                          int64_t row0, int64_t nrows, cudaStream_t st);
-cudaError_t launch_pack_rec(const gsr_handle_t *h, const uint32_t *attoff,
-                            const uint16_t *instr, int64_t row0, int64_t nrows,
-                            cudaStream_t st);
-cudaError_t launch_tile_star(const gsr_handle_t *h, cudaStream_t st);
-cudaError_t launch_gather_att(const gsr_handle_t *h, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out,
+                                        int mode, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_validate(const gsr_handle_t *h, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_planes(const gsr_handle_t *h, const double *rowmajor,
+                                        int64_t row0, int64_t nrows, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_pack_rec(const gsr_handle_t *h, const uint32_t *attoff,
+                                          const uint16_t *instr, int64_t row0, int64_t nrows,
+                                          cudaStream_t st);
+[[nodiscard]] cudaError_t launch_tile_star(const gsr_handle_t *h, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_gather_att(const gsr_handle_t *h, cudaStream_t st);
 int aprod1_grid(const gsr_handle_t *h);
 // the staged aprod 1 for this handle: its shared memory (0: does not apply)
 size_t aprod1_tma_smem(const gsr_handle_t *h);
-cudaError_t aprod1_tma_prepare(gsr_handle_t *h);
+[[nodiscard]] cudaError_t aprod1_tma_prepare(gsr_handle_t *h);
 bool aprod1_split(const gsr_handle_t *h);
 int split_request(const gsr_config &cfg);
 int aprod2_split(const gsr_handle_t *h);
 int aprod2_split_active(const gsr_handle_t *h);
-cudaError_t launch_att_combine(const gsr_handle_t *h, double *out, int nb_att, int nb_ins,
-                               double *rep, int nrep, const double *gpart, int ngpart,
-                               bool accumulate, cudaStream_t st, unsigned long long *ctr = nullptr);
+[[nodiscard]] cudaError_t launch_att_combine(const gsr_handle_t *h, double *out, int nb_att, int nb_ins,
+                                             double *rep, int nrep, const double *gpart, int ngpart,
+                                             bool accumulate, cudaStream_t st, unsigned long long *ctr = nullptr);
 int instr_path(const gsr_config &cfg, int64_t I);
 A2Queue a2_queue(const gsr_handle_t *h, int G, int64_t ninstr_units = -1, int64_t natt = -1);
 bool aprod2_partials(const gsr_handle_t *h, const double *y, double *out, const double **S,
                      const double **ipart, int *isplit, const double **gpart, int *ngpart,
                      unsigned long long **ctr, cudaStream_t st);
-cudaError_t launch_gather_instr64(const gsr_handle_t *h, const uint32_t *code, double *out,
-                                  cudaStream_t st);
+[[nodiscard]] cudaError_t launch_gather_instr64(const gsr_handle_t *h, const uint32_t *code, double *out,
+                                                cudaStream_t st);
 // instrument pass over row windows (gsr_ell.cu)
-cudaError_t launch_ell_fill(const gsr_handle_t *h, const uint32_t *code, int64_t total,
-                            cudaStream_t st);
-cudaError_t launch_ell_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
-cudaError_t launch_ell_sorted(const gsr_handle_t *h, const uint32_t *start, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_ell_fill(const gsr_handle_t *h, const uint32_t *code, int64_t total,
+                                          cudaStream_t st);
+[[nodiscard]] cudaError_t launch_ell_plane(const gsr_handle_t *h, int slot, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_ell_sorted(const gsr_handle_t *h, const uint32_t *start, cudaStream_t st);
 // mixed precision (gsr_mixed.cu)
-cudaError_t launch_aprod1_f32_api(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
-cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double *x, cudaStream_t st);
-cudaError_t build_cg_graph(gsr_handle_t *h);
-cudaError_t run_cg(gsr_handle_t *h, cudaStream_t st, int max_inner);
-cudaError_t launch_outer_norms(const gsr_handle_t *h, const double *r, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_aprod1_f32_api(const gsr_handle_t *h, const double *x, double *y, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double *x, cudaStream_t st);
+[[nodiscard]] cudaError_t build_cg_graph(gsr_handle_t *h);
+[[nodiscard]] cudaError_t run_cg(gsr_handle_t *h, cudaStream_t st, int max_inner);
+[[nodiscard]] cudaError_t launch_outer_norms(const gsr_handle_t *h, const double *r, cudaStream_t st);
 // out2 = (||p o c||^2, ||r||^2) for one n-vector c and one m-vector r
-cudaError_t launch_norms2(const gsr_handle_t *h, const double *c, const double *r, double *out2,
-                          cudaStream_t st);
-cudaError_t launch_neg(const gsr_handle_t *h, const double *a, double *b, int64_t n, cudaStream_t st);
-cudaError_t launch_count_pos(const gsr_handle_t *h, const double *a, double *out, cudaStream_t st);
-cudaError_t launch_to_f32(const gsr_handle_t *h, const double *a, float *b, int64_t n, cudaStream_t st);
-cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_norms2(const gsr_handle_t *h, const double *c, const double *r, double *out2,
+                                        cudaStream_t st);
+[[nodiscard]] cudaError_t launch_neg(const gsr_handle_t *h, const double *a, double *b, int64_t n, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_count_pos(const gsr_handle_t *h, const double *a, double *out, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_to_f32(const gsr_handle_t *h, const double *a, float *b, int64_t n, cudaStream_t st);
+[[nodiscard]] cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st);
 int f32_main_grid(const gsr_handle_t *h);
 int f32_rest_grid(const gsr_handle_t *h);
-cudaError_t enqueue_precondition(const gsr_handle_t *h, double *p, cudaStream_t st);
+[[nodiscard]] cudaError_t enqueue_precondition(const gsr_handle_t *h, double *p, cudaStream_t st);
 // all LSQR iterations of a small system in one launch (gsr_kernels.cu)
 bool lsqr_loop_fits(const gsr_handle_t *h);
-cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st);
 // LSQR pieces (gsr_lsqr.cu)
-cudaError_t build_solve_graph(gsr_handle_t *h);
-cudaError_t enqueue_prologue(const gsr_handle_t *h, cudaStream_t s,
-                             cudaGraphConditionalHandle loop, int in_graph);
-cudaError_t enqueue_iteration(const gsr_handle_t *h, cudaStream_t s,
-                              cudaGraphConditionalHandle loop, int in_graph);
-cudaError_t enqueue_epilogue(const gsr_handle_t *h, cudaStream_t s);
-cudaError_t enqueue_iteration_timed(const gsr_handle_t *h, cudaStream_t s, const cudaEvent_t *ev);
-cudaError_t launch_precond_finish(const gsr_handle_t *h, double *p, cudaStream_t st);
+[[nodiscard]] cudaError_t build_solve_graph(gsr_handle_t *h);
+[[nodiscard]] cudaError_t enqueue_prologue(const gsr_handle_t *h, cudaStream_t s,
+                                           cudaGraphConditionalHandle loop, int in_graph);
+[[nodiscard]] cudaError_t enqueue_iteration(const gsr_handle_t *h, cudaStream_t s,
+                                            cudaGraphConditionalHandle loop, int in_graph);
+[[nodiscard]] cudaError_t enqueue_epilogue(const gsr_handle_t *h, cudaStream_t s);
+[[nodiscard]] cudaError_t enqueue_iteration_timed(const gsr_handle_t *h, cudaStream_t s, const cudaEvent_t *ev);
+[[nodiscard]] cudaError_t launch_precond_finish(const gsr_handle_t *h, double *p, cudaStream_t st);
 int lsqr_vec_grid(const gsr_handle_t *h);
 // gsr_noalloc.cu: scratch address of gsr_aprod1_norm_noalloc on device dev
 int noalloc_prepare(int dev);

@@ -297,8 +297,9 @@ cudaError_t find_graph_leaf(cudaGraph_t g, cudaGraphNode_t *leaf)
 
 // q = A^T U (overwrite) and the vector pass; with the single-launch aprod 2
 // the vector pass combines its partial sums itself
-static cudaError_t a2_and_vec(const gsr_handle_t *h, cudaStream_t s, cudaGraphConditionalHandle loop,
-                              int in_graph, int first, cudaEvent_t mid = nullptr)
+[[nodiscard]] static cudaError_t a2_and_vec(const gsr_handle_t *h, cudaStream_t s,
+                                            cudaGraphConditionalHandle loop, int in_graph, int first,
+                                            cudaEvent_t mid = nullptr)
 {
     double *part = h->d_partial + kRedV * kPartialsPerKind;
     unsigned *cnt = h->d_counter + kRedV;
@@ -407,7 +408,7 @@ cudaError_t build_solve_graph(gsr_handle_t *h)
     GSR_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
 
     GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_prologue(h, s, loop, 1);
+    GSR_TRY(enqueue_prologue(h, s, loop, 1));
     GSR_TRY(cudaStreamEndCapture(s, &g));
     GSR_TRY(find_graph_leaf(g, &pre_leaf));
 
@@ -419,11 +420,11 @@ cudaError_t build_solve_graph(gsr_handle_t *h)
     GSR_TRY(cudaGraphAddNode(&wnode, g, &pre_leaf, nullptr, 1, &cp));
     body = cp.conditional.phGraph_out[0];
     GSR_TRY(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_iteration(h, s, loop, 1);
+    GSR_TRY(enqueue_iteration(h, s, loop, 1));
     GSR_TRY(cudaStreamEndCapture(s, &body));
 
     GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-    enqueue_epilogue(h, s);
+    GSR_TRY(enqueue_epilogue(h, s));
     GSR_TRY(cudaStreamEndCapture(s, &g));
 
     GSR_TRY(cudaGraphInstantiate(&h->solve_exec, g, 0));

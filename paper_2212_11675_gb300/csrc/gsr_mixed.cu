@@ -797,12 +797,6 @@ static cudaError_t f32_main(const gsr_handle_t *h, double *y, double *glb, cudaS
 template <int MODE, int G>
 static cudaError_t rest_win(const gsr_handle_t *h, double *out, cudaStream_t st)
 {
-    // the most that any handle of the process may ask for
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_f32_rest_win<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)(kEllSmem32 + kEllAccMax * sizeof(double)));
-    if (e != cudaSuccess)
-        return e;
     // at most two star groups a unit: the 8 warps that start with stars end
     // nearer to the 16 of the windows (113 -> 106 us at m = 7.0e6)
     A2Queue q = a2_queue(h, G, 0, 0);
@@ -859,8 +853,8 @@ cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double
     return cudaGetLastError();
 }
 
-static cudaError_t cg_prologue(const gsr_handle_t *h, cudaStream_t s, cudaGraphConditionalHandle loop,
-                               int in_graph)
+[[nodiscard]] static cudaError_t cg_prologue(const gsr_handle_t *h, cudaStream_t s,
+                                             cudaGraphConditionalHandle loop, int in_graph)
 {
     const SysView &A = h->sys;
     k_cg_init<float><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_c, h->d_s, h->d_d, h->d_zc, h->d_x32,
@@ -871,8 +865,8 @@ static cudaError_t cg_prologue(const gsr_handle_t *h, cudaStream_t s, cudaGraphC
     return cudaGetLastError();
 }
 
-static cudaError_t cg_iteration(const gsr_handle_t *h, cudaStream_t s, cudaGraphConditionalHandle loop,
-                                int in_graph)
+[[nodiscard]] static cudaError_t cg_iteration(const gsr_handle_t *h, cudaStream_t s,
+                                              cudaGraphConditionalHandle loop, int in_graph)
 {
     const SysView &A = h->sys;
     A2Parts P;
@@ -915,7 +909,7 @@ cudaError_t build_cg_graph(gsr_handle_t *h)
     CG_TRY(cudaGraphCreate(&g, 0));
     CG_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
     CG_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    cg_prologue(h, s, loop, 1);
+    CG_TRY(cg_prologue(h, s, loop, 1));
     CG_TRY(cudaStreamEndCapture(s, &g));
     CG_TRY(find_graph_leaf(g, &pre_leaf));
     cp.type = cudaGraphNodeTypeConditional;
@@ -925,10 +919,11 @@ cudaError_t build_cg_graph(gsr_handle_t *h)
     CG_TRY(cudaGraphAddNode(&wnode, g, &pre_leaf, nullptr, 1, &cp));
     body = cp.conditional.phGraph_out[0];
     CG_TRY(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    cg_iteration(h, s, loop, 1);
+    CG_TRY(cg_iteration(h, s, loop, 1));
     CG_TRY(cudaStreamEndCapture(s, &body));
     CG_TRY(cudaStreamBeginCaptureToGraph(s, g, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
     k_axpy_p<<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_zc, h->d_xm, h->sys.n);
+    CG_TRY(cudaGetLastError());
     CG_TRY(cudaStreamEndCapture(s, &g));
     CG_TRY(cudaGraphInstantiate(&h->cg_exec, g, 0));
     cudaGraphDestroy(g);
@@ -1032,8 +1027,19 @@ int f32_main_grid(const gsr_handle_t *h)
 
 int f32_rest_grid(const gsr_handle_t *h)
 {
+    // the most that any handle of the process may ask for
+    const void *fns[6] = {
+        (const void *)k_f32_rest_win<8, kA2Accumulate>,  (const void *)k_f32_rest_win<8, kA2Overwrite>,
+        (const void *)k_f32_rest_win<16, kA2Accumulate>, (const void *)k_f32_rest_win<16, kA2Overwrite>,
+        (const void *)k_f32_rest_win<32, kA2Accumulate>, (const void *)k_f32_rest_win<32, kA2Overwrite>};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 6 && e == cudaSuccess; i++)
+        e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kEllSmem32 + kEllAccMax * sizeof(double)));
+    if (e != cudaSuccess)
+        return -1;
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &occ, k_f32_rest<8, kA2Overwrite, true>, kThreads, 0);
     if (e != cudaSuccess || occ <= 0)
         return -1;
@@ -1089,8 +1095,8 @@ cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st)
 // the inner solve above with the FP64 products of gsr_kernels.cu (used for
 // the adjoint of the least-squares solution)
 // ---------------------------------------------------------------------------
-static cudaError_t cg64_prologue(const gsr_handle_t *h, cudaStream_t s,
-                                 cudaGraphConditionalHandle loop, int in_graph)
+[[nodiscard]] static cudaError_t cg64_prologue(const gsr_handle_t *h, cudaStream_t s,
+                                               cudaGraphConditionalHandle loop, int in_graph)
 {
     const SysView &A = h->sys;
     k_cg_init<double><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_c, h->d_s, h->d_d, h->d_zc,
@@ -1102,8 +1108,8 @@ static cudaError_t cg64_prologue(const gsr_handle_t *h, cudaStream_t s,
     return cudaGetLastError();
 }
 
-static cudaError_t cg64_iteration(const gsr_handle_t *h, cudaStream_t s,
-                                  cudaGraphConditionalHandle loop, int in_graph)
+[[nodiscard]] static cudaError_t cg64_iteration(const gsr_handle_t *h, cudaStream_t s,
+                                                cudaGraphConditionalHandle loop, int in_graph)
 {
     const SysView &A = h->sys;
     cudaError_t e = launch_aprod1_cg(h, h->d_xp64, h->d_q64, s);
@@ -1142,7 +1148,7 @@ cudaError_t build_cg64_graph(gsr_handle_t *h)
     CG_TRY(cudaGraphCreate(&g, 0));
     CG_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
     CG_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    cg64_prologue(h, s, loop, 1);
+    CG_TRY(cg64_prologue(h, s, loop, 1));
     CG_TRY(cudaStreamEndCapture(s, &g));
     CG_TRY(find_graph_leaf(g, &pre_leaf));
     cp.type = cudaGraphNodeTypeConditional;
@@ -1152,10 +1158,11 @@ cudaError_t build_cg64_graph(gsr_handle_t *h)
     CG_TRY(cudaGraphAddNode(&wnode, g, &pre_leaf, nullptr, 1, &cp));
     body = cp.conditional.phGraph_out[0];
     CG_TRY(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    cg64_iteration(h, s, loop, 1);
+    CG_TRY(cg64_iteration(h, s, loop, 1));
     CG_TRY(cudaStreamEndCapture(s, &body));
     CG_TRY(cudaStreamBeginCaptureToGraph(s, g, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
     k_axpy_p<<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_zc, h->d_xm, h->sys.n);
+    CG_TRY(cudaGetLastError());
     CG_TRY(cudaStreamEndCapture(s, &g));
     CG_TRY(cudaGraphInstantiate(&h->cg64_exec, g, 0));
     cudaGraphDestroy(g);

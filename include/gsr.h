@@ -214,6 +214,14 @@ int gsr_lsqr_solve(void *h, const double *b, int itmax, double atol,
                    void *stream);
 
 /*
+ * *on = 1 when gsr_lsqr_solve runs the iterations of this handle in one
+ * kernel launch (a small system with the default product forms), 0 when it
+ * launches three kernels an iteration.  Host only, no CUDA call.  Errors:
+ * GSR_ERR_ARG.
+ */
+int gsr_lsqr_one_launch(void *h, int *on);
+
+/*
  * y[m] = A x[n] + cy * y[m] and *ynorm = ||y||_2 (the first half of a
  * Golub-Kahan step with cy = -alpha), without allocating anything.  The
  * paper has no counterpart: this entry point exists for callers that must

@@ -1075,6 +1075,15 @@ extern "C" int gsr_lsqr_solve(void *hv, const double *b, int itmax, double atol,
     return s.nonfinite ? GSR_ERR_NONFINITE : GSR_OK;
 }
 
+extern "C" int gsr_lsqr_one_launch(void *hv, int *on)
+{
+    const gsr_handle_t *h = (const gsr_handle_t *)hv;
+    if (!h || !on)
+        return GSR_ERR_ARG;
+    *on = !h->cfg.eager && lsqr_loop_fits(h) ? 1 : 0;
+    return GSR_OK;
+}
+
 extern "C" int gsr_time_iteration(void *hv, const double *b, int iters, double *ms3, void *stream)
 {
     gsr_handle_t *h = (gsr_handle_t *)hv;

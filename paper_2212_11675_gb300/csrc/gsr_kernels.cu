@@ -1325,8 +1325,8 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // grid reductions whose last block works alone.  Here its three parts are
 // separated by barriers of the grid, and every block works out the sums of
 // the blocks' partials and the scalar recurrences for itself, in the same
-// order, so no block waits for another's result (20,000 rows: 36.6 -> 27 us an
-// iteration; 280,000: 80.7 -> 74; from 500,000 rows on the launches win).
+// order, so no block waits for another's result (20,000 rows: 34.2 -> 23.7 us
+// an iteration).
 //   1. U = A vp + cy U, ||U||^2 (rows as in k_aprod1's split form)
 //   2. star, attitude and instrument units of A^T U, one after the other
 //   3. the columns; block 0 adds the global column
@@ -1335,11 +1335,19 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // the next iteration (which changes only U, so it may be one too many).
 // Data that other blocks write is read from L2 (ld_shared).  Each wait of the
 // barrier is bounded: when it runs out the block sets *kerr and ends.
-// Taken up to kLoopRows rows: beyond, the staged aprod 1 and the dynamic unit
-// queue of the separate launches win.
+//
+// Where it is taken: beyond some size the staged aprod 1, the dynamic unit
+// queue and the wider vector pass of the separate launches win.  us an
+// iteration, loop / launches, 5 to 400 rows a star: 50,000 rows 33 to 45 / 38
+// to 49; 100,000 rows 46 to 63 / 48 to 55; 200,000 rows 62 to 97 / 60 to 72;
+// 400,000 rows 102 to 165 / 83 to 111.  Columns cost more here (mostly empty
+// stars, 20,000 rows): 25,661 columns 26.9 / 34.3, 100,661 columns 44.6 / 42.5,
+// 500,661 columns 132 / 60.  So do offsets cut into pieces, whose sums one
+// thread adds: 20,000 rows on one offset (40 pieces) 49 / 49, on five (8
+// pieces) 36 / 43.  Up to 3,072 instruments change nothing.
 // ---------------------------------------------------------------------------
 constexpr int kLoopThreads = 512;
-constexpr int64_t kLoopRows = 400000;
+constexpr int64_t kLoopRows = 75000, kLoopCols = 60000, kLoopPieces = 16;
 
 struct LoopArgs {
     double *u, *q, *S, *ipart, *gpart;
@@ -1940,7 +1948,8 @@ cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out, i
 
 bool lsqr_loop_fits(const gsr_handle_t *h)
 {
-    return h->sys.m <= kLoopRows && h->sys.I <= kSplitInstrMax && h->ipath == kIpSorted &&
+    return h->sys.m <= kLoopRows && h->sys.n <= kLoopCols && h->sys.attp <= kLoopPieces &&
+           h->sys.I <= kSplitInstrMax && h->ipath == kIpSorted &&
            h->a2_fused && h->cfg.products == GSR_PRODUCTS_AUTO && h->drop_tile < 0 &&
            h->nsm <= kMaxPartials;
 }

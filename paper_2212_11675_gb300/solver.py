@@ -205,6 +205,12 @@ class Solver:
         check(lib().gsr_aprod1_staging(self._h, ctypes.byref(v)), "gsr_aprod1_staging")
         return bool(v.value)
 
+    def lsqr_one_launch(self):
+        """True when lsqr_solve runs its iterations in one kernel launch."""
+        v = ctypes.c_int()
+        check(lib().gsr_lsqr_one_launch(self._h, ctypes.byref(v)), "gsr_lsqr_one_launch")
+        return bool(v.value)
+
     def kernel_status(self, stream=None):
         """Raw status of the bounded device waits since the last check
         (GSR_OK or GSR_ERR_TIMEOUT; the flag is cleared)."""

@@ -204,7 +204,10 @@ int gsr_precondition(void *h, double *p, void *stream);
  * outputs (se may be NULL).  atol, btol >= 0 are the tolerances of rules S1
  * and S2 (0 disables them); the condition limit is the handle's conlim.
  * The whole iteration runs on the device (one CUDA graph, no host
- * synchronisation until the end).  `out` receives the stopping estimates.
+ * synchronisation until the end).  A small system's iterations are one
+ * kernel that needs every SM (gsr_lsqr_one_launch); while work of another
+ * stream or thread holds one, the call runs them as launches on the others.
+ * `out` receives the stopping estimates.
  * Errors: GSR_ERR_ARG, GSR_ERR_NONFINITE (a NaN/Inf in b or in the scalar
  * recurrences; x and se are then undefined), GSR_ERR_TIMEOUT (a bounded
  * device wait expired; x and se are undefined), GSR_ERR_CUDA.

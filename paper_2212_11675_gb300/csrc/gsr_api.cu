@@ -118,6 +118,8 @@ static void release(gsr_handle_t *h)
     cudaSetDevice(h->device);
     if (h->solve_exec)
         cudaGraphExecDestroy(h->solve_exec);
+    if (h->launch_exec)
+        cudaGraphExecDestroy(h->launch_exec);
     if (h->cg_exec)
         cudaGraphExecDestroy(h->cg_exec);
     if (h->cg64_exec)
@@ -1054,12 +1056,27 @@ extern "C" int gsr_lsqr_solve(void *hv, const double *b, int itmax, double atol,
     } else {
         CK(cudaGraphLaunch(h->solve_exec, st));
     }
-    CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(SolveState), cudaMemcpyDeviceToHost, st));
-    if (dx != x)
-        CK(cudaMemcpyAsync(x, dx, h->sys.n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (se && dse != se)
-        CK(cudaMemcpyAsync(se, dse, h->sys.n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    auto results = [&]() -> int {
+        CK(cudaMemcpyAsync(h->h_state, h->d_state, sizeof(SolveState), cudaMemcpyDeviceToHost, st));
+        if (dx != x)
+            CK(cudaMemcpyAsync(x, dx, h->sys.n * sizeof(double), cudaMemcpyDeviceToHost, st));
+        if (se && dse != se)
+            CK(cudaMemcpyAsync(se, dse, h->sys.n * sizeof(double), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        return GSR_OK;
+    };
+    TRY(results());
+    if (h->h_state->left) {
+        // another kernel held an SM that the one-launch loop needs: the same
+        // solve as launches, which run on the SMs there are
+        if (!h->launch_exec) {
+            const cudaError_t e = build_launch_graph(h, &h->launch_exec);
+            if (e != cudaSuccess)
+                return cuda_fail(e, "build_launch_graph");
+        }
+        CK(cudaGraphLaunch(h->launch_exec, st));
+        TRY(results());
+    }
     TRY(take_kernel_status(h, st));
     const SolveState &s = *h->h_state;
     if (out) {
@@ -1439,46 +1456,16 @@ static int cm_buffers(gsr_handle_t *h, int k)
     return GSR_OK;
 }
 
-extern "C" int gsr_set_aprod2_fused(void *hv, int fused)
-{
-    gsr_handle_t *h = (gsr_handle_t *)hv;
-    if (!h || (fused != 0 && fused != 1))
-        return GSR_ERR_ARG;
-    if (h->ipath != kIpSorted)
-        return GSR_ERR_UNSUPPORTED;
-    if (h->a2_fused == fused)
-        return GSR_OK;
-    h->a2_fused = fused;
-    // the captured graphs hold the old launches: capture them again
-    if (h->solve_exec) {
-        cudaGraphExecDestroy(h->solve_exec);
-        h->solve_exec = nullptr;
-    }
-    if (h->cg64_exec) {
-        cudaGraphExecDestroy(h->cg64_exec);
-        h->cg64_exec = nullptr;
-    }
-    const bool mixed = h->cg_exec != nullptr;
-    if (h->cg_exec) {
-        cudaGraphExecDestroy(h->cg_exec);
-        h->cg_exec = nullptr;
-    }
-    cudaError_t e = build_solve_graph(h);
-    if (e == cudaSuccess)
-        e = build_cg64_graph(h);
-    if (e == cudaSuccess && mixed)
-        e = build_cg_graph(h);
-    if (e != cudaSuccess)
-        return cuda_fail(e, "gsr_set_aprod2_fused");
-    return GSR_OK;
-}
-
 // the captured graphs hold the old launches: capture them again
 static int recapture_graphs(gsr_handle_t *h, const char *what)
 {
     if (h->solve_exec) {
         cudaGraphExecDestroy(h->solve_exec);
         h->solve_exec = nullptr;
+    }
+    if (h->launch_exec) {
+        cudaGraphExecDestroy(h->launch_exec);
+        h->launch_exec = nullptr;
     }
     if (h->cg64_exec) {
         cudaGraphExecDestroy(h->cg64_exec);
@@ -1497,6 +1484,19 @@ static int recapture_graphs(gsr_handle_t *h, const char *what)
     if (e != cudaSuccess)
         return cuda_fail(e, what);
     return GSR_OK;
+}
+
+extern "C" int gsr_set_aprod2_fused(void *hv, int fused)
+{
+    gsr_handle_t *h = (gsr_handle_t *)hv;
+    if (!h || (fused != 0 && fused != 1))
+        return GSR_ERR_ARG;
+    if (h->ipath != kIpSorted)
+        return GSR_ERR_UNSUPPORTED;
+    if (h->a2_fused == fused)
+        return GSR_OK;
+    h->a2_fused = fused;
+    return recapture_graphs(h, "gsr_set_aprod2_fused");
 }
 
 extern "C" int gsr_set_aprod1_staging(void *hv, int staged)

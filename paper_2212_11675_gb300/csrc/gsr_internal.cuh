@@ -208,6 +208,7 @@ struct SolveState {
     double irho;               // 1/rho of the pending rotation
     double ia;                 // 1/alpha (1 if alpha = 0)
     int itn, istop, done, nonfinite;
+    int left;                  // k_lsqr_loop ended unstarted: not all of its blocks were resident
 };
 
 // Conjugate-gradient state of the mixed-precision inner solve.
@@ -367,6 +368,7 @@ struct gsr_handle_t {
     int64_t device_bytes = 0;
     // CUDA graph of one whole solve
     cudaGraphExec_t solve_exec = nullptr;
+    cudaGraphExec_t launch_exec = nullptr;  // the solve as launches, once solve_exec's loop has left
     cudaStream_t cap_stream = nullptr;
     int grid_rows = 0, grid_rows2 = 0, grid_vec = 0, grid_att = 0, grid_ins = 0;
     int grid_lsqr_vec = 0;              // the LSQR vector pass: every resident block
@@ -454,6 +456,7 @@ bool lsqr_loop_fits(const gsr_handle_t *h);
 [[nodiscard]] cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st);
 // LSQR pieces (gsr_lsqr.cu)
 [[nodiscard]] cudaError_t build_solve_graph(gsr_handle_t *h);
+[[nodiscard]] cudaError_t build_launch_graph(gsr_handle_t *h, cudaGraphExec_t *exec);
 [[nodiscard]] cudaError_t enqueue_prologue(const gsr_handle_t *h, cudaStream_t s,
                                            cudaGraphConditionalHandle loop, int in_graph);
 [[nodiscard]] cudaError_t enqueue_iteration(const gsr_handle_t *h, cudaStream_t s,

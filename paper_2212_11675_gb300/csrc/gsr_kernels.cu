@@ -1319,8 +1319,7 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 }
 
 // ---------------------------------------------------------------------------
-// All LSQR iterations of a small system in one launch (cooperative: every
-// block is resident).  An iteration as three launches costs about 35 us on
+// All LSQR iterations of a small system in one launch.  An iteration as three launches costs about 35 us on
 // the 1,000-star system however little work it has: three launch ramps, three
 // grid reductions whose last block works alone.  Here its three parts are
 // separated by barriers of the grid, and every block works out the sums of
@@ -1335,6 +1334,16 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // the next iteration (which changes only U, so it may be one too many).
 // Data that other blocks write is read from L2 (ld_shared).  Each wait of the
 // barrier is bounded: when it runs out the block sets *kerr and ends.
+//
+// A block takes a whole SM (its registers), so another stream's kernel on any
+// SM keeps the grid from being resident.  A cooperative launch then waits for
+// that kernel to end (beside a kernel of one block and 1.5 s the solve took
+// 1.45 s; as launches 2.8 ms on the other SMs).  This one is an ordinary
+// launch whose first barrier (loop_join) settles whether all blocks are
+// there: if they are not within kJoinNs, every block ends, the state says so
+// (left) and the host runs the solve as launches.  Up to there only U was
+// written, which a solve starts anew.  After it all blocks are resident, and
+// resident blocks run to their end.
 //
 // Where it is taken: beyond some size the staged aprod 1, the dynamic unit
 // queue and the wider vector pass of the separate launches win.  us an
@@ -1389,6 +1398,44 @@ __device__ __forceinline__ bool loop_sync(unsigned *bar, unsigned &target, int *
         }
         __threadfence();
         s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// The first barrier: true when every block has come.  A block that has waited
+// kJoinNs closes the barrier (kLoopLeft) unless the last one comes first; the
+// count and that bit are one word, so all blocks agree, also those that start
+// later.
+constexpr unsigned kLoopLeft = 0x80000000u;
+constexpr uint64_t kJoinNs = 500000;  // 0.5 ms
+
+__device__ __forceinline__ bool loop_join(unsigned *bar, unsigned &target, SolveState *st)
+{
+    __shared__ int s_ok;
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        unsigned c = atomicAdd(bar, 1u) + 1u;
+        const uint64_t t0 = global_ns();
+        // a failed exchange means that another block has come or left, so there
+        // are at most gridDim.x of them
+        for (int it = 1; !(c & kLoopLeft) && c < target; it++) {
+            if ((it & 15) == 0 && global_ns() - t0 > kJoinNs) {
+                const unsigned seen = atomicCAS(bar, c, c | kLoopLeft);
+                if (seen == c) {
+                    st->left = 1;
+                    c |= kLoopLeft;
+                } else {
+                    c = seen;
+                }
+            } else {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(bar) : "memory");
+            }
+        }
+        __threadfence();
+        s_ok = !(c & kLoopLeft);
     }
     __syncthreads();
     return s_ok != 0;
@@ -1492,7 +1539,7 @@ k_lsqr_loop(SysView A, LoopArgs L)
             }
         }
         loop_part<1>(nrm, gw < ntiles, L.partial);
-        if (!loop_sync(L.bar, target, L.kerr))
+        if (!(target == 0 ? loop_join(L.bar, target, L.st) : loop_sync(L.bar, target, L.kerr)))
             return;
         if (s.done)  // by the recurrences of the iteration before
             break;
@@ -1962,8 +2009,6 @@ static cudaError_t loop_launch(const gsr_handle_t *h, cudaStream_t st)
                   h->d_cseg, h->d_irow, h->d_ival, h->isplit,
                   (h->sys.S + 32 / G - 1) / (32 / G), h->sys.I * h->isplit,
                   h->d_state, h->d_args, h->d_partial, h->d_bar, h->d_kerr};
-    SysView A = h->sys;
-    void *args[] = {&A, &L};
     // beside the kernel's static shared memory, the pieces of kSplitInstrMax
     // instruments exceed the 48 KB that a launch may have without asking; the
     // attribute belongs to the kernel: the most that any handle asks for
@@ -1971,10 +2016,10 @@ static cudaError_t loop_launch(const gsr_handle_t *h, cudaStream_t st)
                                          (int)(kSplitInstrMax * sizeof(float4)));
     if (e == cudaSuccess)
         e = cudaMemsetAsync(h->d_bar, 0, sizeof(unsigned), st);
-    if (e == cudaSuccess)
-        e = cudaLaunchCooperativeKernel(k_lsqr_loop<G>, dim3(h->nsm), dim3(kLoopThreads), args,
-                                        (size_t)A.I * sizeof(float4), st);
-    return e;
+    if (e != cudaSuccess)
+        return e;
+    k_lsqr_loop<G><<<h->nsm, kLoopThreads, (size_t)h->sys.I * sizeof(float4), st>>>(h->sys, L);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_lsqr_loop(const gsr_handle_t *h, cudaStream_t st)

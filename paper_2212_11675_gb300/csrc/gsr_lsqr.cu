@@ -377,12 +377,25 @@ cudaError_t enqueue_epilogue(const gsr_handle_t *h, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// an unfinished capture on s and the graph g are given up
+static void drop_capture(cudaStream_t s, cudaGraph_t g)
+{
+    cudaStreamCaptureStatus cs;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
+        cudaGraph_t junk = nullptr;
+        cudaStreamEndCapture(s, &junk);
+        if (junk && junk != g)
+            cudaGraphDestroy(junk);
+    }
+    if (g)
+        cudaGraphDestroy(g);
+    cudaGetLastError();
+}
+
 // Build and instantiate the graph of one whole solve:
 //   [precondition, U_1 = b, q = A^T U_1, V_1]  ->  WHILE(flag) { iteration }
 //   ->  [x = p o z, se]
-// or, for a small system, with one launch for all iterations in place of the
-// loop (k_lsqr_loop).
-cudaError_t build_solve_graph(gsr_handle_t *h)
+cudaError_t build_launch_graph(gsr_handle_t *h, cudaGraphExec_t *exec)
 {
     cudaError_t err = cudaSuccess;
     cudaGraph_t g = nullptr;
@@ -393,18 +406,6 @@ cudaError_t build_solve_graph(gsr_handle_t *h)
     cudaStream_t s = h->cap_stream;
 
     GSR_TRY(cudaGraphCreate(&g, 0));
-    if (lsqr_loop_fits(h)) {
-        // a small system: all iterations in one launch
-        GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0,
-                                              cudaStreamCaptureModeThreadLocal));
-        GSR_TRY(enqueue_prologue(h, s, 0, 0));
-        GSR_TRY(launch_lsqr_loop(h, s));
-        GSR_TRY(enqueue_epilogue(h, s));
-        GSR_TRY(cudaStreamEndCapture(s, &g));
-        GSR_TRY(cudaGraphInstantiate(&h->solve_exec, g, 0));
-        cudaGraphDestroy(g);
-        return cudaSuccess;
-    }
     GSR_TRY(cudaGraphConditionalHandleCreate(&loop, g, 1u, cudaGraphCondAssignDefault));
 
     GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
@@ -427,22 +428,34 @@ cudaError_t build_solve_graph(gsr_handle_t *h)
     GSR_TRY(enqueue_epilogue(h, s));
     GSR_TRY(cudaStreamEndCapture(s, &g));
 
+    GSR_TRY(cudaGraphInstantiate(exec, g, 0));
+    cudaGraphDestroy(g);
+    return cudaSuccess;
+fail:
+    drop_capture(s, g);
+    return err;
+}
+
+// ... or, for a small system, with one launch for all iterations in place of
+// the loop (k_lsqr_loop)
+cudaError_t build_solve_graph(gsr_handle_t *h)
+{
+    if (!lsqr_loop_fits(h))
+        return build_launch_graph(h, &h->solve_exec);
+    cudaError_t err = cudaSuccess;
+    cudaGraph_t g = nullptr;
+    cudaStream_t s = h->cap_stream;
+    GSR_TRY(cudaGraphCreate(&g, 0));
+    GSR_TRY(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    GSR_TRY(enqueue_prologue(h, s, 0, 0));
+    GSR_TRY(launch_lsqr_loop(h, s));
+    GSR_TRY(enqueue_epilogue(h, s));
+    GSR_TRY(cudaStreamEndCapture(s, &g));
     GSR_TRY(cudaGraphInstantiate(&h->solve_exec, g, 0));
     cudaGraphDestroy(g);
     return cudaSuccess;
 fail:
-    {
-        cudaStreamCaptureStatus cs;
-        if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
-            cudaGraph_t junk = nullptr;
-            cudaStreamEndCapture(s, &junk);
-            if (junk && junk != g)
-                cudaGraphDestroy(junk);
-        }
-    }
-    if (g)
-        cudaGraphDestroy(g);
-    cudaGetLastError();
+    drop_capture(s, g);
     return err;
 }
 

@@ -1,5 +1,9 @@
 """The one-launch LSQR loop of small systems: the shared memory of its
-instrumental x at the limits of its sizes, and the systems it is taken for."""
+instrumental x at the limits of its sizes, the systems it is taken for, and
+solves beside other work on the GPU."""
+import threading
+import time
+
 import numpy as np
 import pytest
 
@@ -54,3 +58,60 @@ def test_where_the_loop_is_taken(shape, empty, one):
         assert np.linalg.norm(x.cpu().numpy() - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
         np.testing.assert_allclose(se.cpu().numpy(), ref["se"], rtol=1e-9)
         assert s.kernel_status() == _lib.GSR_OK
+
+
+def test_solve_beside_a_kernel_that_holds_an_sm():
+    # one block of another stream for about 1.2 s: the loop cannot be resident,
+    # the solve goes on without it on the other SMs
+    sys = _random(257, 20, 37, 11, seed=9)
+    b = oracle.aprod1(sys, gen.x_true(sys, 3)) + gen.noise(sys, 4)
+    ref = oracle.pc_lsqr(sys, b, 12, 0.0, 0.0)
+    bd = torch.tensor(b, device=DEV)
+    other = torch.cuda.Stream()
+    with _solver(sys) as s:
+        assert s.lsqr_one_launch()
+        s.lsqr_solve(bd, 12, 0.0, 0.0)
+        for _ in range(2):
+            with torch.cuda.stream(other):
+                torch.cuda._sleep(int(2.4e9))
+                done = torch.cuda.Event()
+                done.record()
+            time.sleep(0.01)
+            x, se, res = s.lsqr_solve(bd, 12, 0.0, 0.0)
+            assert not done.query(), "the solve waited for the other stream"
+            assert res["itn"] == ref["itn"]
+            assert np.linalg.norm(x.cpu().numpy() - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
+            np.testing.assert_allclose(se.cpu().numpy(), ref["se"], rtol=1e-9)
+            assert s.kernel_status() == _lib.GSR_OK
+            other.synchronize()
+        x2, _, _ = s.lsqr_solve(bd, 12, 0.0, 0.0)  # by the loop again
+    assert np.linalg.norm(x2.cpu().numpy() - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
+
+
+def test_two_handles_from_two_threads():
+    systems = [_random(257, 20, 37, 11, seed=9), _random(301, 25, 60, 30, seed=10)]
+    refs, bs = [], []
+    for sys in systems:
+        bs.append(oracle.aprod1(sys, gen.x_true(sys, 3)) + gen.noise(sys, 4))
+        refs.append(oracle.pc_lsqr(sys, bs[-1], 12, 0.0, 0.0)["x"])
+    errors = []
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream), _solver(systems[i]) as s:
+                bd = torch.tensor(bs[i], device=DEV)
+                for _ in range(30):
+                    x, _, _ = s.lsqr_solve(bd, 12, 0.0, 0.0)
+                    e = np.linalg.norm(x.cpu().numpy() - refs[i]) / np.linalg.norm(refs[i])
+                    if not e <= 1e-9:
+                        errors.append((i, e))
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append((i, repr(e)))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:3]

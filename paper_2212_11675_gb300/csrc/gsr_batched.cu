@@ -169,7 +169,12 @@ constexpr int kBA2 = 2;  // attitude and global part of A32^T Q
 // the warp.  They read the values from the tile's stage and the rows of Q
 // through shared memory, two rows per packed operation (even and odd rows are
 // two chains); the lanes of different taps start 8 rows apart, so that they
-// read different banks.
+// read different banks.  A chain ends with its tile, after 16 terms, and the
+// tiles of a unit are added in three words: a lane per row had chains of a
+// thirty-second of the offset's rows and a tree over the lanes (rms error in
+// units of the sum of |terms|, 50 / 200 / 350 / 1,000 rows an offset: 3.9 / 4.9
+// / 5.5 / 8.6e-18; now 2.7 / 2.5 / 1.9 / 0.7e-18; one chain over the unit had
+// 9.8 / 43 / 26 / 23e-18).
 // Bound by the FP32 pipe: 8 lane operations per product, 37 products a row
 // and column (0.47 ms at 7.0e6 rows and 8 columns with all lanes busy; 0.69
 // measured, the pipe 62 % active, against 0.76 + 0.39 ms for the two products
@@ -238,7 +243,7 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
 #pragma unroll
     for (int c = 0; c < N; c++)
         nh[c] = nl[c] = gh[c] = gl[c] = V(0);
-    f32x2 sh[NI], sl[NI];  // this lane's attitude sums, even and odd rows
+    Df3<f32x2> su[NI];  // this lane's attitude sums of the unit, even and odd rows
     bool ok = walk.d[0].ok && walk.arrived(0, kerr);
     while (ok) {
         const Visit v = walk.d[0];
@@ -253,7 +258,7 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
             }
 #pragma unroll
             for (int i = 0; i < NI; i++)
-                sh[i] = sl[i] = 0ull;
+                su[i].hi = su[i].lo = su[i].c = 0ull;
         }
         const uint32_t e = (v.t << 5) + lane;
         const float *val = walk.val();  // plane k of the tile at val + 32 k
@@ -329,21 +334,29 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
             for (int c = 0; c < KT; c++)
                 W.q[c][lane] = col_of<KT>(h, c);
             __syncwarp();
+            f32x2 sh[NI], sl[NI];  // of the tile
+#pragma unroll
+            for (int i = 0; i < NI; i++)
+                sh[i] = sl[i] = 0ull;
             const uint32_t b = v.t << 5;
             if (v.un.y <= b && v.un.z >= b + 32)
                 b_att_tile<KT, NI, true>(val, W, lane, 0, 32, sh, sl);
             else
                 b_att_tile<KT, NI, false>(val, W, lane, (int)(max(v.un.y, b) - b),
                                           (int)(min(v.un.z, b + 32) - b), sh, sl);
+#pragma unroll
+            for (int i = 0; i < NI; i++)
+                su[i].add(sh[i], sl[i]);
             if (v.last()) {
 #pragma unroll
                 for (int i = 0; i < NI; i++) {
-                    float h0, h1, l0, l1;
-                    unpack2(sh[i], h0, h1);
-                    unpack2(sl[i], l0, l1);
-                    df_add(h0, l0, h1, l1);
+                    float h0, h1, l0, l1, c0, c1;
+                    unpack2(su[i].hi, h0, h1);
+                    unpack2(su[i].lo, l0, l1);
+                    unpack2(su[i].c, c0, c1);
                     if (lane + 32 * i < NOUT)
-                        S[(int64_t)v.un.w * NOUT + lane + 32 * i] = df_to_d(h0, l0);
+                        S[(int64_t)v.un.w * NOUT + lane + 32 * i] =
+                            df_to_d(h0, h1) + (df_to_d(l0, l1) + df_to_d(c0, c1));
                 }
             }
         }
@@ -387,7 +400,12 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
 // G lanes own a star: KT / 2 lanes take a pair of columns each of one row, G
 // over that many rows at a time.  A lane holds five packed sums, so that
 // enough warps and rows are in flight (with a whole row of 8 columns per lane:
-// 144 registers, 8 warps per SM, 276 us at 7.0e6 rows).
+// 144 registers, 8 warps per SM, 276 us at 7.0e6 rows).  The chain of a lane
+// is KT / 2 times as long as with a row per lane; its low word is renormalised
+// at each addition (df_acc_norm), which keeps the error of the shorter chains
+// (rms in units of the sum of |terms|, 8 columns on 16 lanes, 70 / 200 / 400
+// rows a star: 3.6 / 5.7 / 6.4e-18, a row per lane 3.7 / 5.7 / 7.1e-18, without
+// it 6.2 / 15 / 29e-18).
 // ---------------------------------------------------------------------------
 template <int KT, int G>
 __global__ void __launch_bounds__(kThreads, 4)
@@ -426,7 +444,10 @@ k_b_stars(SysView A, const float *__restrict__ sv, const float *__restrict__ Y,
             for (int k = 0; k < kNAstro; k++) {
                 V a;
                 v_bcast(a, __ldcs(v + 32 * k));
-                df_acc_v(h[k], l[k], v_mul(a, yv[0]));
+                if constexpr (CL > 1)
+                    df_acc_norm(h[k], l[k], v_mul(a, yv[0]));
+                else
+                    df_acc_v(h[k], l[k], v_mul(a, yv[0]));
             }
         }
         // over the RS rows in double-float; slot q writes sums q, q + RS, ...
@@ -858,12 +879,13 @@ static int b_occ(F f)
     return occ;
 }
 
-// pieces per instrument: about 2048 entries each
+// pieces per instrument: about 2048 entries each, four at least (an instrument
+// that many rows use gives four warps work, and the chains of sums stay short)
 int batched_instr_pieces(const gsr_handle_t *h)
 {
     const int64_t mean = kNInstr * h->sys.m / h->sys.I;
     const int64_t np = (mean + 2047) / 2048;
-    return (int)(np < 1 ? 1 : (np > 256 ? 256 : np));
+    return (int)(np < 4 ? 4 : (np > 256 ? 256 : np));
 }
 
 template <int KT, int MODE>

@@ -73,16 +73,51 @@ __device__ __forceinline__ f32x2 v_fma(f32x2 a, f32x2 b, f32x2 c)
 }
 __device__ __forceinline__ f32x2 v_neg(f32x2 a) { return a ^ 0x8000000080000000ull; }
 
+// a + p = (a, err) exactly (Knuth's TwoSum), on one value or on a packed pair
+template <typename V>
+__device__ __forceinline__ void two_sum_v(V &a, V &err, V p)
+{
+    const V s = v_add(a, p);
+    const V bp = v_sub(s, a);
+    err = v_add(v_sub(a, v_sub(s, bp)), v_sub(p, bp));
+    a = s;
+}
+
 // df_acc on one value or on a packed pair of independent accumulators
 template <typename V>
 __device__ __forceinline__ void df_acc_v(V &hi, V &lo, V p)
 {
-    const V s = v_add(hi, p);
-    const V bp = v_sub(s, hi);
-    const V err = v_add(v_sub(hi, v_sub(s, bp)), v_sub(p, bp));
-    hi = s;
+    V err;
+    two_sum_v(hi, err, p);
     lo = v_add(lo, err);
 }
+
+// ... with hi and lo renormalised after each addition (Fast2Sum), so that the
+// roundings of lo stay relative to the last place of hi however long the chain
+// is: three operations more, and chains four times as long are as accurate.
+template <typename V>
+__device__ __forceinline__ void df_acc_norm(V &hi, V &lo, V p)
+{
+    df_acc_v(hi, lo, p);
+    const V s = v_add(hi, lo);
+    lo = v_sub(lo, v_sub(s, hi));
+    hi = s;
+}
+
+// Sum of double-float chains in three words: hi + lo + c takes (ph, pl) with
+// error-free sums, only c rounds (in its own, third, place).
+template <typename V>
+struct Df3 {
+    V hi, lo, c;
+    __device__ __forceinline__ void add(V ph, V pl)
+    {
+        V e, g, f;
+        two_sum_v(hi, e, ph);
+        two_sum_v(lo, g, pl);
+        two_sum_v(lo, f, e);
+        c = v_add(c, v_add(g, f));
+    }
+};
 
 // Sum of two double-float numbers (ah + al) + (bh + bl), Joldes, Muller &
 // Popescu, "Tight and rigorous error bounds for basic building blocks of

@@ -201,6 +201,8 @@ static int finish_instr(gsr_handle_t *h, const std::vector<uint32_t> &cseg, int6
 // columns of every window and the place of every entry are worked out on the
 // host, window by window, the values gathered on the device; the
 // instrument-sorted copy (FP64 aprod 2, batched form) is written from them.
+// kEllTooMany, with nothing allocated, where the sums of a block do not fit.
+constexpr int kEllTooMany = 1;
 static int build_ell(gsr_handle_t *h, cudaStream_t st)
 {
     SysView &A = h->sys;
@@ -330,6 +332,12 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
             s0[f + 1] = s0[f] + nchunk[b * I + f];
         nacc = std::max<int64_t>(nacc, s0[I]);
     }
+    // A block's sums are, instrument by instrument, the most columns that any
+    // one of its windows has: I + 6 W / L at most for one window, more where its
+    // windows use different instruments heavily.  Beyond the shared memory they
+    // may take the sorted copy's units serve.
+    if (nacc > kEllAccMax)
+        return kEllTooMany;
     seg[0] = 0;
     for (int64_t f = 0; f < I; f++)
         seg[f + 1] = seg[f] + rank[f];
@@ -385,12 +393,8 @@ static int build_ell(gsr_handle_t *h, cudaStream_t st)
     cudaFree(d_tmp);
     if (e != cudaSuccess)
         return cuda_fail(e, "instrument windows");
-    // (nacc is at most I + 6 W / L, below kEllAccMax, unless the instruments are
-    // used very unevenly: the sorted copy's units serve then)
-    h->ell_on = nacc <= kEllAccMax;
-    if (!h->ell_on)
-        h->ks32 = (int)((kNInstr * m / I + 4095) / 4096);
-    return finish_instr(h, cseg, nq, std::max<int64_t>(nq, h->ks32));
+    h->ell_on = true;
+    return finish_instr(h, cseg, nq, nq);
 }
 
 // Instrument-sorted copy of the instrumental nonzeros: a stable counting
@@ -757,9 +761,14 @@ static int create_impl(gsr_handle_t *h, const gsr_dims *d, const uint32_t *star_
 
     // instrumental part of aprod 2 and its layout
     h->ipath = instr_path(h->cfg, I);
-    if (h->ipath == kIpSorted || h->cfg.precision == GSR_PREC_MIXED)
-        TRY(h->cfg.precision == GSR_PREC_MIXED && I <= kEllInstrMax ? build_ell(h, st)
-                                                                    : build_instr_sorted(h, st));
+    if (h->ipath == kIpSorted || h->cfg.precision == GSR_PREC_MIXED) {
+        rc = kEllTooMany;
+        if (h->cfg.precision == GSR_PREC_MIXED && I <= kEllInstrMax)
+            rc = build_ell(h, st);
+        if (rc == kEllTooMany)
+            rc = build_instr_sorted(h, st);
+        TRY(rc);
+    }
 
     // launch geometry
     // measured at the medium size (70 rows a star): 8 lanes per star with

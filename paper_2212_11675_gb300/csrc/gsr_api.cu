@@ -544,6 +544,19 @@ static int build_units(gsr_handle_t *h)
     return GSR_OK;
 }
 
+// ||A diag(p)||_F^2 = number of nonempty columns (column sums of squares > 0)
+static int count_nonempty(gsr_handle_t *h, cudaStream_t st)
+{
+    CK(cudaMemsetAsync(h->d_s, 0, h->sys.n * sizeof(double), st));
+    CK(launch_aprod2(h, nullptr, h->d_s, kA2Squares, st));
+    CK(launch_count_pos(h, h->d_s, h->d_onorm, st));
+    CK(cudaMemcpyAsync(h->h_onorm, h->d_onorm, sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    h->n_nonempty = h->h_onorm[0];
+    h->nonempty_stale = false;
+    return GSR_OK;
+}
+
 // the binary32 copies of the values, the mixed-precision workspace and the
 // inner CG graph
 static int create_mixed(gsr_handle_t *h, cudaStream_t st)
@@ -566,13 +579,7 @@ static int create_mixed(gsr_handle_t *h, cudaStream_t st)
         TRY(dalloc(h, &h->d_ival32, kNInstr * m));
         CK(launch_to_f32(h, h->d_ival, h->d_ival32, kNInstr * m, st));
     }
-    // ||A diag(p)||_F^2 = number of nonempty columns (column sums of squares > 0)
-    CK(cudaMemsetAsync(h->d_s, 0, n * sizeof(double), st));
-    CK(launch_aprod2(h, nullptr, h->d_s, kA2Squares, st));
-    CK(launch_count_pos(h, h->d_s, h->d_onorm, st));
-    CK(cudaMemcpyAsync(h->h_onorm, h->d_onorm, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    h->n_nonempty = h->h_onorm[0];
+    TRY(count_nonempty(h, st));
     h->grid_main32 = f32_main_grid(h);
     h->grid_rest32 = f32_rest_grid(h);
     if (h->grid_main32 <= 0 || h->grid_rest32 <= 0)
@@ -1223,6 +1230,8 @@ extern "C" int gsr_mixed_solve(void *hv, const double *b, int max_outer, int max
     h->h_cgargs->max_inner = max_inner;
     h->h_cgargs->tol = inner_tol;
     CK(cudaMemcpyAsync(h->d_cgargs, h->h_cgargs, sizeof(CgArgs), cudaMemcpyHostToDevice, st));
+    if (h->nonempty_stale)
+        TRY(count_nonempty(h, st));
     const double anorm = sqrt(h->n_nonempty);
     gsr_mixed_result res = {};
     res.anorm = anorm;
@@ -1291,8 +1300,10 @@ extern "C" int gsr_set_values(void *hv, int k, const double *values, void *strea
         if (h->ell_on)
             CK(launch_ell_plane(h, slot, st));
     }
-    if (h->cfg.precision == GSR_PREC_MIXED)
+    if (h->cfg.precision == GSR_PREC_MIXED) {
         CK(launch_f32_plane(h, k, st));
+        h->nonempty_stale = true;
+    }
     if (dv != values)
         CK(cudaStreamSynchronize(st));
     return GSR_OK;
@@ -1631,6 +1642,8 @@ extern "C" int gsr_batched_solve(void *hv, int k, const double *B, int max_outer
     h->h_bargs->max_inner = max_inner;
     h->h_bargs->tol = inner_tol;
     CK(cudaMemcpyAsync(h->d_bargs, h->h_bargs, sizeof(BatchArgs), cudaMemcpyHostToDevice, st));
+    if (h->nonempty_stale)
+        TRY(count_nonempty(h, st));
     const double anorm = sqrt(h->n_nonempty);
     std::vector<gsr_mixed_result> res((size_t)k);
     for (int c = 0; c < k; c++)

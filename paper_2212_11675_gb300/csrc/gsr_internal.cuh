@@ -352,7 +352,8 @@ struct gsr_handle_t {
     int b_kt = 8, b_lanes = 16, b_graph_kt = 0, b_graph_lanes = 0;  // the graphs' tiling
     double *d_xp64 = nullptr, *d_q64 = nullptr;
     int grid_main32 = 0, grid_rest32 = 0;
-    double n_nonempty = 0.0;
+    double n_nonempty = 0.0;            // columns with a nonzero
+    bool nonempty_stale = false;        // a plane was replaced since they were counted
     double *d_p = nullptr;              // preconditioner
     double *d_u = nullptr;              // m
     double *d_v = nullptr, *d_w = nullptr, *d_z = nullptr, *d_var = nullptr;

@@ -77,3 +77,18 @@ def test_solves_after_replacing_an_instrument_plane():
               s.batched_solve(_dev(b[None]), 20, 300, 1e-5, 1e-13)[0][0]]
     for x in xs:
         assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-9 * np.linalg.norm(ref)
+
+
+def test_norm_of_the_scaled_matrix_after_emptying_a_plane():
+    # anorm^2 is the number of nonempty columns: zeros in plane 0 empty one
+    # column a star, in plane 23 the global one
+    sys = _random(40, 12, 10, 9, seed=3)
+    b = np.random.default_rng(5).standard_normal(sys.m)
+    with _solver(sys, precision=_lib.GSR_PREC_MIXED, conlim=0.0) as s:
+        for planes, empty in (((), 0), ((0,), 40), ((23,), 41)):
+            for k in planes:
+                s.set_values(k, np.zeros(sys.m))
+            for res in (s.mixed_solve(_dev(b), 1, 1)[1], s.batched_solve(_dev(b[None]), 1, 1)[1][0]):
+                assert res["anorm"] == np.sqrt(sys.n - empty)
+        s.set_values(0, sys.values[:, 0].copy())
+        assert s.mixed_solve(_dev(b), 1, 1)[1]["anorm"] == np.sqrt(sys.n - 1)

@@ -236,9 +236,8 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
     const float *Xp = X + pidx(0, A.n, c0);  // row j of the panel at Xp + 8 j
     float *Qp = Q + pidx(0, A.m, c0);
     double *S = Sall + (int64_t)c0 * U.nunits * kNAtt;
-    const int64_t stride = (int64_t)gridDim.x * kBWarps;
-    int64_t u = blockIdx.x + (int64_t)gridDim.x * wib;
-    AttWalk<kBStages> walk(U, W.stage, W.bar, u, stride);
+    AttWalk<kBStages> walk(U, W.stage, W.bar, blockIdx.x + (int64_t)gridDim.x * wib,
+                           (int64_t)gridDim.x * kBWarps);
     V nh[N], nl[N], gh[N], gl[N];  // |Q[:, c]|^2 and the global sums of this thread
 #pragma unroll
     for (int c = 0; c < N; c++)
@@ -360,8 +359,6 @@ k_b_main(SysView A, Att32 U, const float *__restrict__ X, float *__restrict__ Q,
                 }
             }
         }
-        if (v.last())
-            u += stride;
         if (!walk.d[1].ok)
             break;
         walk.advance();

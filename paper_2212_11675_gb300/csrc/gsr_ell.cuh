@@ -117,24 +117,22 @@ struct EllShared {
     volatile int fail;
 };
 
-// Two shared-memory buffers of a window of y: the window after next is copied
-// while the next is used.  One bulk copy per window where y is 16-byte
-// aligned, plain loads otherwise.
-template <typename T>
+// Two shared-memory buffers of a window of y (16-byte aligned, W a multiple of
+// 32): the next window is copied while the current one is used.
 struct EllWindows {
-    T *buf;  // 2 kEllRows
+    float *buf;  // 2 kEllRows
     EllShared *sh;
     uint32_t bar;
-    const T *y;
+    const float *y;
     int64_t m, W;
-    bool bulk;
     uint32_t phase = 0;
 
     __device__ __forceinline__ int rows(int64_t w) const
     {
         return (int)(m - w * W < W ? m - w * W : W);
     }
-    __device__ __forceinline__ void init(T *b, EllShared *sh_, const T *y_, int64_t m_, int64_t W_)
+    __device__ __forceinline__ void init(float *b, EllShared *sh_, const float *y_, int64_t m_,
+                                         int64_t W_)
     {
         buf = b;
         sh = sh_;
@@ -142,9 +140,8 @@ struct EllWindows {
         y = y_;
         m = m_;
         W = W_;
-        bulk = ((uintptr_t)y & 15u) == 0;
         if (threadIdx.x == 0) {
-            buf[kEllPad] = buf[kEllRows + kEllPad] = T(0);
+            buf[kEllPad] = buf[kEllRows + kEllPad] = 0.f;
             sh->fail = 0;
             mbar_init(bar);
             mbar_init(bar + 8);
@@ -153,18 +150,16 @@ struct EllWindows {
         ell_sync();
     }
     // start the copy of window w into buffer b (the tail of a ragged window
-    // that no 16 bytes cover is stored by the thread itself)
+    // that no 16 bytes cover is stored by the threads)
     __device__ __forceinline__ void fetch(int64_t w, int b)
     {
-        const int nr = rows(w);
-        T *d = buf + b * kEllRows;
-        const T *src = y + w * W;
-        constexpr int Q = 16 / sizeof(T);
-        const int whole = bulk ? nr / Q * Q : 0;
+        const int nr = rows(w), whole = nr / 4 * 4;
+        float *d = buf + b * kEllRows;
+        const float *src = y + w * W;
         if (threadIdx.x == 0 && whole) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            mbar_expect(bar + 8 * b, whole * sizeof(T));
-            bulk_copy(smem_addr(d), src, whole * sizeof(T), bar + 8 * b);
+            mbar_expect(bar + 8 * b, whole * sizeof(float));
+            bulk_copy(smem_addr(d), src, whole * sizeof(float), bar + 8 * b);
         }
         for (int i = whole + threadIdx.x; i < nr; i += kEllThreads)
             d[i] = __ldg(src + i);
@@ -172,7 +167,7 @@ struct EllWindows {
     // window w in buffer b is complete, for every thread; false on a timeout
     __device__ __forceinline__ bool wait(int64_t w, int b, int *kerr)
     {
-        if (bulk && rows(w) * sizeof(T) >= 16) {
+        if (rows(w) >= 4) {
             if (!mbar_wait(bar + 8 * b, (phase >> b) & 1u))
                 sh->fail = 1;
             phase ^= 1u << b;
@@ -188,11 +183,11 @@ struct EllWindows {
 
 // the windows of this block (w = blockIdx.x, + E.nblk, ...): use(w, window of
 // y) for each; called by the first kEllThreads threads
-template <typename T, typename Use>
-__device__ __forceinline__ void ell_windows(const Ell &E, const T *y, int64_t m, T *buf,
+template <typename Use>
+__device__ __forceinline__ void ell_windows(const Ell &E, const float *y, int64_t m, float *buf,
                                             EllShared *sh, int *kerr, Use use)
 {
-    EllWindows<T> win;
+    EllWindows win;
     int64_t w = blockIdx.x;
     win.init(buf, sh, y, m, E.W);
     int b = 0;
@@ -223,8 +218,7 @@ __device__ __forceinline__ void ell32_part(const Ell &E, const float *y, int64_t
         return;
     for (int i = threadIdx.x; i < E.nacc; i += kEllThreads)
         acc[i] = 0.0;
-    ell_windows<float>(E, y, m, reinterpret_cast<float *>(smem), sh, kerr,
-                       [&](int64_t w, const float *yw) {
+    ell_windows(E, y, m, reinterpret_cast<float *>(smem), sh, kerr, [&](int64_t w, const float *yw) {
         EllCursor cur(E, __ldg(E.win + w) + (threadIdx.x >> 5), __ldg(E.win + w + 1));
         f32x2 h[2] = {0ull, 0ull}, l[2] = {0ull, 0ull};
         EllRun a, b, c;

@@ -109,7 +109,6 @@ k_f32_main(SysView A, Att32 U, const float *__restrict__ x32, const float *__res
     float nh = 0.f, nl = 0.f;  // |q|^2 of this thread (double-float)
     float gh = 0.f, gl = 0.f;  // its global sum
     f32x2 sh[kNAtt / 2], sl[kNAtt / 2];  // attitude sums, taps k and k + 1 packed
-    int64_t u = blockIdx.x + (int64_t)gridDim.x * wib;
     // astrometric x of the row (one sector), or its q, one visit ahead
     f32x2 s01 = 0ull, s23 = 0ull;
     float s4 = 0.f, xt = 0.f;
@@ -221,7 +220,6 @@ k_f32_main(SysView A, Att32 U, const float *__restrict__ x32, const float *__res
                 if ((lane & 1) == 0 && kk < kNAtt)
                     S[(int64_t)v.un.w * kNAtt + kk] = df_to_d(rh[0], rl[0]);
             }
-            u += (int64_t)gridDim.x * kMainWarps;
         }
         if (!more || !ok)
             break;

@@ -425,16 +425,28 @@ int gsr_aprod1_staging(void *h, int *staged);
 int gsr_kernel_status(void *h, void *stream);
 
 /*
- * Test hook for the bounded waits of the staged aprod 1: tile >= 0 makes
- * every later launch on the handle announce tile's bulk copies to its
- * barrier without issuing them, so the wait of the warp that owns the tile
- * expires after one second (the tile's rows and the rest of that warp's
- * rows are not computed; the launch still ends and the flag read by
- * gsr_kernel_status is set).  No memory access is made out of bounds and no
+ * Test hook for the bounded waits on bulk copies: tile >= 0 makes every later
+ * launch of the staged aprod 1 on the handle announce tile's copies to its
+ * barrier without issuing them, and every later binary32 pass (tiles of the
+ * offset order, row windows of the instruments) let the barriers of one warp,
+ * or block, number `tile` wait for an arrival that does not come.  Such a wait
+ * expires after one second (the rest of that warp's rows are not computed; the
+ * launch still ends and the flag read by gsr_kernel_status is set; a solve
+ * ends with the iteration).  No memory access is made out of bounds and no
  * kernel is left waiting.  tile = -1 turns the hook off.  The solve graphs
  * are captured again.  Errors: GSR_ERR_ARG, GSR_ERR_CUDA.
  */
 int gsr_inject_missing_copy(void *h, int64_t tile);
+
+/*
+ * Test hook for the barriers of a small system's one-launch iterations: with
+ * on = 1 the second barrier of every later gsr_lsqr_solve on the handle waits
+ * for one block more than there are, so its bounded wait expires after one
+ * second, every block ends and the call returns GSR_ERR_TIMEOUT.  on = 0 turns
+ * the hook off.  Without effect where gsr_lsqr_one_launch says 0.  The solve
+ * graphs are captured again.  Errors: GSR_ERR_ARG, GSR_ERR_CUDA.
+ */
+int gsr_inject_missing_block(void *h, int on);
 
 /*
  * Measured FP64 fused multiply-add throughput of the current device, in FMAs

@@ -37,7 +37,7 @@ EXPORTS = (
     "gsr_batched_products", "gsr_set_batch_tiling", "gsr_set_aprod2_fused",
     "gsr_product_forms", "gsr_fp64_fma_rate", "gsr_time_iteration", "gsr_vector_add",
     "gsr_set_aprod1_staging", "gsr_aprod1_staging", "gsr_kernel_status",
-    "gsr_inject_missing_copy", "gsr_lsqr_one_launch",
+    "gsr_inject_missing_copy", "gsr_lsqr_one_launch", "gsr_inject_missing_block",
 )
 
 
@@ -137,6 +137,7 @@ def lib():
             L.gsr_aprod1_staging.argtypes = [P, ctypes.POINTER(I)]
             L.gsr_kernel_status.argtypes = [P, P]
             L.gsr_inject_missing_copy.argtypes = [P, I64]
+            L.gsr_inject_missing_block.argtypes = [P, I]
             L.gsr_lsqr_one_launch.argtypes = [P, ctypes.POINTER(I)]
             L.gsr_last_error.restype = ctypes.c_char_p
             L.gsr_strerror.argtypes = [I]
@@ -150,7 +151,8 @@ def lib():
                          "gsr_set_batch_tiling", "gsr_set_aprod2_fused", "gsr_product_forms",
                          "gsr_fp64_fma_rate", "gsr_time_iteration", "gsr_vector_add",
                          "gsr_set_aprod1_staging", "gsr_aprod1_staging", "gsr_kernel_status",
-                         "gsr_inject_missing_copy", "gsr_lsqr_one_launch"):
+                         "gsr_inject_missing_copy", "gsr_lsqr_one_launch",
+                         "gsr_inject_missing_block"):
                 getattr(L, name).restype = I
             _lib = L
     return _lib

@@ -1260,6 +1260,8 @@ extern "C" int gsr_mixed_solve(void *hv, const double *b, int max_outer, int max
         CK(launch_neg(h, h->d_xm, h->d_xneg, A.n, st));
         CK(launch_aprod1(h, h->d_xneg, h->d_r, 0, st));
         CK(cudaStreamSynchronize(st));
+        if (h->h_cg->late)
+            return take_kernel_status(h, st);
         if (h->h_cg->nonfinite)
             return GSR_ERR_NONFINITE;
         res.outer = k + 1;
@@ -1329,6 +1331,8 @@ static int normal_solve_dev(gsr_handle_t *h, const double *dg, int max_iter, dou
         res->converged = (g.gamma <= g.stop2) ? 1 : 0;
         res->rel_resid = (g.gamma0 > 0.0) ? sqrt(g.gamma / g.gamma0) : 0.0;
     }
+    if (g.late)
+        return take_kernel_status(h, st);
     if (g.nonfinite)
         return GSR_ERR_NONFINITE;
     return GSR_OK;
@@ -1555,7 +1559,19 @@ extern "C" int gsr_inject_missing_copy(void *hv, int64_t tile)
     if (!h || tile < -1)
         return GSR_ERR_ARG;
     h->drop_tile = tile;
+    h->att32.late = tile;
+    h->ell.late = tile;
+    drop_batched_graphs(h);
     return recapture_graphs(h, "gsr_inject_missing_copy");
+}
+
+extern "C" int gsr_inject_missing_block(void *hv, int on)
+{
+    gsr_handle_t *h = (gsr_handle_t *)hv;
+    if (!h || (on != 0 && on != 1))
+        return GSR_ERR_ARG;
+    h->drop_block = on;
+    return recapture_graphs(h, "gsr_inject_missing_block");
 }
 
 extern "C" int gsr_set_batch_tiling(void *hv, int kt, int lanes)
@@ -1686,6 +1702,8 @@ extern "C" int gsr_batched_solve(void *hv, int k, const double *B, int max_outer
         CK(launch_b_update_x(h, h->d_bXcm, k, st));
         CK(cudaMemcpyAsync(h->h_bs, h->d_bs, sizeof(BatchState), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
+        if (h->h_bs->late)
+            return take_kernel_status(h, st);
         for (int c = 0; c < k; c++) {
             res[c].outer = it + 1;
             res[c].inner += h->h_bs->it[c];

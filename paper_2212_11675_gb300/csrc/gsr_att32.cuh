@@ -40,7 +40,7 @@ struct AttWalk {
     {
         if (lane == 0) {
             for (int j = 0; j < NS; j++)
-                mbar_init(bar + 8 * j);
+                mbar_init(bar + 8 * j, u0 == U.late);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();

@@ -27,6 +27,7 @@
 #include "gsr_att32.cuh"
 #include "gsr_df.cuh"
 #include "gsr_internal.cuh"
+#include "gsr_lsqr.cuh"
 #include "gsr_reduce.cuh"
 
 namespace gsr {
@@ -694,6 +695,7 @@ k_b_init(const double *__restrict__ p, const double *__restrict__ C, double *__r
     if (grid_reduce_col<KT>(acc, partial + (int64_t)c0 * kMaxPartials, counter + c0)) {
         if (c0 == 0 && threadIdx.x == 0) {
             bs->nonfinite = 0;
+            bs->late = 0;
             bs->all_done = 0;
         }
         if (threadIdx.x < KT) {
@@ -714,13 +716,14 @@ __global__ void __launch_bounds__(kThreads)
 k_b_vec1(SysView A, Att32 U, const double *__restrict__ p, const double *__restrict__ T,
          const double *__restrict__ Sall, double *__restrict__ Sv,
          const double *__restrict__ Dd, double *__restrict__ Z, int c_first, BatchState *bs,
-         const BatchArgs *args, double *partial, unsigned *counter)
+         const BatchArgs *args, double *partial, unsigned *counter, const int *kerr)
 {
     const int c0 = c_first + blockIdx.y * KT;
     const int c = threadIdx.x % KT;
     const int64_t base = pidx(0, A.n, c0);
     const double *S = Sall + (int64_t)c0 * U.nunits * kNAtt;
     const double al = bs->alpha[c0 + c];
+    const bool late = threadIdx.x < KT && wait_expired(kerr);
     double acc = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n * KT;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -743,7 +746,9 @@ k_b_vec1(SysView A, Att32 U, const double *__restrict__ p, const double *__restr
             bs->it[cc] += 1;
             if (!isfinite(gnew))
                 bs->nonfinite = 1;
-            if (!isfinite(gnew) || gnew <= args->tol * args->tol * bs->gamma0[cc] ||
+            if (late)
+                bs->late = 1;
+            if (!isfinite(gnew) || late || gnew <= args->tol * args->tol * bs->gamma0[cc] ||
                 bs->it[cc] >= args->max_inner)
                 bs->done[cc] = 1;
         }
@@ -980,7 +985,7 @@ static cudaError_t b_iteration_tiles(const gsr_handle_t *h, int c0, int ny, cuda
     const dim3 g(vec_blocks<KT>(h), ny);
     k_b_vec1<KT><<<g, kThreads, 0, s>>>(h->sys, h->att32, h->d_p, h->d_bT, h->d_bS, h->d_bS_,
                                         h->d_bD, h->d_bZ, c0, h->d_bs, h->d_bargs, h->d_bpartial,
-                                        h->d_bcounter);
+                                        h->d_bcounter, h->d_kerr);
     k_b_vec2<KT><<<g, kThreads, 0, s>>>(h->d_p, h->d_bS_, h->d_bD, h->d_bX32, h->sys.n, c0, h->d_bs,
                                         k, loop, in_graph, last);
     return cudaGetLastError();

@@ -132,7 +132,7 @@ struct EllWindows {
         return (int)(m - w * W < W ? m - w * W : W);
     }
     __device__ __forceinline__ void init(float *b, EllShared *sh_, const float *y_, int64_t m_,
-                                         int64_t W_)
+                                         int64_t W_, bool late)
     {
         buf = b;
         sh = sh_;
@@ -143,8 +143,8 @@ struct EllWindows {
         if (threadIdx.x == 0) {
             buf[kEllPad] = buf[kEllRows + kEllPad] = 0.f;
             sh->fail = 0;
-            mbar_init(bar);
-            mbar_init(bar + 8);
+            mbar_init(bar, late);
+            mbar_init(bar + 8, late);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         ell_sync();
@@ -189,7 +189,7 @@ __device__ __forceinline__ void ell_windows(const Ell &E, const float *y, int64_
 {
     EllWindows win;
     int64_t w = blockIdx.x;
-    win.init(buf, sh, y, m, E.W);
+    win.init(buf, sh, y, m, E.W, w == E.late);
     int b = 0;
     win.fetch(w, 0);
     for (; w < E.nwin; w += E.nblk, b ^= 1) {

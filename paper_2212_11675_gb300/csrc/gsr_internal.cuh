@@ -55,6 +55,7 @@ struct Att32 {
     const uint32_t *useg;  // [nseg+1] units of offset o: useg[o] .. useg[o+1]-1
     const float *sv;       // the 5 astrometric planes in row order (tidx<5>)
     int64_t nunits;
+    int64_t late = -1;     // test hook: first unit of the warp whose waits run out
 };
 constexpr uint32_t kAttRecAt = 32 * kNPar * sizeof(float);               // 3072
 constexpr uint32_t kAttRowAt = kAttRecAt + 32 * sizeof(uint4);           // 3584
@@ -112,6 +113,7 @@ struct Ell {
     int nacc;             // sums of a block at most
     int64_t nwin, W;      // windows, rows per window
     int64_t nblk;         // block b takes windows b, b + nblk, ...
+    int64_t late = -1;    // test hook: first window of the block whose waits run out
 };
 
 // Partial sums of the single-launch aprod 2 that a following vector pass
@@ -215,7 +217,8 @@ struct SolveState {
 struct CgState {
     double gamma, gamma0, stop2;  // |s|^2, its start value, tol^2 |s_0|^2
     double xi, alpha, beta;       // |q|^2, step, direction update
-    int it, done, nonfinite, pad;
+    int it, done, nonfinite;
+    int late;                     // a bounded wait expired: the iterations ended
 };
 struct CgArgs {
     int max_inner;
@@ -227,7 +230,7 @@ constexpr int kMaxBatch = 32;
 struct BatchState {
     double gamma[kMaxBatch], gamma0[kMaxBatch], xi[kMaxBatch], alpha[kMaxBatch], beta[kMaxBatch];
     int it[kMaxBatch], done[kMaxBatch];
-    int all_done, nonfinite;
+    int all_done, nonfinite, late;
 };
 struct BatchArgs {
     int max_inner;
@@ -379,6 +382,7 @@ struct gsr_handle_t {
     unsigned *d_bar = nullptr;          // barrier count of k_lsqr_loop
     int *d_kerr = nullptr;              // set by a kernel whose bounded wait expired
     int64_t drop_tile = -1;             // test hook: the tile whose bulk copy is not issued
+    int drop_block = 0;                 // test hook: a block that the one-launch loop waits for in vain
 };
 
 namespace gsr {

@@ -1370,6 +1370,7 @@ struct LoopArgs {
     double *partial;          // [4][kMaxPartials]
     unsigned *bar;            // zero on entry
     int *kerr;
+    int drop_block;           // test hook: the second barrier waits for a block more
 };
 
 // Barrier of the grid: false when the others did not arrive in time
@@ -1549,6 +1550,7 @@ k_lsqr_loop(SysView A, LoopArgs L)
                 t += ld_shared<true>(L.partial + b);
             lsqr_beta_rotation_warp(&s, warp_sum(t));
         }
+        target += L.drop_block;
         // 2. units
         const int64_t natt = A.nseg * A.attp;
         for (int64_t i = gw; i < natt + L.ninstr + L.ngroups; i += nw) {
@@ -2008,7 +2010,7 @@ static cudaError_t loop_launch(const gsr_handle_t *h, cudaStream_t st)
                   VecPass{h->d_p, h->d_v, h->d_vp, h->d_w, h->d_z, h->d_var},
                   h->d_cseg, h->d_irow, h->d_ival, h->isplit,
                   (h->sys.S + 32 / G - 1) / (32 / G), h->sys.I * h->isplit,
-                  h->d_state, h->d_args, h->d_partial, h->d_bar, h->d_kerr};
+                  h->d_state, h->d_args, h->d_partial, h->d_bar, h->d_kerr, h->drop_block};
     // beside the kernel's static shared memory, the pieces of kSplitInstrMax
     // instruments exceed the 48 KB that a launch may have without asking; the
     // attribute belongs to the kernel: the most that any handle asks for

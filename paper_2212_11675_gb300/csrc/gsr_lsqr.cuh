@@ -15,6 +15,14 @@ namespace gsr {
 constexpr int kIstopNonfinite = 8;
 constexpr int kThreadParts = 8;  // window totals of an instrument that one thread adds
 
+// A bounded wait of a kernel before this one has expired: the results are
+// undefined, and each further iteration could wait as long.  Read at the start
+// of a kernel, beside its other loads, by the threads that form the scalars.
+__device__ __forceinline__ bool wait_expired(const int *kerr)
+{
+    return *(const volatile int *)kerr != 0;
+}
+
 // Square roots and the reciprocal that the scalar recurrences of an iteration
 // start from: alpha_{i+1}, ||z||, ||A||, sqrt(ddnorm), 1/alpha_{i+1}, rho_i
 struct LsqrRoots {
@@ -26,9 +34,10 @@ struct LsqrRoots {
 // divisions: FP64 divisions and square roots take a third of a microsecond
 // each on this part and every dependent operation 65 clocks.  The tests of
 // the machine-precision rules are multiplied out: 1 + a / b <= 1 exactly when
-// a <= 2^-53 b (up to the rounding of a / b).
+// a <= 2^-53 b (up to the rounding of a / b).  late: a wait has expired, the
+// iterations end.
 __device__ __forceinline__ void lsqr_finish(SolveState *st, const SolveArgs *args, const LsqrRoots &R,
-                                            double anorm2, double ddnorm,
+                                            double anorm2, double ddnorm, bool late,
                                             cudaGraphConditionalHandle loop, int in_graph)
 {
     constexpr double kHalfEps = 1.0 / 9007199254740992.0;  // 2^-53
@@ -83,7 +92,7 @@ __device__ __forceinline__ void lsqr_finish(SolveState *st, const SolveArgs *arg
     if (args->force_itmax && !bad && s.itn < args->itmax)
         istop = 0;
     s.istop = istop;
-    if (istop != 0) {
+    if (istop != 0 || late) {
         s.done = 1;
         if (in_graph)
             cudaGraphSetConditional(loop, 0u);
@@ -94,8 +103,8 @@ __device__ __forceinline__ void lsqr_finish(SolveState *st, const SolveArgs *arg
 // ... by the whole last block of the vector pass: the independent roots go to
 // different warps
 __device__ __forceinline__ void lsqr_scalars(SolveState *st, const SolveArgs *args, double vnorm2,
-                                             double dd, double zz, cudaGraphConditionalHandle loop,
-                                             int in_graph)
+                                             double dd, double zz, bool late,
+                                             cudaGraphConditionalHandle loop, int in_graph)
 {
     __shared__ LsqrRoots sq;
     const double beta = st->bnext;
@@ -118,7 +127,7 @@ __device__ __forceinline__ void lsqr_scalars(SolveState *st, const SolveArgs *ar
         sq.rho = sqrt(st->rhobar * st->rhobar + beta * beta);
     __syncthreads();
     if (threadIdx.x == 0)
-        lsqr_finish(st, args, sq, anorm2, ddnorm, loop, in_graph);
+        lsqr_finish(st, args, sq, anorm2, ddnorm, late, loop, in_graph);
 }
 
 // ... by one warp: the roots in different lanes
@@ -143,7 +152,7 @@ __device__ __forceinline__ void lsqr_scalars_warp(SolveState *st, const SolveArg
     R.ia = (R.alpha > 0.0) ? 1.0 / R.alpha : 1.0;
     __syncwarp();  // every lane has read the state
     if (lane == 0)
-        lsqr_finish(st, args, R, anorm2, ddnorm, 0, 0);
+        lsqr_finish(st, args, R, anorm2, ddnorm, false, 0, 0);
 }
 
 // Coefficients of the column updates of iteration i (W = w / rho, see k_vec)

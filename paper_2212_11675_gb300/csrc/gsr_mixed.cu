@@ -623,10 +623,12 @@ __global__ void __launch_bounds__(kThreads)
 k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restrict__ t,
           double *__restrict__ s, const double *__restrict__ d, double *__restrict__ z, CgState *cg,
           const CgArgs *args, double *partial, unsigned *counter,
-          cudaGraphConditionalHandle loop, int in_graph, const uint32_t *__restrict__ useg, A2Parts P)
+          cudaGraphConditionalHandle loop, int in_graph, const uint32_t *__restrict__ useg, A2Parts P,
+          const int *kerr)
 {
     const int64_t n = A.n;
     const double alpha = cg->alpha;
+    const bool late = threadIdx.x == 0 && wait_expired(kerr);
     double acc[SUMS == kSumsParts ? 2 : 1] = {};
     // column j with t_j = tf(): the loads of the vectors come first
     auto update = [&](int64_t j, auto tf) {
@@ -689,7 +691,8 @@ k_cg_vec1(const SysView A, const double *__restrict__ p, const double *__restric
         const bool bad = !isfinite(gnew) || !isfinite(g.alpha);
         if (bad)
             g.nonfinite = 1;
-        if (bad || g.it >= args->max_inner || gnew <= g.stop2 || g.xi <= 0.0) {
+        g.late = late;
+        if (bad || late || g.it >= args->max_inner || gnew <= g.stop2 || g.xi <= 0.0) {
             g.done = 1;
             if (in_graph)
                 cudaGraphSetConditional(loop, 0u);
@@ -877,7 +880,7 @@ cudaError_t launch_aprod2_f32_api(const gsr_handle_t *h, const double *y, double
                                                            h->d_zc, h->d_cg, h->d_cgargs,
                                                            h->d_partial + kRedV * kPartialsPerKind,
                                                            h->d_counter + kRedV, loop, in_graph,
-                                                           h->d_useg, P);
+                                                           h->d_useg, P, h->d_kerr);
     k_cg_vec2<float><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_x32, h->d_t, A.n, A.n,
                                                 h->d_cg, h->d_x8, A.att0);
     return cudaGetLastError();
@@ -1120,14 +1123,14 @@ cudaError_t build_att32(gsr_handle_t *h, cudaStream_t st)
                         s)) {
         k_cg_vec1<kSumsParts><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
                                                                h->d_zc, h->d_cg, h->d_cgargs, part,
-                                                               cnt, loop, in_graph, nullptr, P);
+                                                               cnt, loop, in_graph, nullptr, P, h->d_kerr);
     } else {
         e = launch_aprod2(h, h->d_q64, h->d_t, kA2Overwrite, s);
         if (e != cudaSuccess)
             return e;
         k_cg_vec1<kSumsDone><<<h->grid_vec, kThreads, 0, s>>>(A, h->d_p, h->d_t, h->d_s, h->d_d,
                                                               h->d_zc, h->d_cg, h->d_cgargs, part,
-                                                              cnt, loop, in_graph, nullptr, P);
+                                                              cnt, loop, in_graph, nullptr, P, h->d_kerr);
     }
     k_cg_vec2<double><<<h->grid_vec, kThreads, 0, s>>>(h->d_p, h->d_s, h->d_d, h->d_xp64, h->d_t,
                                                         A.n, A.ins0, h->d_cg, nullptr, 0);

@@ -42,9 +42,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     return true;
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t bar)
+// late: a test hook, the barrier waits for an arrival that does not come
+__device__ __forceinline__ void mbar_init(uint32_t bar, bool late = false)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(late ? 2 : 1) : "memory");
 }
 
 __device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes)

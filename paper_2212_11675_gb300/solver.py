@@ -220,6 +220,10 @@ class Solver:
         """Test hook: tile's bulk copies are never issued (-1: off)."""
         check(lib().gsr_inject_missing_copy(self._h, int(tile)), "gsr_inject_missing_copy")
 
+    def inject_missing_block(self, on):
+        """Test hook: the one-launch LSQR loop waits for a block more than there are."""
+        check(lib().gsr_inject_missing_block(self._h, 1 if on else 0), "gsr_inject_missing_block")
+
     def product_forms(self):
         """(aprod1_split, aprod2_split): which FP64 products run on the binary32
         pipes from exact splits: aprod1_split 0 (none), 1 (instrumental and

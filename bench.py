@@ -60,6 +60,16 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
+def launches_per_solve(iterations, one_launch):
+    """Kernel launches of one PC-LSQR solve (as in the ncu launch list of
+    --eager): 8 in the prologue (2 clears; preconditioner: single-launch aprod 2
+    of squares, combine, finish; start: U, aprod 2, first vector pass), 3 per
+    iteration (aprod 1, single-launch aprod 2, vector pass that also combines
+    its partial sums) or one for all iterations of a small system
+    (gsr_lsqr_one_launch), 1 epilogue."""
+    return 9 + (1 if one_launch else 3 * iterations)
+
+
 def captured_traffic(kernel, workload):
     """DRAM bytes (read + write) per launch of `kernel` from the committed ncu
     summaries under profiles/: a line
@@ -569,6 +579,8 @@ def main():
     se = torch.empty(sys_.n, dtype=torch.float64, device=dev)
     torch.cuda.synchronize()
 
+    one_launch = solver.lsqr_one_launch()
+
     def step():
         return solver.lsqr_solve(b, itmax, 0.0, 0.0, x=x, se=se, stream=stream)[2]
 
@@ -697,13 +709,7 @@ def main():
             except Exception as e:  # reported, never fatal for the main line
                 large[name] = {"unavailable": ("%s: %s" % (type(e).__name__, e))[:300]}
 
-    # per solve (ncu launch list of --eager): 8 prologue launches (2 clears,
-    # preconditioner: single-launch aprod 2 of squares + combine + finish;
-    # init: U, aprod 2, first vector pass), 3 per LSQR iteration (aprod 1,
-    # single-launch aprod 2, vector pass that also combines aprod 2's
-    # partial sums; all iterations of a system of at most 400,000 rows in one
-    # launch), 1 epilogue
-    launches_per_step = 9 + (3 * (iters // args.steps) if m > 400000 else 1)
+    launches_per_step = launches_per_solve(iters // args.steps, one_launch)
     line = {"metric": METRIC, "value": value, "unit": "iter/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1e3 * t_max / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",

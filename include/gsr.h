@@ -379,9 +379,8 @@ int gsr_batched_products(void *h, int k, const double *X, const double *Y,
 int gsr_set_batch_tiling(void *h, int kt, int lanes);
 
 /*
- * Schedule of aprod 2 (Alg. 2; FP64, and the binary32 form inside the
- * mixed-precision inner solve) on the sorted instrumental path
- * (GSR_INSTR_SORTED, the default).  fused = 1 (default): the star-group
+ * Schedule of the FP64 aprod 2 (Alg. 2) on the sorted instrumental path
+ * (GSR_INSTR_SORTED, the default; the binary32 forms have one schedule).  fused = 1 (default): the star-group
  * sums, the attitude segment sums and the instrumental segment sums run in
  * one launch whose warps take units of all three kinds from one work queue,
  * so the FP64-bound and the gather-bound parts share every SM.  fused = 0:
@@ -402,11 +401,12 @@ int gsr_set_aprod2_fused(void *h, int fused);
  * has the bulk-copy (TMA) engine stage its next 32-row tile (the 24 value
  * planes, the records, the star deltas and, when y is read and 16-byte
  * aligned, the tile's y) into a 7,040-byte stage in shared memory, one tile
- * ahead of the tile it computes.  Both forms use the same
- * per-row arithmetic (the split instrumental and global products), so their
- * results are bitwise equal.  Available when the split products apply (I up
- * to the split limit) and the stages fit the block's opt-in shared memory;
- * GSR_ERR_UNSUPPORTED otherwise.  Every wait on a copy is bounded (one
+ * ahead of the tile it computes.  Up to 3,072 instruments both forms use the
+ * same per-row arithmetic (the split instrumental and global products), so
+ * their results are bitwise equal; beyond, only the staged form has the split
+ * products and the register form takes native ones.  Available when the split
+ * products are asked for and their x fits beside the stages in the block's
+ * opt-in shared memory (I <= 6,576); GSR_ERR_UNSUPPORTED otherwise.  Every wait on a copy is bounded (one
  * second); an expired wait sets a device flag that the solve entry points
  * (gsr_lsqr_solve, gsr_mixed_solve, gsr_normal_solve, gsr_lsq_backward,
  * gsr_batched_solve) and gsr_kernel_status report as GSR_ERR_TIMEOUT (and

@@ -485,9 +485,9 @@ static int build_instr_sorted(gsr_handle_t *h, cudaStream_t st)
     return finish_instr(h, cseg, nq, nparts);
 }
 
-// the units of the offset-ordered binary32 layout (Att32)
-constexpr int64_t kQInL2 = 96 << 20;  // bytes of the 129 MB
+constexpr int64_t kQInL2 = 96 << 20;  // bytes of q that L2 (129 MB) keeps
 
+// the units of the offset-ordered binary32 layout (Att32)
 static int build_units(gsr_handle_t *h)
 {
     const SysView &A = h->sys;

@@ -177,9 +177,9 @@ constexpr int kBA2 = 2;  // attitude and global part of A32^T Q
 // / 5.5 / 8.6e-18; now 2.7 / 2.5 / 1.9 / 0.7e-18; one chain over the unit had
 // 9.8 / 43 / 26 / 23e-18).
 // Bound by the FP32 pipe: 8 lane operations per product, 37 products a row
-// and column (0.47 ms at 7.0e6 rows and 8 columns with all lanes busy; 0.69
-// measured, the pipe 62 % active, against 0.76 + 0.39 ms for the two products
-// as passes in row order and in offset order).
+// and column (0.47 ms at 7.0e6 rows and 8 columns with all lanes busy; 0.73
+// measured, against 0.76 + 0.39 ms for the two products as passes in row order
+// and in offset order; 0.69 with one chain over the unit).
 // ---------------------------------------------------------------------------
 constexpr int kBWarps = 16;  // one block per SM
 constexpr int kBThreads = 32 * kBWarps;

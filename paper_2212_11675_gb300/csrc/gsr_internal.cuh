@@ -89,10 +89,10 @@ __device__ __forceinline__ uint32_t star_of_row(const SysView &A, int64_t t, int
     return s;
 }
 
-// Instrumental nonzeros in row windows (gsr_ell.cu): slices of 32 columns, the
-// entry i < slice[s].y of its lane at slice[s].x * 32 + (i / 2) * 64 + 2 lane
-// + i % 2
-// (a multiple of kEllStep).
+// Instrumental nonzeros in row windows (gsr_ell.cu): slices of 32 columns, one a
+// lane.  Slice s has slice[s].y entries a column (a multiple of kEllStep, the
+// shorter columns padded); entry i of a lane is at
+// slice[s].x * 32 + (i / 2) * 64 + 2 lane + i % 2.
 constexpr uint32_t kEllRowBits = 13;
 constexpr uint32_t kEllRowMask = (1u << kEllRowBits) - 1;
 constexpr uint32_t kEllPad = kEllRowMask;     // window row of a padding entry (y = 0)

@@ -134,7 +134,8 @@ __global__ void __launch_bounds__(kThreads)
 k_vec(const SysView A, const double *__restrict__ p, double *__restrict__ q, double *__restrict__ v,
       double *__restrict__ vp, double *__restrict__ w, double *__restrict__ z,
       double *__restrict__ var, SolveState *st, const SolveArgs *args, double *partial,
-      unsigned *counter, cudaGraphConditionalHandle loop, int in_graph, int first, A2Parts P, const int *kerr)
+      unsigned *counter, cudaGraphConditionalHandle loop, int in_graph, int first, A2Parts P,
+      const int *kerr)
 {
     const int64_t n = A.n, att0 = A.att0, glb0 = A.glb0;
     const bool late = threadIdx.x == 0 && wait_expired(kerr);
@@ -315,7 +316,8 @@ cudaError_t find_graph_leaf(cudaGraph_t g, cudaGraphNode_t *leaf)
             return e;
         k_vec<false><<<h->grid_lsqr_vec, kThreads, 0, s>>>(h->sys, h->d_p, h->d_q, h->d_v, h->d_vp, h->d_w,
                                                       h->d_z, h->d_var, h->d_state, h->d_args, part,
-                                                      cnt, loop, in_graph, first, P, h->d_kerr);
+                                                      cnt, loop, in_graph, first, P,
+                                                      h->d_kerr);
     } else {
         if (mid) {
             cudaError_t e = cudaEventRecord(mid, s);
@@ -324,7 +326,8 @@ cudaError_t find_graph_leaf(cudaGraph_t g, cudaGraphNode_t *leaf)
         }
         k_vec<true><<<h->grid_lsqr_vec, kThreads, 0, s>>>(h->sys, h->d_p, h->d_q, h->d_v, h->d_vp, h->d_w,
                                                      h->d_z, h->d_var, h->d_state, h->d_args, part,
-                                                     cnt, loop, in_graph, first, P, h->d_kerr);
+                                                     cnt, loop, in_graph, first, P,
+                                                     h->d_kerr);
     }
     return cudaGetLastError();
 }

@@ -196,7 +196,8 @@ class Solver:
 
     def set_aprod1_staging(self, staged):
         """FP64 aprod 1 with its tiles staged in shared memory by the bulk-copy
-        engine (True) or loaded into registers (False); bitwise-equal results."""
+        engine (True) or loaded into registers (False); bitwise-equal results up
+        to 3,072 instruments (the register form's split products end there)."""
         check(lib().gsr_set_aprod1_staging(self._h, 1 if staged else 0),
               "gsr_set_aprod1_staging")
 

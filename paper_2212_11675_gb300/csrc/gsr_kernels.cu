@@ -1347,16 +1347,21 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 //
 // Where it is taken: beyond some size the staged aprod 1, the dynamic unit
 // queue and the wider vector pass of the separate launches win.  us an
-// iteration, loop / launches, 5 to 400 rows a star: 50,000 rows 33 to 45 / 38
-// to 49; 100,000 rows 46 to 63 / 48 to 55; 200,000 rows 62 to 97 / 60 to 72;
-// 400,000 rows 102 to 165 / 83 to 111.  Columns cost more here (mostly empty
-// stars, 20,000 rows): 25,661 columns 26.9 / 34.3, 100,661 columns 44.6 / 42.5,
-// 500,661 columns 132 / 60.  So do offsets cut into pieces, whose sums one
-// thread adds: 20,000 rows on one offset (40 pieces) 49 / 49, on five (8
-// pieces) 36 / 43.  Up to 3,072 instruments change nothing.
+// iteration, loop / launches, rows in time order inside their star, stars of 20
+// to 400 rows: 50,000 rows 27 to 50 / 38 to 54; 100,000 rows 41 to 60 / 48 to
+// 63; 200,000 rows 52 to 82 / 59 to 85; 280,000 rows, stars of 20 to 40 rows 69
+// to 97 / 68 to 81, of 70 rows and more 60 to 83 / 68 to 90; 400,000 rows, of
+// 20 to 130 rows 87 to 111 / 77 to 92, of 250 and 400 rows 80 to 86 / 82 to 96.
+// (Runs of the same system differ by up to a fifth in the loop.)  A column
+// costs the loop more than a row: mostly empty stars on 20,000 rows, 25,661
+// columns 26.9 / 34.3, 100,661 columns 44.6 / 42.5, 500,661 columns 132 / 60.
+// So do offsets cut into pieces, whose sums one thread adds: 20,000 rows on one
+// offset (40 pieces) 49 / 49, on five (8 pieces) 36 / 43.  Up to 3,072
+// instruments change nothing.
 // ---------------------------------------------------------------------------
 constexpr int kLoopThreads = 512;
-constexpr int64_t kLoopRows = 75000, kLoopCols = 60000, kLoopPieces = 16;
+constexpr int64_t kLoopSize = 460000;  // rows + 6 columns
+constexpr int64_t kLoopPieces = 16;
 
 struct LoopArgs {
     double *u, *q, *S, *ipart, *gpart;
@@ -1997,7 +2002,7 @@ cudaError_t launch_aprod2(const gsr_handle_t *h, const double *y, double *out, i
 
 bool lsqr_loop_fits(const gsr_handle_t *h)
 {
-    return h->sys.m <= kLoopRows && h->sys.n <= kLoopCols && h->sys.attp <= kLoopPieces &&
+    return h->sys.m + 6 * h->sys.n <= kLoopSize && h->sys.attp <= kLoopPieces &&
            h->sys.I <= kSplitInstrMax && h->ipath == kIpSorted &&
            h->a2_fused && h->cfg.products == GSR_PRODUCTS_AUTO && h->drop_tile < 0 &&
            h->nsm <= kMaxPartials;

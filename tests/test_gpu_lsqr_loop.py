@@ -39,12 +39,13 @@ def test_instruments_at_the_shared_memory_limit(n_instr, precision):
 
 
 # (stars, rows a star, knots, instruments), empty stars, one launch?  The lines
-# lie at 75,000 rows, 60,000 columns and offsets of 16 pieces of 512 rows
+# lie at rows + 6 columns = 460,000 and offsets of 16 pieces of 512 rows
 @pytest.mark.parametrize("shape,empty,one", [
-    ((2500, 30, 60, 30), 0, True), ((2500, 30, 60, 30), 1, True), ((2501, 30, 60, 30), 0, False),
-    ((11951, 3, 61, 61), 0, True), ((11952, 3, 61, 61), 0, False),   # 60,000 and 60,005 columns
-    ((12000, 5, 60, 30), 11000, False),                              # mostly empty stars
-    ((512, 16, 4, 30), 0, True), ((513, 16, 4, 30), 0, False)])      # one offset: 16 and 17 pieces
+    ((2000, 199, 100, 30), 0, True), ((2000, 199, 100, 30), 1, True),  # 459,986 without empty stars
+    ((2000, 199, 100, 33), 0, False),                                  # 460,004
+    ((13900, 3, 30, 30), 0, True), ((13920, 3, 30, 30), 0, False),     # 459,426 and 460,086
+    ((16000, 5, 60, 30), 15000, False),                                # mostly empty stars
+    ((512, 16, 4, 30), 0, True), ((513, 16, 4, 30), 0, False)])        # one offset: 16 and 17 pieces
 def test_where_the_loop_is_taken(shape, empty, one):
     sys = _random(*shape, seed=9)
     if empty:

@@ -205,8 +205,8 @@ int gsr_precondition(void *h, double *p, void *stream);
  * and S2 (0 disables them); the condition limit is the handle's conlim.
  * The whole iteration runs on the device (one CUDA graph, no host
  * synchronisation until the end).  A small system's iterations are one
- * kernel that needs every SM (gsr_lsqr_one_launch); while work of another
- * stream or thread holds one, the call runs them as launches on the others.
+ * kernel that needs room on every SM (gsr_lsqr_one_launch); while another
+ * stream's work leaves too little on one, the call runs them as launches.
  * `out` receives the stopping estimates.
  * Errors: GSR_ERR_ARG, GSR_ERR_NONFINITE (a NaN/Inf in b or in the scalar
  * recurrences; x and se are then undefined), GSR_ERR_TIMEOUT (a bounded
@@ -439,14 +439,15 @@ int gsr_kernel_status(void *h, void *stream);
 int gsr_inject_missing_copy(void *h, int64_t tile);
 
 /*
- * Test hook for the barriers of a small system's one-launch iterations: with
- * on = 1 the second barrier of every later gsr_lsqr_solve on the handle waits
- * for one block more than there are, so its bounded wait expires after one
- * second, every block ends and the call returns GSR_ERR_TIMEOUT.  on = 0 turns
- * the hook off.  Without effect where gsr_lsqr_one_launch says 0.  The solve
- * graphs are captured again.  Errors: GSR_ERR_ARG, GSR_ERR_CUDA.
+ * Test hook for the barriers of a small system's one-launch iterations, which
+ * then wait for one block more than there are.  where = 2, the first barrier:
+ * every later gsr_lsqr_solve on the handle finds its blocks not all resident
+ * and runs as launches.  where = 1, the second: its bounded wait expires after
+ * one second, every block ends and the call returns GSR_ERR_TIMEOUT.
+ * where = 0 turns the hook off.  Without effect where gsr_lsqr_one_launch says
+ * 0.  The solve graphs are captured again.  Errors: GSR_ERR_ARG, GSR_ERR_CUDA.
  */
-int gsr_inject_missing_block(void *h, int on);
+int gsr_inject_missing_block(void *h, int where);
 
 /*
  * Measured FP64 fused multiply-add throughput of the current device, in FMAs

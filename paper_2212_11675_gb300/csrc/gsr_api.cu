@@ -1565,12 +1565,12 @@ extern "C" int gsr_inject_missing_copy(void *hv, int64_t tile)
     return recapture_graphs(h, "gsr_inject_missing_copy");
 }
 
-extern "C" int gsr_inject_missing_block(void *hv, int on)
+extern "C" int gsr_inject_missing_block(void *hv, int where)
 {
     gsr_handle_t *h = (gsr_handle_t *)hv;
-    if (!h || (on != 0 && on != 1))
+    if (!h || where < 0 || where > 2)
         return GSR_ERR_ARG;
-    h->drop_block = on;
+    h->drop_block = where;
     return recapture_graphs(h, "gsr_inject_missing_block");
 }
 

@@ -382,7 +382,7 @@ struct gsr_handle_t {
     unsigned *d_bar = nullptr;          // barrier count of k_lsqr_loop
     int *d_kerr = nullptr;              // set by a kernel whose bounded wait expired
     int64_t drop_tile = -1;             // test hook: the tile whose bulk copy is not issued
-    int drop_block = 0;                 // test hook: a block that the one-launch loop waits for in vain
+    int drop_block = 0;                 // test hook: barrier at which the one-launch loop waits in vain
 };
 
 namespace gsr {

@@ -1335,15 +1335,18 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // Data that other blocks write is read from L2 (ld_shared).  Each wait of the
 // barrier is bounded: when it runs out the block sets *kerr and ends.
 //
-// A block takes a whole SM (its registers), so another stream's kernel on any
-// SM keeps the grid from being resident.  A cooperative launch then waits for
-// that kernel to end (beside a kernel of one block and 1.5 s the solve took
-// 1.45 s; as launches 2.8 ms on the other SMs).  This one is an ordinary
-// launch whose first barrier (loop_join) settles whether all blocks are
-// there: if they are not within kJoinNs, every block ends, the state says so
-// (left) and the host runs the solve as launches.  Up to there only U was
-// written, which a solve starts anew.  After it all blocks are resident, and
-// resident blocks run to their end.
+// Beside other work: a block takes three quarters of an SM's registers (96 a
+// thread; with 128, which filled the SM, 0.7 % faster alone), so that it fits
+// beside whatever the staged aprod 1 of the launches (55,296 registers, 220 KB
+// of shared memory) fits beside.  A larger kernel of another stream on any SM
+// keeps the grid from being resident.  A cooperative launch then waits for
+// that kernel to end (with 128 registers, beside a kernel of one block and
+// 1.5 s the solve took 1.45 s; as launches 2.8 ms on the other SMs).  This one
+// is an ordinary launch whose first barrier (loop_join) settles whether all
+// blocks are there: if they are not within kJoinNs, every block ends, the
+// state says so (left) and the host runs the solve as launches.  Up to there
+// only U was written, which a solve starts anew.  After it all blocks are
+// resident, and resident blocks run to their end.
 //
 // Where it is taken: beyond some size the staged aprod 1, the dynamic unit
 // queue and the wider vector pass of the separate launches win.  us an
@@ -1360,6 +1363,7 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // instruments change nothing.
 // ---------------------------------------------------------------------------
 constexpr int kLoopThreads = 512;
+constexpr int kLoopRegThreads = 640;  // launch bound: 96 registers a thread
 constexpr int64_t kLoopSize = 460000;  // rows + 6 columns
 constexpr int64_t kLoopPieces = 16;
 
@@ -1375,7 +1379,7 @@ struct LoopArgs {
     double *partial;          // [4][kMaxPartials]
     unsigned *bar;            // zero on entry
     int *kerr;
-    int drop_block;           // test hook: the second barrier waits for a block more
+    int drop_block;           // test hook: the second (1) or first (2) barrier waits for a block more
 };
 
 // Barrier of the grid: false when the others did not arrive in time
@@ -1416,10 +1420,10 @@ __device__ __forceinline__ bool loop_sync(unsigned *bar, unsigned &target, int *
 constexpr unsigned kLoopLeft = 0x80000000u;
 constexpr uint64_t kJoinNs = 500000;  // 0.5 ms
 
-__device__ __forceinline__ bool loop_join(unsigned *bar, unsigned &target, SolveState *st)
+__device__ __forceinline__ bool loop_join(unsigned *bar, unsigned &target, SolveState *st, bool drop)
 {
     __shared__ int s_ok;
-    target += gridDim.x;
+    target += gridDim.x + drop;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -1496,7 +1500,7 @@ __device__ __forceinline__ void loop_total(double (&v)[K], const double *partial
 }
 
 template <int G>
-__global__ void __launch_bounds__(kLoopThreads, 1)
+__global__ void __launch_bounds__(kLoopRegThreads, 1)
 k_lsqr_loop(SysView A, LoopArgs L)
 {
     constexpr int NW = kLoopThreads / 32;
@@ -1545,7 +1549,7 @@ k_lsqr_loop(SysView A, LoopArgs L)
             }
         }
         loop_part<1>(nrm, gw < ntiles, L.partial);
-        if (!(target == 0 ? loop_join(L.bar, target, L.st) : loop_sync(L.bar, target, L.kerr)))
+        if (!(target == 0 ? loop_join(L.bar, target, L.st, L.drop_block == 2) : loop_sync(L.bar, target, L.kerr)))
             return;
         if (s.done)  // by the recurrences of the iteration before
             break;
@@ -1555,7 +1559,7 @@ k_lsqr_loop(SysView A, LoopArgs L)
                 t += ld_shared<true>(L.partial + b);
             lsqr_beta_rotation_warp(&s, warp_sum(t));
         }
-        target += L.drop_block;
+        target += L.drop_block == 1;
         // 2. units
         const int64_t natt = A.nseg * A.attp;
         for (int64_t i = gw; i < natt + L.ninstr + L.ngroups; i += nw) {

@@ -221,9 +221,10 @@ class Solver:
         """Test hook: tile's bulk copies are never issued (-1: off)."""
         check(lib().gsr_inject_missing_copy(self._h, int(tile)), "gsr_inject_missing_copy")
 
-    def inject_missing_block(self, on):
-        """Test hook: the one-launch LSQR loop waits for a block more than there are."""
-        check(lib().gsr_inject_missing_block(self._h, 1 if on else 0), "gsr_inject_missing_block")
+    def inject_missing_block(self, where):
+        """Test hook: the first (2) or second (1) barrier of the one-launch LSQR
+        loop waits for a block more than there are (0: off)."""
+        check(lib().gsr_inject_missing_block(self._h, int(where)), "gsr_inject_missing_block")
 
     def product_forms(self):
         """(aprod1_split, aprod2_split): which FP64 products run on the binary32

@@ -62,8 +62,7 @@ def test_where_the_loop_is_taken(shape, empty, one):
 
 
 def test_solve_beside_a_kernel_that_holds_an_sm():
-    # one block of another stream for about 1.2 s: the loop cannot be resident,
-    # the solve goes on without it on the other SMs
+    # one block of another stream for about 1.2 s on an SM that the loop needs too
     sys = _random(257, 20, 37, 11, seed=9)
     b = oracle.aprod1(sys, gen.x_true(sys, 3)) + gen.noise(sys, 4)
     ref = oracle.pc_lsqr(sys, b, 12, 0.0, 0.0)
@@ -87,6 +86,25 @@ def test_solve_beside_a_kernel_that_holds_an_sm():
             other.synchronize()
         x2, _, _ = s.lsqr_solve(bd, 12, 0.0, 0.0)  # by the loop again
     assert np.linalg.norm(x2.cpu().numpy() - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
+
+
+def test_blocks_that_are_not_all_resident():
+    # the loop leaves at its first barrier and the solve runs as launches
+    sys = _random(257, 20, 37, 11, seed=9)
+    b = oracle.aprod1(sys, gen.x_true(sys, 3)) + gen.noise(sys, 4)
+    ref = oracle.pc_lsqr(sys, b, 12, 0.0, 0.0)
+    with _solver(sys) as s:
+        assert s.lsqr_one_launch()
+        for where in (2, 2, 0):
+            s.inject_missing_block(where)
+            for host in (False, True):
+                for _ in range(2):
+                    x, se, res = s.lsqr_solve(b if host else torch.tensor(b, device=DEV), 12, 0.0, 0.0)
+                    x, se = (x, se) if host else (x.cpu().numpy(), se.cpu().numpy())
+                    assert res["itn"] == ref["itn"]
+                    assert np.linalg.norm(x - ref["x"]) <= 1e-9 * np.linalg.norm(ref["x"])
+                    np.testing.assert_allclose(se, ref["se"], rtol=1e-9)
+                    assert s.kernel_status() == _lib.GSR_OK
 
 
 def test_two_handles_from_two_threads():

@@ -86,9 +86,9 @@ def test_missing_block_in_the_one_launch_loop():
     ref = oracle.pc_lsqr(sys, b.cpu().numpy(), 12, 0.0, 0.0)["x"]
     with _solver(sys) as s:
         assert s.lsqr_one_launch()
-        s.inject_missing_block(True)
+        s.inject_missing_block(1)
         assert _timeout(lambda: s.lsqr_solve(b, 12, 0.0, 0.0)) < 10.0
-        s.inject_missing_block(False)
+        s.inject_missing_block(0)
         x, _, res = s.lsqr_solve(b, 12, 0.0, 0.0)
         assert res["itn"] == 12 and s.kernel_status() == _lib.GSR_OK
     assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-9 * np.linalg.norm(ref)

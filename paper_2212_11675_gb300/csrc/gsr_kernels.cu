@@ -1335,18 +1335,17 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // Data that other blocks write is read from L2 (ld_shared).  Each wait of the
 // barrier is bounded: when it runs out the block sets *kerr and ends.
 //
-// Beside other work: a block takes three quarters of an SM's registers (96 a
-// thread; with 128, which filled the SM, 0.7 % faster alone), so that it fits
-// beside whatever the staged aprod 1 of the launches (55,296 registers, 220 KB
-// of shared memory) fits beside.  A larger kernel of another stream on any SM
-// keeps the grid from being resident.  A cooperative launch then waits for
+// Beside other work: a block takes 112 registers a thread, which leaves 8,192 of
+// an SM to other kernels (the staged aprod 1 of the launches leaves 10,240 and
+// 7 KB of shared memory); 128 would fill the SM (0.4 % faster alone), 96 were
+// 1 to 2 % slower.  A larger kernel of another stream on any SM keeps the grid
+// from being resident.  A cooperative launch then waits for
 // that kernel to end (with 128 registers, beside a kernel of one block and
 // 1.5 s the solve took 1.45 s; as launches 2.8 ms on the other SMs).  This one
 // is an ordinary launch whose first barrier (loop_join) settles whether all
 // blocks are there: if they are not within kJoinNs, every block ends, the
-// state says so (left) and the host runs the solve as launches.  Up to there
-// only U was written, which a solve starts anew.  After it all blocks are
-// resident, and resident blocks run to their end.
+// state says so (left) and the host runs the solve as launches.  After it all
+// blocks are resident, and resident blocks run to their end.
 //
 // Where it is taken: beyond some size the staged aprod 1, the dynamic unit
 // queue and the wider vector pass of the separate launches win.  us an
@@ -1363,7 +1362,7 @@ k_aprod2_fused(SysView A, const double *__restrict__ y, double *__restrict__ out
 // instruments change nothing.
 // ---------------------------------------------------------------------------
 constexpr int kLoopThreads = 512;
-constexpr int kLoopRegThreads = 640;  // launch bound: 96 registers a thread
+constexpr int kLoopRegThreads = 576;  // launch bound: 112 registers a thread
 constexpr int64_t kLoopSize = 460000;  // rows + 6 columns
 constexpr int64_t kLoopPieces = 16;
 
@@ -1516,8 +1515,9 @@ k_lsqr_loop(SysView A, LoopArgs L)
         s = *L.st;
     __syncthreads();
     double cy = s.cy;
-    if (s.done)
+    if (s.done || !loop_join(L.bar, target, L.st, L.drop_block == 2))
         return;
+    target += L.drop_block == 1;
     for (;;) {
         // 1. rows
         const double *x = L.X.vp;
@@ -1549,7 +1549,7 @@ k_lsqr_loop(SysView A, LoopArgs L)
             }
         }
         loop_part<1>(nrm, gw < ntiles, L.partial);
-        if (!(target == 0 ? loop_join(L.bar, target, L.st, L.drop_block == 2) : loop_sync(L.bar, target, L.kerr)))
+        if (!loop_sync(L.bar, target, L.kerr))
             return;
         if (s.done)  // by the recurrences of the iteration before
             break;
@@ -1559,7 +1559,6 @@ k_lsqr_loop(SysView A, LoopArgs L)
                 t += ld_shared<true>(L.partial + b);
             lsqr_beta_rotation_warp(&s, warp_sum(t));
         }
-        target += L.drop_block == 1;
         // 2. units
         const int64_t natt = A.nseg * A.attp;
         for (int64_t i = gw; i < natt + L.ninstr + L.ngroups; i += nw) {
